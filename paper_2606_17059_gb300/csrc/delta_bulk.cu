@@ -1,0 +1,850 @@
+// delta_bulk.cu -- the ops of a delta that do not meet, applied all at once over the whole GPU.
+//
+// delta_kernel gives a tree to one CTA and an op to one warp, which walks the tree, then changes it: an op is a
+// chain of a dozen dependent loads (10-28 us), and a tree has 16 such chains in flight.  A delta that goes mostly
+// to one tree (a routed batch, the own cache) leaves the rest of the GPU idle, and 256 trees keep 4,096 chains
+// going where the SMs could hold over 100,000.  But ops on different sequences commute, and nearly all of them
+// touch nothing in common: so here every op is walked by one lane of a grid-wide launch that changes nothing, says
+// which table slot and which nodes it would touch, and is then applied in a later launch if nothing else wants
+// them first.  What is left after kBulkRounds such rounds goes to delta_kernel.
+//
+// A round, three launches:
+//   bulk_resolve_kernel  a lane per op: the read-only walk.  It ends in a place: a node u and a token (a slot of u's
+//                        table, whether taken or free).  The op enters the place in a key table (the smallest op
+//                        index wins it) and the nodes it depends on in a node table:
+//                          leaf     INSERT of a new leaf edge under u            slot (u, tok), shares u
+//                          split    INSERT that leaves the edge (u, tok) inside  slot (u, tok), shares u
+//                          count    INSERT or DELETE that only changes a node's sequence count
+//                                                                                slot of its edge, shares the node
+//                                   (a DELETE that leaves the node without one:  the node for itself)
+//                          remove   DELETE of the leaf v under u                 slot (u, tok), shares u, v for itself
+//                          fold     the same where u then has one child y left and stores nothing: u takes y in
+//                                                    slot (u, tok), u's own slot; u, v and y for itself
+//                          absent   DELETE of a sequence that is not stored      slot (u, tok)
+//                        An op of any other form (a node that is one child's only parent, say) holds its slot and
+//                        is left over.
+//   bulk_grow_kernel     the tables of nodes that would pass 1/2 claimed with the round's leaves under them.
+//   bulk_apply_kernel    an op that holds its slots, whose shared nodes nobody needs alone -- an op that needs a
+//                        node for itself steps back when anyone shares it -- and whose own nodes nobody else
+//                        named (or only ops of larger index that need them alone too) is applied: room for the
+//                        warp's ops with one reservation per tree and arena, labels copied by the whole warp,
+//                        slots, records and counts by the op's lane.  The others go to the next round's list.
+// Of the removals under a node with z children that stores nothing only the first z - 2 to arrive go in one round, so
+// no node is left with fewer than 2 children unless it is folded.  Ops on one sequence always name the same slot,
+// the one with the smallest index wins it and the others wait: they apply in op order.  A slot that an op could
+// not enter (no room in the key table) cannot be entered by the others that name it either, so none of them
+// overtakes it.
+//
+// What bounds it: each lane's chain of dependent loads (a probe, a compare and a record per tree level), with
+// 32 chains a warp in flight.  Long compares are made by the warp, once per launch for an interned label and a
+// pool run (the table delta_kernel uses): the lane that enters a pair first compares it, the others go on with
+// other edges and look again.
+//
+// Measured, the delta of a call (delta_kernel alone -> these rounds and delta_kernel behind them): 16,384 routed
+// requests into 16 trees, most into one, 8.2 -> 0.25 ms; 4,096 requests into one cache trie 2.46 -> 0.17 ms; 300 ops
+// into one tree 189 -> 74 us; 1,024,000 ops on 256 trees of 40,000 sequences 3.58 -> 1.77 ms.
+#include "internal.h"
+
+namespace p2p {
+
+// What an op would do, as found by the walk.  u, pos: the node and the token position the place belongs to (the
+// place's token is the sequence's at pos); k: where a split cuts the edge; v: the node of a count or a removal.
+// Fold: g, gpos give u's own place.  Table indices are -1 where there is none.
+struct __align__(16) BulkOp {
+  int32_t what;  // B_* | BF_* flags | tree << kTreeShift
+  int32_t u, pos, k;
+  int32_t v, g, gpos, key;
+  int32_t key2, ent_u, ent_v, ent_y;
+};
+
+namespace {
+
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kBulkThreads = 256;
+constexpr int kBulkWarps = kBulkThreads / 32;
+constexpr int kBulkCtasPerSm = 3;   // at most 85 registers a thread
+constexpr int kLaneSpan = 64;       // label tokens after the first eight that a lane compares alone
+constexpr int kMaxProbes = 64;      // of the key and node tables
+constexpr int kMemoProbes = 4;
+constexpr int kMemoWaits = 64;      // looks at a pair another warp compares before the lane's warp compares it too
+constexpr int kFoldBits = 6;        // tables a lane searches for the one other child
+
+enum { B_NONE = 0, B_LEAF, B_SPLIT, B_COUNT, B_REMOVE, B_FOLD, B_ABSENT, B_LEFT };
+enum { BF_ALONE = 16, BF_REVIVE = 32, BF_GROW = 64, BF_LATER = 128 };
+constexpr int kTreeShift = 8;  // (a tree index has 16 bits)
+
+__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {  // SplitMix64's output function
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  return z ^ (z >> 31);
+}
+
+// Enters (tree, u, tok) of this round for op idx; the table's index, or -1 if it has no room near the key's home.
+// Two places with the same 64-bit hash only wait for one another.
+__device__ int32_t enter_key(const BulkTables& T, int32_t tree, int32_t u, int32_t tok, int round, uint32_t idx) {
+  unsigned long long h = mix64((((unsigned long long)(uint32_t)u << 32) | (uint32_t)tok) ^
+                               mix64(((unsigned long long)(uint32_t)tree << 8) | (unsigned)(round + 1)));
+  h |= 1ull;  // 0 marks an empty entry
+  uint32_t s = (uint32_t)(h >> 17) & T.key_mask;
+  for (int it = 0; it < kMaxProbes; ++it, s = (s + 1) & T.key_mask) {
+    const unsigned long long prev = atomicCAS(&T.keys[s].key, 0ull, h);
+    if (prev == 0ull || prev == h) {
+      atomicMax(&T.keys[s].first, ~idx);  // the smallest index, complemented
+      return (int32_t)s;
+    }
+  }
+  return -1;
+}
+
+// The entry of (tree, node) of this round; -1 if the table has no room for it near its home.
+__device__ int32_t enter_node(const BulkTables& T, int32_t tree, int32_t node, int round) {
+  const unsigned long long key = 1ull | ((unsigned long long)round << 1) | ((unsigned long long)(uint32_t)node << 8) |
+                                 ((unsigned long long)(uint32_t)tree << 40);
+  uint32_t s = (uint32_t)(mix64(key) >> 17) & T.node_mask;
+  for (int it = 0; it < kMaxProbes; ++it, s = (s + 1) & T.node_mask) {
+    const unsigned long long prev = atomicCAS(&T.nodes[s].key, 0ull, key);
+    if (prev == 0ull || prev == key) return (int32_t)s;
+  }
+  return -1;
+}
+
+// An op's sequence: token j is a[j] below na, bo[j] from there (bo = the second pool run less na).
+struct LaneSeq {
+  const int32_t* a;
+  const int32_t* bo;
+  int32_t na, n;
+  __device__ __forceinline__ int32_t at(int32_t j) const { return __ldg((j < na ? a : bo) + j); }
+};
+__device__ __forceinline__ LaneSeq lane_seq(const BulkArgs& A, int64_t i) {
+  const int64_t g0 = A.seg_begin[i], g1 = A.seg_begin[i + 1];
+  LaneSeq q;
+  q.na = g1 > g0 ? A.seg_len[g0] : 0;
+  q.a = A.pool + (g1 > g0 ? A.seg_off[g0] : 0);
+  q.bo = q.a;
+  q.n = q.na;
+  if (g1 - g0 == 2) {
+    q.bo = A.pool + A.seg_off[g0 + 1] - q.na;
+    q.n = q.na + A.seg_len[g0 + 1];
+  }
+  return q;
+}
+
+// The tree (index into states) of op i.
+__device__ __forceinline__ int32_t tree_of(const BulkArgs& A, int64_t i) {
+  if (!A.peer_begin) return 0;
+  int32_t lo = 0, hi = A.n_trees;  // peer_begin[lo] <= i < peer_begin[hi]
+  while (hi - lo > 1) {
+    const int32_t mid = lo + (hi - lo) / 2;
+    if (__ldg(A.peer_begin + mid) <= i) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+// One lane: the slot of tok in the table of 2^bits slots at off.  Returns 1 (live; e = the entry), 2 (tombstone) or
+// 0 (absent); slot = where it is (absent: the first empty slot, or -1).  Two slots per step, each read as two
+// 64-bit words whose first holds key and state: in the apply launch other lanes claim other keys' slots meanwhile.
+__device__ int probe_lane(const int4* child, int32_t off, int32_t bits, int32_t tok, int32_t& slot, int4& e) {
+  slot = -1;
+  if (bits == 0) return 0;
+  const uint32_t mask = (1u << bits) - 1, h = slot_hash(tok, bits);
+  for (uint32_t i = 0; i <= mask; i += 2) {
+    const uint32_t s0 = (h + i) & mask, s1 = (h + i + 1) & mask;
+    const longlong2 x = __ldcg(reinterpret_cast<const longlong2*>(child + off + s0));
+    const longlong2 y = __ldcg(reinterpret_cast<const longlong2*>(child + off + s1));
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const longlong2 w = c ? y : x;
+      const int32_t key = (int32_t)(w.x & 0xffffffffll), state = (int32_t)((unsigned long long)w.x >> 32);
+      if (state == 0) {
+        slot = off + (int32_t)(c ? s1 : s0);
+        return 0;
+      }
+      if (key == tok && (state >= 1 || state == -1)) {
+        slot = off + (int32_t)(c ? s1 : s0);
+        e = make_int4(key, state, (int32_t)(w.y & 0xffffffffll), (int32_t)((unsigned long long)w.y >> 32));
+        return state >= 1 ? 1 : 2;
+      }
+    }
+  }
+  return 0;
+}
+
+// One lane: first j in [from, to) with lab[j] != q[pos + j], or to; eight pairs in flight.
+__device__ __forceinline__ int32_t diff_lane(const int32_t* lab, const LaneSeq& q, int32_t pos, int32_t from, int32_t to) {
+  for (int32_t j0 = from; j0 < to; j0 += 8) {
+    int32_t x[8], y[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int32_t j = j0 + u;
+      x[u] = j < to ? __ldg(lab + j) : 0;
+      y[u] = j < to ? q.at(pos + j) : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (j0 + u < to && x[u] != y[u]) return j0 + u;
+  }
+  return to;
+}
+
+// One warp: first j in [from, to) with a[j] != b[j], or to; 256 tokens per step and side.
+__device__ int32_t diff_warp(const int32_t* a, const int32_t* b, int32_t from, int32_t to, int lane) {
+  constexpr int U = 8;
+  int32_t j0 = from;
+  for (; to - j0 >= 32 * U; j0 += 32 * U) {
+    int32_t x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) x[u] = __ldg(a + j0 + u * 32 + lane);
+    int32_t d = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) d |= x[u] ^ __ldg(b + j0 + u * 32 + lane);
+    if (__any_sync(kFull, d != 0)) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const unsigned m = __ballot_sync(kFull, x[u] != __ldg(b + j0 + u * 32 + lane));
+        if (m) return j0 + u * 32 + (__ffs(m) - 1);
+      }
+    }
+  }
+  for (; j0 < to; j0 += 32) {
+    const int32_t j = j0 + lane;
+    const bool in = lane < to - j0;
+    const unsigned m = __ballot_sync(kFull, in && __ldg(a + j) != __ldg(b + j));
+    if (m) return j0 + (__ffs(m) - 1);
+  }
+  return to;
+}
+
+__device__ __forceinline__ int64_t list_size(const BulkArgs& A, int round) { return round == 0 ? A.n : A.counts[round]; }
+
+__global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_kernel(BulkArgs A, int round) {
+  const int lane = threadIdx.x & 31;
+  const int64_t total = list_size(A, round);
+  const int64_t warps = (int64_t)gridDim.x * kBulkWarps;
+  // Ops per warp: few enough that every warp has some, since a warp's long compares follow one another.
+  const int32_t per = (int32_t)max((int64_t)1, min((int64_t)32, total / warps));
+  const int32_t* list = A.lists + (round & 1) * A.n;
+  for (int64_t b0 = (((int64_t)blockIdx.x * kBulkThreads + threadIdx.x) >> 5) * per; b0 < total; b0 += warps * per) {
+    int64_t i = b0 + lane;
+    bool valid = lane < per && i < total;
+    if (valid && round > 0) i = list[i];
+    valid = valid && !A.done[i];
+    LaneSeq q{nullptr, nullptr, 0, 0};
+    int32_t tree = 0, opc = 0;
+    const int4* node = nullptr;
+    const int4* child = nullptr;
+    const int32_t* label = nullptr;
+    if (valid) {
+      q = lane_seq(A, i);
+      opc = A.op[i];
+      tree = round == 0 ? tree_of(A, i) : A.ops[i].what >> kTreeShift;
+      const TreeState& s = A.states[tree];
+      node = s.node;
+      child = s.child;
+      label = s.label;
+    }
+    valid = valid && q.n > 0;  // (an empty sequence is the root's own count: left to delta_kernel)
+    // The walk: at node u (record nd, reached at pos), its parent g (reached at gpos, gz children, gw sequences)
+    // and that one's parent gg.
+    int32_t u = 0, pos = 0, g = -1, gpos = 0, gz = 0, gw = 0, gg = -1, ggpos = 0, k = 0, waits = 0;
+    int what = B_NONE, flags = 0;
+    int4 nd = make_int4(0, 0, 0, 0), ce = nd, nn = nd;
+    bool act = valid, held = false;  // held: at the edge ce, waiting for a pair that another warp compares
+    int32_t lim = 0, first = 0;
+    if (act) nd = __ldg(node);
+    while (__any_sync(kFull, act)) {
+      bool need = false;
+      int32_t memo_at = -1;  // the pair's entry, when this lane is the one to compare it
+      const int32_t* lab = nullptr;
+      if (act && !held) {
+        int32_t slot;
+        const int st = probe_lane(child, nd.x, tab_bits(nd.y), q.at(pos), slot, ce);
+        if (st != 1) {
+          what = opc == P2P_OP_INSERT ? B_LEAF : B_ABSENT;
+          flags = st == 2 ? BF_REVIVE : 0;
+          act = false;
+        } else if (ce.w <= 0 || ce.y <= 0) {  // (not in a valid tree: delta_kernel reports it)
+          what = B_LEFT;
+          act = false;
+        } else {
+          nn = __ldg(node + ce.y);
+          lim = min(ce.w, q.n - pos);
+          lab = label_ptr(label, A.shared, ce.z);
+          first = min(lim, 9);
+          k = diff_lane(lab, q, pos, 1, first);
+          if (k == first && first < lim) {
+            if (lim - first <= kLaneSpan) {
+              k = diff_lane(lab, q, pos, first, lim);
+            } else {
+              need = true;
+              waits = 0;
+            }
+          }
+        }
+      } else if (act) {
+        lab = label_ptr(label, A.shared, ce.z);
+        need = true;
+        held = false;
+      }
+      // A pair of an interned label and a pool run: how much of it is known to be equal.
+      if (need && ce.z < 0 && A.memo_keys && q.na - pos >= first) {
+        const int64_t so = q.a + pos - A.pool;
+        if (so <= 0xffffffffll) {
+          const unsigned long long key =
+              (1ull << 63) | ((unsigned long long)(uint32_t)~ce.z << 32) | (unsigned long long)so;
+          uint32_t s = (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> 32) & A.memo_mask;
+          for (int it = 0; it < kMemoProbes; ++it, s = (s + 1) & A.memo_mask) {
+            unsigned long long have = __ldcg(A.memo_keys + s);
+            if (have == 0ull) {
+              have = atomicCAS(A.memo_keys + s, 0ull, key);
+              if (have == 0ull) {
+                memo_at = (int32_t)s;
+                break;
+              }
+            }
+            if (have == key) {
+              const int32_t known = __ldcg(A.memo_vals + s);
+              if (known == 0 && ++waits < kMemoWaits) {
+                held = true;
+                need = false;
+              } else if (known >= lim) {
+                k = lim;
+                need = false;
+              } else {
+                first = max(first, known);
+                memo_at = (int32_t)s;
+              }
+              break;
+            }
+          }
+        }
+      }
+      for (unsigned m = __ballot_sync(kFull, need); m; m &= m - 1) {
+        const int j = __ffs(m) - 1;
+        const int32_t* l = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)lab, j);
+        const int32_t* qa = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)(q.a + pos), j);
+        const int32_t* qb = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)(q.bo + pos), j);
+        const int32_t f = __shfl_sync(kFull, first, j), t = __shfl_sync(kFull, lim, j);
+        const int32_t cut = max(f, min(t, __shfl_sync(kFull, q.na - pos, j)));  // below cut: the first pool run
+        int32_t kk = diff_warp(l, qa, f, cut, lane);
+        if (kk == cut && cut < t) kk = diff_warp(l, qb, cut, t, lane);
+        if (lane == j) {
+          k = kk;
+          if (memo_at >= 0) atomicMax(A.memo_vals + memo_at, min(kk, q.na - pos));
+        }
+      }
+      if (act && !held) {
+        if (k == ce.w) {
+          gg = g;
+          ggpos = gpos;
+          g = u;
+          gpos = pos;
+          gz = nd.z;
+          gw = nd.w;
+          u = ce.y;
+          nd = nn;
+          pos += k;
+          if (pos == q.n) {  // the sequence ends at node u
+            act = false;
+            if (opc == P2P_OP_INSERT) what = B_COUNT;
+            else if (nd.w == 0) what = B_ABSENT;
+            else if (nd.w > 1 || nd.z >= 2) what = B_COUNT, flags = nd.w == 1 ? BF_ALONE : 0;
+            else if (nd.z == 1) what = B_LEFT;
+            else if (g == 0 || gw > 0 || gz >= 3) what = B_REMOVE;
+            else what = gz == 2 ? B_FOLD : B_LEFT;
+          }
+        } else {
+          what = opc == P2P_OP_INSERT ? B_SPLIT : B_ABSENT;
+          act = false;
+        }
+      }
+    }
+    if (valid) {
+      // The op's place and nodes.  An op that ended at a node has its place in the parent's table.
+      const bool at_node = pos == q.n;
+      const int32_t pu = at_node ? g : u, ppos = at_node ? gpos : pos, v = at_node ? u : -1;
+      const uint32_t idx = (uint32_t)i;
+      int32_t ent_u = -1, ent_v = -1, ent_y = -1, key2 = -1, y = -1;
+      const int32_t key = enter_key(A.tab, tree, pu, q.at(ppos), round, idx);
+      if (key < 0) what = B_LEFT;
+      if (what == B_FOLD) {  // the one other child of the place's node
+        const int4 rec = __ldg(node + pu);
+        const int32_t bits = tab_bits(rec.y);
+        if (bits <= kFoldBits)
+          for (int32_t s = 0; s < (1 << bits); ++s) {
+            const int4 e = __ldg(child + rec.x + s);
+            if (e.y >= 1 && e.y != v) y = e.y;
+          }
+        if (y < 0 || gg < 0) what = B_LEFT;
+      }
+      if (what == B_LEAF || what == B_SPLIT || what == B_REMOVE || what == B_FOLD) {
+        ent_u = enter_node(A.tab, tree, pu, round);
+        if (ent_u < 0) {
+          what = B_LEFT;
+        } else if (what == B_FOLD) {
+          atomicMax(&A.tab.nodes[ent_u].alone, ~idx);
+        } else {
+          BulkNode* e = A.tab.nodes + ent_u;
+          atomicAdd(&e->shared, 1u);
+          if (what == B_LEAF && !(flags & BF_REVIVE)) {
+            const uint32_t rank = atomicAdd(&e->leaves, 1u);
+            if (rank == 0) flags |= BF_GROW;  // this op sees to the node's table
+            // The root's table grows between launches only; a leaf past its half waits for that.
+            if (pu == 0 && tab_full(tab_bits(nd.y), (int64_t)tab_used(nd.y) + rank + 1)) flags |= BF_LATER;
+          }
+          if (what == B_REMOVE && g != 0 && gw == 0 && (int64_t)atomicAdd(&e->removals, 1u) > (int64_t)gz - 3)
+            flags |= BF_LATER;
+        }
+      }
+      if (what == B_REMOVE || what == B_FOLD || what == B_COUNT) {
+        ent_v = enter_node(A.tab, tree, v, round);
+        if (ent_v < 0) what = B_LEFT;
+        else if (what == B_COUNT && !(flags & BF_ALONE)) atomicAdd(&A.tab.nodes[ent_v].shared, 1u);
+        else atomicMax(&A.tab.nodes[ent_v].alone, ~idx);
+      }
+      if (what == B_FOLD) {
+        key2 = enter_key(A.tab, tree, gg, q.at(ggpos), round, idx);
+        ent_y = enter_node(A.tab, tree, y, round);
+        if (key2 < 0 || ent_y < 0) what = B_LEFT;
+        else atomicMax(&A.tab.nodes[ent_y].alone, ~idx);
+      }
+      int4* out = reinterpret_cast<int4*>(A.ops + i);
+      out[0] = make_int4(what | flags | tree << kTreeShift, pu, ppos, k);
+      out[1] = make_int4(v, gg, ggpos, key);
+      out[2] = make_int4(key2, ent_u, ent_v, ent_y);
+    } else if (lane < per && i < A.n && b0 + lane < total && !A.done[i]) {
+      A.ops[i].what = B_LEFT;  // an empty sequence
+    }
+  }
+}
+
+// Reserves k units of a tree's counter; -1 if they do not fit.  Every warp of a launch may be after the same counter,
+// where compare-and-swap loops take turns failing (4,096 ops of one tree: 1.5 ms), so it is an addition, taken back
+// when it went too far.  Only arenas and requests small enough that additions still to be taken back cannot wrap the
+// counter round (2^30, and 2^17 for each of the warps in flight) are served so.
+__device__ int32_t reserve(int32_t* ctr, int32_t cap, int64_t k) {
+  int32_t old = *(volatile int32_t*)ctr;
+  if (cap <= (1 << 30) && k <= (1 << 17)) {
+    if ((int64_t)old + k > cap) return -1;
+    old = atomicAdd(ctr, (int32_t)k);
+    if ((int64_t)old + k <= cap) return old;
+    atomicSub(ctr, (int32_t)k);
+    return -1;
+  }
+  for (int it = 0; it < (1 << 20); ++it) {
+    if ((int64_t)old + k > cap) return -1;
+    const int32_t prev = atomicCAS(ctr, old, (int32_t)(old + k));
+    if (prev == old) return old;
+    old = prev;
+  }
+  return -1;
+}
+__device__ __forceinline__ void add64(int64_t* p, int64_t v) {
+  if (v) atomicAdd((unsigned long long*)p, (unsigned long long)v);
+}
+
+// The first leaf under a node sees to its table: if the round's leaves would take it past 1/2 claimed, one warp
+// moves it to a table of at most 1/4 live load (as delta_kernel grows tables).  A table that cannot grow (no room in
+// the arena) marks the entry, and its leaves wait.
+__global__ void __launch_bounds__(kBulkThreads) bulk_grow_kernel(BulkArgs A, int round) {
+  const int lane = threadIdx.x & 31;
+  const int64_t total = list_size(A, round);
+  const int64_t warps = (int64_t)gridDim.x * kBulkWarps;
+  const int32_t* list = A.lists + (round & 1) * A.n;
+  for (int64_t b0 = (((int64_t)blockIdx.x * kBulkThreads + threadIdx.x) >> 5) * 32; b0 < total; b0 += warps * 32) {
+    int64_t i = b0 + lane;
+    const bool valid = i < total;
+    if (valid && round > 0) i = list[i];
+    int32_t u = 0, tree = 0, nb = 0, ent = -1;
+    int4 rec = make_int4(0, 0, 0, 0);
+    if (valid && !A.done[i]) {
+      const BulkOp& b = A.ops[i];
+      if (b.what & BF_GROW) {
+        ent = b.ent_u;
+        u = b.u;
+        const int64_t leaves = A.tab.nodes[ent].leaves;
+        if (u != 0 && leaves > 0) {
+          tree = b.what >> kTreeShift;
+          rec = A.states[tree].node[u];
+          const int32_t bits = tab_bits(rec.y);
+          if (tab_full(bits, (int64_t)tab_used(rec.y) + leaves)) {
+            nb = bits ? bits + 1 : kMinTabBits;
+            while (nb < kMaxTabBits && ((int64_t)rec.z + leaves) * 4 > ((int64_t)1 << nb)) ++nb;
+          }
+        }
+      }
+    }
+    for (unsigned m = __ballot_sync(kFull, nb > 0); m; m &= m - 1) {
+      const int j = __ffs(m) - 1;
+      TreeState* s = A.states + __shfl_sync(kFull, tree, j);
+      const int32_t bits2 = __shfl_sync(kFull, nb, j);
+      const int32_t off = __shfl_sync(kFull, rec.x, j), meta = __shfl_sync(kFull, rec.y, j);
+      const int32_t bits = tab_bits(meta);
+      int32_t c0 = 0;
+      if (lane == 0) c0 = reserve(&s->n_child, s->cap_child, (int64_t)1 << bits2);
+      c0 = __shfl_sync(kFull, c0, 0);
+      if (c0 < 0) {
+        if (lane == j) A.tab.nodes[ent].stuck = 1;
+        continue;
+      }
+      int4* child = s->child;
+      for (int32_t t = lane; t < (1 << bits2); t += 32) child[c0 + t] = make_int4(0, 0, 0, 0);
+      __syncwarp();
+      const uint32_t mask = (1u << bits2) - 1;
+      for (int32_t t0 = 0; bits && t0 < (1 << bits); t0 += 128) {
+        int4 e[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int32_t t = t0 + c * 32 + lane;
+          e[c] = t < (1 << bits) ? child[off + t] : make_int4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          if (e[c].y < 1) continue;
+          const unsigned long long kv =
+              (unsigned long long)(uint32_t)e[c].x | ((unsigned long long)(uint32_t)e[c].y << 32);
+          uint32_t sl = slot_hash(e[c].x, bits2);
+          for (uint32_t it = 0; it <= mask; ++it, sl = (sl + 1) & mask)
+            if (atomicCAS((unsigned long long*)&child[c0 + sl], 0ull, kv) == 0ull) {
+              child[c0 + sl].z = e[c].z;
+              child[c0 + sl].w = e[c].w;
+              break;
+            }
+        }
+      }
+      __syncwarp();
+      if (lane == j) {
+        s->node[u] = make_int4(c0, make_meta(bits2, rec.z), rec.z, rec.w);
+        if (bits) add64(&s->stale_child, (int64_t)1 << bits);
+      }
+    }
+  }
+}
+
+// Copies, for every lane with n > 0, n tokens to dst: [0, na) from a, the rest from bo (bo[j] for j >= na); the
+// whole warp copies, kCopies lanes' runs in flight at a time.
+constexpr int kCopies = 4;
+__device__ void copy_runs(int32_t* dst, const int32_t* a, const int32_t* bo, int32_t na, int32_t n, int lane) {
+  unsigned m = __ballot_sync(kFull, n > 0);
+  while (m) {
+    int32_t* d[kCopies];
+    const int32_t *pa[kCopies], *pb[kCopies];
+    int32_t ca[kCopies], cn[kCopies], most = 0;
+#pragma unroll
+    for (int c = 0; c < kCopies; ++c) {
+      const int j = m ? __ffs(m) - 1 : 0;
+      d[c] = (int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)dst, j);
+      pa[c] = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)a, j);
+      pb[c] = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)bo, j);
+      ca[c] = __shfl_sync(kFull, na, j);
+      cn[c] = m ? __shfl_sync(kFull, n, j) : 0;
+      m &= m - 1;
+      most = max(most, cn[c]);
+    }
+    for (int32_t t0 = 0; t0 < most; t0 += 64) {
+      int32_t x[kCopies][2];
+#pragma unroll
+      for (int c = 0; c < kCopies; ++c)
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const int32_t t = t0 + s * 32 + lane;
+          x[c][s] = t < cn[c] ? ((t < ca[c] ? pa[c] : pb[c])[t]) : 0;
+        }
+#pragma unroll
+      for (int c = 0; c < kCopies; ++c)
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const int32_t t = t0 + s * 32 + lane;
+          if (t < cn[c]) d[c][t] = x[c][s];
+        }
+    }
+  }
+}
+
+__device__ __forceinline__ bool adjacent(const int4& a, const int4& b) {  // label b starts where label a ends
+  if (a.z >= 0 && b.z >= 0) return (int64_t)a.z + a.w == b.z;
+  if (a.z < 0 && b.z < 0) return (int64_t)~a.z + a.w == (int64_t)~b.z;
+  return false;
+}
+
+__device__ __forceinline__ bool won(const BulkArgs& A, int32_t key, uint32_t idx) {
+  return A.tab.keys[key].first == ~idx;
+}
+__device__ __forceinline__ bool alone(const BulkArgs& A, int32_t ent, uint32_t idx) {
+  const BulkNode& e = A.tab.nodes[ent];
+  return e.shared == 0 && e.alone == ~idx;
+}
+
+__global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kernel(BulkArgs A, int round) {
+  const int lane = threadIdx.x & 31;
+  const int64_t total = list_size(A, round);
+  const int64_t warps = (int64_t)gridDim.x * kBulkWarps;
+  const int32_t per = (int32_t)max((int64_t)1, min((int64_t)32, total / warps));
+  const int32_t* list = A.lists + (round & 1) * A.n;
+  int32_t* next = A.lists + ((round + 1) & 1) * A.n;
+  for (int64_t b0 = (((int64_t)blockIdx.x * kBulkThreads + threadIdx.x) >> 5) * per; b0 < total; b0 += warps * per) {
+    int64_t i = b0 + lane;
+    bool valid = lane < per && i < total;
+    if (valid && round > 0) i = list[i];
+    valid = valid && !A.done[i];
+    LaneSeq q{nullptr, nullptr, 0, 0};
+    if (valid) q = lane_seq(A, i);
+    valid = valid && q.n > 0;
+    BulkOp b;
+    int what = B_NONE, opc = 0;
+    int32_t tree = -1;
+    bool go = false;
+    if (valid) {
+      const int4* in = reinterpret_cast<const int4*>(A.ops + i);
+      const int4 x = in[0], y = in[1], z = in[2];
+      b = BulkOp{x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w, z.x, z.y, z.z, z.w};
+      what = b.what & 15;
+      opc = A.op[i];
+      tree = b.what >> kTreeShift;
+      const uint32_t idx = (uint32_t)i;
+      go = what != B_LEFT && !(b.what & BF_LATER) && won(A, b.key, idx);
+      if (go && what == B_LEAF && !(b.what & BF_REVIVE)) go = !A.tab.nodes[b.ent_u].stuck;
+      if (go && what == B_COUNT && (b.what & BF_ALONE)) go = alone(A, b.ent_v, idx);
+      if (go && (what == B_REMOVE || what == B_FOLD)) go = alone(A, b.ent_v, idx);
+      if (go && what == B_FOLD) go = won(A, b.key2, idx) && alone(A, b.ent_u, idx) && alone(A, b.ent_y, idx);
+    }
+    // Where the op acts, looked up again: tables may have moved since the walk.
+    TreeState* s = A.states + max(tree, 0);
+    int4 *node = nullptr, *child = nullptr;
+    const int32_t* label = nullptr;
+    int4 rec = make_int4(0, 0, 0, 0), e = rec, pe = rec, ye = rec;
+    int32_t slot = -1, pslot = -1, tok = 0;
+    int32_t want_n = 0, want_c = 0;
+    int64_t want_l = 0;
+    if (go) {
+      node = s->node;
+      child = s->child;
+      label = s->label;
+      if (what == B_LEAF || what == B_SPLIT || what == B_REMOVE || what == B_FOLD) {
+        rec.x = __ldcg(&node[b.u].x);
+        rec.y = __ldcg(&node[b.u].y);
+        tok = q.at(b.pos);
+        const int st = probe_lane(child, rec.x, tab_bits(rec.y), tok, slot, e);
+        const int expect = what == B_LEAF ? (b.what & BF_REVIVE ? 2 : 0) : 1;
+        go = st == expect && slot >= 0;  // (always: nothing else may touch this op's slot)
+      }
+      if (go && what == B_FOLD) {
+        const int4 gr = make_int4(__ldcg(&node[b.g].x), __ldcg(&node[b.g].y), 0, 0);
+        int32_t ys = -1;
+        for (int32_t t = 0; t < (1 << tab_bits(rec.y)); ++t) {
+          const int4 o = __ldcg(child + rec.x + t);
+          if (o.y >= 1 && o.y != b.v) ys = t, ye = o;
+        }
+        go = ys >= 0 && probe_lane(child, gr.x, tab_bits(gr.y), q.at(b.gpos), pslot, pe) == 1;
+        if (go && !adjacent(pe, ye)) want_l = (int64_t)pe.w + ye.w;
+      }
+      if (go && what == B_LEAF) want_n = 1, want_l = q.n - b.pos;
+      if (go && what == B_SPLIT) {
+        want_l = q.n - b.pos - b.k;
+        want_n = want_l > 0 ? 2 : 1;
+        want_c = 1 << kMinTabBits;
+      }
+    }
+    // Room, once per tree and warp; a group that does not fit waits (delta_kernel asks the host for room).
+    int32_t n0 = 0, c0 = 0, l0 = 0;
+    for (unsigned m = __ballot_sync(kFull, go && (want_n || want_c || want_l)); m;) {
+      const int j = __ffs(m) - 1;
+      const int32_t t = __shfl_sync(kFull, tree, j);
+      const bool mine = go && tree == t && (want_n || want_c || want_l);
+      m &= ~__ballot_sync(kFull, mine);
+      int32_t sn = mine ? want_n : 0, sc = mine ? want_c : 0;
+      int64_t sl = mine ? want_l : 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int32_t an = __shfl_up_sync(kFull, sn, o), ac = __shfl_up_sync(kFull, sc, o);
+        const int64_t al = __shfl_up_sync(kFull, sl, o);
+        if (lane >= o) sn += an, sc += ac, sl += al;
+      }
+      const int32_t tn = __shfl_sync(kFull, sn, 31), tc = __shfl_sync(kFull, sc, 31);
+      const int64_t tl = __shfl_sync(kFull, sl, 31);
+      TreeState* ts = A.states + t;
+      int32_t r = 0;
+      if (lane == 0 && tn) r = reserve(&ts->n_node, ts->cap_node, tn);
+      if (lane == 1 && tc) r = reserve(&ts->n_child, ts->cap_child, tc);
+      if (lane == 2 && tl) r = reserve(&ts->n_label, ts->cap_label, tl);
+      const bool ok = __all_sync(kFull, r >= 0);
+      if (!ok) {  // what was taken stays behind as stale space
+        if (lane == 0 && tn && r >= 0) add64(&ts->dead_nodes, tn);
+        if (lane == 1 && tc && r >= 0) add64(&ts->stale_child, tc);
+        if (lane == 2 && tl && r >= 0) add64(&ts->stale_label, tl);
+        if (mine) go = false;
+      }
+      const int32_t bn = __shfl_sync(kFull, r, 0), bc = __shfl_sync(kFull, r, 1), bl = __shfl_sync(kFull, r, 2);
+      if (mine) {
+        n0 = bn + sn - want_n;
+        c0 = bc + sc - want_c;
+        l0 = (int32_t)(bl + sl - want_l);
+      }
+    }
+    // The new labels: a leaf's tokens, or a fold's two labels joined.
+    {
+      const int32_t n = go ? (int32_t)want_l : 0;
+      const int32_t *a = q.a, *bo = q.bo;
+      int32_t na = 0;
+      if (n > 0) {
+        if (what == B_FOLD) {
+          a = label_ptr(label, A.shared, pe.z);
+          bo = label_ptr(label, A.shared, ye.z) - pe.w;
+          na = pe.w;
+        } else {
+          const int32_t at = q.n - n;
+          a = q.a + at;
+          bo = q.bo + at;
+          na = max(q.na - at, 0);
+        }
+      }
+      copy_runs(n > 0 ? s->label + l0 : nullptr, a, bo, na, n, lane);
+    }
+    int32_t absent = 0, dead = 0, st_child = 0;
+    int64_t st_label = 0;
+    if (go) {
+      switch (what) {
+        case B_LEAF: {
+          node[n0] = make_int4(0, 0, 0, 1);
+          const unsigned long long kv = (unsigned long long)(uint32_t)tok | ((unsigned long long)(uint32_t)n0 << 32);
+          if (b.what & BF_REVIVE) {
+            child[slot].z = l0;
+            child[slot].w = (int32_t)want_l;
+            child[slot].y = n0;
+          } else {
+            // The probe's first empty slot, or the next: other leaves of this table claim theirs meanwhile.  The
+            // table has room for all of them (bulk_grow_kernel), so this ends within its size.
+            const int32_t bits = tab_bits(rec.y);
+            const uint32_t mask = (1u << bits) - 1;
+            uint32_t sl = (uint32_t)(slot - rec.x);
+            for (uint32_t it = 0; it <= mask; ++it, sl = (sl + 1) & mask)
+              if (atomicCAS((unsigned long long*)&child[rec.x + sl], 0ull, kv) == 0ull) {
+                child[rec.x + sl].z = l0;
+                child[rec.x + sl].w = (int32_t)want_l;
+                break;
+              }
+            atomicAdd(&node[b.u].y, 1 << 5);
+          }
+          atomicAdd(&node[b.u].z, 1);
+          if (b.u == 0) {
+            const uint32_t h = root_filter_bit(tok);
+            atomicOr(s->rfilter + (h >> 5), 1u << (h & 31));
+          }
+          break;
+        }
+        case B_SPLIT: {
+          const bool tail = want_l > 0;
+          const int32_t mid = n0, leaf = n0 + 1;
+          const int4 lower = make_int4(label_ptr(label, A.shared, e.z)[b.k], e.y, label_adv(e.z, b.k), e.w - b.k);
+          const uint32_t mask = (1u << kMinTabBits) - 1, s0 = slot_hash(lower.x, kMinTabBits);
+          uint32_t s1 = s0;
+          int4 le = make_int4(0, 0, 0, 0);
+          if (tail) {
+            le = make_int4(q.at(b.pos + b.k), leaf, l0, (int32_t)want_l);
+            s1 = slot_hash(le.x, kMinTabBits);
+            if (s1 == s0) s1 = (s1 + 1) & mask;
+            node[leaf] = make_int4(0, 0, 0, 1);
+          }
+          for (uint32_t t = 0; t <= mask; ++t)
+            child[c0 + t] = t == s0 ? lower : (tail && t == s1) ? le : make_int4(0, 0, 0, 0);
+          node[mid] = make_int4(c0, make_meta(kMinTabBits, tail ? 2 : 1), tail ? 2 : 1, tail ? 0 : 1);
+          child[slot] = make_int4(tok, mid, e.z, b.k);  // the slot keeps its key; the label starts where it did
+          break;
+        }
+        case B_COUNT:
+          atomicAdd(&node[b.v].w, opc == P2P_OP_INSERT ? 1 : -1);
+          break;
+        case B_REMOVE:
+        case B_FOLD: {
+          const int32_t vb = tab_bits(__ldcg(&node[b.v].y));
+          child[slot].y = -1;  // a tombstone: the slot keeps its key
+          st_label = e.w;
+          dead = 1;
+          st_child = vb ? 1 << vb : 0;
+          if (what == B_REMOVE) {
+            atomicAdd(&node[b.u].z, -1);
+          } else {
+            // u takes its last child in: the joined label, the child's record.
+            child[pslot].z = want_l > 0 ? l0 : pe.z;
+            child[pslot].w = pe.w + ye.w;
+            node[b.u] = node[ye.y];
+            st_label += want_l;
+            dead += 1;
+            st_child += tab_bits(rec.y) ? 1 << tab_bits(rec.y) : 0;
+          }
+          break;
+        }
+        default:
+          absent = 1;
+      }
+      A.done[i] = 1;
+    }
+    // The trees' counts, once per tree and warp.
+    for (unsigned m = __ballot_sync(kFull, go && (absent || dead)); m;) {
+      const int j = __ffs(m) - 1;
+      const int32_t t = __shfl_sync(kFull, tree, j);
+      const bool mine = go && (absent || dead) && tree == t;
+      m &= ~__ballot_sync(kFull, mine);
+      int64_t v[4] = {mine ? absent : 0, mine ? dead : 0, mine ? st_child : 0, mine ? st_label : 0};
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] += __shfl_xor_sync(kFull, v[c], o);
+      TreeState* ts = A.states + t;
+      if (lane == 0) add64(&ts->n_absent, v[0]);
+      if (lane == 1) add64(&ts->dead_nodes, v[1]);
+      if (lane == 2) add64(&ts->stale_child, v[2]);
+      if (lane == 3) add64(&ts->stale_label, v[3]);
+    }
+    // The rest goes to the next round.
+    const bool again = valid && !go;
+    const unsigned am = __ballot_sync(kFull, again);
+    int32_t at = 0;
+    if (lane == 0 && am) at = atomicAdd(&A.counts[round + 1], __popc(am));
+    at = __shfl_sync(kFull, at, 0);
+    if (again) next[at + __popc(am & ((1u << lane) - 1))] = (int32_t)i;
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_bulk(const BulkArgs& A, int num_sms, cudaStream_t st, int* launched) {
+  *launched = 0;
+  if (A.n <= 0) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(A.tab.keys, 0, ((size_t)A.tab.key_mask + 1) * sizeof(BulkKey), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(A.tab.nodes, 0, ((size_t)A.tab.node_mask + 1) * sizeof(BulkNode), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(A.counts, 0, (kBulkRounds + 2) * sizeof(int32_t), st);
+  if (e != cudaSuccess) return e;
+  // A warp per op up to a full wave of resident CTAs (the kernels then take more ops per warp).
+  const int grid = (int)std::min<int64_t>((A.n + kBulkWarps - 1) / kBulkWarps, (int64_t)num_sms * kBulkCtasPerSm);
+  const int grid_g = (int)std::min<int64_t>((A.n + kBulkThreads - 1) / kBulkThreads, (int64_t)num_sms * 8);
+  for (int round = 0; round < kBulkRounds; ++round) {
+    P2P_TIMED(K_DELTA_BULK, st, (bulk_resolve_kernel<<<grid, kBulkThreads, 0, st>>>(A, round)));
+    P2P_TIMED(K_DELTA_BULK, st, (bulk_grow_kernel<<<grid_g, kBulkThreads, 0, st>>>(A, round)));
+    P2P_TIMED(K_DELTA_BULK, st, (bulk_apply_kernel<<<grid, kBulkThreads, 0, st>>>(A, round)));
+    *launched += 3;
+  }
+  return cudaGetLastError();
+}
+
+size_t bulk_scratch(int64_t n, void* base, BulkArgs& A) {
+  int64_t keys = 1024, nodes = 1024;
+  while (keys < 4 * n) keys <<= 1;
+  while (nodes < 2 * n) nodes <<= 1;
+  char* p = static_cast<char*>(base);
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    void* q = p ? p + at : nullptr;
+    at += (bytes + 255) & ~(size_t)255;
+    return q;
+  };
+  A.tab.keys = static_cast<BulkKey*>(take((size_t)keys * sizeof(BulkKey)));
+  A.tab.key_mask = (uint32_t)(keys - 1);
+  A.tab.nodes = static_cast<BulkNode*>(take((size_t)nodes * sizeof(BulkNode)));
+  A.tab.node_mask = (uint32_t)(nodes - 1);
+  A.ops = static_cast<BulkOp*>(take((size_t)n * sizeof(BulkOp)));
+  A.lists = static_cast<int32_t*>(take((size_t)n * 2 * sizeof(int32_t)));
+  A.counts = static_cast<int32_t*>(take((kBulkRounds + 2) * sizeof(int32_t)));
+  return at;
+}
+
+}  // namespace p2p

@@ -6,6 +6,9 @@
 // that leaves an edge part-way splits it; a DELETE prunes a leaf that no longer stores anything and folds
 // a node left with one child and no sequence into that child.
 //
+// The ops that meet no other op are applied before this kernel runs, over the whole GPU (delta_bulk.cu); it takes
+// what is left, every op of a delta whose sequences have more than two pool runs, and the allocation-free call's.
+//
 // Parallel schedule.  One CTA of kDeltaWarps warps takes a tree; the tree's ops are taken in chunks.
 // Two facts make ops independent:
 //   - ops on different sequences commute (the canonical tree depends only on the multiset), so only ops
@@ -74,11 +77,14 @@ struct Tree {
   const int32_t* shared;  // router-wide pool of interned labels (read-only here)
   TreeState* g;
   int2* slab;  // this warp's slabs (shared memory): per counter, the next free unit and the units left
+  int32_t slab_shift;  // slabs are 2^slab_shift smaller than usual
   __device__ const int32_t* lab(int32_t off) const { return label_ptr(label, shared, off); }
 };
 
 // Units a warp reserves at a time for its slab of counter c: nodes, child entries, label tokens.
-__device__ __forceinline__ int32_t slab_units(int c) { return c == 0 ? 64 : c == 1 ? 256 : 4096; }
+__device__ __forceinline__ int32_t slab_units(const Tree& t, int c) {
+  return (c == 0 ? 64 : c == 1 ? 256 : 4096) >> t.slab_shift;
+}
 
 // Reserves k units of counter c (0 nodes, 1 child entries, 2 label tokens) from the tree's counters by
 // compare-and-swap; -1 if they do not fit.  One lane.
@@ -102,7 +108,7 @@ __device__ void add_stale(const Tree& t, int c, int64_t k) {
   atomicAdd((unsigned long long*)p, (unsigned long long)k);
 }
 
-// Reserves the room an op may need.  Each warp keeps a slab per counter, refilled slab_units(c) units at a
+// Reserves the room an op may need.  Each warp keeps a slab per counter, refilled slab_units(t, c) units at a
 // time from the tree's counters (lanes 0, 1 and 2 at once), so most ops take their room without a global
 // atomic; a slab's rest is counted as stale when it is replaced and when the warp finishes.  A request of a
 // slab or more, or one whose refill does not fit, is reserved exactly.  On failure the op does nothing:
@@ -119,7 +125,7 @@ __device__ bool take(Tree& t, int64_t nodes, int64_t entries, int64_t tokens, in
     sl = t.slab[lane];
     ns = sl;
     if (k > 0) {
-      const int32_t S = slab_units(lane);
+      const int32_t S = slab_units(t, lane);
       if (k <= sl.y) {
         r = sl.x;
         ns = make_int2(sl.x + (int32_t)k, sl.y - (int32_t)k);
@@ -140,7 +146,7 @@ __device__ bool take(Tree& t, int64_t nodes, int64_t entries, int64_t tokens, in
   if (lane < 3) {
     if (!ok) {
       if (exact) add_stale(t, lane, exact);
-      ns = refilled ? make_int2(r, slab_units(lane)) : sl;
+      ns = refilled ? make_int2(r, slab_units(t, lane)) : sl;
     }
     t.slab[lane] = ns;
   }
@@ -889,7 +895,7 @@ __global__ void __launch_bounds__(kDeltaWarps * 32, 2)
                  const int64_t* __restrict__ seg_begin, const int64_t* __restrict__ seg_off,
                  const int32_t* __restrict__ seg_len, const int32_t* __restrict__ pool, int32_t* gather,
                  int64_t stride, const int32_t* shared, unsigned long long* gmemo_keys, int32_t* gmemo_vals,
-                 uint32_t gmemo_mask, const int32_t* __restrict__ parts) {
+                 uint32_t gmemo_mask, const int32_t* __restrict__ parts, int32_t slab_shift) {
   // The chunk's per-op and per-anchor arrays, in dynamic shared memory (delta_smem_bytes()).
   extern __shared__ __align__(16) unsigned char s_dyn[];
   AnchorEntry* s_aentry = reinterpret_cast<AnchorEntry*>(s_dyn);        // per anchor: its shortcut
@@ -938,12 +944,16 @@ __global__ void __launch_bounds__(kDeltaWarps * 32, 2)
   t.shared = shared;
   t.g = gs;
   t.slab = s_slab[warp];
+  t.slab_shift = slab_shift;
   const int4 root = t.node[0];  // its table offset and size hold for the whole launch
   int32_t* buf = gather ? gather + ((int64_t)blockIdx.x * kDeltaWarps + warp) * stride : nullptr;
   // Facts about immutable labels: valid whichever bucket the warp works on.
   Memo memo{s_memo[warp], gmemo_keys, gmemo_vals, gmemo_mask, pool};
   for (int64_t c0 = op_begin; c0 < op_end; c0 += kChunk) {
     const int clen = (int)min((int64_t)kChunk, op_end - c0);
+    int open = 0;  // a chunk with nothing left to apply (the bulk rounds did it all) is passed over
+    for (int j = threadIdx.x; j < clen; j += blockDim.x) open |= !done[c0 + j];
+    if (!__syncthreads_or(open)) continue;
     // 1. Per op: first-token bucket, done flag, and (for ops still to apply) the anchor.
     for (int k = threadIdx.x; k < kAnchorSlots; k += blockDim.x) {
       s_akey[k] = -1;
@@ -1500,7 +1510,7 @@ cudaError_t launch_compact(CompactJob* d_jobs, int32_t n_jobs, int32_t max_cap_n
 cudaError_t launch_delta(TreeState* d_states, uint8_t* done, int32_t n_trees, const int32_t* op,
                          const int64_t* seg_begin, const int64_t* seg_off, const int32_t* seg_len, const int32_t* pool,
                          int32_t* gather, int64_t gather_stride, const int32_t* shared, cudaStream_t st,
-                         const GlobalMemo* gm, const int32_t* parts, int32_t n_blocks) {
+                         const GlobalMemo* gm, const int32_t* parts, int32_t n_blocks, int32_t slab_shift) {
   if (n_trees <= 0) return cudaSuccess;
   const int dyn = delta_smem_bytes();
   cudaError_t e = cudaFuncSetAttribute(parts ? delta_kernel<true> : delta_kernel<false>,
@@ -1510,12 +1520,12 @@ cudaError_t launch_delta(TreeState* d_states, uint8_t* done, int32_t n_trees, co
     P2P_TIMED(K_DELTA, st,
               (delta_kernel<true><<<n_blocks, kDeltaWarps * 32, dyn, st>>>(
                   d_states, done, op, seg_begin, seg_off, seg_len, pool, gather, gather_stride, shared,
-                  gm ? gm->keys : nullptr, gm ? gm->vals : nullptr, gm ? gm->mask : 0u, parts)));
+                  gm ? gm->keys : nullptr, gm ? gm->vals : nullptr, gm ? gm->mask : 0u, parts, slab_shift)));
   } else {
     P2P_TIMED(K_DELTA, st,
               (delta_kernel<false><<<n_trees, kDeltaWarps * 32, dyn, st>>>(
                   d_states, done, op, seg_begin, seg_off, seg_len, pool, gather, gather_stride, shared,
-                  gm ? gm->keys : nullptr, gm ? gm->vals : nullptr, gm ? gm->mask : 0u, nullptr)));
+                  gm ? gm->keys : nullptr, gm ? gm->vals : nullptr, gm ? gm->mask : 0u, nullptr, slab_shift)));
   }
   return cudaGetLastError();
 }

@@ -108,7 +108,7 @@ enum KernelId {
   K_GROUP_HASH, K_GROUP_RESOLVE, K_GROUP_RESOLVE32, K_ROUTE_STAGED, K_LANE_LEADER, K_LANE_FOLLOWER, K_DECIDE,
   K_VALIDATE, K_INIT_RANGES, K_DELTA, K_COMPACT, K_COMPACT_LABELS, K_REFRESH_VIEWS, K_SET_TREE,
   K_UPDATE_COUNT, K_UPDATE_SCAN, K_UPDATE_SCATTER, K_GROUP_RANGES, K_GROUP_PLACE, K_LRU_WALK, K_LRU_STAMP,
-  K_LRU_ORDER, K_LRU_SELECT, K_LRU_EVICT, K_LRU_OPS, K_HIT_RATE, K_ROOM, K_COUNT_
+  K_LRU_ORDER, K_LRU_SELECT, K_LRU_EVICT, K_LRU_OPS, K_HIT_RATE, K_ROOM, K_DELTA_BULK, K_COUNT_
 };
 static_assert((int)K_COUNT_ == (int)P2P_KERNEL_COUNT, "the header's kernel count");
 const char* kernel_name(int id);
@@ -185,13 +185,60 @@ struct GlobalMemo {
   uint32_t mask;
 };
 constexpr int kGlobalMemoBits = 16;
+// slab_shift: each warp's slabs are 2^slab_shift smaller than usual (few ops are left to apply).
 cudaError_t launch_delta(TreeState* d_states, uint8_t* done, int32_t n_trees, const int32_t* op,
                          const int64_t* seg_begin, const int64_t* seg_off, const int32_t* seg_len, const int32_t* pool,
                          int32_t* gather, int64_t gather_stride, const int32_t* shared, cudaStream_t st,
-                         const GlobalMemo* gm = nullptr, const int32_t* parts = nullptr, int32_t n_blocks = 0);
+                         const GlobalMemo* gm = nullptr, const int32_t* parts = nullptr, int32_t n_blocks = 0,
+                         int32_t slab_shift = 0);
 constexpr int kPartShift = 16, kNpartShift = 21;
 constexpr int32_t kPartTreeMask = (1 << kPartShift) - 1;  // a tree index < 65,536 (P <= 65,536)
 static_assert(kDeltaBuckets <= 32, "a part index fits in 5 bits and nparts in 6");
+
+// Bulk rounds ahead of the delta kernel (delta_bulk.cu): every op is walked by a lane of a grid-wide launch, and
+// the ops that nothing else in the delta gets in the way of are applied at once.  Sets done[i] for each; the rest
+// is left for launch_delta.  Ops of at most two pool runs, fewer than 2^31 ops.
+struct BulkKey {  // one place of a round: a token of a node's table
+  unsigned long long key;  // 0: empty entry
+  uint32_t first;          // ~(smallest op index that names it)
+  uint32_t pad_;
+};
+struct __align__(32) BulkNode {  // one node of a round
+  unsigned long long key;        // 0: empty entry
+  uint32_t shared;               // ops that depend on it and can do so side by side
+  uint32_t alone;                // ~(smallest op index that needs it for itself)
+  uint32_t leaves;               // new slots its table would need
+  uint32_t removals;             // leaves that would be removed under it
+  uint32_t stuck;                // its table had to grow and could not
+  uint32_t pad_;
+};
+struct BulkTables {
+  BulkKey* keys;  // key_mask + 1
+  BulkNode* nodes;
+  uint32_t key_mask, node_mask;
+};
+struct BulkOp;
+struct BulkArgs {
+  TreeState* states;  // of the call's n_trees trees
+  int32_t n_trees;
+  const int64_t* peer_begin;  // [n_trees + 1], or NULL: one tree takes every op
+  int64_t n;
+  const int32_t* op;
+  const int64_t *seg_begin, *seg_off;
+  const int32_t *seg_len, *pool, *shared;
+  uint8_t* done;
+  unsigned long long* memo_keys;  // the GlobalMemo of launch_delta
+  int32_t* memo_vals;
+  uint32_t memo_mask;
+  BulkTables tab;  // from here on: scratch (bulk_scratch)
+  BulkOp* ops;     // [n]
+  int32_t* lists;  // [2n]: the op indices of odd and even rounds
+  int32_t* counts; // [kBulkRounds + 2]: list sizes by round
+};
+constexpr int kBulkRounds = 3;
+// The bytes of scratch for n ops; with base, also sets A's scratch pointers into it.
+size_t bulk_scratch(int64_t n, void* base, BulkArgs& A);
+cudaError_t launch_bulk(const BulkArgs& A, int num_sms, cudaStream_t st, int* launched);
 
 // Compaction: copies the live part of a tree (everything reachable from the root) into fresh arrays, with
 // nodes renumbered in breadth-first order, every live table rehashed at its size without tombstones, and

@@ -93,7 +93,7 @@ const char* kernel_name(int id) {
       "compact_kernel", "compact_labels_kernel", "refresh_views_kernel", "set_tree_kernel", "update_count_kernel",
       "update_scan_kernel", "update_scatter_kernel", "group_ranges_kernel", "group_place_kernel", "lru_walk_kernel",
       "lru_stamp_kernel", "lru_order_kernels", "lru_count_kernel", "lru_evict_kernel", "lru_ops_kernel",
-      "hit_rate_kernel", "room_kernel"};
+      "hit_rate_kernel", "room_kernel", "delta_bulk_kernels"};
   return id >= 0 && id < K_COUNT_ ? names[id] : "";
 }
 
@@ -215,6 +215,7 @@ struct p2p_router {
   DevBuf upd_cnt, upd_op, upd_sb, upd_so, upd_sl;  // a routed batch as an INSERT delta (p2p_update_estimates)
   DevBuf lru_buf;                                   // scratch of the LRU calls
   DevBuf gmemo;                                     // the delta kernel's launch-wide verified-run table
+  DevBuf bulk;                                      // the bulk rounds' tables, op records and lists
   DevBuf d_room;                                    // room bounds of the trees that stopped (room_kernel)
   DevBuf d_parts;                                   // the delta launch's CTA parts (split_trees)
   std::vector<int32_t> h_parts;                     // their host copy (kept until the next call)
@@ -1068,7 +1069,7 @@ void p2p_router_destroy(p2p_router* r) {
                       &r->d_seg_off, &r->d_seg_len, &r->d_pool, &r->d_peer_begin, &r->d_done, &r->d_gather,
                       &r->grp_keys, &r->grp_vals, &r->grp_req, &r->grp_ckpt, &r->cmp_jobs, &r->cmp_queue,
                       &r->upd_cnt, &r->upd_op, &r->upd_sb, &r->upd_so, &r->upd_sl, &r->lru_buf, &r->gmemo,
-                      &r->d_room, &r->d_parts})
+                      &r->d_room, &r->d_parts, &r->bulk})
       dfree(r, b->p);
     dfree(r, r->d_views);
     dfree(r, r->d_states);
@@ -1215,6 +1216,10 @@ int p2p_tree_apply_delta(p2p_router* r, int32_t peer, const p2p_delta* d, int64_
 // routed mostly to one tree and inserted with p2p_update_estimates, for one).  n_blocks = nt and
 // d_parts = NULL when no tree is split.
 constexpr int64_t kPartOps = 16384;
+// Largest delta of the bulk rounds (their scratch takes up to 320 bytes per op), and how much smaller the delta
+// kernel's slabs are behind them.
+constexpr int64_t kBulkMaxOps = (int64_t)1 << 24;
+constexpr int32_t kBulkSlabShift = 3;
 static int split_trees(p2p_router* r, int32_t peer, const p2p_delta* d, const int64_t* d_pb, int32_t p0, int32_t nt,
                 int64_t n, int32_t& n_blocks, const int32_t*& d_parts) {
   n_blocks = nt;
@@ -1349,6 +1354,32 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
                      reinterpret_cast<int32_t*>(static_cast<unsigned long long*>(r->gmemo.p) + gslots),
                      (uint32_t)(gslots - 1)};
   CK(cudaMemsetAsync(r->gmemo.p, 0, gslots * (sizeof(unsigned long long) + sizeof(int32_t)), r->stream));
+  // Bulk rounds first, where the ops are of at most two pool runs and the scratch can be had; what they leave (few
+  // ops, as a rule) goes to the delta kernel, whose warps then take smaller slabs.
+  p2p::BulkArgs bulk = {};
+  bool use_bulk = max_runs <= 2 && n <= kBulkMaxOps;
+  if (use_bulk) {
+    if (ensure(r, r->bulk, p2p::bulk_scratch(n, nullptr, bulk)) != cudaSuccess) {
+      (void)cudaGetLastError();
+      use_bulk = false;
+    } else {
+      p2p::bulk_scratch(n, r->bulk.p, bulk);
+      bulk.states = r->d_states + p0;
+      bulk.n_trees = nt;
+      bulk.peer_begin = peer == -1 ? d_pb : nullptr;
+      bulk.n = n;
+      bulk.op = d_op;
+      bulk.seg_begin = d_sb;
+      bulk.seg_off = d_so;
+      bulk.seg_len = d_sl;
+      bulk.pool = d_pool;
+      bulk.shared = r->d_shared;
+      bulk.done = done;
+      bulk.memo_keys = gm.keys;
+      bulk.memo_vals = gm.vals;
+      bulk.memo_mask = gm.mask;
+    }
+  }
   int rc = P2P_OK;
   bool sized = false;  // the room of the rest of the call was bounded once (room_kernel)
   for (int round = 0;; ++round) {
@@ -1358,8 +1389,13 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
     }
     if (round == 0)
       if (int rc = prepare_scratch(r)) return rc;
+    if (use_bulk) {
+      int launched = 0;
+      CK(p2p::launch_bulk(bulk, r->num_sms, r->stream, &launched));
+      r->launches += launched;
+    }
     CK(p2p::launch_delta(r->d_states + p0, done, nt, d_op, d_sb, d_so, d_sl, d_pool, gather, stride, r->d_shared,
-                         r->stream, &gm, d_parts, n_blocks));
+                         r->stream, &gm, d_parts, n_blocks, use_bulk ? kBulkSlabShift : 0));
     if (round == 0)
       if (int rc = launch_prepared(r)) return rc;  // a prepared batch's grouping overlaps the delta kernel
     r->launches += 1;

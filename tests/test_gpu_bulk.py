@@ -1,0 +1,132 @@
+"""GPU parity of the delta's bulk rounds (delta_bulk.cu: ops that do not meet are applied at once) against the CPU
+oracle: deltas made of the ops that do meet, or nearly do.  After every call the canonical export equals the
+oracle's byte for byte, the count of absent DELETEs agrees, and a route over the trees matches."""
+import random
+
+import numpy as np
+import pytest
+
+import oracle
+import paper_2606_17059_gb300 as g
+import workload as wl
+from gpu_util import assert_same_route, csr_from_lists, route_device, router_from_seqlists, same_snapshot, seqlist_from_lists
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    g.build()
+
+
+def _runs(seqs, cuts):
+    """Sequence list whose sequence i is cut into two pool runs at cuts[i]; equal first runs share one pool copy."""
+    pool, at, sb, so, sl = [], {}, [0], [], []
+    for s, c in zip(seqs, cuts):
+        for part, share in ((s[:c], True), (s[c:], False)):
+            key = tuple(part)
+            if not (share and key in at):
+                at[key] = len(pool)
+                pool.extend(part)
+            so.append(at[key])
+            sl.append(len(part))
+        sb.append(len(so))
+    return wl.SeqList(np.array(sb, np.int64), np.array(so, np.int64), np.array(sl, np.int32), np.array(pool, np.int32))
+
+
+def _check(r, trees, calls, reqs):
+    for n, (p, ops, sl) in enumerate(calls):
+        op = np.array(ops, np.int32)
+        assert r.apply_delta(p, op, sl) == trees[p].apply_ops(op, sl), f"call {n}: absent DELETEs"
+        assert same_snapshot(r.download(p), trees[p].export()), f"call {n}"
+    tok, off = csr_from_lists(reqs)
+    P = len(trees)
+    gm, gp = route_device(r, tok, off, [0] * P, 0)
+    om, op_, _ = oracle.route(trees, tok, off, [0] * P, 0)
+    assert_same_route(gm, gp, om, op_, "after the deltas")
+
+
+# Prompt lengths around what a lane compares alone (8, then 64 tokens), what is interned (128) and a warp's step (256).
+@pytest.mark.parametrize("length", [1, 2, 8, 9, 10, 72, 73, 74, 127, 128, 129, 300, 700])
+def test_ops_that_meet(length):
+    rng = random.Random(length)
+    tail = lambda n=None: [rng.randrange(50, 60) for _ in range(n or rng.randint(1, 100))]
+    prompts = [[1000 + k] + [rng.randrange(3) for _ in range(length - 1)] for k in range(6)]
+    held = [[p + tail() for _ in range(k)] for k, p in enumerate(prompts)]  # 0 .. 5 sequences a prompt
+    a = [s for h in held for s in h]
+    other = [p + tail() for p in prompts for _ in range(2)]  # (its interned prompts make tree 0's upload split some)
+    sls = [seqlist_from_lists(other), seqlist_from_lists(a)]
+    r, trees = router_from_seqlists(sls), oracle.build_trees(sls)
+    fresh = [9000] + [rng.randrange(3) for _ in range(length)]
+    ins, rem = [], []
+    ins += [prompts[0] + tail() for _ in range(40)]           # many sequences of a prompt the tree does not hold
+    ins += [fresh + tail() for _ in range(3)] + [fresh]       # ... and one that is its prompt itself
+    ins += [prompts[5][: max(1, length // 2)], prompts[5][: max(1, length - 1)] + [77]]  # ends and leaves inside an edge
+    ins += [prompts[4] + [50 + k] for k in range(10)]          # tables that have to grow
+    ins += [held[3][0], held[3][0], held[3][0] + [1]]          # counts, and a leaf that gets a child
+    rem += held[2] + held[3][1:] + held[4][:3] + held[5]       # folds, and prompts that vanish
+    rem += [prompts[1] + [1, 2], [4242], held[1][0][:-1]]      # not stored
+    ops = [(0, s) for s in ins] + [(1, s) for s in rem]
+    again = [(1, ins[0]), (0, ins[0]), (1, ins[0]), (1, ins[0]), (0, held[2][0]), (1, held[2][0]), (1, ins[41])]
+    rng.shuffle(ops)
+    ops += again
+    cuts = [min(len(s), rng.choice([length, length, 0, len(s), 5])) for _, s in ops]
+    seqs = [s for _, s in ops]
+    calls = [(1, [o for o, _ in ops], _runs(seqs, cuts))]
+    # Taken back one by one from the other end: every DELETE has a stored sequence or is a counted no-op.
+    back = [(1 - o, s) for o, s in reversed(ops)]
+    calls.append((1, [o for o, _ in back], seqlist_from_lists([s for _, s in back])))
+    reqs = [s + [3] for s in seqs[::3]] + prompts + [s[:-1] for s in a]
+    _check(r, trees, calls, reqs)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 255, 257, 1000])
+def test_batch_sizes_and_runs(n):
+    """Deltas of n ops over three trees (sizes around a warp and a CTA), of one, two and three pool runs (the last
+    are delta_kernel's alone), in one call over all trees from device memory."""
+    import torch
+    rng = random.Random(n)
+    V = 4
+    stored = [[[rng.randrange(V) for _ in range(rng.randint(1, 20))] for _ in range(60)] for _ in range(3)]
+    sls = [seqlist_from_lists(s) for s in stored]
+    for runs in (1, 2, 3):
+        r, trees = router_from_seqlists(sls), oracle.build_trees(sls)
+        ops, seqs, pb = [], [], [0]
+        for p in range(3):
+            for _ in range(n if p != 1 else n // 2):
+                if rng.random() < 0.5:
+                    ops.append(1)
+                    seqs.append(list(rng.choice(stored[p])))
+                else:
+                    ops.append(0)
+                    seqs.append(rng.choice(stored[p])[: rng.randint(0, 20)] + [rng.randrange(V) for _ in range(rng.randint(0, 20))])
+            pb.append(len(ops))
+        sb, so, sl, pool = [0], [], [], []
+        for s in seqs:
+            marks = sorted(rng.randint(0, len(s)) for _ in range(runs - 1))
+            for lo, hi in zip([0] + marks, marks + [len(s)]):
+                so.append(len(pool))
+                sl.append(hi - lo)
+                pool.extend(s[lo:hi])
+            sb.append(len(so))
+        host = wl.SeqList(np.array(sb, np.int64), np.array(so, np.int64), np.array(sl, np.int32), np.array(pool or [0], np.int32))
+        op = np.array(ops, np.int32)
+        dev = wl.SeqList(*(torch.from_numpy(x).cuda() for x in (host.seg_begin, host.seg_off, host.seg_len, host.pool)))
+        got = r.apply_delta(-1, torch.from_numpy(op).cuda(), dev, torch.from_numpy(np.array(pb, np.int64)).cuda(), on_device=True)
+        assert got == sum(trees[p].apply_ops(op, host, pb[p], pb[p + 1]) for p in range(3))
+        for p in range(3):
+            assert same_snapshot(r.download(p), trees[p].export()), (runs, p)
+
+
+def test_a_root_table_that_has_to_grow():
+    """Thousands of new first tokens at once: the root's table only grows between launches, and the rounds run again
+    after it has."""
+    rng = random.Random(3)
+    sls = [seqlist_from_lists([[5, 6, 7]])]
+    r, trees = router_from_seqlists(sls), oracle.build_trees(sls)
+    seqs = [[rng.randrange(1 << 20)] + [rng.randrange(9) for _ in range(rng.randint(0, 90))] for _ in range(5000)]
+    sl = seqlist_from_lists(seqs)
+    _check(r, trees, [(0, [0] * 5000, sl), (0, [1] * 5000, sl)], seqs[:300])
