@@ -818,9 +818,9 @@ cudaError_t launch_bulk(const BulkArgs& A, int num_sms, cudaStream_t st, int* la
   const int grid = (int)std::min<int64_t>((A.n + kBulkWarps - 1) / kBulkWarps, (int64_t)num_sms * kBulkCtasPerSm);
   const int grid_g = (int)std::min<int64_t>((A.n + kBulkThreads - 1) / kBulkThreads, (int64_t)num_sms * 8);
   for (int round = 0; round < kBulkRounds; ++round) {
-    P2P_TIMED(K_DELTA_BULK, st, (bulk_resolve_kernel<<<grid, kBulkThreads, 0, st>>>(A, round)));
-    P2P_TIMED(K_DELTA_BULK, st, (bulk_grow_kernel<<<grid_g, kBulkThreads, 0, st>>>(A, round)));
-    P2P_TIMED(K_DELTA_BULK, st, (bulk_apply_kernel<<<grid, kBulkThreads, 0, st>>>(A, round)));
+    P2P_TIMED(K_BULK_RESOLVE, st, (bulk_resolve_kernel<<<grid, kBulkThreads, 0, st>>>(A, round)));
+    P2P_TIMED(K_BULK_GROW, st, (bulk_grow_kernel<<<grid_g, kBulkThreads, 0, st>>>(A, round)));
+    P2P_TIMED(K_BULK_APPLY, st, (bulk_apply_kernel<<<grid, kBulkThreads, 0, st>>>(A, round)));
     *launched += 3;
   }
   return cudaGetLastError();

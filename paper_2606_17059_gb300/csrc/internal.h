@@ -108,7 +108,7 @@ enum KernelId {
   K_GROUP_HASH, K_GROUP_RESOLVE, K_GROUP_RESOLVE32, K_ROUTE_STAGED, K_LANE_LEADER, K_LANE_FOLLOWER, K_DECIDE,
   K_VALIDATE, K_INIT_RANGES, K_DELTA, K_COMPACT, K_COMPACT_LABELS, K_REFRESH_VIEWS, K_SET_TREE,
   K_UPDATE_COUNT, K_UPDATE_SCAN, K_UPDATE_SCATTER, K_GROUP_RANGES, K_GROUP_PLACE, K_LRU_WALK, K_LRU_STAMP,
-  K_LRU_ORDER, K_LRU_SELECT, K_LRU_EVICT, K_LRU_OPS, K_HIT_RATE, K_ROOM, K_DELTA_BULK, K_COUNT_
+  K_LRU_EVICT, K_LRU_OPS, K_HIT_RATE, K_ROOM, K_BULK_RESOLVE, K_BULK_GROW, K_BULK_APPLY, K_COUNT_
 };
 static_assert((int)K_COUNT_ == (int)P2P_KERNEL_COUNT, "the header's kernel count");
 const char* kernel_name(int id);
@@ -301,35 +301,32 @@ cudaError_t launch_update_scatter(const int32_t* peer, const int64_t* offsets, i
                                   int32_t* cursor, int32_t* op, int64_t* seg_begin, int64_t* seg_off, int32_t* seg_len,
                                   int num_sms, cudaStream_t st);
 
-// LRU trees (lru_kernel.cu): walk + stamp (an access), BFS order, the level passes, the selection counts and
-// the eviction; see that file for the method.  lvl_begin (host) holds n_levels + 1 offsets into order.
+// LRU trees (lru_kernel.cu): walk + stamp (an access), and the eviction; see that file for the method.
 cudaError_t launch_lru_walk(const TreeState& s, const int32_t* shared, const int32_t* tokens, int64_t n_tokens,
                             const int64_t* offsets, int64_t B, int32_t* touch, int32_t* pslot, int32_t* out_match,
                             int32_t* err, int num_sms, cudaStream_t st);
 cudaError_t launch_lru_stamp(const TreeState& s, TreeState* d_state, const int32_t* shared, const int32_t* touch,
                              const int32_t* pslot, int32_t n_node, uint32_t time, int num_sms, cudaStream_t st);
-cudaError_t launch_lru_bfs(const TreeState& s, const int32_t* front, int32_t n_front, int32_t* next, int32_t* n_next,
-                           int32_t cap, int32_t* parent, int32_t* cslot, int num_sms, cudaStream_t st);
-cudaError_t launch_lru_init(const int32_t* order, int32_t n, int64_t* size, int64_t* off, int64_t* rank,
-                            unsigned long long* best, uint8_t* gone, int num_sms, cudaStream_t st);
-// Scratch of the sibling-offset sort (n2 = the live non-root nodes rounded up to a power of two; N = node slots).
-struct LruSortScratch {
-  unsigned long long* key;  // [n2]
-  int32_t* val;             // [n2]
-  int32_t* first;           // [N]
-  int64_t* scan;            // [n2]
+// Scratch of an eviction from a tree of N node slots (lru_scratch lays it out; its first `zeroed` bytes, from cnt on,
+// are cleared by the launch).
+struct LruScratch {
+  int32_t *cnt, *big_cnt;     // [N + 2]: nodes found for a level, and its nodes with large tables
+  unsigned long long* hist;   // [4 * 256]
+  unsigned long long* out;    // [8]: tokens of the tree, 1 if it is inconsistent, depth, cut level and cut
+  size_t zeroed;
+  unsigned long long* sum;    // [N], by node: tokens of the threshold's stamp in its subtree
+  int32_t *order, *parent, *cslot, *len;  // [N], by position in breadth-first order
+  uint32_t* stamp;            // [N], likewise
+  int32_t *surv, *big;        // [N]
+  int32_t* lvl;               // [N + 2]: where each level starts in the order
+  int32_t *path_node, *path_tok, *path_len;  // [N + 2], by level
+  uint8_t* state;             // [N], by node
 };
-cudaError_t launch_lru_levels(const TreeState& s, const int32_t* order, const int32_t* lvl_begin, int32_t n_levels,
-                              const int32_t* parent, const int32_t* cslot, int64_t* size, int64_t* off, int64_t* rank,
-                              unsigned long long* best, int32_t* end, const LruSortScratch& sc, int num_sms,
-                              cudaStream_t st);
-cudaError_t launch_lru_count(const TreeState& s, const int32_t* nodes, int32_t n, const int32_t* cslot,
-                             const int64_t* rank, const int32_t* end, int mode, uint32_t S, unsigned long long K,
-                             unsigned long long* out, int num_sms, cudaStream_t st);
-cudaError_t launch_lru_evict(const TreeState& s, TreeState* d_state, const int32_t* order, const int32_t* lvl_begin,
-                             int32_t n_levels, const int32_t* parent, const int32_t* cslot, const int64_t* rank,
-                             const int32_t* end, uint32_t S, unsigned long long K, int32_t cut, uint8_t* gone,
-                             int32_t* surv, int num_sms, cudaStream_t st);
+size_t lru_scratch(int64_t N, void* base, LruScratch& s);
+// Evicts `want` tokens (all, if the tree holds fewer); s.out[0] = the tokens the tree held, s.out[1] = 1 if the tree
+// is inconsistent (nothing is removed then).
+cudaError_t launch_lru_evict(const TreeState& tree, TreeState* d_state, const LruScratch& s, int32_t N,
+                             unsigned long long want, cudaStream_t st);
 cudaError_t launch_lru_ops(const int64_t* offsets, int64_t B, int64_t n_tokens, int32_t* op, int64_t* seg_begin,
                            int64_t* seg_off, int32_t* seg_len, int num_sms, cudaStream_t st);
 cudaError_t launch_hit_rate(const int32_t* match, int32_t P, const int64_t* offsets, int64_t B, const int32_t* peer,

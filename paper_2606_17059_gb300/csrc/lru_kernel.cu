@@ -17,20 +17,22 @@
 // removes the tokens in increasing order of (stamp, path of end, deeper first): a node becomes a leaf only
 // after its descendants go, those of other stamps are older (removed before it) and those of its stamp
 // include end(v), which precedes v in that order.  All tokens of one edge share the key, the deepest first.
-// So n tokens are removed at once: the nodes whose key is below a threshold found by binary search on
-// token counts, and the tail of the one node at the threshold.  The key's path order is the preorder rank
-// of end(v) with children taken by first token.
+// So n tokens are removed at once: the nodes whose key is below a threshold, and the tail of the one node at it.
 //
-// Kernels (all data-parallel; the host drives the level loops and the binary search):
-//   lru_walk_kernel        warp per request: PrefixMatch, and per node the deepest touched position
-//   lru_stamp_kernel       thread per node: stamp fully touched nodes, split partially touched edges
-//   lru_bfs_kernel         warp per frontier node: children, parent links, child slots, next frontier
-//   lru_size_kernel        subtree sizes, one level at a time from the deepest
-//   lru_pairs/bitonic/runs/scan/off_kernel  sibling offsets: the (parent, first token) pairs sorted, sizes scanned
-//   lru_rank_kernel        preorder ranks, one level at a time from the top
-//   lru_end_kernel         end(v), one level at a time from the deepest
-//   lru_count_kernel       token count of the nodes below a key (binary search steps)
-//   lru_evict_kernel       one level at a time from the top: remove, cut the boundary edge, move terms
+// The threshold needs no sort and no rank of the nodes.  Its stamp S comes from a radix selection over the stamps,
+// weighted by edge lengths; the r tokens left over are the first r of stamp S in the order of (end, deeper first), found
+// by walking down from the root.  At a node u, `carry` is the length of the edges above (u's included) whose end
+// lies in u's subtree: they are a run of stamp S down to u, each the largest same-stamp child of the one before.
+// A child c then stands for T(c) tokens, the edge lengths of stamp S in its subtree, and for carry too if it is u's
+// largest same-stamp child; the children are taken in token order, and the walk goes on in the one that holds token r.
+// At a u of stamp S without a same-stamp child the carried edges end: the r tokens are taken from the deepest up.  A
+// node of stamp S is removed if it precedes the walked path x in preorder or is one of those whole edges: one that
+// follows x is not, nor is an ancestor on x that is not carried (its end follows x).
+//
+// Kernels:
+//   lru_walk_kernel    warp per request: the match, and per node the deepest touched position (atomicMax)
+//   lru_stamp_kernel   thread per node: stamp fully touched nodes, split partially touched edges
+//   lru_evict_kernel   one cluster of CTAs does an eviction: breadth-first order, threshold, removal
 #include "internal.h"
 
 namespace p2p {
@@ -75,11 +77,29 @@ __device__ int find_live(const LruTree& t, int32_t off, int32_t bits, int32_t to
   return 0;
 }
 
-// First j in [0, lim) with a[j] != b[j], or lim (one warp).
+// First j in [0, lim) with a[j] != b[j], or lim (one warp): 256 tokens per step and side, so that a prompt of a
+// thousand tokens takes a handful of round trips (32 per step: the walk of 4,096 requests 39 us, now 19).
 __device__ int32_t first_mismatch(const int32_t* a, const int32_t* b, int32_t lim, int lane) {
-  for (int32_t j0 = 0; j0 < lim; j0 += 32) {
+  constexpr int U = 8;
+  int32_t j0 = 0;
+  for (; lim - j0 >= 32 * U; j0 += 32 * U) {
+    int32_t x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) x[u] = a[j0 + u * 32 + lane];
+    int32_t d = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) d |= x[u] ^ b[j0 + u * 32 + lane];
+    if (__any_sync(kFull, d != 0)) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const unsigned m = __ballot_sync(kFull, x[u] != b[j0 + u * 32 + lane]);
+        if (m) return j0 + u * 32 + __ffs(m) - 1;
+      }
+    }
+  }
+  for (; j0 < lim; j0 += 32) {
     const int32_t j = j0 + lane;
-    const unsigned m = __ballot_sync(kFull, j < lim && a[j] != b[j]);
+    const unsigned m = __ballot_sync(kFull, lane < lim - j0 && a[j] != b[j]);
     if (m) return j0 + __ffs(m) - 1;
   }
   return lim;
@@ -153,239 +173,361 @@ __global__ void __launch_bounds__(kLruThreads) lru_stamp_kernel(LruTree t, TreeS
   }
 }
 
-// Warp per node of the frontier: its live children get parent and slot, and go to the next frontier (at most
-// cap entries are written; the host checks the count against it).
-__global__ void __launch_bounds__(kLruThreads) lru_bfs_kernel(LruTree t, const int32_t* __restrict__ front,
-                                                              int32_t n_front, int32_t* next, int32_t* n_next,
-                                                              int32_t cap, int32_t* parent, int32_t* cslot) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (kLruThreads / 32);
-  for (int64_t i = ((int64_t)blockIdx.x * kLruThreads + threadIdx.x) >> 5; i < n_front; i += warps) {
-    const int32_t v = front[i];
-    const int4 nd = t.node[v];
-    const int32_t bits = tab_bits(nd.y);
-    if (bits == 0) continue;
-    for (int32_t b0 = 0; b0 < (1 << bits); b0 += 32) {
-      const int32_t s = b0 + lane;
-      const int4 x = s < (1 << bits) ? t.child[nd.x + s] : make_int4(0, 0, 0, 0);
-      const bool live = x.y >= 1;
-      const unsigned m = __ballot_sync(kFull, live);
-      if (!m) continue;
-      int32_t base = 0;
-      if (lane == 0) base = atomicAdd(n_next, __popc(m));
-      base = __shfl_sync(kFull, base, 0);
-      const int32_t at = base + __popc(m & ((1u << lane) - 1));
-      if (live && at < cap) {
-        next[at] = x.y;
-        parent[x.y] = v;
-        cslot[x.y] = nd.x + s;
+// ---- eviction ---------------------------------------------------------------------------------------------
+//
+// One cluster of kEvictCtas CTAs, so that its steps are ordered by the cluster's hardware barrier: an eviction has
+// about three steps per tree level and eight for the threshold.  With a launch per step (and per step of a global
+// bitonic sort of all siblings, and a host read per step of a binary search for the threshold) an eviction from
+// a trie of ~20,000 nodes took 240 launches and 100 host reads, 2.6 ms; now 0.2 ms.  What bounds it: the barriers and the
+// dependent loads between them (a level's records, tables, stamps); 16 of the SMs stream the tables at ~1 TB/s,
+// which large tries need less than the steps do.
+constexpr int kEvictThreads = 1024;
+constexpr int kEvictCtas = 16;
+constexpr int kLaneBits = 4;    // tables of up to 16 slots are read by one lane,
+constexpr int kWarpBits = 8;    // up to 256 slots by one warp, larger ones by the whole cluster
+constexpr int kStBefore = 0, kStAfter = 1, kStOnPath = 2, kStGone = 4;
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+
+struct EvictShared {
+  unsigned long long hist[256];
+  unsigned long long below, sum, best;
+  int bin, child, len, tok;
+};
+
+// The bin of the 256 that holds unit r (0 <= r < the bins' sum) of the weights in S.hist, and the sum before it
+// (S.bin, S.below; S.sum = all).  Every thread of the CTA calls it.
+__device__ void pick_bin(EvictShared& S, unsigned long long r) {
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    unsigned long long w[8], mine = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) mine += w[c] = S.hist[threadIdx.x * 8 + c];
+    unsigned long long incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(kFull, incl, o);
+      if ((int)threadIdx.x >= o) incl += y;
+    }
+    unsigned long long at = incl - mine;
+    if (r >= at && r < incl) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        if (r >= at && r < at + w[c]) {
+          S.bin = threadIdx.x * 8 + c;
+          S.below = at;
+        }
+        at += w[c];
       }
     }
+    if (threadIdx.x == 31) S.sum = incl;
   }
-}
-
-// Nodes of one level add their subtree sizes to their parents (size starts at 1).
-__global__ void __launch_bounds__(kLruThreads) lru_size_kernel(const int32_t* __restrict__ lvl, int32_t n,
-                                                               const int32_t* __restrict__ parent, int64_t* size) {
-  const int64_t stride = (int64_t)gridDim.x * kLruThreads;
-  for (int64_t i = (int64_t)blockIdx.x * kLruThreads + threadIdx.x; i < n; i += stride) {
-    const int32_t v = lvl[i];
-    atomicAdd((unsigned long long*)&size[parent[v]], (unsigned long long)size[v]);
-  }
-}
-
-// Sibling offsets for the preorder ranks: off[c] = the total subtree size of c's siblings whose first token
-// is smaller (signed order).  All (parent, first token) pairs of the tree are sorted at once (a bitonic sort:
-// a pair per live non-root node, padded to a power of two with the largest key), so each parent's children
-// form one run in first-token order; off[c] is then an exclusive scan of the sizes in that order, less the
-// scan at the start of c's run.  O(n log^2 n) for any fan-out.
-__global__ void __launch_bounds__(kLruThreads) lru_pairs_kernel(LruTree t, const int32_t* __restrict__ nodes, int32_t n,
-                                                                int64_t n2, const int32_t* __restrict__ parent,
-                                                                const int32_t* __restrict__ cslot,
-                                                                unsigned long long* key, int32_t* val) {
-  const int64_t stride = (int64_t)gridDim.x * kLruThreads;
-  for (int64_t i = (int64_t)blockIdx.x * kLruThreads + threadIdx.x; i < n2; i += stride) {
-    if (i < n) {
-      const int32_t v = nodes[i];
-      const uint32_t tok = (uint32_t)t.child[cslot[v]].x ^ 0x80000000u;  // signed order as unsigned
-      key[i] = ((unsigned long long)(uint32_t)parent[v] << 32) | tok;
-      val[i] = v;
-    } else {
-      key[i] = ~0ull;
-      val[i] = -1;
-    }
-  }
-}
-
-// One compare-exchange step of the bitonic sort of (key, val) over n2 (a power of two) entries.
-__global__ void __launch_bounds__(kLruThreads) lru_bitonic_kernel(unsigned long long* key, int32_t* val, int64_t n2,
-                                                                  int64_t j, int64_t k) {
-  const int64_t stride = (int64_t)gridDim.x * kLruThreads;
-  for (int64_t i = (int64_t)blockIdx.x * kLruThreads + threadIdx.x; i < n2; i += stride) {
-    const int64_t l = i ^ j;
-    if (l <= i) continue;
-    const unsigned long long a = key[i], b = key[l];
-    if ((a > b) == ((i & k) == 0)) {
-      key[i] = b;
-      key[l] = a;
-      const int32_t va = val[i];
-      val[i] = val[l];
-      val[l] = va;
-    }
-  }
-}
-
-// For the sorted pairs [0, n): the first position of each parent's run (first[parent]) and the sizes in
-// sorted order (into scan, scanned next).
-__global__ void __launch_bounds__(kLruThreads) lru_runs_kernel(const unsigned long long* __restrict__ key,
-                                                               const int32_t* __restrict__ val, int32_t n,
-                                                               const int64_t* __restrict__ size, int32_t* first,
-                                                               int64_t* scan) {
-  const int64_t stride = (int64_t)gridDim.x * kLruThreads;
-  for (int64_t i = (int64_t)blockIdx.x * kLruThreads + threadIdx.x; i < n; i += stride) {
-    if (i == 0 || (key[i] >> 32) != (key[i - 1] >> 32)) first[(int32_t)(key[i] >> 32)] = (int32_t)i;
-    scan[i] = size[val[i]];
-  }
-}
-
-// Exclusive scan of scan[0, n) in place, one CTA: each thread sums a contiguous stretch, the CTA scans the
-// stretch sums, each thread rewrites its stretch.
-__global__ void __launch_bounds__(1024) lru_scan_kernel(int64_t* scan, int32_t n) {
-  __shared__ int64_t s_part[1024];
-  const int32_t per = (n + 1023) / 1024, a = min(n, (int32_t)threadIdx.x * per), b = min(n, a + per);
-  int64_t sum = 0;
-  for (int32_t i = a; i < b; ++i) sum += scan[i];
-  s_part[threadIdx.x] = sum;
   __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {  // inclusive scan of the stretch sums (Hillis-Steele)
-    const int64_t x = threadIdx.x >= (unsigned)o ? s_part[threadIdx.x - o] : 0;
+}
+
+// Adds w to bin k of S.hist: one addition for the warp when all of its lanes have the same bin (the high bytes
+// of the keys usually agree).  Every lane of the warp calls it; w = 0 adds nothing.
+__device__ __forceinline__ void add_bin(EvictShared& S, int k, unsigned long long w) {
+  const unsigned has = __ballot_sync(kFull, w != 0);
+  if (!has) return;
+  const int k0 = __shfl_sync(kFull, k, __ffs(has) - 1);
+  if (__all_sync(kFull, w == 0 || k == k0)) {
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(kFull, w, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&S.hist[k0], w);
+  } else if (w) {
+    atomicAdd(&S.hist[k], w);
+  }
+}
+
+__global__ void __launch_bounds__(kEvictThreads, 1) lru_evict_kernel(LruTree t, TreeState* st, LruScratch s, int32_t N,
+                                                                     unsigned long long want) {
+  __shared__ EvictShared S;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t rank = cluster_rank();
+  const int n_warps = (int)cluster_size() * (kEvictThreads / 32), gw = (int)rank * (kEvictThreads / 32) + warp;
+  const int n_threads = n_warps * 32, gt = gw * 32 + lane;
+  const bool lead = rank == 0 && threadIdx.x == 0;
+  if (lead) {
+    s.order[0] = 0;
+    s.lvl[0] = 0;
+    s.lvl[1] = 1;
+    s.sum[0] = 0;
+    s.state[0] = kStOnPath;
+  }
+  cluster_sync();
+  // Breadth-first order, a level at a time.  By position in the order: node, parent, slot, edge length, stamp.
+  auto put = [&](int32_t at, int32_t v, int32_t slot, const int4& e) {
+    if (at >= N) return;  // (more nodes than the tree has: reported below)
+    s.order[at] = e.y;
+    s.parent[at] = v;
+    s.cslot[at] = slot;
+    s.len[at] = e.w;
+    s.stamp[at] = t.stamp[e.y];
+    s.sum[e.y] = 0;
+  };
+  int32_t begin = 0, end = 1, L = 0;
+  for (;;) {
+    for (int32_t b0 = begin + gw * 32; b0 < end; b0 += n_warps * 32) {
+      const int32_t i = b0 + lane;
+      const int32_t v = i < end ? __ldcg(s.order + i) : -1;
+      const int4 nd = v >= 0 ? t.node[v] : make_int4(0, 0, 0, 0);
+      const int32_t bits = tab_bits(nd.y);
+      const int32_t z = bits > 0 && bits <= kWarpBits ? max(nd.z, 0) : 0;  // its children, placed side by side
+      int32_t incl = z;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const int32_t total = __shfl_sync(kFull, incl, 31);
+      int32_t base = 0;
+      if (lane == 31 && total) base = atomicAdd(&s.cnt[L + 1], total);
+      base = __shfl_sync(kFull, base, 31);
+      int32_t at = end + base + incl - z;
+      const int32_t stop = at + z;
+      if (bits > kWarpBits) {
+        const int32_t k = atomicAdd(&s.big_cnt[L], 1);
+        if (k < N) s.big[k] = v;
+      } else if (bits > 0 && bits <= kLaneBits) {
+        for (int32_t j0 = 0; j0 < (1 << bits) && at < stop; j0 += 4) {
+          int4 e[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) e[c] = t.child[nd.x + j0 + c];
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (e[c].y >= 1 && at < stop) put(at++, v, nd.x + j0 + c, e[c]);
+        }
+      }
+      for (unsigned m = __ballot_sync(kFull, bits > kLaneBits && bits <= kWarpBits); m; m &= m - 1) {
+        const int j = __ffs(m) - 1;
+        const int32_t x = __shfl_sync(kFull, nd.x, j), size = 1 << __shfl_sync(kFull, bits, j);
+        const int32_t vj = __shfl_sync(kFull, v, j), sj = __shfl_sync(kFull, stop, j);
+        int32_t aj = __shfl_sync(kFull, at, j);
+        for (int32_t j0 = 0; j0 < size; j0 += 32) {
+          const int4 e = t.child[x + j0 + lane];
+          const unsigned lm = __ballot_sync(kFull, e.y >= 1);
+          const int32_t pos = aj + __popc(lm & ((1u << lane) - 1));
+          if (e.y >= 1 && pos < sj) put(pos, vj, x + j0 + lane, e);
+          aj += __popc(lm);
+        }
+      }
+    }
+    cluster_sync();
+    const int32_t nb = min(__ldcg(s.big_cnt + L), N);
+    if (nb) {
+      for (int32_t k = 0; k < nb; ++k) {
+        const int32_t v = __ldcg(s.big + k);
+        const int4 nd = t.node[v];
+        for (int32_t j0 = gw * 32; j0 < (1 << tab_bits(nd.y)); j0 += n_warps * 32) {
+          const int4 e = t.child[nd.x + j0 + lane];
+          const unsigned lm = __ballot_sync(kFull, e.y >= 1);
+          int32_t base = 0;
+          if (lane == 0 && lm) base = atomicAdd(&s.cnt[L + 1], __popc(lm));
+          base = __shfl_sync(kFull, base, 0);
+          if (e.y >= 1) put(end + base + __popc(lm & ((1u << lane) - 1)), v, nd.x + j0 + lane, e);
+        }
+      }
+      cluster_sync();
+    }
+    const int32_t c = __ldcg(s.cnt + L + 1);
+    if (c <= 0) break;
+    if ((int64_t)end + c > N) {  // an inconsistent tree: nothing is removed
+      if (lead) s.out[1] = 1;
+      return;
+    }
+    begin = end;
+    end += c;
+    ++L;
+    if (lead) s.lvl[L + 1] = end;
+  }
+  const int32_t total = end;
+  // The stamp S of the threshold: a radix selection of unit `want` of the edge lengths by stamp.
+  uint32_t cut_stamp = 0;
+  unsigned long long rest = want;
+  bool all = false;
+  for (int pass = 0; pass < 4; ++pass) {
+    const int shift = 24 - 8 * pass;
+    for (int k = threadIdx.x; k < 256; k += kEvictThreads) S.hist[k] = 0;
     __syncthreads();
-    s_part[threadIdx.x] += x;
+    for (int32_t i0 = 1 + gw * 32; i0 < total; i0 += n_threads) {
+      const int32_t i = i0 + lane;
+      const uint32_t x = i < total ? __ldcg(s.stamp + i) : 0u;
+      const bool in = i < total && (pass == 0 || (x >> (shift + 8)) == cut_stamp);
+      add_bin(S, (int)((x >> shift) & 255u), in ? (unsigned long long)__ldcg(s.len + i) : 0ull);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < 256; k += kEvictThreads)
+      if (S.hist[k]) atomicAdd(&s.hist[pass * 256 + k], S.hist[k]);
+    cluster_sync();
+    for (int k = threadIdx.x; k < 256; k += kEvictThreads) S.hist[k] = __ldcg(&s.hist[pass * 256 + k]);
+    pick_bin(S, rest);
+    if (pass == 0) {
+      if (lead) s.out[0] = S.sum;
+      if (rest >= S.sum) {
+        all = true;
+        break;
+      }
+    }
+    rest -= S.below;
+    cut_stamp = (cut_stamp << 8) | (uint32_t)S.bin;
     __syncthreads();
   }
-  int64_t run = s_part[threadIdx.x] - sum;
-  for (int32_t i = a; i < b; ++i) {
-    const int64_t x = scan[i];
-    scan[i] = run;
-    run += x;
-  }
-}
-
-// off[c] for every sorted pair: the scan at c less the scan at the start of its parent's run.
-__global__ void __launch_bounds__(kLruThreads) lru_off_kernel(const unsigned long long* __restrict__ key,
-                                                              const int32_t* __restrict__ val, int32_t n,
-                                                              const int32_t* __restrict__ first,
-                                                              const int64_t* __restrict__ scan, int64_t* off) {
-  const int64_t stride = (int64_t)gridDim.x * kLruThreads;
-  for (int64_t i = (int64_t)blockIdx.x * kLruThreads + threadIdx.x; i < n; i += stride)
-    off[val[i]] = scan[i] - scan[first[(int32_t)(key[i] >> 32)]];
-}
-
-// Preorder ranks of one level: rank[v] = rank[parent] + 1 + the sizes of v's earlier siblings.
-__global__ void __launch_bounds__(kLruThreads) lru_rank_kernel(const int32_t* __restrict__ lvl, int32_t n,
-                                                               const int32_t* __restrict__ parent,
-                                                               const int64_t* __restrict__ off, int64_t* rank) {
-  const int64_t stride = (int64_t)gridDim.x * kLruThreads;
-  for (int64_t i = (int64_t)blockIdx.x * kLruThreads + threadIdx.x; i < n; i += stride) {
-    const int32_t v = lvl[i];
-    rank[v] = rank[parent[v]] + 1 + off[v];
-  }
-}
-
-// end(v) for one level (its children's ends are final): the end of the same-stamp child with the largest
-// first token, or v.  Then v offers itself to its parent when their stamps agree (best[] holds the offer
-// with the largest first token: sign-flipped token in the high word, node in the low word).
-__global__ void __launch_bounds__(kLruThreads) lru_end_kernel(LruTree t, const int32_t* __restrict__ lvl, int32_t n,
-                                                              const int32_t* __restrict__ parent,
-                                                              const int32_t* __restrict__ cslot,
-                                                              unsigned long long* best, int32_t* end) {
-  const int64_t stride = (int64_t)gridDim.x * kLruThreads;
-  for (int64_t i = (int64_t)blockIdx.x * kLruThreads + threadIdx.x; i < n; i += stride) {
-    const int32_t v = lvl[i];
-    const unsigned long long bv = best[v];
-    const int32_t e = bv ? end[(int32_t)(bv & 0xffffffffull)] : v;
-    end[v] = e;
-    const int32_t p = parent[v];
-    if (p != 0 && t.stamp[v] == t.stamp[p]) {
-      const uint32_t key = (uint32_t)t.child[cslot[v]].x ^ 0x80000000u;
-      atomicMax(&best[p], ((unsigned long long)key << 32) | (uint32_t)v);
+  // The place of token `rest` of stamp S: T bottom-up, then the walk down from the root (the first CTA).
+  const bool walk = !all && rest > 0;
+  int32_t depth = 0, cut_level = 0, cut = 0;
+  if (walk) {
+    for (int32_t l = L; l >= 1; --l) {
+      const int32_t hi = __ldcg(s.lvl + l + 1);
+      for (int32_t i = __ldcg(s.lvl + l) + gt; i < hi; i += n_threads) {
+        const int32_t v = __ldcg(s.order + i);
+        const unsigned long long own = __ldcg(s.stamp + i) == cut_stamp ? (unsigned long long)__ldcg(s.len + i) : 0ull;
+        const unsigned long long T = __ldcg(s.sum + v) + own;
+        if (own) s.sum[v] = T;
+        if (T) atomicAdd(&s.sum[__ldcg(s.parent + i)], T);
+      }
+      cluster_sync();
     }
-  }
-}
-
-// The eviction key below stamp: (preorder rank of end(v), deeper first), one 64-bit word.
-__device__ __forceinline__ unsigned long long key2_of(const int64_t* rank, const int32_t* end, int32_t v) {
-  return ((unsigned long long)rank[end[v]] << 32) | (unsigned long long)(0xffffffffu - (uint32_t)rank[v]);
-}
-
-// Token count (edge lengths) of the non-root nodes nodes[0 .. n) with stamp < S (mode 0), or with stamp == S
-// and key2 < K (mode 1), added to *out.
-__global__ void __launch_bounds__(kLruThreads) lru_count_kernel(LruTree t, const int32_t* __restrict__ nodes, int32_t n,
-                                                                const int32_t* __restrict__ cslot,
-                                                                const int64_t* __restrict__ rank,
-                                                                const int32_t* __restrict__ end, int mode, uint32_t S,
-                                                                unsigned long long K, unsigned long long* out) {
-  unsigned long long sum = 0;
-  const int64_t stride = (int64_t)gridDim.x * kLruThreads;
-  for (int64_t i = (int64_t)blockIdx.x * kLruThreads + threadIdx.x; i < n; i += stride) {
-    const int32_t v = nodes[i];
-    const uint32_t s = t.stamp[v];
-    const bool in = mode == 0 ? s < S : (s == S && key2_of(rank, end, v) < K);
-    if (in) sum += (unsigned long long)t.child[cslot[v]].w;
-  }
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
-  if ((threadIdx.x & 31) == 0 && sum) atomicAdd(out, sum);
-}
-
-// One level, from the top: a node below the threshold (stamp < S, or stamp == S and key2 < K) is removed --
-// tombstoned in its parent's table when the parent stays -- and its stored sequences move to the nearest
-// node that stays (surv); the node at the threshold (stamp == S, key2 == K) loses its last `cut` tokens.
-__global__ void __launch_bounds__(kLruThreads) lru_evict_kernel(LruTree t, TreeState* st, const int32_t* __restrict__ lvl,
-                                                                int32_t n, const int32_t* __restrict__ parent,
-                                                                const int32_t* __restrict__ cslot,
-                                                                const int64_t* __restrict__ rank,
-                                                                const int32_t* __restrict__ end, uint32_t S,
-                                                                unsigned long long K, int32_t cut, uint8_t* gone,
-                                                                int32_t* surv) {
-  const int64_t stride = (int64_t)gridDim.x * kLruThreads;
-  for (int64_t i = (int64_t)blockIdx.x * kLruThreads + threadIdx.x; i < n; i += stride) {
-    const int32_t v = lvl[i];
-    const uint32_t s = t.stamp[v];
-    const unsigned long long k2 = s == S ? key2_of(rank, end, v) : 0ull;
-    const bool out = s < S || (s == S && k2 < K);
-    gone[v] = out;
-    if (!out) {
-      if (s == S && k2 == K && cut > 0) t.child[cslot[v]].w -= cut;
-      continue;
+    if (rank == 0) {
+      int32_t u = 0, lev = 0, len_u = 0;
+      unsigned long long carry = 0, r = rest;
+      for (; lev <= L; ++lev) {
+        const int4 nd = t.node[u];
+        const int32_t size = tab_bits(nd.y) ? 1 << tab_bits(nd.y) : 0;
+        const bool same = u != 0 && t.stamp[u] == cut_stamp;
+        if (same) carry += (unsigned long long)len_u;
+        // A table of up to one slot per thread is read once; larger ones once per step.
+        const bool held = size <= kEvictThreads;
+        int4 e0 = make_int4(0, 0, 0, 0);
+        if (held && (int)threadIdx.x < size) e0 = t.child[nd.x + threadIdx.x];
+        unsigned long long T0 = e0.y >= 1 ? __ldcg(s.sum + e0.y) : 0ull;
+        if (threadIdx.x == 0) {
+          S.best = 0;
+          S.child = S.len = S.tok = 0;
+        }
+        __syncthreads();
+        if (same)
+          for (int32_t j = threadIdx.x; j < size; j += kEvictThreads) {
+            const int4 e = held ? e0 : t.child[nd.x + j];
+            if (e.y >= 1 && t.stamp[e.y] == cut_stamp)
+              atomicMax(&S.best, ((unsigned long long)((uint32_t)e.x ^ 0x80000000u) << 32) | (uint32_t)e.y);
+          }
+        __syncthreads();
+        const int32_t best = (int32_t)(S.best & 0xffffffffull);
+        if (same && best == 0) break;  // the carried edges end here
+        if (held && same && e0.y == best && e0.y >= 1) T0 += carry;
+        uint32_t key = 0;
+        for (int pass = 0; pass < 4; ++pass) {
+          const int shift = 24 - 8 * pass;
+          for (int k = threadIdx.x; k < 256; k += kEvictThreads) S.hist[k] = 0;
+          __syncthreads();
+          for (int32_t j0 = 0; j0 < size; j0 += kEvictThreads) {
+            const int32_t j = j0 + (int32_t)threadIdx.x;
+            const int4 e = held ? e0 : j < size ? t.child[nd.x + j] : make_int4(0, 0, 0, 0);
+            const uint32_t x = (uint32_t)e.x ^ 0x80000000u;
+            const bool in = j < size && e.y >= 1 && (pass == 0 || (x >> (shift + 8)) == key);
+            unsigned long long w = 0;
+            if (in) w = held ? T0 : __ldcg(s.sum + e.y) + (same && e.y == best ? carry : 0ull);
+            add_bin(S, (int)((x >> shift) & 255u), w);
+          }
+          pick_bin(S, r);
+          r -= S.below;
+          key = (key << 8) | (uint32_t)S.bin;
+          __syncthreads();
+        }
+        for (int32_t j = threadIdx.x; j < size; j += kEvictThreads) {
+          const int4 e = held ? e0 : t.child[nd.x + j];
+          if (e.y >= 1 && ((uint32_t)e.x ^ 0x80000000u) == key) {
+            S.child = e.y;
+            S.len = e.w;
+            S.tok = e.x;
+          }
+        }
+        __syncthreads();
+        if (!(same && S.child == best)) carry = 0;
+        u = S.child;
+        len_u = S.len;
+        if (threadIdx.x == 0) {
+          s.path_node[lev + 1] = u;
+          s.path_tok[lev + 1] = S.tok;
+          s.path_len[lev + 1] = len_u;
+        }
+        __syncthreads();
+      }
+      if (threadIdx.x == 0) {
+        // r < carry: whole edges from the deepest up, then r tokens of the next.
+        int32_t l = lev;
+        while (l > 1 && r >= (unsigned long long)s.path_len[l]) r -= (unsigned long long)s.path_len[l--];
+        s.out[2] = (unsigned long long)lev;
+        s.out[3] = (unsigned long long)l;
+        s.out[4] = r;
+      }
     }
-    const int32_t p = parent[v];
-    const int32_t sv = gone[p] ? surv[p] : p;
-    surv[v] = sv;
-    const int4 e = t.child[cslot[v]];
-    if (!gone[p]) {
-      t.child[cslot[v]].y = -1;  // tombstone: the slot keeps its key
-      atomicSub(&t.node[p].z, 1);
-    }
-    const int4 nd = t.node[v];
-    if (nd.w) atomicAdd(&t.node[sv].w, nd.w);
-    atomicAdd((unsigned long long*)&st->dead_nodes, 1ull);
-    if (e.z >= 0) atomicAdd((unsigned long long*)&st->stale_label, (unsigned long long)e.w);
-    if (tab_bits(nd.y)) atomicAdd((unsigned long long*)&st->stale_child, 1ull << tab_bits(nd.y));
+    cluster_sync();
+    depth = (int32_t)__ldcg(s.out + 2);
+    cut_level = (int32_t)__ldcg(s.out + 3);
+    cut = (int32_t)__ldcg(s.out + 4);
   }
-}
-
-// Node arrays of an eviction: size 1, the rest 0 (nodes of the BFS order).
-__global__ void __launch_bounds__(kLruThreads) lru_init_kernel(const int32_t* __restrict__ order, int32_t n, int64_t* size,
-                                                               int64_t* off, int64_t* rank, unsigned long long* best,
-                                                               uint8_t* gone) {
-  const int64_t stride = (int64_t)gridDim.x * kLruThreads;
-  for (int64_t i = (int64_t)blockIdx.x * kLruThreads + threadIdx.x; i < n; i += stride) {
-    const int32_t v = order[i];
-    size[v] = 1;
-    off[v] = 0;
-    rank[v] = 0;
-    best[v] = 0;
-    gone[v] = 0;
+  // Removal, from the top: a node that goes is tombstoned in its parent's table when the parent stays, and its stored
+  // sequences move to the nearest node that stays; the node at the threshold loses its last `cut` tokens.
+  unsigned long long dead = 0, st_label = 0, st_child = 0;
+  for (int32_t l = 1; l <= L; ++l) {
+    const int32_t hi = __ldcg(s.lvl + l + 1);
+    const int32_t x = walk && l <= depth ? __ldcg(s.path_node + l) : -1;
+    const uint32_t xt = x >= 0 ? (uint32_t)__ldcg(s.path_tok + l) ^ 0x80000000u : 0u;
+    for (int32_t i = __ldcg(s.lvl + l) + gt; i < hi; i += n_threads) {
+      const int32_t v = __ldcg(s.order + i), p = __ldcg(s.parent + i), slot = __ldcg(s.cslot + i);
+      const uint32_t stamp = __ldcg(s.stamp + i);
+      const int up = __ldcg(s.state + p);
+      int where = up & 3;
+      if (walk && where == kStOnPath) {
+        if (x < 0) where = kStAfter;
+        else if (v != x) where = ((uint32_t)t.child[slot].x ^ 0x80000000u) < xt ? kStBefore : kStAfter;
+      }
+      const bool out = all || stamp < cut_stamp ||
+                       (walk && stamp == cut_stamp &&
+                        (where == kStBefore || (where == kStOnPath && l > cut_level)));
+      s.state[v] = (uint8_t)(where | (out ? kStGone : 0));
+      if (!out) {
+        if (walk && where == kStOnPath && l == cut_level && cut > 0) t.child[slot].w -= cut;
+        continue;
+      }
+      const bool orphan = up & kStGone;
+      const int32_t sv = orphan ? __ldcg(s.surv + p) : p;
+      s.surv[v] = sv;
+      const int4 e = t.child[slot];
+      if (!orphan) {
+        t.child[slot].y = -1;  // a tombstone: the slot keeps its key
+        atomicSub(&t.node[p].z, 1);
+      }
+      const int4 nd = t.node[v];
+      if (nd.w) atomicAdd(&t.node[sv].w, nd.w);
+      dead += 1;
+      if (e.z >= 0) st_label += (unsigned long long)e.w;
+      if (tab_bits(nd.y)) st_child += 1ull << tab_bits(nd.y);
+    }
+    cluster_sync();
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    dead += __shfl_xor_sync(kFull, dead, o);
+    st_label += __shfl_xor_sync(kFull, st_label, o);
+    st_child += __shfl_xor_sync(kFull, st_child, o);
+  }
+  if (lane == 0 && dead) {
+    atomicAdd((unsigned long long*)&st->dead_nodes, dead);
+    if (st_label) atomicAdd((unsigned long long*)&st->stale_label, st_label);
+    if (st_child) atomicAdd((unsigned long long*)&st->stale_child, st_child);
   }
 }
 
@@ -447,97 +589,60 @@ cudaError_t launch_lru_stamp(const TreeState& s, TreeState* d_state, const int32
   return cudaGetLastError();
 }
 
-cudaError_t launch_lru_bfs(const TreeState& s, const int32_t* front, int32_t n_front, int32_t* next, int32_t* n_next,
-                           int32_t cap, int32_t* parent, int32_t* cslot, int num_sms, cudaStream_t st) {
-  if (n_front <= 0) return cudaSuccess;
-  P2P_TIMED(K_LRU_ORDER, st,
-            (lru_bfs_kernel<<<grid_for(n_front, kLruThreads / 32, num_sms), kLruThreads, 0, st>>>(
-                lru_tree(s, nullptr), front, n_front, next, n_next, cap, parent, cslot)));
-  return cudaGetLastError();
+size_t lru_scratch(int64_t N, void* base, LruScratch& s) {
+  char* p = static_cast<char*>(base);
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    void* q = p ? p + at : nullptr;
+    at += (bytes + 15) & ~(size_t)15;
+    return q;
+  };
+  const size_t n = (size_t)N, levels = (size_t)N + 2;
+  s.cnt = static_cast<int32_t*>(take(levels * 4));
+  s.big_cnt = static_cast<int32_t*>(take(levels * 4));
+  s.hist = static_cast<unsigned long long*>(take(4 * 256 * 8));
+  s.out = static_cast<unsigned long long*>(take(8 * 8));
+  s.zeroed = at;
+  s.sum = static_cast<unsigned long long*>(take(n * 8));
+  s.order = static_cast<int32_t*>(take(n * 4));
+  s.parent = static_cast<int32_t*>(take(n * 4));
+  s.cslot = static_cast<int32_t*>(take(n * 4));
+  s.len = static_cast<int32_t*>(take(n * 4));
+  s.stamp = static_cast<uint32_t*>(take(n * 4));
+  s.surv = static_cast<int32_t*>(take(n * 4));
+  s.big = static_cast<int32_t*>(take(n * 4));
+  s.lvl = static_cast<int32_t*>(take(levels * 4));
+  s.path_node = static_cast<int32_t*>(take(levels * 4));
+  s.path_tok = static_cast<int32_t*>(take(levels * 4));
+  s.path_len = static_cast<int32_t*>(take(levels * 4));
+  s.state = static_cast<uint8_t*>(take(n));
+  return at;
 }
 
-cudaError_t launch_lru_levels(const TreeState& s, const int32_t* order, const int32_t* lvl_begin, int32_t n_levels,
-                              const int32_t* parent, const int32_t* cslot, int64_t* size, int64_t* off, int64_t* rank,
-                              unsigned long long* best, int32_t* end, const LruSortScratch& sc, int num_sms,
-                              cudaStream_t st) {
-  const LruTree t = lru_tree(s, nullptr);
-  // Sizes, from the deepest level up (level 0 is the root).
-  for (int32_t l = n_levels - 1; l >= 1; --l) {
-    const int32_t n = lvl_begin[l + 1] - lvl_begin[l];
-    P2P_TIMED(K_LRU_ORDER, st,
-              (lru_size_kernel<<<grid_for(n, kLruThreads, num_sms), kLruThreads, 0, st>>>(order + lvl_begin[l], n,
-                                                                                          parent, size)));
+cudaError_t launch_lru_evict(const TreeState& tree, TreeState* d_state, const LruScratch& s, int32_t N,
+                             unsigned long long want, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(s.cnt, 0, s.zeroed, st);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(lru_evict_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kEvictCtas;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(kEvictCtas);
+  cfg.blockDim = dim3(kEvictThreads);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int fit = 0;
+  if (cudaOccupancyMaxActiveClusters(&fit, lru_evict_kernel, &cfg) != cudaSuccess || fit < 1) {
+    (void)cudaGetLastError();
+    attr[0].val.clusterDim.x = 8;  // the portable size
+    cfg.gridDim = dim3(8);
   }
-  // Sibling offsets (all parents at once, by a sort of the (parent, first token) pairs), then preorder ranks
-  // from the top.
-  const int32_t m = lvl_begin[n_levels] - 1;  // the live non-root nodes: order[1 .. m]
-  if (m > 0) {
-    int64_t n2 = 1;
-    while (n2 < m) n2 <<= 1;
-    P2P_TIMED(K_LRU_ORDER, st,
-              (lru_pairs_kernel<<<grid_for(n2, kLruThreads, num_sms), kLruThreads, 0, st>>>(
-                  t, order + 1, m, n2, parent, cslot, sc.key, sc.val)));
-    for (int64_t k = 2; k <= n2; k <<= 1)
-      for (int64_t j = k >> 1; j > 0; j >>= 1)
-        P2P_TIMED(K_LRU_ORDER, st,
-                  (lru_bitonic_kernel<<<grid_for(n2, kLruThreads, num_sms), kLruThreads, 0, st>>>(sc.key, sc.val, n2,
-                                                                                                  j, k)));
-    P2P_TIMED(K_LRU_ORDER, st,
-              (lru_runs_kernel<<<grid_for(m, kLruThreads, num_sms), kLruThreads, 0, st>>>(sc.key, sc.val, m, size,
-                                                                                         sc.first, sc.scan)));
-    P2P_TIMED(K_LRU_ORDER, st, (lru_scan_kernel<<<1, 1024, 0, st>>>(sc.scan, m)));
-    P2P_TIMED(K_LRU_ORDER, st,
-              (lru_off_kernel<<<grid_for(m, kLruThreads, num_sms), kLruThreads, 0, st>>>(sc.key, sc.val, m, sc.first,
-                                                                                        sc.scan, off)));
-  }
-  for (int32_t l = 1; l < n_levels; ++l) {
-    const int32_t n = lvl_begin[l + 1] - lvl_begin[l];
-    P2P_TIMED(K_LRU_ORDER, st,
-              (lru_rank_kernel<<<grid_for(n, kLruThreads, num_sms), kLruThreads, 0, st>>>(order + lvl_begin[l], n,
-                                                                                          parent, off, rank)));
-  }
-  // end(v), from the deepest level up.
-  for (int32_t l = n_levels - 1; l >= 1; --l) {
-    const int32_t n = lvl_begin[l + 1] - lvl_begin[l];
-    P2P_TIMED(K_LRU_ORDER, st,
-              (lru_end_kernel<<<grid_for(n, kLruThreads, num_sms), kLruThreads, 0, st>>>(t, order + lvl_begin[l], n,
-                                                                                         parent, cslot, best, end)));
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_lru_count(const TreeState& s, const int32_t* nodes, int32_t n, const int32_t* cslot,
-                             const int64_t* rank, const int32_t* end, int mode, uint32_t S, unsigned long long K,
-                             unsigned long long* out, int num_sms, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long), st);
-  if (e != cudaSuccess || n <= 0) return e;
-  P2P_TIMED(K_LRU_SELECT, st,
-            (lru_count_kernel<<<grid_for(n, kLruThreads, num_sms), kLruThreads, 0, st>>>(
-                lru_tree(s, nullptr), nodes, n, cslot, rank, end, mode, S, K, out)));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_lru_evict(const TreeState& s, TreeState* d_state, const int32_t* order, const int32_t* lvl_begin,
-                             int32_t n_levels, const int32_t* parent, const int32_t* cslot, const int64_t* rank,
-                             const int32_t* end, uint32_t S, unsigned long long K, int32_t cut, uint8_t* gone,
-                             int32_t* surv, int num_sms, cudaStream_t st) {
-  for (int32_t l = 1; l < n_levels; ++l) {
-    const int32_t n = lvl_begin[l + 1] - lvl_begin[l];
-    P2P_TIMED(K_LRU_EVICT, st,
-              (lru_evict_kernel<<<grid_for(n, kLruThreads, num_sms), kLruThreads, 0, st>>>(
-                  lru_tree(s, nullptr), d_state, order + lvl_begin[l], n, parent, cslot, rank, end, S, K, cut, gone,
-                  surv)));
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_lru_init(const int32_t* order, int32_t n, int64_t* size, int64_t* off, int64_t* rank,
-                            unsigned long long* best, uint8_t* gone, int num_sms, cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  P2P_TIMED(K_LRU_ORDER, st,
-            (lru_init_kernel<<<grid_for(n, kLruThreads, num_sms), kLruThreads, 0, st>>>(order, n, size, off, rank, best,
-                                                                                        gone)));
-  return cudaGetLastError();
+  P2P_TIMED(K_LRU_EVICT, st, (e = cudaLaunchKernelEx(&cfg, lru_evict_kernel, lru_tree(tree, nullptr), d_state, s, N, want)));
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 cudaError_t launch_lru_ops(const int64_t* offsets, int64_t B, int64_t n_tokens, int32_t* op, int64_t* seg_begin,

@@ -92,8 +92,8 @@ const char* kernel_name(int id) {
       "lane_kernel<false>", "decide_kernel", "validate_kernel", "init_ranges_kernel", "delta_kernel",
       "compact_kernel", "compact_labels_kernel", "refresh_views_kernel", "set_tree_kernel", "update_count_kernel",
       "update_scan_kernel", "update_scatter_kernel", "group_ranges_kernel", "group_place_kernel", "lru_walk_kernel",
-      "lru_stamp_kernel", "lru_order_kernels", "lru_count_kernel", "lru_evict_kernel", "lru_ops_kernel",
-      "hit_rate_kernel", "room_kernel", "delta_bulk_kernels"};
+      "lru_stamp_kernel", "lru_evict_kernel", "lru_ops_kernel", "hit_rate_kernel", "room_kernel", "bulk_resolve_kernel",
+      "bulk_grow_kernel", "bulk_apply_kernel"};
   return id >= 0 && id < K_COUNT_ ? names[id] : "";
 }
 
@@ -1747,100 +1747,20 @@ int p2p_lru_evict(p2p_router* r, int32_t tree, int64_t n_tokens, int64_t* n_evic
   if (n_tokens == 0) return P2P_OK;
   DeviceGuard g(r);
   const TreeState& t = r->hs[(size_t)tree];
-  const int64_t N = std::max<int32_t>(t.n_node, 1);
-  // Scratch, per node slot: order, parent, cslot, end, surv (int32); size, off, rank, best (64-bit); gone; two
-  // counters; then the sibling-offset sort (a power of two of entries at least N - 1: key, scan 64-bit; val;
-  // and first per node slot).
-  int64_t n2 = 1;
-  while (n2 < N - 1) n2 <<= 1;
-  const size_t main_bytes = ((size_t)N * (5 * 4 + 4 * 8 + 1) + 64 + 15) & ~(size_t)15;
-  const size_t bytes = main_bytes + (size_t)n2 * (8 + 8 + 4) + (size_t)N * 4;
-  CK(ensure(r, r->lru_buf, bytes));
-  char* base = static_cast<char*>(r->lru_buf.p);
-  p2p::LruSortScratch sc;
-  sc.key = reinterpret_cast<unsigned long long*>(base + main_bytes);
-  sc.scan = reinterpret_cast<int64_t*>(sc.key + n2);
-  sc.val = reinterpret_cast<int32_t*>(sc.scan + n2);
-  sc.first = sc.val + n2;
-  int64_t* size = reinterpret_cast<int64_t*>(base);
-  int64_t* off = size + N;
-  int64_t* rank = off + N;
-  unsigned long long* best = reinterpret_cast<unsigned long long*>(rank + N);
-  unsigned long long* ctr = best + N;                      // [0]: token count, [1]: the BFS frontier size
-  int32_t* order = reinterpret_cast<int32_t*>(ctr + 2);
-  int32_t* parent = order + N;
-  int32_t* cslot = parent + N;
-  int32_t* end = cslot + N;
-  int32_t* surv = end + N;
-  uint8_t* gone = reinterpret_cast<uint8_t*>(surv + N);
-  int32_t* n_next = reinterpret_cast<int32_t*>(ctr + 1);
-  // Breadth-first order of the live nodes, level by level (order[0] = the root).
-  CK(cudaMemsetAsync(order, 0, sizeof(int32_t), r->stream));
-  std::vector<int32_t> lvl{0, 1};
-  for (;;) {
-    const int32_t l = (int32_t)lvl.size() - 2;
-    CK(cudaMemsetAsync(n_next, 0, sizeof(int32_t), r->stream));
-    CK(p2p::launch_lru_bfs(t, order + lvl[(size_t)l], lvl[(size_t)l + 1] - lvl[(size_t)l], order + lvl[(size_t)l + 1],
-                           n_next, (int32_t)(N - lvl[(size_t)l + 1]), parent, cslot, r->num_sms, r->stream));
-    r->launches += 1;
-    int32_t h = 0;
-    CK(d2h(r, &h, n_next, sizeof(h)));
-    if (h == 0) break;
-    if ((int64_t)lvl.back() + h > N) return fail(r, P2P_E_DEVICE, "the LRU tree is inconsistent");
-    lvl.push_back(lvl.back() + h);
-  }
-  const int32_t n_levels = (int32_t)lvl.size() - 1, total = lvl.back();
-  CK(p2p::launch_lru_init(order, total, size, off, rank, best, gone, r->num_sms, r->stream));
-  CK(p2p::launch_lru_levels(t, order, lvl.data(), n_levels, parent, cslot, size, off, rank, best, end, sc, r->num_sms,
-                            r->stream));
-  {
-    int64_t stages = 0, m = total - 1, k2 = 1;
-    for (int32_t lg = 0; k2 < m; ++lg, k2 <<= 1) stages += lg + 1;  // bitonic steps: L (L + 1) / 2 for n2 = 2^L
-    r->launches += 1 + 3 * (n_levels - 1) + (m > 0 ? 4 + stages : 0);
-  }
-  auto count = [&](int mode, uint32_t S, unsigned long long K, unsigned long long& out) -> int {
-    CK(p2p::launch_lru_count(t, order + 1, total - 1, cslot, rank, end, mode, S, K, ctr, r->num_sms, r->stream));
-    r->launches += 1;
-    CK(d2h(r, &out, ctr, sizeof(out)));
-    return P2P_OK;
-  };
-  // The threshold: stamps first, then the (end rank, deeper first) key inside the boundary stamp.
-  unsigned long long all = 0, c = 0;
-  if (int rc = count(0, 0xFFFFFFFFu, 0, all)) return rc;
-  uint32_t S = 0xFFFFFFFFu;
-  unsigned long long K = 0;
-  int32_t cut = 0;
-  const unsigned long long want = (unsigned long long)n_tokens;
-  if (want < all) {
-    uint32_t lo = 0, hi = 0xFFFFFFFFu;  // count(stamp < lo) <= want < count(stamp < hi)
-    while (hi - lo > 1) {
-      const uint32_t mid = lo + (hi - lo) / 2;
-      if (int rc = count(0, mid, 0, c)) return rc;
-      if (c <= want) lo = mid; else hi = mid;
-    }
-    S = lo;
-    if (int rc = count(0, S, 0, c)) return rc;
-    const unsigned long long rest = want - c;
-    if (rest > 0) {
-      unsigned long long lo2 = 0, hi2 = ~0ull;
-      while (hi2 - lo2 > 1) {
-        const unsigned long long mid = lo2 + (hi2 - lo2) / 2;
-        if (int rc = count(1, S, mid, c)) return rc;
-        if (c <= rest) lo2 = mid; else hi2 = mid;
-      }
-      K = lo2;
-      if (int rc = count(1, S, K, c)) return rc;
-      cut = (int32_t)(rest - c);
-    }
-  }
+  const int32_t N = std::max<int32_t>(t.n_node, 1);
+  p2p::LruScratch sc = {};
+  CK(ensure(r, r->lru_buf, p2p::lru_scratch(N, nullptr, sc)));
+  p2p::lru_scratch(N, r->lru_buf.p, sc);
   if (int rc = push_states(r, tree, tree + 1)) return rc;
-  CK(p2p::launch_lru_evict(t, r->d_states + tree, order, lvl.data(), n_levels, parent, cslot, rank, end, S, K, cut, gone,
-                           surv, r->num_sms, r->stream));
-  r->launches += n_levels - 1;
+  CK(p2p::launch_lru_evict(t, r->d_states + tree, sc, N, (unsigned long long)n_tokens, r->stream));
+  r->launches += 1;
+  unsigned long long out[2] = {0, 0};
+  CK(cudaMemcpyAsync(out, sc.out, sizeof(out), cudaMemcpyDeviceToHost, r->stream));
   if (int rc = pull_states(r, tree, tree + 1)) return rc;
+  if (out[1]) return fail(r, P2P_E_DEVICE, "the LRU tree is inconsistent");
   CK(p2p::launch_refresh_views(r->d_states + tree, r->d_views + tree, 1, r->d_shared, r->stream));
   r->launches += 1;
-  if (n_evicted) *n_evicted = (int64_t)std::min(want, all);
+  if (n_evicted) *n_evicted = std::min<int64_t>(n_tokens, (int64_t)out[0]);
   return P2P_OK;
 }
 
