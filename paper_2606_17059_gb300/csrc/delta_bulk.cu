@@ -358,12 +358,13 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
         }
       }
     }
+    int3 want = make_int3(0, 0, 0);
     if (valid) {
       // The op's place and nodes.  An op that ended at a node has its place in the parent's table.
       const bool at_node = pos == q.n;
       const int32_t pu = at_node ? g : u, ppos = at_node ? gpos : pos, v = at_node ? u : -1;
       const uint32_t idx = (uint32_t)i;
-      int32_t ent_u = -1, ent_v = -1, ent_y = -1, key2 = -1, y = -1;
+      int32_t ent_u = -1, ent_v = -1, ent_y = -1, key2 = -1, y = -1, y_len = 0;
       const int32_t key = enter_key(A.tab, tree, pu, q.at(ppos), round, idx);
       if (key < 0) what = B_LEFT;
       if (what == B_FOLD) {  // the one other child of the place's node
@@ -372,7 +373,7 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
         if (bits <= kFoldBits)
           for (int32_t s = 0; s < (1 << bits); ++s) {
             const int4 e = __ldg(child + rec.x + s);
-            if (e.y >= 1 && e.y != v) y = e.y;
+            if (e.y >= 1 && e.y != v) y = e.y, y_len = e.w;
           }
         if (y < 0 || gg < 0) what = B_LEFT;
       }
@@ -407,6 +408,10 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
         if (key2 < 0 || ent_y < 0) what = B_LEFT;
         else atomicMax(&A.tab.nodes[ent_y].alone, ~idx);
       }
+      // At most this much room.
+      if (what == B_LEAF) want = make_int3(1, 0, q.n - ppos);
+      if (what == B_SPLIT) want = make_int3(2, 1 << kMinTabBits, q.n - ppos - k);
+      if (what == B_FOLD) want = make_int3(0, 0, ppos - ggpos + y_len);
       int4* out = reinterpret_cast<int4*>(A.ops + i);
       out[0] = make_int4(what | flags | tree << kTreeShift, pu, ppos, k);
       out[1] = make_int4(v, gg, ggpos, key);
@@ -414,22 +419,28 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
     } else if (lane < per && i < A.n && b0 + lane < total && !A.done[i]) {
       A.ops[i].what = B_LEFT;  // an empty sequence
     }
+    // The room the round may take, once per tree and warp.
+    for (unsigned m = __ballot_sync(kFull, want.x | want.y | want.z); m;) {
+      const int32_t t = __shfl_sync(kFull, tree, __ffs(m) - 1);
+      const bool mine = (want.x | want.y | want.z) && tree == t;
+      m &= ~__ballot_sync(kFull, mine);
+      unsigned n = mine ? want.x : 0, c = mine ? want.y : 0;
+      unsigned long long l = mine ? want.z : 0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        n += __shfl_xor_sync(kFull, n, o);
+        c += __shfl_xor_sync(kFull, c, o);
+        l += __shfl_xor_sync(kFull, l, o);
+      }
+      const unsigned long long v = lane == 0 ? n : lane == 1 ? c : l;
+      if (lane < 3 && v) atomicAdd(&A.want[((int64_t)round * A.n_trees + t) * 3 + lane], v);
+    }
   }
 }
 
-// Reserves k units of a tree's counter; -1 if they do not fit.  Every warp of a launch may be after the same counter,
-// where compare-and-swap loops take turns failing (4,096 ops of one tree: 1.5 ms), so it is an addition, taken back
-// when it went too far.  Only arenas and requests small enough that additions still to be taken back cannot wrap the
-// counter round (2^30, and 2^17 for each of the warps in flight) are served so.
+// Reserves k units of a tree's counter; -1 if they do not fit.
 __device__ int32_t reserve(int32_t* ctr, int32_t cap, int64_t k) {
   int32_t old = *(volatile int32_t*)ctr;
-  if (cap <= (1 << 30) && k <= (1 << 17)) {
-    if ((int64_t)old + k > cap) return -1;
-    old = atomicAdd(ctr, (int32_t)k);
-    if ((int64_t)old + k <= cap) return old;
-    atomicSub(ctr, (int32_t)k);
-    return -1;
-  }
   for (int it = 0; it < (1 << 20); ++it) {
     if ((int64_t)old + k > cap) return -1;
     const int32_t prev = atomicCAS(ctr, old, (int32_t)(old + k));
@@ -437,6 +448,13 @@ __device__ int32_t reserve(int32_t* ctr, int32_t cap, int64_t k) {
     old = prev;
   }
   return -1;
+}
+// The same where every reservation of the launch together asks for at most `most` units.  Warps that all compare and
+// swap one counter take turns failing (4,096 ops of one tree: 1.5 ms); while there is room for all of them, now and so
+// to the launch's end, an addition cannot go too far and none has to be taken back.
+__device__ int32_t reserve(int32_t* ctr, int32_t cap, int64_t k, unsigned long long most) {
+  if ((unsigned long long)*(volatile int32_t*)ctr + most <= (unsigned long long)cap) return atomicAdd(ctr, (int32_t)k);
+  return reserve(ctr, cap, k);
 }
 __device__ __forceinline__ void add64(int64_t* p, int64_t v) {
   if (v) atomicAdd((unsigned long long*)p, (unsigned long long)v);
@@ -662,10 +680,11 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
       const int32_t tn = __shfl_sync(kFull, sn, 31), tc = __shfl_sync(kFull, sc, 31);
       const int64_t tl = __shfl_sync(kFull, sl, 31);
       TreeState* ts = A.states + t;
+      const unsigned long long* most = A.want + ((int64_t)round * A.n_trees + t) * 3;
       int32_t r = 0;
-      if (lane == 0 && tn) r = reserve(&ts->n_node, ts->cap_node, tn);
-      if (lane == 1 && tc) r = reserve(&ts->n_child, ts->cap_child, tc);
-      if (lane == 2 && tl) r = reserve(&ts->n_label, ts->cap_label, tl);
+      if (lane == 0 && tn) r = reserve(&ts->n_node, ts->cap_node, tn, most[0]);
+      if (lane == 1 && tc) r = reserve(&ts->n_child, ts->cap_child, tc, most[1]);
+      if (lane == 2 && tl) r = reserve(&ts->n_label, ts->cap_label, tl, most[2]);
       const bool ok = __all_sync(kFull, r >= 0);
       if (!ok) {  // what was taken stays behind as stale space
         if (lane == 0 && tn && r >= 0) add64(&ts->dead_nodes, tn);
@@ -812,7 +831,7 @@ cudaError_t launch_bulk(const BulkArgs& A, int num_sms, cudaStream_t st, int* la
   if (A.n <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(A.tab.keys, 0, ((size_t)A.tab.key_mask + 1) * sizeof(BulkKey), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(A.tab.nodes, 0, ((size_t)A.tab.node_mask + 1) * sizeof(BulkNode), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(A.counts, 0, (kBulkRounds + 2) * sizeof(int32_t), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(A.want, 0, A.n_want * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   // A warp per op up to a full wave of resident CTAs (the kernels then take more ops per warp).
   const int grid = (int)std::min<int64_t>((A.n + kBulkWarps - 1) / kBulkWarps, (int64_t)num_sms * kBulkCtasPerSm);
@@ -826,7 +845,7 @@ cudaError_t launch_bulk(const BulkArgs& A, int num_sms, cudaStream_t st, int* la
   return cudaGetLastError();
 }
 
-size_t bulk_scratch(int64_t n, void* base, BulkArgs& A) {
+size_t bulk_scratch(int64_t n, int32_t n_trees, void* base, BulkArgs& A) {
   int64_t keys = 1024, nodes = 1024;
   while (keys < 4 * n) keys <<= 1;
   while (nodes < 2 * n) nodes <<= 1;
@@ -843,7 +862,9 @@ size_t bulk_scratch(int64_t n, void* base, BulkArgs& A) {
   A.tab.node_mask = (uint32_t)(nodes - 1);
   A.ops = static_cast<BulkOp*>(take((size_t)n * sizeof(BulkOp)));
   A.lists = static_cast<int32_t*>(take((size_t)n * 2 * sizeof(int32_t)));
-  A.counts = static_cast<int32_t*>(take((kBulkRounds + 2) * sizeof(int32_t)));
+  A.n_want = (size_t)kBulkRounds * n_trees * 3 + (kBulkRounds + 3) / 2;  // the counts behind them
+  A.want = static_cast<unsigned long long*>(take(A.n_want * sizeof(unsigned long long)));
+  A.counts = reinterpret_cast<int32_t*>(A.want + (size_t)kBulkRounds * n_trees * 3);
   return at;
 }
 

@@ -233,11 +233,13 @@ struct BulkArgs {
   BulkTables tab;  // from here on: scratch (bulk_scratch)
   BulkOp* ops;     // [n]
   int32_t* lists;  // [2n]: the op indices of odd and even rounds
-  int32_t* counts; // [kBulkRounds + 2]: list sizes by round
+  unsigned long long* want;  // [kBulkRounds * n_trees * 3]: nodes, slots and tokens a round may take, at most
+  size_t n_want;             // words from want on, counts included
+  int32_t* counts;           // [kBulkRounds + 2]: list sizes by round
 };
 constexpr int kBulkRounds = 3;
-// The bytes of scratch for n ops; with base, also sets A's scratch pointers into it.
-size_t bulk_scratch(int64_t n, void* base, BulkArgs& A);
+// The bytes of scratch for n ops of n_trees trees; with base, also sets A's scratch pointers into it.
+size_t bulk_scratch(int64_t n, int32_t n_trees, void* base, BulkArgs& A);
 cudaError_t launch_bulk(const BulkArgs& A, int num_sms, cudaStream_t st, int* launched);
 
 // Compaction: copies the live part of a tree (everything reachable from the root) into fresh arrays, with

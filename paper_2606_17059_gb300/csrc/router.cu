@@ -1359,11 +1359,11 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
   p2p::BulkArgs bulk = {};
   bool use_bulk = max_runs <= 2 && n <= kBulkMaxOps;
   if (use_bulk) {
-    if (ensure(r, r->bulk, p2p::bulk_scratch(n, nullptr, bulk)) != cudaSuccess) {
+    if (ensure(r, r->bulk, p2p::bulk_scratch(n, nt, nullptr, bulk)) != cudaSuccess) {
       (void)cudaGetLastError();
       use_bulk = false;
     } else {
-      p2p::bulk_scratch(n, r->bulk.p, bulk);
+      p2p::bulk_scratch(n, nt, r->bulk.p, bulk);
       bulk.states = r->d_states + p0;
       bulk.n_trees = nt;
       bulk.peer_begin = peer == -1 ? d_pb : nullptr;

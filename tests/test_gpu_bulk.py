@@ -130,3 +130,15 @@ def test_a_root_table_that_has_to_grow():
     seqs = [[rng.randrange(1 << 20)] + [rng.randrange(9) for _ in range(rng.randint(0, 90))] for _ in range(5000)]
     sl = seqlist_from_lists(seqs)
     _check(r, trees, [(0, [0] * 5000, sl), (0, [1] * 5000, sl)], seqs[:300])
+
+
+@pytest.mark.parametrize("seed", range(12))
+def test_room_running_out(seed):
+    """INSERTs that run out of node, slot and label room again and again while other warps still find some: every
+    reservation keeps its own room."""
+    rng = random.Random(seed)
+    sls = [seqlist_from_lists([[1, 2, 3]]) for _ in range(4)]
+    r, trees = router_from_seqlists(sls), oracle.build_trees(sls)
+    for p in range(4):
+        seqs = [[rng.randrange(60) for _ in range(rng.randint(1, 90))] for _ in range(2500)]
+        _check(r, trees, [(p, [0] * 2500, seqlist_from_lists(seqs))], seqs[:50])
