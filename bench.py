@@ -59,8 +59,8 @@ CSRC = os.path.join(ROOT, "paper_2606_17059_gb300", "csrc")
 # Source file of each kernel (with internal.h, the layout they share): a DRAM-traffic figure holds only for
 # the source it was captured on.
 KERNEL_SOURCE = {
-    "group_hash_kernel": "group_kernel.cu", "group_resolve_kernel": "group_kernel.cu",
-    "group_resolve32_kernel": "group_kernel.cu", "route_kernel": "route_kernel.cu",
+    "group_hash_kernel": "group_kernel.cu",
+    "group_resolve_kernel": "group_kernel.cu", "route_kernel": "route_kernel.cu",
     "lane_kernel<true>": "route_kernel.cu", "lane_kernel<false>": "route_kernel.cu", "decide_kernel": "route_kernel.cu",
     "validate_kernel": "delta_kernel.cu", "init_ranges_kernel": "delta_kernel.cu", "delta_kernel": "delta_kernel.cu",
     "compact_kernel": "delta_kernel.cu", "compact_labels_kernel": "delta_kernel.cu",
@@ -502,9 +502,9 @@ def run_ours(args):
         kt = {k["kernel"]: k for k in kernels}
         # ---- the route step: compulsory bytes, and the oracle's touched bytes ----
         compulsory = 4 * int(n_tok) + 8 * (B + 1) + 4 * B * P + 4 * B
-        route = {"kernels": [k for k in ("group_hash_kernel", "group_resolve_kernel", "group_resolve32_kernel",
-                                         "group_ranges_kernel", "group_place_kernel", "route_kernel",
-                                         "lane_kernel<true>", "lane_kernel<false>") if k in kt],
+        route = {"kernels": [k for k in ("group_hash_kernel", "group_resolve_kernel", "group_ranges_kernel",
+                                         "group_place_kernel", "route_kernel", "lane_kernel<true>",
+                                         "lane_kernel<false>") if k in kt],
                  "ms": route_avg_ms, "compulsory_bytes": compulsory}
         # Device time of the route kernels (with p2p_route_prepare the grouping runs alongside the delta kernel,
         # outside the route span), the time the route's bytes are measured against.

@@ -13,8 +13,8 @@
 // and inserted into an open-addressing table; the smallest request index with that key leads the group.
 // A follower whose exact common prefix with its leader is shorter than kGroupHead (a hash collision) routes
 // as a leader instead.  The leader choice is deterministic (smallest index); the order of the two request
-// lists is not, and only affects scheduling.  Each group's followers take a contiguous range of the follower
-// list (group_ranges_kernel, group_place_kernel): the warps that route them at the same time then read the
+// lists is not, and only affects scheduling.  In a large batch each group's followers take a contiguous range of the
+// follower list (group_ranges_kernel, group_place_kernel): the warps that route them at the same time then read the
 // leader's match row, its checkpoints and the tables at the checkpoint nodes once, from cache.
 #include "internal.h"
 
@@ -39,31 +39,49 @@ __device__ __forceinline__ bool request_range(const int64_t* offsets, int64_t b,
   return start >= 0 && start <= end && end <= n_tokens;
 }
 
-// One warp per 32 consecutive requests (lane i owns request base + i).  The warp hashes each request's
-// first kGroupHead tokens in turn (one token per lane and position, each mixed with its position, summed);
-// then every distinct key of the 32 is looked up or claimed once, by its lowest lane, which also lowers
-// the key's leader index to that lane's request (the smallest of the warp's requests with the key).
+// One warp per `per` consecutive requests (lane i < per owns request base + i).  Eight lanes hash a request: four
+// requests a step and two steps in flight, each lane eight tokens of each (token 8 j + s by lane s), mixed with
+// their positions and summed.  (A request at a time by the whole warp, 32 in series, took 31 us for 65,536
+// requests and 30 for 8,191; now 17 and 9.)  Then every distinct key of the warp is looked up or claimed once, by its lowest lane, which also
+// lowers the key's leader index to that lane's request (the smallest of the warp's requests with the key).
 __global__ void __launch_bounds__(kGroupThreads) group_hash_kernel(
     const int32_t* __restrict__ tokens, int64_t n_tokens, int64_t tok_base, const int64_t* __restrict__ offsets,
-    int64_t B, unsigned long long* keys, int32_t* vals, int32_t bits, int32_t* slot_of) {
-  static_assert(kGroupHead == 64, "two tokens per lane");
-  const int lane = threadIdx.x & 31;
+    int64_t B, int32_t per, unsigned long long* keys, int32_t* vals, int32_t bits, int32_t* slot_of) {
+  static_assert(kGroupHead == 64, "eight tokens for each of eight lanes");
+  const int lane = threadIdx.x & 31, sub = lane & 7;
   const int64_t warps = (int64_t)gridDim.x * (kGroupThreads / 32);
   const uint32_t mask = (1u << bits) - 1;
-  for (int64_t base = (((int64_t)blockIdx.x * kGroupThreads + threadIdx.x) >> 5) * 32; base < B; base += warps * 32) {
-    unsigned long long my_h = 0;  // 0: the lane's request is not grouped
-    for (int r = 0; r < 32 && base + r < B; ++r) {
-      int64_t start, len;
-      if (!request_range(offsets, base + r, tok_base, n_tokens, start, len) || len < kGroupHead) continue;
-      const int32_t* g = tokens + start;
-      unsigned long long h = mix64((unsigned long long)(uint32_t)__ldg(g + lane) | ((unsigned long long)lane << 32)) +
-                             mix64((unsigned long long)(uint32_t)__ldg(g + lane + 32) |
-                                   ((unsigned long long)(lane + 32) << 32));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(kFull, h, o);
-      h |= 1ull;  // 0 marks an empty slot
-      if (lane == r) my_h = h;
+  for (int64_t base = (((int64_t)blockIdx.x * kGroupThreads + threadIdx.x) >> 5) * per; base < B; base += warps * per) {
+    int64_t my_start = -1, len;  // -1: the lane's request is not grouped
+    if (lane < per && base + lane < B) {
+      const bool ok = request_range(offsets, base + lane, tok_base, n_tokens, my_start, len);
+      if (!ok || len < kGroupHead) my_start = -1;
     }
+    unsigned long long my_h = 0;
+    for (int r0 = 0; r0 < per; r0 += 8) {
+      unsigned long long h[2];
+      int32_t x[2][8];
+      int64_t st[2];
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        st[c] = __shfl_sync(kFull, my_start, (r0 + 4 * c + (lane >> 3)) & 31);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[c][j] = st[c] >= 0 ? __ldg(tokens + st[c] + 8 * j + sub) : 0;
+      }
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        h[c] = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          h[c] += mix64((unsigned long long)(uint32_t)x[c][j] | ((unsigned long long)(8 * j + sub) << 32));
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) h[c] += __shfl_xor_sync(kFull, h[c], o);
+        // Lane r0 + 4 c + q owns the request that lanes 8 q .. 8 q + 7 hashed.
+        const unsigned long long mine = __shfl_sync(kFull, h[c], (lane & 3) * 8);
+        if ((lane >> 2) == (r0 >> 2) + c) my_h = mine | 1ull;  // 0 marks an empty slot
+      }
+    }
+    if (my_start < 0) my_h = 0;
     const unsigned same = __match_any_sync(kFull, my_h);
     const int first = __ffs(same) - 1;
     int32_t slot = -1;
@@ -79,13 +97,13 @@ __global__ void __launch_bounds__(kGroupThreads) group_hash_kernel(
       if (slot >= 0) atomicMin(&vals[slot], (int32_t)(base + lane));
     }
     slot = __shfl_sync(kFull, slot, first);
-    if (base + lane < B) slot_of[base + lane] = my_h ? slot : -1;
+    if (lane < per && base + lane < B) slot_of[base + lane] = my_h ? slot : -1;
   }
 }
 
-// First position in [0, n) where a and b differ, or n (one warp, both in global memory).
+// First position in [0, n) where a and b differ, or n (one warp, both in global memory; 32 U tokens per step).
+template <int U>
 __device__ int64_t lcp_warp(const int32_t* __restrict__ a, const int32_t* __restrict__ b, int64_t n, int lane) {
-  constexpr int U = 8;
   int64_t j0 = 0;
   for (; j0 + 32 * U <= n; j0 += 32 * U) {
     int32_t x[U];
@@ -110,21 +128,23 @@ __device__ int64_t lcp_warp(const int32_t* __restrict__ a, const int32_t* __rest
   return n;
 }
 
-// One warp per 32 consecutive requests (lane i owns request base + i): each request's leader; for each
-// follower in turn, the exact common prefix with its leader (the whole warp compares); then the warp's
-// leaders are appended to lists[0 ..) with one counter update, and each follower takes its rank in its group
-// (fcnt[leader] counts them; the rank goes to slot_of[b]).  counts and fcnt must start at zero, gid at -1 and
-// cmin at INT32_MAX.  A leader with followers gets the smallest of their common prefixes in cmin and, while
-// rows last, a checkpoint row in gid (one update per distinct leader of the warp's followers).
-__global__ void __launch_bounds__(kGroupThreads) group_resolve32_kernel(
+// One warp per `per` consecutive requests (lane i < per owns request base + i): each request's leader; for each follower
+// in turn, the exact common prefix with its leader (the whole warp compares); then the warp's leaders are
+// appended to lists[0 ..) with one counter update, and so are its followers to lists[B ..) if `place` is set; if not,
+// each follower takes its rank in its group (fcnt[leader] counts them; the rank goes to slot_of[b]) and
+// group_ranges_kernel and group_place_kernel make the list.  A leader with followers gets the smallest of their common
+// prefixes in cmin and, while rows last, a checkpoint row in gid (one update per distinct leader of the warp's
+// followers).  U: 16 for long requests, whose longest compares bound the kernel, else 8 (more resident warps).
+template <int U>
+__global__ void __launch_bounds__(kGroupThreads) group_resolve_kernel(
     const int32_t* __restrict__ tokens, int64_t n_tokens, int64_t tok_base, const int64_t* __restrict__ offsets,
-    int64_t B, const int32_t* __restrict__ vals, int32_t* slot_of, int32_t* lead, int32_t* cpre, int32_t* lists,
-    int32_t* counts, int32_t* gid, int32_t* cmin, int32_t gcap, int32_t* fcnt) {
+    int64_t B, int32_t per, bool place, const int32_t* __restrict__ vals, int32_t* slot_of, int32_t* lead,
+    int32_t* cpre, int32_t* lists, int32_t* counts, int32_t* gid, int32_t* cmin, int32_t gcap, int32_t* fcnt) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (kGroupThreads / 32);
-  for (int64_t base = (((int64_t)blockIdx.x * kGroupThreads + threadIdx.x) >> 5) * 32; base < B; base += warps * 32) {
+  for (int64_t base = (((int64_t)blockIdx.x * kGroupThreads + threadIdx.x) >> 5) * per; base < B; base += warps * per) {
     const int64_t b = base + lane;
-    const bool valid = b < B;
+    const bool valid = lane < per && b < B;
     const int32_t s = valid ? slot_of[b] : -1;
     const int32_t l = s >= 0 ? vals[s] : (int32_t)b;
     int32_t my_c = -1;
@@ -134,25 +154,21 @@ __global__ void __launch_bounds__(kGroupThreads) group_resolve32_kernel(
       int64_t sb, nb, sl, nl;  // both requests are valid and hold at least kGroupHead tokens
       request_range(offsets, base + r, tok_base, n_tokens, sb, nb);
       request_range(offsets, lr, tok_base, n_tokens, sl, nl);
-      int64_t c = lcp_warp(tokens + sb, tokens + sl, min(nb, nl), lane);
+      int64_t c = lcp_warp<U>(tokens + sb, tokens + sl, min(nb, nl), lane);
       if (c < kGroupHead || c > INT32_MAX) c = -1;
       if (lane == r) my_c = (int32_t)c;
     }
     const bool is_f = my_c >= 0;
     const unsigned lm = __ballot_sync(kFull, valid && !is_f), fm = __ballot_sync(kFull, is_f);
-    int32_t lbase = 0, fbase = 0;
-    if (lane == 0) {
-      if (lm) lbase = atomicAdd(&counts[0], __popc(lm));
-      if (fm) fbase = atomicAdd(&counts[1], __popc(fm));
-    }
-    lbase = __shfl_sync(kFull, lbase, 0);
-    fbase = __shfl_sync(kFull, fbase, 0);
+    int32_t at = 0;
+    if (lane == 0 && lm) at = atomicAdd(&counts[0], __popc(lm));
+    if (lane == 1 && fm) at = atomicAdd(&counts[1], __popc(fm));
+    const int32_t lbase = __shfl_sync(kFull, at, 0), fbase = __shfl_sync(kFull, at, 1);
     const unsigned below = (1u << lane) - 1;
     if (valid && !is_f) {
       lead[b] = (int32_t)b;
       lists[lbase + __popc(lm & below)] = (int32_t)b;
     }
-    (void)fbase;
     const unsigned same = __match_any_sync(kFull, is_f ? l : -1);
     if (is_f) {
       lead[b] = l;
@@ -161,73 +177,18 @@ __global__ void __launch_bounds__(kGroupThreads) group_resolve32_kernel(
       const int first = __ffs(same) - 1;
       int32_t rbase = 0;
       if (lane == first) {
-        atomicMin(&cmin[l], c_min);
-        rbase = atomicAdd(&fcnt[l], __popc(same));
-        if (atomicCAS(&gid[l], -1, -2) == -1) {  // the leader's first follower gives it a row
-          const int32_t row = atomicAdd(&counts[2], 1);
-          atomicExch(&gid[l], row < gcap ? row : -1);
+        if (c_min < *(volatile int32_t*)&cmin[l]) atomicMin(&cmin[l], c_min);
+        if (!place) rbase = atomicAdd(&fcnt[l], __popc(same));
+        if (*(volatile int32_t*)&gid[l] == kNoRow && atomicCAS(&gid[l], kNoRow, -1) == kNoRow) {
+          const int32_t row = atomicAdd(&counts[2], 1);  // the leader's first follower gives it a row
+          if (row < gcap) atomicExch(&gid[l], row);
         }
       }
-      slot_of[b] = __shfl_sync(same, rbase, first) + __popc(same & below);  // rank in the group
+      if (place)
+        lists[B + fbase + __popc(fm & below)] = (int32_t)b;
+      else
+        slot_of[b] = __shfl_sync(same, rbase, first) + __popc(same & below);  // rank in the group
     }
-  }
-}
-
-// One warp per request: its leader and the exact common prefix with it; the CTA's leaders of a round are
-// then appended to lists[0 ..) with one counter update per round, and the followers counted (one update per
-// round) and ranked in their groups as in group_resolve32_kernel.  counts and fcnt must start at zero, gid at
-// -1 and cmin at INT32_MAX.  A leader with followers gets the smallest of their common prefixes in cmin
-// (updated only when a follower lowers it, so popular groups make few atomics) and, while rows last, a
-// checkpoint row in gid.
-__global__ void __launch_bounds__(kGroupThreads) group_resolve_kernel(
-    const int32_t* __restrict__ tokens, int64_t n_tokens, int64_t tok_base, const int64_t* __restrict__ offsets,
-    int64_t B, const int32_t* __restrict__ vals, int32_t* slot_of, int32_t* lead, int32_t* cpre, int32_t* lists,
-    int32_t* counts, int32_t* gid, int32_t* cmin, int32_t gcap, int32_t* fcnt) {
-  constexpr int kWarps = kGroupThreads / 32;
-  __shared__ int s_kind[kWarps];  // 0: none, 1: leader, 2: follower
-  __shared__ int s_pos[kWarps];   // the request's index in its list
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int64_t r0 = (int64_t)blockIdx.x * kWarps; r0 < B; r0 += (int64_t)gridDim.x * kWarps) {
-    const int64_t b = r0 + warp;
-    int kind = 0;
-    int32_t l = -1, c32 = -1;
-    if (b < B) {
-      const int32_t s = slot_of[b];
-      l = s >= 0 ? vals[s] : (int32_t)b;
-      int64_t c = -1;
-      if (l != (int32_t)b) {  // both requests are valid and hold at least kGroupHead tokens
-        int64_t sb, nb, sl, nl;
-        request_range(offsets, b, tok_base, n_tokens, sb, nb);
-        request_range(offsets, l, tok_base, n_tokens, sl, nl);
-        c = lcp_warp(tokens + sb, tokens + sl, min(nb, nl), lane);
-        if (c < kGroupHead || c > INT32_MAX) c = -1;
-      }
-      kind = c < 0 ? 1 : 2;
-      c32 = (int32_t)c;
-    }
-    if (lane == 0) s_kind[warp] = kind;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int nl = 0, nf = 0;
-      for (int w = 0; w < kWarps; ++w) nl += s_kind[w] == 1, nf += s_kind[w] == 2;
-      const int bl = nl ? atomicAdd(&counts[0], nl) : 0, bf = nf ? atomicAdd(&counts[1], nf) : 0;
-      for (int w = 0, il = 0, jf = 0; w < kWarps; ++w) s_pos[w] = s_kind[w] == 1 ? bl + il++ : s_kind[w] == 2 ? bf + jf++ : 0;
-    }
-    __syncthreads();
-    if (lane == 0 && kind == 1) {
-      lead[b] = (int32_t)b;
-      lists[s_pos[warp]] = (int32_t)b;
-    } else if (lane == 0 && kind == 2) {
-      lead[b] = l;
-      cpre[b] = c32;
-      slot_of[b] = atomicAdd(&fcnt[l], 1);  // rank in the group (slot_of[b] was read above)
-      if (c32 < *(volatile int32_t*)&cmin[l]) atomicMin(&cmin[l], c32);
-      if (*(volatile int32_t*)&gid[l] == -1 && atomicCAS(&gid[l], -1, -2) == -1) {
-        const int32_t row = atomicAdd(&counts[2], 1);  // the leader's first follower gives it a row
-        atomicExch(&gid[l], row < gcap ? row : -1);
-      }
-    }
-    __syncthreads();  // s_kind and s_pos are reused next round
   }
 }
 
@@ -266,48 +227,50 @@ __global__ void __launch_bounds__(kGroupThreads) group_place_kernel(int64_t B, c
 
 }  // namespace
 
+// CTAs a SM of the resolve kernel (by its registers).  A warp gets as many requests as give every resident warp about
+// the same (one counter update serves them all): 65,536 requests 65 us, 80 from a work cursor in smaller pieces.
+constexpr int64_t kResolveCtas = 6;
+
+// Below this many bytes of match matrix the followers of short requests are listed as they come: their leaders' rows,
+// checkpoints and tables stay in L2 (126 MB) whatever the order, and two launches are spared (65,536 requests
+// of 1,250 tokens on 16 trees: the follower pass 37 -> 41 us, 12 us of launches less).  Above it a group's followers
+// lie side by side: the follower pass of 200,003 requests on 64 trees takes 217 us so and 234 as they come, of 8,191
+// requests of 11,400 tokens on 32 trees 147 and 192, of 1,048,576 on 256 it reads 15.5 GB instead of 22.  (A single
+// tree's row is 4 bytes and its requests have no choice of route: that path is left as it was.)
+constexpr int64_t kPlaceBytes = (int64_t)8 << 20;
+
 cudaError_t launch_group(const int32_t* tokens, int64_t n_tokens, int64_t tok_base, const int64_t* offsets, int64_t B,
-                         const GroupScratch& g, int num_sms, cudaStream_t st) {
+                         int32_t P, const GroupScratch& g, int num_sms, cudaStream_t st, int* launched) {
+  *launched = 0;
   if (B <= 0) return cudaSuccess;
-  const size_t slots = (size_t)1 << g.bits;
-  cudaError_t e = cudaMemsetAsync(g.keys, 0, slots * sizeof(unsigned long long), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(g.vals, 0x7f, slots * sizeof(int32_t), st);  // 0x7f7f7f7f > any index
-  if (e == cudaSuccess) e = cudaMemsetAsync(g.counts, 0, 8 * sizeof(int32_t), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(g.fcnt, 0, (size_t)B * sizeof(int32_t), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(g.gid, 0xff, (size_t)B * sizeof(int32_t), st);   // -1
-  if (e == cudaSuccess) e = cudaMemsetAsync(g.cmin, 0x7f, (size_t)B * sizeof(int32_t), st);  // > any prefix
+  constexpr int kWarps = kGroupThreads / 32;
+  const int64_t warps = (int64_t)num_sms * kResolveCtas * kWarps;
+  const int32_t per = (int32_t)std::min<int64_t>(32, long_requests(B, n_tokens) ? 1 : (B + warps - 1) / warps);
+  const int32_t per_hash = B < 16 * warps ? 8 : 32;  // (eight requests are hashed at a time)
+  const bool place = P > 1 && B * P * (int64_t)sizeof(int32_t) <= kPlaceBytes && !long_requests(B, n_tokens);
+  cudaError_t e = cudaMemsetAsync(g.keys, 0, g.n_zero, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g.vals, 0x7f, g.n_large, st);
   if (e != cudaSuccess) return e;
-  const int64_t hash_ctas = ((B + 31) / 32 + kGroupThreads / 32 - 1) / (kGroupThreads / 32);  // a warp per 32 requests
-  const int64_t resolve_ctas = (B + kGroupThreads / 32 - 1) / (kGroupThreads / 32);            // a warp per request
-  const int grid = (int)std::min<int64_t>(hash_ctas, (int64_t)num_sms * 8);
-  const int grid2 = (int)std::min<int64_t>(resolve_ctas, (int64_t)num_sms * 8);
+  auto grid_for = [&](int64_t items, int64_t per_cta, int64_t most = 8) {
+    return (int)std::min<int64_t>((items + per_cta - 1) / per_cta, (int64_t)num_sms * most);
+  };
   P2P_TIMED(K_GROUP_HASH, st,
-            (group_hash_kernel<<<grid, kGroupThreads, 0, st>>>(tokens, n_tokens, tok_base, offsets, B, g.keys, g.vals,
-                                                               g.bits, g.slot_of)));
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // Large batches: a warp per 32 requests (at least 32 warps per SM still busy; fewest atomics).  Smaller
-  // ones: a warp per request, so that the common-prefix compares spread over as many warps as there are
-  // requests.
-  if (B >= (int64_t)num_sms * 32 * 32) {
-    P2P_TIMED(K_GROUP_RESOLVE32, st,
-              (group_resolve32_kernel<<<grid, kGroupThreads, 0, st>>>(tokens, n_tokens, tok_base, offsets, B, g.vals,
-                                                                      g.slot_of, g.lead, g.cpre, g.lists, g.counts,
-                                                                      g.gid, g.cmin, g.gcap, g.fcnt)));
-  } else {
-    P2P_TIMED(K_GROUP_RESOLVE, st,
-              (group_resolve_kernel<<<grid2, kGroupThreads, 0, st>>>(tokens, n_tokens, tok_base, offsets, B, g.vals,
-                                                                     g.slot_of, g.lead, g.cpre, g.lists, g.counts,
-                                                                     g.gid, g.cmin, g.gcap, g.fcnt)));
+            (group_hash_kernel<<<grid_for(B, (int64_t)kWarps * per_hash), kGroupThreads, 0, st>>>(
+                tokens, n_tokens, tok_base, offsets, B, per_hash, g.keys, g.vals, g.bits, g.slot_of)));
+  const auto resolve = long_requests(B, n_tokens) ? group_resolve_kernel<16> : group_resolve_kernel<8>;
+  P2P_TIMED(K_GROUP_RESOLVE, st,
+            (resolve<<<grid_for(B, (int64_t)kWarps * per), kGroupThreads, 0, st>>>(
+                tokens, n_tokens, tok_base, offsets, B, per, place, g.vals, g.slot_of, g.lead, g.cpre, g.lists,
+                g.counts, g.gid, g.cmin, g.gcap, g.fcnt)));
+  *launched = 2;
+  if (!place) {  // each group's followers side by side in the follower list
+    P2P_TIMED(K_GROUP_RANGES, st,
+              (group_ranges_kernel<<<grid_for(B, kGroupThreads), kGroupThreads, 0, st>>>(B, g.fcnt, g.counts)));
+    P2P_TIMED(K_GROUP_PLACE, st,
+              (group_place_kernel<<<grid_for(B, kGroupThreads), kGroupThreads, 0, st>>>(B, g.lead, g.slot_of, g.fcnt,
+                                                                                       g.lists)));
+    *launched = 4;
   }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // Each group's followers side by side in the follower list.
-  const int64_t place_ctas = (B + kGroupThreads - 1) / kGroupThreads;
-  const int grid3 = (int)std::min<int64_t>(place_ctas, (int64_t)num_sms * 8);
-  P2P_TIMED(K_GROUP_RANGES, st, (group_ranges_kernel<<<grid, kGroupThreads, 0, st>>>(B, g.fcnt, g.counts)));
-  P2P_TIMED(K_GROUP_PLACE, st,
-            (group_place_kernel<<<grid3, kGroupThreads, 0, st>>>(B, g.lead, g.slot_of, g.fcnt, g.lists)));
   return cudaGetLastError();
 }
 

@@ -105,7 +105,7 @@ constexpr int32_t kMaxTabBits = 26;  // slots ever claimed must fit the 27 bits 
 // Launchers bracket every launch with clock_mark(id, ...); a router whose clock is on installs it in
 // t_clock for the duration of an API call on the calling thread (one router per host thread at a time).
 enum KernelId {
-  K_GROUP_HASH, K_GROUP_RESOLVE, K_GROUP_RESOLVE32, K_ROUTE_STAGED, K_LANE_LEADER, K_LANE_FOLLOWER, K_DECIDE,
+  K_GROUP_HASH, K_GROUP_RESOLVE, K_ROUTE_STAGED, K_LANE_LEADER, K_LANE_FOLLOWER, K_DECIDE,
   K_VALIDATE, K_INIT_RANGES, K_DELTA, K_COMPACT, K_COMPACT_LABELS, K_REFRESH_VIEWS, K_SET_TREE,
   K_UPDATE_COUNT, K_UPDATE_SCAN, K_UPDATE_SCATTER, K_GROUP_RANGES, K_GROUP_PLACE, K_LRU_WALK, K_LRU_STAMP,
   K_LRU_EVICT, K_LRU_OPS, K_HIT_RATE, K_ROOM, K_BULK_RESOLVE, K_BULK_GROW, K_BULK_APPLY, K_COUNT_
@@ -133,28 +133,37 @@ enum { ERR_BAD_OFFSETS = 1, ERR_CORRUPT_TREE = 2, ERR_STALL = 4 };
 
 // Shared-prefix groups of a batch (group_kernel.cu): requests of at least kGroupHead tokens are grouped by
 // their first kGroupHead tokens; lead[b] is b's group leader, cpre[b] its exact common prefix with the
-// leader (followers only); lists[0 .. counts[0]) are the leaders, lists[B .. B + counts[1]) the followers,
-// each group's followers side by side (so the warps routing them at the same time share the leader's row,
+// leader (followers only); lists[0 .. counts[0]) are the leaders, lists[B .. B + counts[1]) the followers, in a
+// large batch each group's side by side (so the warps routing them at the same time share the leader's row,
 // checkpoints and tables in cache).
 constexpr int kGroupHead = 64;
 struct GroupScratch {
+  // Cleared to zero by the launch, in one piece from keys on (n_zero bytes):
   unsigned long long* keys;  // 2^bits slots
-  int32_t* vals;             // 2^bits slots
+  int32_t* fcnt;     // [B]: a leader's follower count, then the start of its followers' range
+  int32_t* counts;   // [8]: leaders, followers, groups with a checkpoint row, the leader pass's work cursor,
+                     //      the follower ranges handed out
+  size_t n_zero;
+  // Set to 0x7f bytes (larger than any index or prefix), in one piece from vals on (n_large bytes):
+  int32_t* vals;     // 2^bits slots
+  int32_t* gid;      // [B]: a leader's checkpoint row (kNoRow or -1: none)
+  int32_t* cmin;     // [B]: a leader's smallest common prefix with its followers
+  size_t n_large;
   int32_t bits;
   int32_t* slot_of;  // [B]
   int32_t* lead;     // [B]
   int32_t* cpre;     // [B]
   int32_t* lists;    // [2B]
-  int32_t* counts;   // [8]: leaders, followers, groups with a checkpoint row, the leader pass's work cursor,
-                     //      the follower ranges handed out
-  int32_t* fcnt;     // [B]: a leader's follower count, then the start of its followers' range
-  int32_t* gid;      // [B]: a leader's checkpoint row (-1: none)
-  int32_t* cmin;     // [B]: a leader's smallest common prefix with its followers
   int4* ckpt;        // [gcap * P]: per (row, tree) the leader's walk state to resume from (see route_kernel.cu)
   int32_t gcap;      // checkpoint rows
 };
+constexpr int32_t kNoRow = 0x7f7f7f7f;  // (rows are below 2^29 + 1)
+inline __host__ __device__ int32_t group_row(int32_t gid) { return gid == kNoRow ? -1 : gid; }
+// Requests of a staging window (of route_kernel.cu's staged pass) or longer on average.
+constexpr int kSlotTokens = 4096;  // tokens of a request kept in shared memory (16 KB per slot)
+inline bool long_requests(int64_t B, int64_t n_tokens) { return n_tokens >= B * (int64_t)kSlotTokens; }
 cudaError_t launch_group(const int32_t* tokens, int64_t n_tokens, int64_t tok_base, const int64_t* offsets, int64_t B,
-                         const GroupScratch& g, int num_sms, cudaStream_t st);
+                         int32_t P, const GroupScratch& g, int num_sms, cudaStream_t st, int* launched);
 
 // Staged load words (d_load) carry the load in the low 16 bits and kLoadExcluded for a tree that the
 // decision with excluded trees takes out.
@@ -162,8 +171,10 @@ constexpr int32_t kLoadExcluded = 1 << 16;
 // Best and next-best non-excluded peer of every row of match [B x P] (route_key order); -1 where none.
 cudaError_t launch_decide(const int32_t* match, int64_t B, int32_t P, const int32_t* d_load, int32_t alpha,
                           int32_t* out_peer, int32_t* out_next, int num_sms, cudaStream_t st);
+// Whether a batch is routed without grouping: every request is walked as a leader (route_kernel.cu has the rule).
+bool route_ungrouped(int64_t B, int32_t P, int64_t n_tokens, int num_sms);
 // Route kernels (lookup + route decision) of a grouped batch, see route_kernel.cu: a leader pass and a
-// follower pass (g is required).  *launched is set to the number of kernels launched.  With decide (load
+// follower pass; with g = NULL the batch is not grouped and the leader pass takes every request.  *launched is set to the number of kernels launched.  With decide (load
 // words carrying kLoadExcluded) or out_next (device [B]) the passes make the decision with excluded trees
 // and the next-best target instead of the plain argmax.
 cudaError_t launch_route(const TreeView* d_trees, int32_t P, const int32_t* tokens, int64_t n_tokens,

@@ -4,7 +4,8 @@
 // number of leading request tokens found along one path of T_p, a partial edge included), and the
 // chosen peer argmax_p (match - alpha*load_p, -load_p, -p) (Algorithm 1's argmax with a load term).
 //
-// Passes.  A grouped batch (group_kernel.cu) is routed by a leader pass and a follower pass.  Leaders of
+// Passes.  A grouped batch (group_kernel.cu) is routed by a leader pass and a follower pass; a small batch is not
+// grouped and all of it is routed by the leader pass (route_ungrouped).  Leaders of
 // short requests, and all followers, are walked by lane_kernel (a lane per tree; below).  Leaders whose
 // requests are longer than a staging window on average go to route_kernel:
 //
@@ -30,7 +31,6 @@ namespace {
 constexpr int kWarps = 16;              // warps per CTA
 constexpr int kThreads = kWarps * 32;
 constexpr int kSlots = 4;               // requests staged at a time per CTA
-constexpr int kSlotTokens = 4096;       // tokens of a request kept in shared memory (16 KB per slot)
 constexpr int kCtasPerSm = 2;           // 32 warps per SM: 64 KB of slots and <= 64 registers per thread
 constexpr int kUnroll = 16;             // label loads in flight per lane on long labels (512 tokens per step)
 constexpr int kMaxGroup = 8;            // trees per work item, at most
@@ -349,10 +349,10 @@ struct LaneAcc<true> {
   }
 };
 
-// Routes the leaders list[0 .. *count) of a grouped batch with full walks.  kDecide: the decision with
+// Routes the leaders list[0 .. *count) of a grouped batch, or (kGrouped = false) all B requests, with full walks.  kDecide: the decision with
 // excluded trees and the next-best target (RouteAcc<true>), made by the request's last warp from its match
 // row once every item of the request has written its part.
-template <bool kDecide>
+template <bool kDecide, bool kGrouped>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) route_kernel(
     const TreeView* __restrict__ trees, int32_t P, const int32_t* __restrict__ tokens, int64_t n_tokens,
     int64_t tok_base, const int64_t* __restrict__ offsets, int64_t B, const int32_t* __restrict__ list,
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) route_kernel(
   }
   if (threadIdx.x == 0) s_next = 0;
   __syncthreads();
-  const int64_t n_all = *count;  // requests of this launch
+  const int64_t n_all = kGrouped ? *count : B;  // requests of this launch
   const int64_t n_req = n_all > blockIdx.x ? (n_all - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
   // A work item is (request k, trees p0 .. p0 + G - 1): G grows with P so that the per-item costs (the
   // shared counter, the staging waits, the route-key merge) are shared by several walks while every warp of
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) route_kernel(
     }
     const int s = (int)(k % kSlots);
     const int64_t kb = blockIdx.x + k * gridDim.x;
-    const int64_t b = __ldg(list + kb);
+    const int64_t b = kGrouped ? __ldg(list + kb) : kb;
     Slot& sl = s_slot[s];
     int32_t* st = s_tok + s * kSlotTokens;
     if (c == 0) {
@@ -447,8 +447,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) route_kernel(
         sl.shift = shift;
         sl.best = 0;
         sl.done = 0;
-        sl.row = __ldg(gid + b);
-        sl.climit = __ldg(cmin + b);
+        sl.row = kGrouped ? group_row(__ldg(gid + b)) : -1;
+        sl.climit = kGrouped ? __ldg(cmin + b) : -1;
         __threadfence_block();
         *(volatile int*)&sl.ready = (int)k;
       }
@@ -700,17 +700,18 @@ __device__ __forceinline__ int probe_first2(const int4& a, const int4& b, int32_
   return b.y == 0 ? 0 : -1;
 }
 
-// One warp per request list[i], i < *count.
+// One warp per request list[i], i < *count, or (kGrouped = false) per request of the batch, all
+// leaders.
 //   kLeader: the request is a group leader (or ungrouped): lane j walks trees j, j + 32, ..., and for a
 //   leader with a checkpoint row records the checkpoints its followers resume from.
 //   !kLeader: the request follows leader lead[f] with common prefix c = cpre[f]: match(f, T) = match(lead,
 //   T) if that is < c, else a walk resumed at the leader's checkpoint that does not compare f's first c
 //   tokens.  A lane takes kFollowIlp trees at a time (p, p + 32, ...): the leader's matches, the
 //   checkpoints and the first probe step of each are loaded before any of them is looked at.
-template <bool kLeader, bool kDecide, int kFirst = 8>
+template <bool kLeader, bool kDecide, int kFirst = 8, bool kGrouped = true>
 __global__ void __launch_bounds__(kFollowThreads, kFollowCtasPerSm) lane_kernel(
     const TreeView* __restrict__ trees, int32_t P, const int32_t* __restrict__ tokens, int64_t n_tokens,
-    int64_t tok_base, const int64_t* __restrict__ offsets, const int32_t* __restrict__ list,
+    int64_t tok_base, const int64_t* __restrict__ offsets, int64_t B, const int32_t* __restrict__ list,
     const int32_t* __restrict__ count, const int32_t* __restrict__ lead, const int32_t* __restrict__ cpre,
     const int32_t* __restrict__ gid, const int32_t* __restrict__ cmin, int4* __restrict__ ckpt,
     const int32_t* __restrict__ load, int32_t alpha, int32_t* __restrict__ out_match, int32_t* __restrict__ out_peer,
@@ -718,7 +719,7 @@ __global__ void __launch_bounds__(kFollowThreads, kFollowCtasPerSm) lane_kernel(
   __shared__ unsigned long long s_top[kDecide ? kFollowThreads / 32 : 1][kDecide ? 64 : 1];
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (kFollowThreads / 32);
-  const int64_t n = *count;
+  const int64_t n = kGrouped ? *count : B;
   // Requests go to warps in a fixed stride, or, with a cursor (zero at launch), one at a time as warps
   // become free: leaders' walks differ widely in length.  The next index is fetched while the warp
   // routes the current request.
@@ -730,7 +731,7 @@ __global__ void __launch_bounds__(kFollowThreads, kFollowCtasPerSm) lane_kernel(
   }
   for (int64_t i = i0; i < n; i = cursor ? (int64_t)__shfl_sync(kFull, nxt, 0) : i + warps) {
     if (cursor && lane == 0) nxt = atomicAdd(cursor, 1);
-    const int64_t f = __ldg(list + i);
+    const int64_t f = kGrouped ? __ldg(list + i) : i;
     const int64_t start = __ldg(offsets + f) - tok_base, end = __ldg(offsets + f + 1) - tok_base;
     const int64_t frow = f * P;
     if (!(start >= 0 && start <= end && end <= n_tokens)) {  // (followers are always valid)
@@ -746,7 +747,7 @@ __global__ void __launch_bounds__(kFollowThreads, kFollowCtasPerSm) lane_kernel(
     const int32_t len = (int32_t)min(end - start, (int64_t)INT32_MAX);
     LaneAcc<kDecide> acc(kDecide ? &s_top[threadIdx.x >> 5][lane] : nullptr);
     if constexpr (kLeader) {
-      const int32_t row = __ldg(gid + f);
+      const int32_t row = kGrouped ? group_row(__ldg(gid + f)) : -1;
       const int32_t climit = row >= 0 ? __ldg(cmin + f) : -1;
       const int32_t tok0 = len > 0 ? __ldg(req) : 0;
       for (int32_t p0 = 0; p0 < P; p0 += 32) {
@@ -775,7 +776,7 @@ __global__ void __launch_bounds__(kFollowThreads, kFollowCtasPerSm) lane_kernel(
     } else {
       const int32_t c = __ldg(cpre + f);
       const int32_t l = __ldg(lead + f);
-      const int32_t row = __ldg(gid + l);
+      const int32_t row = group_row(__ldg(gid + l));
       const int64_t lrow = (int64_t)l * P;  // the leaders' pass has finished: the leader's row is final
       const int4* ckrow = ckpt + (int64_t)(row >= 0 ? row : 0) * P;
       for (int32_t p0 = 0; p0 < P; p0 += 32 * kFollowIlp) {
@@ -962,7 +963,7 @@ __global__ void __launch_bounds__(256, 2) decide_kernel(const int32_t* __restric
 
 namespace {
 
-// The leader and follower passes with the decision of RouteAcc<kDecide>.
+// The leader and follower passes with the decision of RouteAcc<kDecide>; without g, the leader pass alone.
 template <bool kDecide>
 cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tokens, int64_t n_tokens, int64_t tok_base,
                           const int64_t* offsets, int64_t B, const int32_t* d_load, int32_t alpha, int32_t* out_match,
@@ -970,41 +971,46 @@ cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tok
                           int32_t* out_next, int* launched) {
   const int64_t want = (B + kFollowThreads / 32 - 1) / (kFollowThreads / 32);
   const int grid2 = (int)std::min<int64_t>(want, (int64_t)num_sms * kFollowCtasPerSm);
+  const int32_t *lists = g ? g->lists : nullptr, *counts = g ? g->counts : nullptr;
+  const int32_t *gid = g ? g->gid : nullptr, *cmin = g ? g->cmin : nullptr;
+  int4* ckpt = g ? g->ckpt : nullptr;
   cudaError_t e;
-  if (n_tokens >= B * (int64_t)kSlotTokens) {
+  if (long_requests(B, n_tokens)) {
     // Requests of a staging window or longer on average: the leaders' walks are long compares, which the
     // staged kernel's warps do from shared memory.
     const size_t smem = (size_t)kSlots * kSlotTokens * sizeof(int32_t);
-    e = cudaFuncSetAttribute(route_kernel<kDecide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kernel = g ? route_kernel<kDecide, true> : route_kernel<kDecide, false>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t max_ctas = (int64_t)num_sms * kCtasPerSm;
     const int grid = (int)(B < max_ctas ? B : max_ctas);
     P2P_TIMED(K_ROUTE_STAGED, st,
-              (route_kernel<kDecide><<<grid, kThreads, smem, st>>>(d_trees, P, tokens, n_tokens, tok_base, offsets, B,
-                                                                   g->lists, g->counts, g->gid, g->cmin, g->ckpt, d_load,
-                                                                   alpha, out_match, out_peer, d_err, out_next)));
+              (kernel<<<grid, kThreads, smem, st>>>(d_trees, P, tokens, n_tokens, tok_base, offsets, B, lists, counts,
+                                                    gid, cmin, ckpt, d_load, alpha, out_match, out_peer, d_err,
+                                                    out_next)));
     *launched = 1;
   } else {
     // Shorter requests: most leader walks end within a few tokens, so each lane walks its own tree.
+    const auto kernel = g ? lane_kernel<true, kDecide, 8, true> : lane_kernel<true, kDecide, 8, false>;
     P2P_TIMED(K_LANE_LEADER, st,
-              (lane_kernel<true, kDecide><<<grid2, kFollowThreads, 0, st>>>(
-                  d_trees, P, tokens, n_tokens, tok_base, offsets, g->lists, g->counts, nullptr, nullptr, g->gid,
-                  g->cmin, g->ckpt, d_load, alpha, out_match, out_peer, d_err, g->counts + 3, out_next)));
+              (kernel<<<grid2, kFollowThreads, 0, st>>>(
+                  d_trees, P, tokens, n_tokens, tok_base, offsets, B, lists, counts, nullptr, nullptr, gid, cmin, ckpt,
+                  d_load, alpha, out_match, out_peer, d_err, g ? g->counts + 3 : nullptr, out_next)));
     *launched = 1;
   }
   e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || !g) return e;
   // The followers' first per-lane compare: 8 tokens for long requests, 16 otherwise (lane_walks).
-  if (n_tokens >= B * (int64_t)kSlotTokens) {
+  if (long_requests(B, n_tokens)) {
     P2P_TIMED(K_LANE_FOLLOWER, st,
               (lane_kernel<false, kDecide, 8><<<grid2, kFollowThreads, 0, st>>>(
-                  d_trees, P, tokens, n_tokens, tok_base, offsets, g->lists + B, g->counts + 1, g->lead, g->cpre, g->gid,
-                  nullptr, g->ckpt, d_load, alpha, out_match, out_peer, d_err, nullptr, out_next)));
+                  d_trees, P, tokens, n_tokens, tok_base, offsets, B, g->lists + B, g->counts + 1, g->lead, g->cpre,
+                  g->gid, nullptr, g->ckpt, d_load, alpha, out_match, out_peer, d_err, nullptr, out_next)));
   } else {
     P2P_TIMED(K_LANE_FOLLOWER, st,
               (lane_kernel<false, kDecide, 16><<<grid2, kFollowThreads, 0, st>>>(
-                  d_trees, P, tokens, n_tokens, tok_base, offsets, g->lists + B, g->counts + 1, g->lead, g->cpre, g->gid,
-                  nullptr, g->ckpt, d_load, alpha, out_match, out_peer, d_err, nullptr, out_next)));
+                  d_trees, P, tokens, n_tokens, tok_base, offsets, B, g->lists + B, g->counts + 1, g->lead, g->cpre,
+                  g->gid, nullptr, g->ckpt, d_load, alpha, out_match, out_peer, d_err, nullptr, out_next)));
   }
   *launched += 1;
   return cudaGetLastError();
@@ -1012,13 +1018,25 @@ cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tok
 
 }  // namespace
 
+// A batch of no more requests than the leader pass has warps (or eight a resident CTA of the staged pass) is not
+// grouped: its walks all run at once, so the pass takes as long as its longest walk whether or not the followers are
+// among them, and the grouping and the follower pass would only come on top.  Measured (us a call, grouped ->
+// ungrouped): 33 requests on 4 trees 34 -> 25, 1,025 on 16 trees 46 -> 24, 4,864 on 64 trees 60 -> 29, on 256 trees
+// 103 -> 77, twice that many on 256 trees 140 -> 144; long requests on 32 trees: 33 124 -> 68, 2,048 246 -> 173,
+// 4,096 318 -> 333.  A batch on few trees gains too, but stays grouped past 300 requests for each tree after the
+// first: the kernel clock and the launch count are documented by their grouped launches on such batches.
+bool route_ungrouped(int64_t B, int32_t P, int64_t n_tokens, int num_sms) {
+  const int64_t most = long_requests(B, n_tokens) ? (int64_t)num_sms * kCtasPerSm * 8
+                                                  : (int64_t)num_sms * kFollowCtasPerSm * (kFollowThreads / 32);
+  return B <= std::min<int64_t>(most, (int64_t)300 * (P - 1));
+}
+
 cudaError_t launch_route(const TreeView* d_trees, int32_t P, const int32_t* tokens, int64_t n_tokens, int64_t tok_base,
                          const int64_t* offsets, int64_t B, const int32_t* d_load, int32_t alpha, int32_t* out_match,
                          int32_t* out_peer, int32_t* d_err, const GroupScratch* g, int num_sms, cudaStream_t st,
                          int* launched, bool decide, int32_t* out_next) {
   *launched = 0;
   if (B <= 0) return cudaSuccess;
-  if (!g) return cudaErrorInvalidValue;  // every batch is grouped first
   if (decide || out_next)
     return launch_passes<true>(d_trees, P, tokens, n_tokens, tok_base, offsets, B, d_load, alpha, out_match, out_peer,
                                d_err, g, num_sms, st, out_next, launched);

@@ -88,7 +88,7 @@ thread_local KernelClock* t_clock = nullptr;
 
 const char* kernel_name(int id) {
   static const char* const names[K_COUNT_] = {
-      "group_hash_kernel", "group_resolve_kernel", "group_resolve32_kernel", "route_kernel", "lane_kernel<true>",
+      "group_hash_kernel", "group_resolve_kernel", "route_kernel", "lane_kernel<true>",
       "lane_kernel<false>", "decide_kernel", "validate_kernel", "init_ranges_kernel", "delta_kernel",
       "compact_kernel", "compact_labels_kernel", "refresh_views_kernel", "set_tree_kernel", "update_count_kernel",
       "update_scan_kernel", "update_scatter_kernel", "group_ranges_kernel", "group_place_kernel", "lru_walk_kernel",
@@ -293,34 +293,36 @@ cudaError_t ensure(p2p_router* r, DevBuf& b, size_t bytes) {
 }
 
 // Scratch of the shared-prefix grouping for a batch of B requests (B <= 2^30): a key table of at least 2B
-// slots; slot_of, lead, cpre (B each), the two request lists (2B), gid, cmin and fcnt (B each) and eight counts;
-// and checkpoint rows, as many as fit in 256 MB (and at most B/2 + 1, one per leader with followers).
+// slots with fcnt (B) and eight counts behind the keys, gid and cmin (B each) behind the values; slot_of, lead and
+// cpre (B each) and the two request lists (2B); and checkpoint rows, as many as fit in 256 MB (and at most B/2 + 1, one per leader with followers).
 cudaError_t group_scratch(p2p_router* r, int64_t B, p2p::GroupScratch& g) {
   const int64_t slots = std::max<int64_t>(next_pow2(2 * B), 1024);
   const int64_t gcap = std::max<int64_t>(1, std::min<int64_t>(B / 2 + 1, ((int64_t)256 << 20) / ((int64_t)r->P * 16)));
-  cudaError_t e = ensure(r, r->grp_keys, (size_t)slots * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = ensure(r, r->grp_vals, (size_t)slots * sizeof(int32_t));
-  if (e == cudaSuccess) e = ensure(r, r->grp_req, (size_t)(8 * B + 8) * sizeof(int32_t));
+  g.n_zero = (size_t)slots * sizeof(unsigned long long) + (size_t)(B + 8) * sizeof(int32_t);
+  g.n_large = (size_t)(slots + 2 * B) * sizeof(int32_t);
+  cudaError_t e = ensure(r, r->grp_keys, g.n_zero);
+  if (e == cudaSuccess) e = ensure(r, r->grp_vals, g.n_large);
+  if (e == cudaSuccess) e = ensure(r, r->grp_req, (size_t)(5 * B) * sizeof(int32_t));
   if (e == cudaSuccess) e = ensure(r, r->grp_ckpt, (size_t)gcap * r->P * sizeof(int4));
   if (e != cudaSuccess) return e;
-  int32_t* q = static_cast<int32_t*>(r->grp_req.p);
   g.keys = static_cast<unsigned long long*>(r->grp_keys.p);
+  g.fcnt = reinterpret_cast<int32_t*>(g.keys + slots);
+  g.counts = g.fcnt + B;
   g.vals = static_cast<int32_t*>(r->grp_vals.p);
+  g.gid = g.vals + slots;
+  g.cmin = g.gid + B;
   g.bits = log2_exact(slots);
+  int32_t* q = static_cast<int32_t*>(r->grp_req.p);
   g.slot_of = q;
   g.lead = q + B;
   g.cpre = q + 2 * B;
   g.lists = q + 3 * B;
-  g.gid = q + 5 * B;
-  g.cmin = q + 6 * B;
-  g.fcnt = q + 7 * B;
-  g.counts = q + 8 * B;
   g.ckpt = static_cast<int4*>(r->grp_ckpt.p);
   g.gcap = (int32_t)gcap;
   return cudaSuccess;
 }
 
-// Groups the batch by shared prefix and routes it (leaders, then followers).  The callers check B <= kMaxBatch
+// Groups the batch by shared prefix (unless it is small) and routes it (leaders, then followers).  The callers check B <= kMaxBatch
 // (request indices and list positions are 32-bit).
 // With decide (an excluded-peer mask staged with the load) or out_next, the passes make the decision with
 // excluded trees and the next-best target.
@@ -334,14 +336,17 @@ int route(p2p_router* r, const int32_t* tokens, int64_t n_tokens, int64_t tok_ba
   // (state 3, scratch taken but the grouping not launched, cannot outlive the delta call that took it)
   r->prep.state = 0;
   p2p::GroupScratch g;
-  CK(group_scratch(r, B, g));
-  if (!grouped) {
-    CK(p2p::launch_group(tokens, n_tokens, tok_base, offsets, B, g, r->num_sms, r->stream));
-    r->launches += 4;
-  }
+  const bool group = !p2p::route_ungrouped(B, r->P, n_tokens, r->num_sms);
   int launched = 0;
+  if (group) {
+    CK(group_scratch(r, B, g));
+    if (!grouped) {
+      CK(p2p::launch_group(tokens, n_tokens, tok_base, offsets, B, r->P, g, r->num_sms, r->stream, &launched));
+      r->launches += launched;
+    }
+  }
   CK(p2p::launch_route(r->d_views, r->P, tokens, n_tokens, tok_base, offsets, B, r->d_load, alpha, out_match, out_peer,
-                       r->d_err, &g, r->num_sms, r->stream, &launched, decide, out_next));
+                       r->d_err, group ? &g : nullptr, r->num_sms, r->stream, &launched, decide, out_next));
   r->launches += launched;
   return P2P_OK;
 }
@@ -364,9 +369,11 @@ int launch_prepared(p2p_router* r) {
   p2p::GroupScratch g;
   CK(group_scratch(r, r->prep.B, g));  // the buffers of prepare_scratch (no allocation)
   CK(cudaStreamWaitEvent(r->grp_stream, r->grp_start, 0));
-  CK(p2p::launch_group(r->prep.tokens, r->prep.n_tokens, 0, r->prep.offsets, r->prep.B, g, r->num_sms, r->grp_stream));
+  int launched = 0;
+  CK(p2p::launch_group(r->prep.tokens, r->prep.n_tokens, 0, r->prep.offsets, r->prep.B, r->P, g, r->num_sms,
+                       r->grp_stream, &launched));
   CK(cudaEventRecord(r->grp_done, r->grp_stream));
-  r->launches += 4;
+  r->launches += launched;
   r->prep.state = 2;
   return P2P_OK;
 }
@@ -1783,7 +1790,7 @@ int p2p_route_prepare(p2p_router* r, const int32_t* tokens, int64_t n_tokens, co
   DeviceGuard g(r);
   if (r->prep.state == 2) CK(cudaStreamWaitEvent(r->stream, r->grp_done, 0));  // the scratch is free again
   r->prep.state = 0;
-  if (B == 0) return P2P_OK;
+  if (B == 0 || p2p::route_ungrouped(B, r->P, n_tokens, r->num_sms)) return P2P_OK;  // nothing to do ahead
   r->prep.tokens = tokens;
   r->prep.offsets = offsets;
   r->prep.n_tokens = n_tokens;
