@@ -1349,19 +1349,44 @@ __device__ void compact_range_warp(CompactJob& J, CompactShared& S, const int4& 
   }
 }
 
-// One CTA per tree: level-synchronous breadth-first copy of the structure from the root.  New ids are
+// One cluster of kC CTAs per tree (kC = 1: a CTA): level-synchronous breadth-first copy of the structure from the root.  New ids are
 // handed out level by level, so the nodes of the next level are the ids [end, S.node) and the scratch
 // entry of id c (old id, old and new label offsets, own-arena label length) is written by the parent's
 // copy.  A thread takes each node of the level.  A node whose table has more than 2^kSmallBits slots gets
 // its new table range and record from that thread, and its slots are cut into units of kUnitSlots that all
 // warps then zero and fill; smaller tables are copied by the thread.  A big table's record counts its
 // children from the old record (the live-child count), so no pass has to count them.
+//
+// Few trees are compacted by clusters: one tree's levels keep 512 threads busy for long (a tree of ~50,000 nodes
+// 0.61 ms by a CTA), while a wave of 256 trees fills the GPU with a CTA each.  The cluster's counters and units are
+// in its first CTA's shared memory.
+// The cluster's shared counters, and a barrier of the cluster (or of the CTA).
+template <int kC>
+__device__ __forceinline__ CompactShared* compact_shared(CompactShared* own) {
+  if constexpr (kC == 1) return own;
+  unsigned long long at;
+  asm("mapa.u64 %0, %1, 0;" : "=l"(at) : "l"((unsigned long long)own));
+  return reinterpret_cast<CompactShared*>(at);
+}
+template <int kC>
+__device__ __forceinline__ void compact_sync() {
+  if constexpr (kC == 1) {
+    __syncthreads();
+  } else {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+}
+
+template <int kC>
 __global__ void __launch_bounds__(kCompactThreads) compact_kernel(CompactJob* jobs) {
-  CompactJob& J = jobs[blockIdx.x];
-  __shared__ CompactShared S;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int kWarps = kCompactThreads / 32;
-  if (threadIdx.x == 0) {
+  CompactJob& J = jobs[blockIdx.x / kC];
+  __shared__ CompactShared S_own;
+  CompactShared& S = *compact_shared<kC>(&S_own);
+  const int rank = kC > 1 ? (int)(blockIdx.x % kC) : 0;
+  const int lane = threadIdx.x & 31, warp = rank * (kCompactThreads / 32) + (threadIdx.x >> 5);
+  constexpr int kThreads = kCompactThreads * kC, kWarps = kThreads / 32;
+  const int thread = rank * kCompactThreads + (int)threadIdx.x;
+  if (thread == 0) {
     S.node = 1;
     S.child = 0;
     S.label = 0;
@@ -1369,11 +1394,11 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(CompactJob* jo
     S.nunits = 0;
     J.queue[0] = make_int4(0, 0, 0, 0);
   }
-  __syncthreads();
+  compact_sync<kC>();
   int begin = 0, end = 1;
   while (begin < end) {
-    for (int cid = begin + threadIdx.x; cid < end; cid += kCompactThreads) {
-      const int4 rec = __ldg(J.node + J.queue[cid].x);
+    for (int cid = begin + thread; cid < end; cid += kThreads) {
+      const int4 rec = __ldg(J.node + __ldcg(&J.queue[cid].x));
       const int32_t bits = tab_bits(rec.y);
       if (bits > kSmallBits) {
         const int32_t size = 1 << bits, nu = (size + kUnitSlots - 1) / kUnitSlots;
@@ -1393,30 +1418,30 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(CompactJob* jo
       }
       compact_node_thread(J, S, cid, rec);
     }
-    __syncthreads();
+    compact_sync<kC>();
     const int nunits = min(S.nunits, kUnitCap);
     for (int k = warp; k < nunits; k += kWarps) {  // zero every unit's slots first: inserts may wrap into them
       const int2 u = S.units[k];
       if (u.x < 0) continue;
-      const int4 nrec = J.nnode[u.x];
+      const int4 nrec = __ldcg(J.nnode + u.x);
       const int32_t n = min(kUnitSlots, (1 << tab_bits(nrec.y)) - u.y);
       for (int32_t j = lane; j < n; j += 32) J.nchild[nrec.x + u.y + j] = make_int4(0, 0, 0, 0);
     }
-    __syncthreads();
+    compact_sync<kC>();
     for (int k = warp; k < nunits; k += kWarps) {
       const int2 u = S.units[k];
       if (u.x < 0 || __shfl_sync(kFull, *(volatile int*)&S.fail, 0)) continue;
-      const int4 rec = __ldg(J.node + J.queue[u.x].x);
-      const int32_t noff = J.nnode[u.x].x;
+      const int4 rec = __ldg(J.node + __ldcg(&J.queue[u.x].x));
+      const int32_t noff = __ldcg(&J.nnode[u.x].x);
       compact_range_warp(J, S, rec, noff, u.y, min(u.y + kUnitSlots, 1 << tab_bits(rec.y)), lane);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) S.nunits = 0;
+    compact_sync<kC>();
+    if (thread == 0) S.nunits = 0;
     begin = end;
     end = *(volatile int*)&S.fail ? end : *(volatile int*)&S.node;
-    __syncthreads();
+    compact_sync<kC>();
   }
-  if (threadIdx.x == 0) {
+  if (thread == 0) {
     J.n_node = S.node;
     J.n_child = S.child;
     J.n_label = S.label;
@@ -1497,9 +1522,34 @@ cudaError_t launch_refresh_views(const TreeState* d_states, TreeView* d_views, i
   return cudaGetLastError();
 }
 
+namespace {
+template <int kC>
+cudaError_t compact_structure(CompactJob* d_jobs, int32_t n_jobs, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kC;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(n_jobs * kC));
+  cfg.blockDim = dim3(kCompactThreads);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = kC > 1 ? 1 : 0;
+  cudaError_t e = cudaSuccess;
+  P2P_TIMED(K_COMPACT, st, (e = cudaLaunchKernelEx(&cfg, compact_kernel<kC>, d_jobs)));
+  return e;
+}
+}  // namespace
+
 cudaError_t launch_compact(CompactJob* d_jobs, int32_t n_jobs, int32_t max_cap_node, int num_sms, cudaStream_t st) {
   if (n_jobs <= 0) return cudaSuccess;
-  P2P_TIMED(K_COMPACT, st, (compact_kernel<<<n_jobs, kCompactThreads, 0, st>>>(d_jobs)));
+  // CTAs per tree: as many as the SMs hold once, up to the portable cluster size.
+  const int per = std::max(num_sms, 1) / n_jobs;
+  cudaError_t e = per >= 8   ? compact_structure<8>(d_jobs, n_jobs, st)
+                  : per >= 4 ? compact_structure<4>(d_jobs, n_jobs, st)
+                  : per >= 2 ? compact_structure<2>(d_jobs, n_jobs, st)
+                             : compact_structure<1>(d_jobs, n_jobs, st);
+  if (e != cudaSuccess) return e;
   const int32_t groups = (max_cap_node + 31) / 32;
   P2P_TIMED(K_COMPACT_LABELS, st,
             (compact_labels_kernel<<<std::max(num_sms, 1) * kLabelCtasPerSm, kLabelThreads, 0, st>>>(
