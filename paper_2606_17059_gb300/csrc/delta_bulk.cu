@@ -141,28 +141,37 @@ __device__ __forceinline__ int32_t tree_of(const BulkArgs& A, int64_t i) {
 }
 
 // One lane: the slot of tok in the table of 2^bits slots at off.  Returns 1 (live; e = the entry), 2 (tombstone) or
-// 0 (absent); slot = where it is (absent: the first empty slot, or -1).  Two slots per step, each read as two
-// 64-bit words whose first holds key and state: in the apply launch other lanes claim other keys' slots meanwhile.
+// 0 (absent); slot = where it is (absent: the first empty slot, or -1).  Two slots per step; kLive: each read as two
+// 64-bit words whose first holds key and state, since other lanes claim other keys' slots meanwhile.
+template <bool kLive>
 __device__ int probe_lane(const int4* child, int32_t off, int32_t bits, int32_t tok, int32_t& slot, int4& e) {
   slot = -1;
   if (bits == 0) return 0;
   const uint32_t mask = (1u << bits) - 1, h = slot_hash(tok, bits);
   for (uint32_t i = 0; i <= mask; i += 2) {
     const uint32_t s0 = (h + i) & mask, s1 = (h + i + 1) & mask;
-    const longlong2 x = __ldcg(reinterpret_cast<const longlong2*>(child + off + s0));
-    const longlong2 y = __ldcg(reinterpret_cast<const longlong2*>(child + off + s1));
+    int4 x, y;
+    if constexpr (kLive) {
+      const longlong2 u = __ldcg(reinterpret_cast<const longlong2*>(child + off + s0));
+      const longlong2 v = __ldcg(reinterpret_cast<const longlong2*>(child + off + s1));
+      x = make_int4((int32_t)u.x, (int32_t)((unsigned long long)u.x >> 32), (int32_t)u.y,
+                    (int32_t)((unsigned long long)u.y >> 32));
+      y = make_int4((int32_t)v.x, (int32_t)((unsigned long long)v.x >> 32), (int32_t)v.y,
+                    (int32_t)((unsigned long long)v.y >> 32));
+    } else {
+      load_slots(child + off + s0, x, y);
+    }
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const longlong2 w = c ? y : x;
-      const int32_t key = (int32_t)(w.x & 0xffffffffll), state = (int32_t)((unsigned long long)w.x >> 32);
-      if (state == 0) {
+      const int4 w = c ? y : x;
+      if (w.y == 0) {
         slot = off + (int32_t)(c ? s1 : s0);
         return 0;
       }
-      if (key == tok && (state >= 1 || state == -1)) {
+      if (w.x == tok && (w.y >= 1 || w.y == -1)) {
         slot = off + (int32_t)(c ? s1 : s0);
-        e = make_int4(key, state, (int32_t)(w.y & 0xffffffffll), (int32_t)((unsigned long long)w.y >> 32));
-        return state >= 1 ? 1 : 2;
+        e = w;
+        return w.y >= 1 ? 1 : 2;
       }
     }
   }
@@ -257,7 +266,7 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
       const int32_t* lab = nullptr;
       if (act && !held) {
         int32_t slot;
-        const int st = probe_lane(child, nd.x, tab_bits(nd.y), q.at(pos), slot, ce);
+        const int st = probe_lane<false>(child, nd.x, tab_bits(nd.y), q.at(pos), slot, ce);
         if (st != 1) {
           what = opc == P2P_OP_INSERT ? B_LEAF : B_ABSENT;
           flags = st == 2 ? BF_REVIVE : 0;
@@ -641,7 +650,7 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
         rec.x = __ldcg(&node[b.u].x);
         rec.y = __ldcg(&node[b.u].y);
         tok = q.at(b.pos);
-        const int st = probe_lane(child, rec.x, tab_bits(rec.y), tok, slot, e);
+        const int st = probe_lane<true>(child, rec.x, tab_bits(rec.y), tok, slot, e);
         const int expect = what == B_LEAF ? (b.what & BF_REVIVE ? 2 : 0) : 1;
         go = st == expect && slot >= 0;  // (always: nothing else may touch this op's slot)
       }
@@ -652,7 +661,7 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
           const int4 o = __ldcg(child + rec.x + t);
           if (o.y >= 1 && o.y != b.v) ys = t, ye = o;
         }
-        go = ys >= 0 && probe_lane(child, gr.x, tab_bits(gr.y), q.at(b.gpos), pslot, pe) == 1;
+        go = ys >= 0 && probe_lane<true>(child, gr.x, tab_bits(gr.y), q.at(b.gpos), pslot, pe) == 1;
         if (go && !adjacent(pe, ye)) want_l = (int64_t)pe.w + ye.w;
       }
       if (go && what == B_LEAF) want_n = 1, want_l = q.n - b.pos;

@@ -575,14 +575,14 @@ constexpr int kFollowCtasPerSm = 4;
 constexpr int kThreadSpan = 64;
 constexpr int kFollowIlp = 2;  // trees a follower's lane takes per iteration (their first loads overlap; 3 or 4 spill)
 
-// One thread: the child with first token tok in a table of 2^bits (>= 4, even) slots, two slots per step of
+// One thread: the child with first token tok in a table of 2^bits (>= 4) slots, two slots (a sector) per step of
 // the linear probe.  Returns false if there is none.
 __device__ __forceinline__ bool find_child_1(const int4* __restrict__ tab, int32_t bits, int32_t tok, int4& out) {
   if (bits == 0) return false;
   const uint32_t mask = (1u << bits) - 1, h = slot_hash(tok, bits);
   for (uint32_t i = 0; i <= mask; i += 2) {
-    const int4 a = __ldg(tab + ((h + i) & mask));
-    const int4 b = __ldg(tab + ((h + i + 1) & mask));
+    int4 a, b;
+    load_slots(tab + ((h + i) & mask), a, b);
     if (a.y >= 1 && a.x == tok) {
       out = a;
       return true;
@@ -809,10 +809,9 @@ __global__ void __launch_bounds__(kFollowThreads, kFollowCtasPerSm) lane_kernel(
           tab[g] = nullptr;
           if (act[g]) {
             const int32_t bits = tab_bits(st[g].z);
-            const uint32_t mask = (1u << bits) - 1, h = slot_hash(tk[g], bits);
+            const uint32_t h = slot_hash(tk[g], bits);
             tab[g] = trees[pt[g]].child + st[g].y;
-            e0[g] = __ldg(tab[g] + h);
-            e1[g] = __ldg(tab[g] + ((h + 1) & mask));
+            load_slots(tab[g] + h, e0[g], e1[g]);
           }
         }
 #pragma unroll
