@@ -10,30 +10,34 @@
 //
 // A round, three launches:
 //   bulk_resolve_kernel  a lane per op: the read-only walk.  It ends in a place: a node u and a token (a slot of u's
-//                        table, whether taken or free).  The op enters the place in a key table (the smallest op
-//                        index wins it) and the nodes it depends on in a node table:
-//                          leaf     INSERT of a new leaf edge under u            slot (u, tok), shares u
-//                          split    INSERT that leaves the edge (u, tok) inside  slot (u, tok), shares u
+//                        table, whether taken or free).  The op enters the places it needs for itself in a key table
+//                        (the smallest op index wins each), its own place first, and the node it depends on in a
+//                        node table:
+//                          leaf     INSERT of a new leaf edge under u            (u, tok), shares u; if u is a leaf
+//                                                                                itself, u's own place too
+//                          split    INSERT that leaves the edge (u, tok) inside  (u, tok), shares u
 //                          count    INSERT or DELETE that only changes a node's sequence count
-//                                                                                slot of its edge, shares the node
-//                                   (a DELETE that leaves the node without one:  the node for itself)
-//                          remove   DELETE of the leaf v under u                 slot (u, tok), shares u, v for itself
+//                                                                                its place, shares the node (a DELETE
+//                                                                                that leaves it without one: alone)
+//                          remove   DELETE of the leaf v under u                 (u, tok), shares u
 //                          fold     the same where u then has one child y left and stores nothing: u takes y in
-//                                                    slot (u, tok), u's own slot; u, v and y for itself
-//                          absent   DELETE of a sequence that is not stored      slot (u, tok)
-//                        An op of any other form (a node that is one child's only parent, say) holds its slot and
+//                                                                                (u, tok), u's own place, u alone;
+//                                                                                y's place if it is a leaf, else y
+//                                                                                alone
+//                          absent   DELETE of a sequence that is not stored      (u, tok)
+//                        An op of any other form (a DELETE that takes in a node's only child, say) holds its place and
 //                        is left over.
 //   bulk_grow_kernel     the tables of nodes that would pass 1/2 claimed with the round's leaves under them.
-//   bulk_apply_kernel    an op that holds its slots, whose shared nodes nobody needs alone -- an op that needs a
-//                        node for itself steps back when anyone shares it -- and whose own nodes nobody else
-//                        named (or only ops of larger index that need them alone too) is applied: room for the
-//                        warp's ops with one reservation per tree and arena, labels copied by the whole warp,
-//                        slots, records and counts by the op's lane.  The others go to the next round's list.
+//   bulk_apply_kernel    an op that won its places, and whose node nobody shares if it needs it alone (and no op of
+//                        smaller index needs it alone too), is applied: room for the warp's ops with one reservation
+//                        per tree and arena, labels copied by the whole warp, slots, records and counts by the op's
+//                        lane.  The others go to the next round's list.  A tree whose arenas may not hold what the
+//                        round asks for is grown by the host first: its ops that need room all wait.
 // Of the removals under a node with z children that stores nothing only the first z - 2 to arrive go in one round, so
-// no node is left with fewer than 2 children unless it is folded.  Ops on one sequence always name the same slot,
-// the one with the smallest index wins it and the others wait: they apply in op order.  A slot that an op could
-// not enter (no room in the key table) cannot be entered by the others that name it either, so none of them
-// overtakes it.
+// no node is left with fewer than 2 children unless it is folded.  A leaf's record and what hangs from it are
+// changed only by ops that hold its place.  Ops on one sequence always name the same place first, the one with the
+// smallest index wins it and the others wait: they apply in op order.  A place that an op could not enter (no room in
+// the key table) cannot be entered by the others that name it either, so none of them overtakes it.
 //
 // What bounds it: each lane's chain of dependent loads (a probe, a compare and a record per tree level), with
 // 32 chains a warp in flight.  Long compares are made by the warp, once per launch for an interned label and a
@@ -41,20 +45,22 @@
 // other edges and look again.
 //
 // Measured, the delta of a call (delta_kernel alone -> these rounds and delta_kernel behind them): 16,384 routed
-// requests into 16 trees, most into one, 8.2 -> 0.25 ms; 4,096 requests into one cache trie 2.46 -> 0.17 ms; 300 ops
-// into one tree 189 -> 74 us; 1,024,000 ops on 256 trees of 40,000 sequences 3.58 -> 1.77 ms.
+// requests into 16 trees, most into one, 8.2 -> 0.21 ms; 4,096 requests into one cache trie 2.46 -> 0.12 ms; 300 ops
+// into one tree 189 -> 77 us; 1,024,000 ops on 256 trees of 40,000 sequences 3.58 -> 1.46 ms.
 #include "internal.h"
 
 namespace p2p {
 
-// What an op would do, as found by the walk.  u, pos: the node and the token position the place belongs to (the
-// place's token is the sequence's at pos); k: where a split cuts the edge; v: the node of a count or a removal.
-// Fold: g, gpos give u's own place.  Table indices are -1 where there is none.
-struct __align__(16) BulkOp {
+// What an op would do, as found by the walk.  u, tok: its place, which was slot `slot` of u's table at table offset
+// `tab` then; key: its entry.  Then by kind: k where a split cuts the edge, the leaf a removal takes, the node of a
+// count (arg) and its entry (ent); a leaf's entry of u (ent).  The second half only for a fold (v = arg; g, gpos: u's own
+// place) and a leaf under a leaf (key2).
+struct __align__(32) BulkOp {
   int32_t what;  // B_* | BF_* flags | tree << kTreeShift
-  int32_t u, pos, k;
-  int32_t v, g, gpos, key;
-  int32_t key2, ent_u, ent_v, ent_y;
+  int32_t u, tok, slot;
+  int32_t key, arg, ent, pos;
+  int32_t key2, key3, ent_u, ent_y;
+  int32_t g, gpos, pad0, pad1;
 };
 
 namespace {
@@ -62,15 +68,17 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kBulkThreads = 256;
 constexpr int kBulkWarps = kBulkThreads / 32;
-constexpr int kBulkCtasPerSm = 3;   // at most 85 registers a thread
-constexpr int kLaneSpan = 64;       // label tokens after the first eight that a lane compares alone
+constexpr int kBulkCtasPerSm = 4;   // at most 64 registers a thread (80 and 3 CTAs: the resolve launches of a step of
+                                    // 1,024,000 ops 0.90 ms instead of 0.81)
+constexpr int kLaneSpan = 128;      // label tokens after the first eight that a lane compares alone
+constexpr int kLaneBits = 5;        // tables up to 32 slots are moved by one lane
 constexpr int kMaxProbes = 64;      // of the key and node tables
 constexpr int kMemoProbes = 4;
-constexpr int kMemoWaits = 64;      // looks at a pair another warp compares before the lane's warp compares it too
+constexpr int kMemoWaits = 256;     // looks at a pair another warp compares before the lane's warp compares it too
 constexpr int kFoldBits = 6;        // tables a lane searches for the one other child
 
 enum { B_NONE = 0, B_LEAF, B_SPLIT, B_COUNT, B_REMOVE, B_FOLD, B_ABSENT, B_LEFT };
-enum { BF_ALONE = 16, BF_REVIVE = 32, BF_GROW = 64, BF_LATER = 128 };
+enum { BF_ALONE = 16, BF_REVIVE = 32, BF_MORE = 64, BF_LATER = 128 };  // BF_MORE: the record's second half holds
 constexpr int kTreeShift = 8;  // (a tree index has 16 bits)
 
 __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {  // SplitMix64's output function
@@ -79,17 +87,20 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {  // 
   return z ^ (z >> 31);
 }
 
-// Enters (tree, u, tok) of this round for op idx; the table's index, or -1 if it has no room near the key's home.
-// Two places with the same 64-bit hash only wait for one another.
+// Enters (tree, u, tok) of this round for op idx; the table's index, or -1 if it has no room near the key's home.  An
+// entry is 32 bits of the place's hash over the complement of the smallest op index.  Two places that share those
+// bits and the neighbourhood only wait for one another.
 __device__ int32_t enter_key(const BulkTables& T, int32_t tree, int32_t u, int32_t tok, int round, uint32_t idx) {
-  unsigned long long h = mix64((((unsigned long long)(uint32_t)u << 32) | (uint32_t)tok) ^
-                               mix64(((unsigned long long)(uint32_t)tree << 8) | (unsigned)(round + 1)));
-  h |= 1ull;  // 0 marks an empty entry
-  uint32_t s = (uint32_t)(h >> 17) & T.key_mask;
+  const unsigned long long h = mix64((((unsigned long long)(uint32_t)u << 32) | (uint32_t)tok) ^
+                                     mix64(((unsigned long long)(uint32_t)tree << 8) | (unsigned)(round + 1)));
+  const uint32_t mark = (uint32_t)(h >> 32) | 1u;  // 0 marks an empty entry
+  const unsigned long long mine = ((unsigned long long)mark << 32) | (uint32_t)~idx;
+  uint32_t s = (uint32_t)h & T.key_mask;
   for (int it = 0; it < kMaxProbes; ++it, s = (s + 1) & T.key_mask) {
-    const unsigned long long prev = atomicCAS(&T.keys[s].key, 0ull, h);
-    if (prev == 0ull || prev == h) {
-      atomicMax(&T.keys[s].first, ~idx);  // the smallest index, complemented
+    const unsigned long long prev = atomicCAS(&T.keys[s], 0ull, mine);
+    if (prev == 0ull) return (int32_t)s;
+    if ((uint32_t)(prev >> 32) == mark) {
+      if (prev < mine) atomicMax(&T.keys[s], mine);
       return (int32_t)s;
     }
   }
@@ -129,14 +140,17 @@ __device__ __forceinline__ LaneSeq lane_seq(const BulkArgs& A, int64_t i) {
   return q;
 }
 
-// The tree (index into states) of op i.
+// The tree (index into states) of op i, where the ops of lower lanes come before it: a search for the warp's first op,
+// and from there a step per tree passed.  The whole warp calls it.
 __device__ __forceinline__ int32_t tree_of(const BulkArgs& A, int64_t i) {
   if (!A.peer_begin) return 0;
-  int32_t lo = 0, hi = A.n_trees;  // peer_begin[lo] <= i < peer_begin[hi]
+  const int64_t i0 = __shfl_sync(kFull, i, 0);
+  int32_t lo = 0, hi = A.n_trees;  // peer_begin[lo] <= i0 < peer_begin[hi]
   while (hi - lo > 1) {
     const int32_t mid = lo + (hi - lo) / 2;
-    if (__ldg(A.peer_begin + mid) <= i) lo = mid; else hi = mid;
+    if (__ldg(A.peer_begin + mid) <= i0) lo = mid; else hi = mid;
   }
+  while (lo + 1 < A.n_trees && __ldg(A.peer_begin + lo + 1) <= i) ++lo;
   return lo;
 }
 
@@ -178,19 +192,36 @@ __device__ int probe_lane(const int4* child, int32_t off, int32_t bits, int32_t 
   return 0;
 }
 
-// One lane: first j in [from, to) with lab[j] != q[pos + j], or to; eight pairs in flight.
+// A token of a label or a pool run that a lane reads on from: the whole 256 bytes come to L2 with the first one, where
+// a lane's next steps find them.
+__device__ __forceinline__ int32_t ld_ahead(const int32_t* p) {
+  int32_t x;
+  asm("ld.global.nc.L2::256B.b32 %0, [%1];" : "=r"(x) : "l"(p));
+  return x;
+}
+
+// One lane: first j in [from, to) with lab[j] != q[pos + j], or to; lab[0 .. from) is known to agree.  Eight pairs in
+// flight and no test per token: the last step ends at `to` and looks at tokens before it again instead of stopping
+// short, so that lanes with ends of their own stay together (with a tested tail per lane the resolve launch had
+// three times the instructions in this loop).  Only labels under eight tokens and steps across the two pool runs take
+// a token at a time.
 __device__ __forceinline__ int32_t diff_lane(const int32_t* lab, const LaneSeq& q, int32_t pos, int32_t from, int32_t to) {
   for (int32_t j0 = from; j0 < to; j0 += 8) {
-    int32_t x[8], y[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int32_t j = j0 + u;
-      x[u] = j < to ? __ldg(lab + j) : 0;
-      y[u] = j < to ? q.at(pos + j) : 0;
+    const int32_t s0 = min(j0, to - 8), p0 = pos + s0;
+    if (s0 < 0 || (p0 < q.na && q.na - p0 < 8)) {
+      const int32_t e = min(to, j0 + 8);
+      for (int32_t j = j0; j < e; ++j)
+        if (__ldg(lab + j) != q.at(pos + j)) return j;
+      continue;
     }
+    const int32_t* y = (p0 < q.na ? q.a : q.bo) + p0;
+    int32_t x[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (j0 + u < to && x[u] != y[u]) return j0 + u;
+    for (int u = 0; u < 8; ++u) x[u] = ld_ahead(lab + s0 + u);
+    unsigned d = 0;  // bit u: token u differs
+#pragma unroll
+    for (int u = 0; u < 8; ++u) d |= (x[u] != ld_ahead(y + u) ? 1u : 0u) << u;
+    if (d) return s0 + __ffs(d) - 1;
   }
   return to;
 }
@@ -214,11 +245,19 @@ __device__ int32_t diff_warp(const int32_t* a, const int32_t* b, int32_t from, i
       }
     }
   }
-  for (; j0 < to; j0 += 32) {
-    const int32_t j = j0 + lane;
-    const bool in = lane < to - j0;
-    const unsigned m = __ballot_sync(kFull, in && __ldg(a + j) != __ldg(b + j));
-    if (m) return j0 + (__ffs(m) - 1);
+  for (; j0 < to; j0 += 128) {
+    int32_t x[4], y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const bool in = u * 32 + lane < to - j0;
+      x[u] = in ? __ldg(a + j0 + u * 32 + lane) : 0;
+      y[u] = in ? __ldg(b + j0 + u * 32 + lane) : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const unsigned m = __ballot_sync(kFull, x[u] != y[u]);
+      if (m) return j0 + u * 32 + (__ffs(m) - 1);
+    }
   }
   return to;
 }
@@ -232,20 +271,27 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
   // Ops per warp: few enough that every warp has some, since a warp's long compares follow one another.
   const int32_t per = (int32_t)max((int64_t)1, min((int64_t)32, total / warps));
   const int32_t* list = A.lists + (round & 1) * A.n;
+  for (int64_t t = (int64_t)blockIdx.x * kBulkThreads + threadIdx.x; t < A.n_trees; t += (int64_t)gridDim.x * kBulkThreads) {
+    const TreeState& s = A.states[t];  // the arenas' use ahead of this round's reservations
+    A.base[3 * t] = s.n_node;
+    A.base[3 * t + 1] = s.n_child;
+    A.base[3 * t + 2] = s.n_label;
+  }
   for (int64_t b0 = (((int64_t)blockIdx.x * kBulkThreads + threadIdx.x) >> 5) * per; b0 < total; b0 += warps * per) {
     int64_t i = b0 + lane;
     bool valid = lane < per && i < total;
+    int32_t tree = round == 0 ? tree_of(A, min(i, total - 1)) : 0;
     if (valid && round > 0) i = list[i];
     valid = valid && !A.done[i];
     LaneSeq q{nullptr, nullptr, 0, 0};
-    int32_t tree = 0, opc = 0;
+    int32_t opc = 0;
     const int4* node = nullptr;
     const int4* child = nullptr;
     const int32_t* label = nullptr;
     if (valid) {
       q = lane_seq(A, i);
       opc = A.op[i];
-      tree = round == 0 ? tree_of(A, i) : A.ops[i].what >> kTreeShift;
+      if (round > 0) tree = A.ops[i].what >> kTreeShift;
       const TreeState& s = A.states[tree];
       node = s.node;
       child = s.child;
@@ -255,6 +301,7 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
     // The walk: at node u (record nd, reached at pos), its parent g (reached at gpos, gz children, gw sequences)
     // and that one's parent gg.
     int32_t u = 0, pos = 0, g = -1, gpos = 0, gz = 0, gw = 0, gg = -1, ggpos = 0, k = 0, waits = 0;
+    int32_t slot = -1;  // where the last probe ended
     int what = B_NONE, flags = 0;
     int4 nd = make_int4(0, 0, 0, 0), ce = nd, nn = nd;
     bool act = valid, held = false;  // held: at the edge ce, waiting for a pair that another warp compares
@@ -265,7 +312,6 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
       int32_t memo_at = -1;  // the pair's entry, when this lane is the one to compare it
       const int32_t* lab = nullptr;
       if (act && !held) {
-        int32_t slot;
         const int st = probe_lane<false>(child, nd.x, tab_bits(nd.y), q.at(pos), slot, ce);
         if (st != 1) {
           what = opc == P2P_OP_INSERT ? B_LEAF : B_ABSENT;
@@ -294,27 +340,26 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
         need = true;
         held = false;
       }
-      // A pair of an interned label and a pool run: how much of it is known to be equal.
+      // A pair of an interned label and a pool run: how much of it is known to be equal.  One lane of the warp at a time
+      // takes on a pair that nobody has compared yet, so that a launch's first compares spread over all warps (a
+      // warp that took on each of its lanes' pairs had 20 of them to do, one after another, with the others waiting).
+      int32_t free_at = -1;
+      unsigned long long key = 0;
       if (need && ce.z < 0 && A.memo_keys && q.na - pos >= first) {
         const int64_t so = q.a + pos - A.pool;
         if (so <= 0xffffffffll) {
-          const unsigned long long key =
-              (1ull << 63) | ((unsigned long long)(uint32_t)~ce.z << 32) | (unsigned long long)so;
+          key = (1ull << 63) | ((unsigned long long)(uint32_t)~ce.z << 32) | (unsigned long long)so;
           uint32_t s = (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> 32) & A.memo_mask;
           for (int it = 0; it < kMemoProbes; ++it, s = (s + 1) & A.memo_mask) {
-            unsigned long long have = __ldcg(A.memo_keys + s);
+            const unsigned long long have = __ldcg(A.memo_keys + s);
             if (have == 0ull) {
-              have = atomicCAS(A.memo_keys + s, 0ull, key);
-              if (have == 0ull) {
-                memo_at = (int32_t)s;
-                break;
-              }
+              free_at = (int32_t)s;
+              break;
             }
             if (have == key) {
               const int32_t known = __ldcg(A.memo_vals + s);
               if (known == 0 && ++waits < kMemoWaits) {
                 held = true;
-                need = false;
               } else if (known >= lim) {
                 k = lim;
                 need = false;
@@ -327,6 +372,13 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
           }
         }
       }
+      const unsigned fm = __ballot_sync(kFull, free_at >= 0);
+      if (free_at >= 0) {
+        if (lane == __ffs(fm) - 1 && atomicCAS(A.memo_keys + free_at, 0ull, key) == 0ull) memo_at = free_at;
+        else if (++waits < kMemoWaits) held = true;
+      }
+      if (held) need = false;
+      if (!__any_sync(kFull, act && !held)) __nanosleep(200);  // (bounded by kMemoWaits looks)
       for (unsigned m = __ballot_sync(kFull, need); m; m &= m - 1) {
         const int j = __ffs(m) - 1;
         const int32_t* l = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)lab, j);
@@ -368,65 +420,91 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
       }
     }
     int3 want = make_int3(0, 0, 0);
+    bool grow = false;
+    int4 mine_grow = make_int4(0, 0, 0, 0);
     if (valid) {
-      // The op's place and nodes.  An op that ended at a node has its place in the parent's table.
+      // The op's place and nodes.  An op that ended at a node has its place in the parent's table (the last slot found
+      // led to it).
       const bool at_node = pos == q.n;
-      const int32_t pu = at_node ? g : u, ppos = at_node ? gpos : pos, v = at_node ? u : -1;
+      const int32_t pu = at_node ? g : u, ppos = at_node ? gpos : pos;
+      const int32_t tok = q.at(ppos);
       const uint32_t idx = (uint32_t)i;
-      int32_t ent_u = -1, ent_v = -1, ent_y = -1, key2 = -1, y = -1, y_len = 0;
-      const int32_t key = enter_key(A.tab, tree, pu, q.at(ppos), round, idx);
+      int32_t arg = k, ent = -1;
+      const int32_t key = enter_key(A.tab, tree, pu, tok, round, idx);
       if (key < 0) what = B_LEFT;
-      if (what == B_FOLD) {  // the one other child of the place's node
-        const int4 rec = __ldg(node + pu);
-        const int32_t bits = tab_bits(rec.y);
-        if (bits <= kFoldBits)
-          for (int32_t s = 0; s < (1 << bits); ++s) {
-            const int4 e = __ldg(child + rec.x + s);
-            if (e.y >= 1 && e.y != v) y = e.y, y_len = e.w;
-          }
-        if (y < 0 || gg < 0) what = B_LEFT;
-      }
-      if (what == B_LEAF || what == B_SPLIT || what == B_REMOVE || what == B_FOLD) {
-        ent_u = enter_node(A.tab, tree, pu, round);
-        if (ent_u < 0) {
+      int4* out = reinterpret_cast<int4*>(A.ops + i);
+      if (what == B_LEAF || what == B_SPLIT || what == B_REMOVE) {
+        ent = enter_node(A.tab, tree, pu, round);
+        if (ent < 0) {
           what = B_LEFT;
-        } else if (what == B_FOLD) {
-          atomicMax(&A.tab.nodes[ent_u].alone, ~idx);
         } else {
-          BulkNode* e = A.tab.nodes + ent_u;
+          BulkNode* e = A.tab.nodes + ent;
           atomicAdd(&e->shared, 1u);
           if (what == B_LEAF && !(flags & BF_REVIVE)) {
             const uint32_t rank = atomicAdd(&e->leaves, 1u);
-            if (rank == 0) flags |= BF_GROW;  // this op sees to the node's table
-            // The root's table grows between launches only; a leaf past its half waits for that.
-            if (pu == 0 && tab_full(tab_bits(nd.y), (int64_t)tab_used(nd.y) + rank + 1)) flags |= BF_LATER;
+            // The first leaf under a node puts its table on the list of those that may have to grow.  The root's table
+            // grows between launches only; a leaf past its half waits for that.
+            if (pu != 0) grow = rank == 0;
+            else if (tab_full(tab_bits(nd.y), (int64_t)tab_used(nd.y) + rank + 1)) flags |= BF_LATER;
           }
           if (what == B_REMOVE && g != 0 && gw == 0 && (int64_t)atomicAdd(&e->removals, 1u) > (int64_t)gz - 3)
             flags |= BF_LATER;
         }
-      }
-      if (what == B_REMOVE || what == B_FOLD || what == B_COUNT) {
-        ent_v = enter_node(A.tab, tree, v, round);
-        if (ent_v < 0) what = B_LEFT;
-        else if (what == B_COUNT && !(flags & BF_ALONE)) atomicAdd(&A.tab.nodes[ent_v].shared, 1u);
-        else atomicMax(&A.tab.nodes[ent_v].alone, ~idx);
-      }
-      if (what == B_FOLD) {
-        key2 = enter_key(A.tab, tree, gg, q.at(ggpos), round, idx);
-        ent_y = enter_node(A.tab, tree, y, round);
-        if (key2 < 0 || ent_y < 0) what = B_LEFT;
-        else atomicMax(&A.tab.nodes[ent_y].alone, ~idx);
+        if (what == B_REMOVE) arg = u;
+        if (what == B_LEAF && pu != 0 && nd.z == 0) {
+          const int32_t key2 = enter_key(A.tab, tree, g, q.at(gpos), round, idx);
+          if (key2 < 0) what = B_LEFT;
+          flags |= BF_MORE;
+          out[2] = make_int4(key2, -1, -1, -1);
+        }
+      } else if (what == B_COUNT) {
+        arg = u;
+        ent = enter_node(A.tab, tree, u, round);
+        if (ent < 0) what = B_LEFT;
+        else if (flags & BF_ALONE) atomicMax(&A.tab.nodes[ent].alone, ~idx);
+        else atomicAdd(&A.tab.nodes[ent].shared, 1u);
+      } else if (what == B_FOLD) {
+        arg = u;
+        const int4 rec = __ldg(node + pu);
+        const int32_t bits = tab_bits(rec.y);
+        int4 y = make_int4(0, -1, 0, 0);  // the one other child
+        if (bits <= kFoldBits)
+          for (int32_t s = 0; s < (1 << bits); ++s) {
+            const int4 e = __ldg(child + rec.x + s);
+            if (e.y >= 1 && e.y != u) y = e;
+          }
+        int32_t key2 = -1, key3 = -1, ent_u = -1, ent_y = -1;
+        if (y.y >= 1 && gg >= 0) {
+          key2 = enter_key(A.tab, tree, gg, q.at(ggpos), round, idx);
+          ent_u = enter_node(A.tab, tree, pu, round);
+          if (ent_u >= 0) atomicMax(&A.tab.nodes[ent_u].alone, ~idx);
+          if (__ldg(node + y.y).z == 0) {
+            key3 = enter_key(A.tab, tree, pu, y.x, round, idx);
+          } else if ((ent_y = enter_node(A.tab, tree, y.y, round)) >= 0) {
+            atomicMax(&A.tab.nodes[ent_y].alone, ~idx);
+          }
+        }
+        if (key2 < 0 || ent_u < 0 || (key3 < 0 && ent_y < 0)) what = B_LEFT;
+        flags |= BF_MORE;
+        out[2] = make_int4(key2, key3, ent_u, ent_y);
+        out[3] = make_int4(gg, ggpos, 0, 0);
+        if (what == B_FOLD) want = make_int3(0, 0, ppos - ggpos + y.w);
       }
       // At most this much room.
       if (what == B_LEAF) want = make_int3(1, 0, q.n - ppos);
       if (what == B_SPLIT) want = make_int3(2, 1 << kMinTabBits, q.n - ppos - k);
-      if (what == B_FOLD) want = make_int3(0, 0, ppos - ggpos + y_len);
-      int4* out = reinterpret_cast<int4*>(A.ops + i);
-      out[0] = make_int4(what | flags | tree << kTreeShift, pu, ppos, k);
-      out[1] = make_int4(v, gg, ggpos, key);
-      out[2] = make_int4(key2, ent_u, ent_v, ent_y);
+      out[0] = make_int4(what | flags | tree << kTreeShift, pu, tok, slot);
+      out[1] = make_int4(key, arg, ent, ppos);
+      if (grow) mine_grow = make_int4(tree, pu, ent, 0);
     } else if (lane < per && i < A.n && b0 + lane < total && !A.done[i]) {
       A.ops[i].what = B_LEFT;  // an empty sequence
+    }
+    const unsigned gm = __ballot_sync(kFull, grow);
+    if (gm) {
+      int32_t at = 0;
+      if (lane == 0) at = atomicAdd(&A.counts[kBulkRounds + 1 + round], __popc(gm));
+      at = __shfl_sync(kFull, at, 0);
+      if (grow) A.grow[at + __popc(gm & ((1u << lane) - 1))] = mine_grow;
     }
     // The room the round may take, once per tree and warp.
     for (unsigned m = __ballot_sync(kFull, want.x | want.y | want.z); m;) {
@@ -447,111 +525,167 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
   }
 }
 
-// Reserves k units of a tree's counter; -1 if they do not fit.
-__device__ int32_t reserve(int32_t* ctr, int32_t cap, int64_t k) {
-  int32_t old = *(volatile int32_t*)ctr;
-  for (int it = 0; it < (1 << 20); ++it) {
-    if ((int64_t)old + k > cap) return -1;
-    const int32_t prev = atomicCAS(ctr, old, (int32_t)(old + k));
-    if (prev == old) return old;
-    old = prev;
-  }
-  return -1;
-}
-// The same where every reservation of the launch together asks for at most `most` units.  Warps that all compare and
-// swap one counter take turns failing (4,096 ops of one tree: 1.5 ms); while there is room for all of them, now and so
-// to the launch's end, an addition cannot go too far and none has to be taken back.
-__device__ int32_t reserve(int32_t* ctr, int32_t cap, int64_t k, unsigned long long most) {
-  if ((unsigned long long)*(volatile int32_t*)ctr + most <= (unsigned long long)cap) return atomicAdd(ctr, (int32_t)k);
-  return reserve(ctr, cap, k);
-}
 __device__ __forceinline__ void add64(int64_t* p, int64_t v) {
   if (v) atomicAdd((unsigned long long*)p, (unsigned long long)v);
 }
 
-// The first leaf under a node sees to its table: if the round's leaves would take it past 1/2 claimed, one warp
-// moves it to a table of at most 1/4 live load (as delta_kernel grows tables).  A table that cannot grow (no room in
-// the arena) marks the entry, and its leaves wait.
+// Moves the table of 2^bits slots at off to the fresh one of 2^nb <= 32 slots at dst, one lane: four slots at a time,
+// placed by the bit mask of the slots it has filled.
+__device__ void move_table_lane(int4* child, int32_t off, int32_t bits, int32_t dst, int32_t nb) {
+  const uint32_t mask = (1u << nb) - 1;
+  uint32_t used = 0;
+  for (int32_t t0 = 0; bits && t0 < (1 << bits); t0 += 4) {
+    int4 e[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) e[c] = __ldcg(child + off + t0 + c);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (e[c].y < 1) continue;
+      uint32_t sl = slot_hash(e[c].x, nb);
+      while ((used >> sl) & 1u) sl = (sl + 1) & mask;
+      used |= 1u << sl;
+      child[dst + sl] = e[c];
+    }
+  }
+  for (uint32_t t = 0; t <= mask; ++t)
+    if (!((used >> t) & 1u)) child[dst + t] = make_int4(0, 0, 0, 0);
+}
+
+// The same for any size, one warp.
+__device__ void move_table_warp(int4* child, int32_t off, int32_t bits, int32_t dst, int32_t nb, int lane) {
+  const uint32_t mask = (1u << nb) - 1;
+  for (int32_t t = lane; t < (1 << nb); t += 32) child[dst + t] = make_int4(0, 0, 0, 0);
+  __syncwarp();
+  for (int32_t t0 = 0; bits && t0 < (1 << bits); t0 += 128) {
+    int4 e[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int32_t t = t0 + c * 32 + lane;
+      e[c] = t < (1 << bits) ? __ldcg(child + off + t) : make_int4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (e[c].y < 1) continue;
+      const unsigned long long kv = (unsigned long long)(uint32_t)e[c].x | ((unsigned long long)(uint32_t)e[c].y << 32);
+      uint32_t sl = slot_hash(e[c].x, nb);
+      for (uint32_t it = 0; it <= mask; ++it, sl = (sl + 1) & mask)
+        if (atomicCAS((unsigned long long*)&child[dst + sl], 0ull, kv) == 0ull) {
+          child[dst + sl].z = e[c].z;
+          child[dst + sl].w = e[c].w;
+          break;
+        }
+    }
+  }
+  __syncwarp();
+}
+
+// A lane per listed node: if the round's leaves would take its table past 1/2 claimed, it moves to one of at most 1/4
+// live load (as delta_kernel grows tables), small ones by the lane and larger ones by the warp.  A table that cannot
+// grow (no room in the arena) marks the node's entry, and its leaves wait.
 __global__ void __launch_bounds__(kBulkThreads) bulk_grow_kernel(BulkArgs A, int round) {
   const int lane = threadIdx.x & 31;
-  const int64_t total = list_size(A, round);
-  const int64_t warps = (int64_t)gridDim.x * kBulkWarps;
-  const int32_t* list = A.lists + (round & 1) * A.n;
-  for (int64_t b0 = (((int64_t)blockIdx.x * kBulkThreads + threadIdx.x) >> 5) * 32; b0 < total; b0 += warps * 32) {
-    int64_t i = b0 + lane;
-    const bool valid = i < total;
-    if (valid && round > 0) i = list[i];
-    int32_t u = 0, tree = 0, nb = 0, ent = -1;
+  const int32_t total = A.counts[kBulkRounds + 1 + round];
+  const int32_t stride = (int32_t)gridDim.x * kBulkThreads;
+  for (int32_t b0 = ((int32_t)blockIdx.x * kBulkWarps + (int32_t)(threadIdx.x >> 5)) * 32; b0 < total; b0 += stride) {
+    const bool valid = b0 + lane < total;
+    const int4 gr = valid ? A.grow[b0 + lane] : make_int4(-1, 0, 0, 0);
+    const int32_t tree = gr.x, u = gr.y;
+    int32_t nb = 0, c0 = 0;
     int4 rec = make_int4(0, 0, 0, 0);
-    if (valid && !A.done[i]) {
-      const BulkOp& b = A.ops[i];
-      if (b.what & BF_GROW) {
-        ent = b.ent_u;
-        u = b.u;
-        const int64_t leaves = A.tab.nodes[ent].leaves;
-        if (u != 0 && leaves > 0) {
-          tree = b.what >> kTreeShift;
-          rec = A.states[tree].node[u];
-          const int32_t bits = tab_bits(rec.y);
-          if (tab_full(bits, (int64_t)tab_used(rec.y) + leaves)) {
-            nb = bits ? bits + 1 : kMinTabBits;
-            while (nb < kMaxTabBits && ((int64_t)rec.z + leaves) * 4 > ((int64_t)1 << nb)) ++nb;
+    TreeState* s = A.states + max(tree, 0);
+    if (valid) {
+      const int64_t leaves = A.tab.nodes[gr.z].leaves;
+      rec = s->node[u];
+      const int32_t bits = tab_bits(rec.y);
+      if (tab_full(bits, (int64_t)tab_used(rec.y) + leaves)) {
+        nb = bits ? bits + 1 : kMinTabBits;
+        while (nb < kMaxTabBits && ((int64_t)rec.z + leaves) * 4 > ((int64_t)1 << nb)) ++nb;
+      }
+    }
+    const int32_t bits = tab_bits(rec.y);
+    // Slots, once per tree and warp.
+    for (unsigned m = __ballot_sync(kFull, nb > 0); m;) {
+      const int32_t t = __shfl_sync(kFull, tree, __ffs(m) - 1);
+      const bool mine = nb > 0 && tree == t;
+      const unsigned mm = __ballot_sync(kFull, mine);
+      m &= ~mm;
+      int64_t sum = mine ? (int64_t)1 << nb : 0, old = mine && bits ? (int64_t)1 << bits : 0;
+      const int64_t own = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(kFull, sum, o);
+        if (lane >= o) sum += y;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) old += __shfl_xor_sync(kFull, old, o);
+      const int64_t all = __shfl_sync(kFull, sum, 31);
+      TreeState* ts = A.states + t;
+      int32_t at = -1;
+      if (lane == 0) {
+        int32_t have = *(volatile int32_t*)&ts->n_child;
+        for (int it = 0; it < (1 << 20) && (int64_t)have + all <= ts->cap_child; ++it) {
+          const int32_t prev = atomicCAS(&ts->n_child, have, (int32_t)(have + all));
+          if (prev == have) {
+            at = have;
+            break;
           }
+          have = prev;
+        }
+        if (at >= 0) {
+          atomicAdd(&A.base[3 * t + 1], (int32_t)all);
+          add64(&ts->stale_child, old);
+        }
+      }
+      at = __shfl_sync(kFull, at, 0);
+      if (mine) {
+        if (at < 0) {
+          A.tab.nodes[gr.z].stuck = 1;
+          nb = 0;
+        } else {
+          c0 = (int32_t)(at + sum - own);
         }
       }
     }
-    for (unsigned m = __ballot_sync(kFull, nb > 0); m; m &= m - 1) {
+    int4* child = s->child;
+    if (nb > 0 && nb <= kLaneBits) move_table_lane(child, rec.x, bits, c0, nb);
+    for (unsigned m = __ballot_sync(kFull, nb > kLaneBits); m; m &= m - 1) {
       const int j = __ffs(m) - 1;
-      TreeState* s = A.states + __shfl_sync(kFull, tree, j);
-      const int32_t bits2 = __shfl_sync(kFull, nb, j);
-      const int32_t off = __shfl_sync(kFull, rec.x, j), meta = __shfl_sync(kFull, rec.y, j);
-      const int32_t bits = tab_bits(meta);
-      int32_t c0 = 0;
-      if (lane == 0) c0 = reserve(&s->n_child, s->cap_child, (int64_t)1 << bits2);
-      c0 = __shfl_sync(kFull, c0, 0);
-      if (c0 < 0) {
-        if (lane == j) A.tab.nodes[ent].stuck = 1;
-        continue;
-      }
-      int4* child = s->child;
-      for (int32_t t = lane; t < (1 << bits2); t += 32) child[c0 + t] = make_int4(0, 0, 0, 0);
-      __syncwarp();
-      const uint32_t mask = (1u << bits2) - 1;
-      for (int32_t t0 = 0; bits && t0 < (1 << bits); t0 += 128) {
-        int4 e[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int32_t t = t0 + c * 32 + lane;
-          e[c] = t < (1 << bits) ? child[off + t] : make_int4(0, 0, 0, 0);
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          if (e[c].y < 1) continue;
-          const unsigned long long kv =
-              (unsigned long long)(uint32_t)e[c].x | ((unsigned long long)(uint32_t)e[c].y << 32);
-          uint32_t sl = slot_hash(e[c].x, bits2);
-          for (uint32_t it = 0; it <= mask; ++it, sl = (sl + 1) & mask)
-            if (atomicCAS((unsigned long long*)&child[c0 + sl], 0ull, kv) == 0ull) {
-              child[c0 + sl].z = e[c].z;
-              child[c0 + sl].w = e[c].w;
-              break;
-            }
-        }
-      }
-      __syncwarp();
-      if (lane == j) {
-        s->node[u] = make_int4(c0, make_meta(bits2, rec.z), rec.z, rec.w);
-        if (bits) add64(&s->stale_child, (int64_t)1 << bits);
-      }
+      move_table_warp((int4*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)child, j), __shfl_sync(kFull, rec.x, j),
+                      __shfl_sync(kFull, bits, j), __shfl_sync(kFull, c0, j), __shfl_sync(kFull, nb, j), lane);
     }
+    if (nb > 0) s->node[u] = make_int4(c0, make_meta(nb, rec.z), rec.z, rec.w);
   }
 }
 
 // Copies, for every lane with n > 0, n tokens to dst: [0, na) from a, the rest from bo (bo[j] for j >= na); the
-// whole warp copies, kCopies lanes' runs in flight at a time.
-constexpr int kCopies = 4;
+// whole warp copies.  Long runs (whole prompts) go one after another, 512 tokens per step, the others four at a time,
+// 128 tokens of each per step: 16 loads a lane in flight both ways.  (Four at a time throughout, 64 tokens of each,
+// every prompt among them took 35 round trips: the apply launch of 1,024,000 ops
+// 0.42 -> 0.32 ms.)
+constexpr int kCopies = 4, kCopySteps = 4;
+constexpr int32_t kLongCopy = 256;
 __device__ void copy_runs(int32_t* dst, const int32_t* a, const int32_t* bo, int32_t na, int32_t n, int lane) {
-  unsigned m = __ballot_sync(kFull, n > 0);
+  for (unsigned m = __ballot_sync(kFull, n > kLongCopy); m; m &= m - 1) {
+    const int j = __ffs(m) - 1;
+    int32_t* d = (int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)dst, j);
+    const int32_t* pa = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)a, j);
+    const int32_t* pb = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)bo, j);
+    const int32_t ca = __shfl_sync(kFull, na, j), cn = __shfl_sync(kFull, n, j);
+    for (int32_t t0 = 0; t0 < cn; t0 += 32 * kCopies * kCopySteps) {
+      int32_t x[kCopies * kCopySteps];
+#pragma unroll
+      for (int s = 0; s < kCopies * kCopySteps; ++s) {
+        const int32_t t = t0 + s * 32 + lane;
+        x[s] = t < cn ? ((t < ca ? pa : pb)[t]) : 0;
+      }
+#pragma unroll
+      for (int s = 0; s < kCopies * kCopySteps; ++s) {
+        const int32_t t = t0 + s * 32 + lane;
+        if (t < cn) d[t] = x[s];
+      }
+    }
+  }
+  unsigned m = __ballot_sync(kFull, n > 0 && n <= kLongCopy);
   while (m) {
     int32_t* d[kCopies];
     const int32_t *pa[kCopies], *pb[kCopies];
@@ -567,19 +701,19 @@ __device__ void copy_runs(int32_t* dst, const int32_t* a, const int32_t* bo, int
       m &= m - 1;
       most = max(most, cn[c]);
     }
-    for (int32_t t0 = 0; t0 < most; t0 += 64) {
-      int32_t x[kCopies][2];
+    for (int32_t t0 = 0; t0 < most; t0 += 32 * kCopySteps) {
+      int32_t x[kCopies][kCopySteps];
 #pragma unroll
       for (int c = 0; c < kCopies; ++c)
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
+        for (int s = 0; s < kCopySteps; ++s) {
           const int32_t t = t0 + s * 32 + lane;
           x[c][s] = t < cn[c] ? ((t < ca[c] ? pa[c] : pb[c])[t]) : 0;
         }
 #pragma unroll
       for (int c = 0; c < kCopies; ++c)
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
+        for (int s = 0; s < kCopySteps; ++s) {
           const int32_t t = t0 + s * 32 + lane;
           if (t < cn[c]) d[c][t] = x[c][s];
         }
@@ -594,7 +728,7 @@ __device__ __forceinline__ bool adjacent(const int4& a, const int4& b) {  // lab
 }
 
 __device__ __forceinline__ bool won(const BulkArgs& A, int32_t key, uint32_t idx) {
-  return A.tab.keys[key].first == ~idx;
+  return (uint32_t)__ldcg(A.tab.keys + key) == ~idx;
 }
 __device__ __forceinline__ bool alone(const BulkArgs& A, int32_t ent, uint32_t idx) {
   const BulkNode& e = A.tab.nodes[ent];
@@ -613,70 +747,91 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
     bool valid = lane < per && i < total;
     if (valid && round > 0) i = list[i];
     valid = valid && !A.done[i];
-    LaneSeq q{nullptr, nullptr, 0, 0};
-    if (valid) q = lane_seq(A, i);
-    valid = valid && q.n > 0;
-    BulkOp b;
-    int what = B_NONE, opc = 0;
-    int32_t tree = -1;
+    int what = B_NONE, flags = 0, opc = 0;
+    int32_t tree = -1, u = 0, tok = 0, slot = -1, arg = 0, pos = 0;
     bool go = false;
-    if (valid) {
-      const int4* in = reinterpret_cast<const int4*>(A.ops + i);
-      const int4 x = in[0], y = in[1], z = in[2];
-      b = BulkOp{x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w, z.x, z.y, z.z, z.w};
-      what = b.what & 15;
-      opc = A.op[i];
-      tree = b.what >> kTreeShift;
-      const uint32_t idx = (uint32_t)i;
-      go = what != B_LEFT && !(b.what & BF_LATER) && won(A, b.key, idx);
-      if (go && what == B_LEAF && !(b.what & BF_REVIVE)) go = !A.tab.nodes[b.ent_u].stuck;
-      if (go && what == B_COUNT && (b.what & BF_ALONE)) go = alone(A, b.ent_v, idx);
-      if (go && (what == B_REMOVE || what == B_FOLD)) go = alone(A, b.ent_v, idx);
-      if (go && what == B_FOLD) go = won(A, b.key2, idx) && alone(A, b.ent_u, idx) && alone(A, b.ent_y, idx);
-    }
-    // Where the op acts, looked up again: tables may have moved since the walk.
-    TreeState* s = A.states + max(tree, 0);
+    LaneSeq q{nullptr, nullptr, 0, 0};
+    const uint32_t idx = (uint32_t)i;
+    const int4* in = reinterpret_cast<const int4*>(A.ops + i);
+    TreeState* s = A.states;
     int4 *node = nullptr, *child = nullptr;
     const int32_t* label = nullptr;
-    int4 rec = make_int4(0, 0, 0, 0), e = rec, pe = rec, ye = rec;
-    int32_t slot = -1, pslot = -1, tok = 0;
-    int32_t want_n = 0, want_c = 0;
-    int64_t want_l = 0;
-    if (go) {
+    int4 rec = make_int4(0, 0, 0, 0), e = rec;
+    if (valid) {
+      const int4 x = in[0], y = in[1];
+      what = x.x & 15;
+      flags = x.x & 0xf0;
+      tree = x.x >> kTreeShift;
+      u = x.y;
+      tok = x.z;
+      slot = x.w;
+      arg = y.y;
+      pos = y.w;
+      opc = A.op[i];
+      s += tree;
       node = s->node;
       child = s->child;
       label = s->label;
-      if (what == B_LEAF || what == B_SPLIT || what == B_REMOVE || what == B_FOLD) {
-        rec.x = __ldcg(&node[b.u].x);
-        rec.y = __ldcg(&node[b.u].y);
-        tok = q.at(b.pos);
-        const int st = probe_lane<true>(child, rec.x, tab_bits(rec.y), tok, slot, e);
-        const int expect = what == B_LEAF ? (b.what & BF_REVIVE ? 2 : 0) : 1;
-        go = st == expect && slot >= 0;  // (always: nothing else may touch this op's slot)
+      go = what != B_LEFT && !(flags & BF_LATER) && won(A, y.x, idx);
+      if (go && what == B_LEAF && !(flags & BF_REVIVE)) go = !A.tab.nodes[y.z].stuck;
+      if (go && what == B_COUNT && (flags & BF_ALONE)) go = alone(A, y.z, idx);
+      if (go && (flags & BF_MORE)) {
+        const int4 z = in[2];
+        go = won(A, z.x, idx);
+        if (go && what == B_FOLD)
+          go = alone(A, z.z, idx) && (z.y >= 0 ? won(A, z.y, idx) : alone(A, z.w, idx));
       }
-      if (go && what == B_FOLD) {
-        const int4 gr = make_int4(__ldcg(&node[b.g].x), __ldcg(&node[b.g].y), 0, 0);
-        int32_t ys = -1;
-        for (int32_t t = 0; t < (1 << tab_bits(rec.y)); ++t) {
-          const int4 o = __ldcg(child + rec.x + t);
-          if (o.y >= 1 && o.y != b.v) ys = t, ye = o;
+      if (what == B_LEFT) valid = A.seg_begin[i + 1] > A.seg_begin[i] && lane_seq(A, i).n > 0;  // (not an empty sequence)
+      if (go && (what == B_LEAF || what == B_SPLIT || what == B_FOLD)) q = lane_seq(A, i);
+      // The place, as the walk found it or, where the table has moved since, looked up again.
+      if (go && what <= B_FOLD && what != B_COUNT) {
+        rec.x = __ldcg(&node[u].x);
+        rec.y = __ldcg(&node[u].y);
+        const int32_t bits = tab_bits(rec.y);
+        const bool there = slot >= rec.x && slot < rec.x + (bits ? 1 << bits : 0);
+        if (!there || (what != B_LEAF && what != B_FOLD) || (flags & BF_REVIVE)) {
+          if (there && !(flags & BF_REVIVE)) {
+            const longlong2 w = __ldcg(reinterpret_cast<const longlong2*>(child + slot));
+            e = make_int4((int32_t)w.x, (int32_t)((unsigned long long)w.x >> 32), (int32_t)w.y,
+                          (int32_t)((unsigned long long)w.y >> 32));
+            go = e.x == tok && e.y >= 1;  // (always: nothing else may touch this op's slot)
+          } else {
+            const int st = probe_lane<true>(child, rec.x, bits, tok, slot, e);
+            const int expect = what == B_LEAF ? (flags & BF_REVIVE ? 2 : 0) : 1;
+            go = st == expect && slot >= 0;
+          }
         }
-        go = ys >= 0 && probe_lane<true>(child, gr.x, tab_bits(gr.y), q.at(b.gpos), pslot, pe) == 1;
-        if (go && !adjacent(pe, ye)) want_l = (int64_t)pe.w + ye.w;
-      }
-      if (go && what == B_LEAF) want_n = 1, want_l = q.n - b.pos;
-      if (go && what == B_SPLIT) {
-        want_l = q.n - b.pos - b.k;
-        want_n = want_l > 0 ? 2 : 1;
-        want_c = 1 << kMinTabBits;
       }
     }
-    // Room, once per tree and warp; a group that does not fit waits (delta_kernel asks the host for room).
+    // A fold: u's own slot, and the child it takes in.
+    int4 pe = make_int4(0, 0, 0, 0), ye = pe;
+    int32_t pslot = -1;
+    int32_t want_n = 0, want_c = 0, want_l = 0;
+    if (go && what == B_FOLD) {
+      const int4 gp = in[3];
+      const int32_t gx = __ldcg(&node[gp.x].x), gy = __ldcg(&node[gp.x].y);
+      int32_t ys = -1;
+      slot = -1;
+      for (int32_t t = 0; t < (1 << tab_bits(rec.y)); ++t) {
+        const int4 o = __ldcg(child + rec.x + t);
+        if (o.y >= 1 && o.y != arg) ys = t, ye = o;
+        if (o.y == arg) slot = rec.x + t, e = o;
+      }
+      go = ys >= 0 && slot >= 0 && probe_lane<true>(child, gx, tab_bits(gy), q.at(gp.y), pslot, pe) == 1;
+      if (go && !adjacent(pe, ye)) want_l = pe.w + ye.w;
+    }
+    if (go && what == B_LEAF) want_n = 1, want_l = q.n - pos;
+    if (go && what == B_SPLIT) {
+      want_l = q.n - pos - arg;
+      want_n = want_l > 0 ? 2 : 1;
+      want_c = 1 << kMinTabBits;
+    }
+    // Room, once per tree and warp.  Everything the round may take fits (an addition then cannot go too far, so none
+    // has to be taken back), or the tree's ops that need room all wait until the host has grown it.
     int32_t n0 = 0, c0 = 0, l0 = 0;
-    for (unsigned m = __ballot_sync(kFull, go && (want_n || want_c || want_l)); m;) {
-      const int j = __ffs(m) - 1;
-      const int32_t t = __shfl_sync(kFull, tree, j);
-      const bool mine = go && tree == t && (want_n || want_c || want_l);
+    for (unsigned m = __ballot_sync(kFull, want_n | want_c | want_l); m;) {
+      const int32_t t = __shfl_sync(kFull, tree, __ffs(m) - 1);
+      const bool mine = (want_n | want_c | want_l) && tree == t;
       m &= ~__ballot_sync(kFull, mine);
       int32_t sn = mine ? want_n : 0, sc = mine ? want_c : 0;
       int64_t sl = mine ? want_l : 0;
@@ -689,20 +844,26 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
       const int32_t tn = __shfl_sync(kFull, sn, 31), tc = __shfl_sync(kFull, sc, 31);
       const int64_t tl = __shfl_sync(kFull, sl, 31);
       TreeState* ts = A.states + t;
-      const unsigned long long* most = A.want + ((int64_t)round * A.n_trees + t) * 3;
       int32_t r = 0;
-      if (lane == 0 && tn) r = reserve(&ts->n_node, ts->cap_node, tn, most[0]);
-      if (lane == 1 && tc) r = reserve(&ts->n_child, ts->cap_child, tc, most[1]);
-      if (lane == 2 && tl) r = reserve(&ts->n_label, ts->cap_label, tl, most[2]);
-      const bool ok = __all_sync(kFull, r >= 0);
-      if (!ok) {  // what was taken stays behind as stale space
-        if (lane == 0 && tn && r >= 0) add64(&ts->dead_nodes, tn);
-        if (lane == 1 && tc && r >= 0) add64(&ts->stale_child, tc);
-        if (lane == 2 && tl && r >= 0) add64(&ts->stale_label, tl);
-        if (mine) go = false;
+      bool fits = true;
+      if (lane < 3) {
+        const unsigned long long most = A.want[((int64_t)round * A.n_trees + t) * 3 + lane];
+        const int32_t cap = lane == 0 ? ts->cap_node : lane == 1 ? ts->cap_child : ts->cap_label;
+        fits = most == 0 || (unsigned long long)A.base[3 * t + lane] + most <= (unsigned long long)cap;
+        if (!fits) {
+          atomicOr(&ts->status, DELTA_NEED_SPACE | DELTA_NEED_BULK);
+          atomicMax(lane == 0 ? &ts->need_node : lane == 1 ? &ts->need_child : &ts->need_label,
+                    (int32_t)min(most, (unsigned long long)INT32_MAX));
+        }
+      }
+      const bool ok = __all_sync(kFull, fits);
+      if (ok && lane < 3) {
+        const int32_t k = lane == 0 ? tn : lane == 1 ? tc : (int32_t)tl;
+        if (k) r = atomicAdd(lane == 0 ? &ts->n_node : lane == 1 ? &ts->n_child : &ts->n_label, k);
       }
       const int32_t bn = __shfl_sync(kFull, r, 0), bc = __shfl_sync(kFull, r, 1), bl = __shfl_sync(kFull, r, 2);
       if (mine) {
+        go = ok;
         n0 = bn + sn - want_n;
         c0 = bc + sc - want_c;
         l0 = (int32_t)(bl + sl - want_l);
@@ -710,7 +871,7 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
     }
     // The new labels: a leaf's tokens, or a fold's two labels joined.
     {
-      const int32_t n = go ? (int32_t)want_l : 0;
+      const int32_t n = go ? want_l : 0;
       const int32_t *a = q.a, *bo = q.bo;
       int32_t na = 0;
       if (n > 0) {
@@ -734,9 +895,9 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
         case B_LEAF: {
           node[n0] = make_int4(0, 0, 0, 1);
           const unsigned long long kv = (unsigned long long)(uint32_t)tok | ((unsigned long long)(uint32_t)n0 << 32);
-          if (b.what & BF_REVIVE) {
+          if (flags & BF_REVIVE) {
             child[slot].z = l0;
-            child[slot].w = (int32_t)want_l;
+            child[slot].w = want_l;
             child[slot].y = n0;
           } else {
             // The probe's first empty slot, or the next: other leaves of this table claim theirs meanwhile.  The
@@ -747,13 +908,13 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
             for (uint32_t it = 0; it <= mask; ++it, sl = (sl + 1) & mask)
               if (atomicCAS((unsigned long long*)&child[rec.x + sl], 0ull, kv) == 0ull) {
                 child[rec.x + sl].z = l0;
-                child[rec.x + sl].w = (int32_t)want_l;
+                child[rec.x + sl].w = want_l;
                 break;
               }
-            atomicAdd(&node[b.u].y, 1 << 5);
+            atomicAdd(&node[u].y, 1 << 5);
           }
-          atomicAdd(&node[b.u].z, 1);
-          if (b.u == 0) {
+          atomicAdd(&node[u].z, 1);
+          if (u == 0) {
             const uint32_t h = root_filter_bit(tok);
             atomicOr(s->rfilter + (h >> 5), 1u << (h & 31));
           }
@@ -762,12 +923,12 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
         case B_SPLIT: {
           const bool tail = want_l > 0;
           const int32_t mid = n0, leaf = n0 + 1;
-          const int4 lower = make_int4(label_ptr(label, A.shared, e.z)[b.k], e.y, label_adv(e.z, b.k), e.w - b.k);
+          const int4 lower = make_int4(label_ptr(label, A.shared, e.z)[arg], e.y, label_adv(e.z, arg), e.w - arg);
           const uint32_t mask = (1u << kMinTabBits) - 1, s0 = slot_hash(lower.x, kMinTabBits);
           uint32_t s1 = s0;
           int4 le = make_int4(0, 0, 0, 0);
           if (tail) {
-            le = make_int4(q.at(b.pos + b.k), leaf, l0, (int32_t)want_l);
+            le = make_int4(q.at(pos + arg), leaf, l0, want_l);
             s1 = slot_hash(le.x, kMinTabBits);
             if (s1 == s0) s1 = (s1 + 1) & mask;
             node[leaf] = make_int4(0, 0, 0, 1);
@@ -775,26 +936,26 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
           for (uint32_t t = 0; t <= mask; ++t)
             child[c0 + t] = t == s0 ? lower : (tail && t == s1) ? le : make_int4(0, 0, 0, 0);
           node[mid] = make_int4(c0, make_meta(kMinTabBits, tail ? 2 : 1), tail ? 2 : 1, tail ? 0 : 1);
-          child[slot] = make_int4(tok, mid, e.z, b.k);  // the slot keeps its key; the label starts where it did
+          child[slot] = make_int4(tok, mid, e.z, arg);  // the slot keeps its key; the label starts where it did
           break;
         }
         case B_COUNT:
-          atomicAdd(&node[b.v].w, opc == P2P_OP_INSERT ? 1 : -1);
+          atomicAdd(&node[arg].w, opc == P2P_OP_INSERT ? 1 : -1);
           break;
         case B_REMOVE:
         case B_FOLD: {
-          const int32_t vb = tab_bits(__ldcg(&node[b.v].y));
+          const int32_t vb = tab_bits(__ldcg(&node[arg].y));
           child[slot].y = -1;  // a tombstone: the slot keeps its key
           st_label = e.w;
           dead = 1;
           st_child = vb ? 1 << vb : 0;
           if (what == B_REMOVE) {
-            atomicAdd(&node[b.u].z, -1);
+            atomicAdd(&node[u].z, -1);
           } else {
             // u takes its last child in: the joined label, the child's record.
             child[pslot].z = want_l > 0 ? l0 : pe.z;
             child[pslot].w = pe.w + ye.w;
-            node[b.u] = node[ye.y];
+            node[u] = node[ye.y];
             st_label += want_l;
             dead += 1;
             st_child += tab_bits(rec.y) ? 1 << tab_bits(rec.y) : 0;
@@ -838,13 +999,11 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
 cudaError_t launch_bulk(const BulkArgs& A, int num_sms, cudaStream_t st, int* launched) {
   *launched = 0;
   if (A.n <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(A.tab.keys, 0, ((size_t)A.tab.key_mask + 1) * sizeof(BulkKey), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(A.tab.nodes, 0, ((size_t)A.tab.node_mask + 1) * sizeof(BulkNode), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(A.want, 0, A.n_want * sizeof(unsigned long long), st);
+  cudaError_t e = cudaMemsetAsync(A.tab.keys, 0, A.n_zero, st);
   if (e != cudaSuccess) return e;
   // A warp per op up to a full wave of resident CTAs (the kernels then take more ops per warp).
   const int grid = (int)std::min<int64_t>((A.n + kBulkWarps - 1) / kBulkWarps, (int64_t)num_sms * kBulkCtasPerSm);
-  const int grid_g = (int)std::min<int64_t>((A.n + kBulkThreads - 1) / kBulkThreads, (int64_t)num_sms * 8);
+  const int grid_g = (int)std::min<int64_t>((A.n + kBulkThreads - 1) / kBulkThreads, (int64_t)num_sms * 4);
   for (int round = 0; round < kBulkRounds; ++round) {
     P2P_TIMED(K_BULK_RESOLVE, st, (bulk_resolve_kernel<<<grid, kBulkThreads, 0, st>>>(A, round)));
     P2P_TIMED(K_BULK_GROW, st, (bulk_grow_kernel<<<grid_g, kBulkThreads, 0, st>>>(A, round)));
@@ -855,9 +1014,10 @@ cudaError_t launch_bulk(const BulkArgs& A, int num_sms, cudaStream_t st, int* la
 }
 
 size_t bulk_scratch(int64_t n, int32_t n_trees, void* base, BulkArgs& A) {
+  // Entries: a place per op and a few more for folds, a node per op at most, over all rounds.
   int64_t keys = 1024, nodes = 1024;
-  while (keys < 4 * n) keys <<= 1;
-  while (nodes < 2 * n) nodes <<= 1;
+  while (keys < 2 * n) keys <<= 1;
+  while (nodes < n + n / 4) nodes <<= 1;
   char* p = static_cast<char*>(base);
   size_t at = 0;
   auto take = [&](size_t bytes) {
@@ -865,15 +1025,17 @@ size_t bulk_scratch(int64_t n, int32_t n_trees, void* base, BulkArgs& A) {
     at += (bytes + 255) & ~(size_t)255;
     return q;
   };
-  A.tab.keys = static_cast<BulkKey*>(take((size_t)keys * sizeof(BulkKey)));
+  A.tab.keys = static_cast<unsigned long long*>(take((size_t)keys * sizeof(unsigned long long)));
   A.tab.key_mask = (uint32_t)(keys - 1);
   A.tab.nodes = static_cast<BulkNode*>(take((size_t)nodes * sizeof(BulkNode)));
   A.tab.node_mask = (uint32_t)(nodes - 1);
+  A.want = static_cast<unsigned long long*>(take((size_t)kBulkRounds * n_trees * 3 * sizeof(unsigned long long)));
+  A.counts = static_cast<int32_t*>(take((2 * kBulkRounds + 1) * sizeof(int32_t)));
+  A.n_zero = at;  // cleared by the launch up to here
+  A.base = static_cast<int32_t*>(take((size_t)n_trees * 3 * sizeof(int32_t)));
   A.ops = static_cast<BulkOp*>(take((size_t)n * sizeof(BulkOp)));
   A.lists = static_cast<int32_t*>(take((size_t)n * 2 * sizeof(int32_t)));
-  A.n_want = (size_t)kBulkRounds * n_trees * 3 + (kBulkRounds + 3) / 2;  // the counts behind them
-  A.want = static_cast<unsigned long long*>(take(A.n_want * sizeof(unsigned long long)));
-  A.counts = reinterpret_cast<int32_t*>(A.want + (size_t)kBulkRounds * n_trees * 3);
+  A.grow = static_cast<int4*>(take((size_t)n * sizeof(int4)));
   return at;
 }
 

@@ -927,7 +927,13 @@ __global__ void __launch_bounds__(kDeltaWarps * 32, 2)
   TreeState* gs = states + (kParts ? (pw & kPartTreeMask) : pw);
   if (lane < kMemoSlots) s_memo[warp][lane] = MemoEntry{nullptr, nullptr, 0};
   const int64_t op_begin = gs->op_begin, op_end = gs->op_end;
-  if (threadIdx.x == 0) s_any = 0;
+  // A tree found inconsistent, or one the host has to grow for the bulk rounds first, is left alone (one thread
+  // reads the status: the tree's other CTAs may be setting it).
+  __shared__ int s_skip;
+  if (threadIdx.x == 0) {
+    s_any = 0;
+    s_skip = *(volatile int32_t*)&gs->status & (DELTA_CORRUPT | DELTA_NEED_BULK);
+  }
   if (threadIdx.x < kDeltaBuckets) s_stop[threadIdx.x] = 0;
   __syncthreads();
   for (int64_t i = op_begin + threadIdx.x; i < op_end; i += blockDim.x)
@@ -936,7 +942,7 @@ __global__ void __launch_bounds__(kDeltaWarps * 32, 2)
       break;
     }
   __syncthreads();
-  if (!s_any || gs->status & DELTA_CORRUPT) return;
+  if (!s_any || s_skip) return;
   Tree t;
   t.node = gs->node;
   t.child = gs->child;

@@ -81,7 +81,8 @@ struct TreeState {
   int64_t stale_child, stale_label, dead_nodes;  // unreachable arena space
 };
 
-enum { DELTA_OK = 0, DELTA_NEED_SPACE = 1, DELTA_CORRUPT = 2 };
+// DELTA_NEED_BULK: the room asked for (need_*) is what a bulk round takes in all, not the largest op.
+enum { DELTA_OK = 0, DELTA_NEED_SPACE = 1, DELTA_CORRUPT = 2, DELTA_NEED_BULK = 4 };
 
 // Delta kernel: ops are bucketed by a hash of their first token (kDeltaBuckets per tree); one CTA of
 // kDeltaWarps warps per tree takes the buckets heaviest first.
@@ -209,11 +210,6 @@ static_assert(kDeltaBuckets <= 32, "a part index fits in 5 bits and nparts in 6"
 // Bulk rounds ahead of the delta kernel (delta_bulk.cu): every op is walked by a lane of a grid-wide launch, and
 // the ops that nothing else in the delta gets in the way of are applied at once.  Sets done[i] for each; the rest
 // is left for launch_delta.  Ops of at most two pool runs, fewer than 2^31 ops.
-struct BulkKey {  // one place of a round: a token of a node's table
-  unsigned long long key;  // 0: empty entry
-  uint32_t first;          // ~(smallest op index that names it)
-  uint32_t pad_;
-};
 struct __align__(32) BulkNode {  // one node of a round
   unsigned long long key;        // 0: empty entry
   uint32_t shared;               // ops that depend on it and can do so side by side
@@ -224,7 +220,7 @@ struct __align__(32) BulkNode {  // one node of a round
   uint32_t pad_;
 };
 struct BulkTables {
-  BulkKey* keys;  // key_mask + 1
+  unsigned long long* keys;  // [key_mask + 1]: the places of a round, 0: empty entry
   BulkNode* nodes;
   uint32_t key_mask, node_mask;
 };
@@ -244,9 +240,11 @@ struct BulkArgs {
   BulkTables tab;  // from here on: scratch (bulk_scratch)
   BulkOp* ops;     // [n]
   int32_t* lists;  // [2n]: the op indices of odd and even rounds
+  int4* grow;      // [n]: (tree, node, node entry) of the tables that may have to grow in a round
+  int32_t* base;   // [3 * n_trees]: the arenas' use ahead of the round's ops
   unsigned long long* want;  // [kBulkRounds * n_trees * 3]: nodes, slots and tokens a round may take, at most
-  size_t n_want;             // words from want on, counts included
-  int32_t* counts;           // [kBulkRounds + 2]: list sizes by round
+  int32_t* counts;           // [2 * kBulkRounds + 1]: list sizes by round, then the sizes of its grow lists
+  size_t n_zero;             // bytes from tab.keys on that the launch clears
 };
 constexpr int kBulkRounds = 3;
 // The bytes of scratch for n ops of n_trees trees; with base, also sets A's scratch pointers into it.

@@ -1223,7 +1223,7 @@ int p2p_tree_apply_delta(p2p_router* r, int32_t peer, const p2p_delta* d, int64_
 // routed mostly to one tree and inserted with p2p_update_estimates, for one).  n_blocks = nt and
 // d_parts = NULL when no tree is split.
 constexpr int64_t kPartOps = 16384;
-// Largest delta of the bulk rounds (their scratch takes up to 320 bytes per op), and how much smaller the delta
+// Largest delta of the bulk rounds (their scratch takes up to 200 bytes per op), and how much smaller the delta
 // kernel's slabs are behind them.
 constexpr int64_t kBulkMaxOps = (int64_t)1 << 24;
 constexpr int32_t kBulkSlabShift = 3;
@@ -1365,6 +1365,7 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
   // ops, as a rule) goes to the delta kernel, whose warps then take smaller slabs.
   p2p::BulkArgs bulk = {};
   bool use_bulk = max_runs <= 2 && n <= kBulkMaxOps;
+  int32_t bulk_grown = 0;
   if (use_bulk) {
     if (ensure(r, r->bulk, p2p::bulk_scratch(n, nt, nullptr, bulk)) != cudaSuccess) {
       (void)cudaGetLastError();
@@ -1408,7 +1409,8 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
     r->launches += 1;
     if (int e = pull_states(r, p0, p1)) return e;
     bool again = false, stopped = false;
-    for (int32_t p = p0; p < p1; ++p) stopped = stopped || (r->hs[(size_t)p].status & p2p::DELTA_NEED_SPACE);
+    for (int32_t p = p0; p < p1; ++p)
+      stopped = stopped || (r->hs[(size_t)p].status & (p2p::DELTA_NEED_SPACE | p2p::DELTA_NEED_BULK)) == p2p::DELTA_NEED_SPACE;
     // The first stop for room: the room every op not yet applied may take, per tree (room_kernel), so that a
     // tree is grown once for the rest of the call (a delta that brings many new sequences to one tree would
     // otherwise stop at every doubling).  The bound counts INSERTs only; a later stop (a DELETE's fold needs
@@ -1427,6 +1429,19 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
       TreeState& t = r->hs[(size_t)p];
       if (t.status & p2p::DELTA_CORRUPT) {
         rc = fail(r, P2P_E_DEVICE, "tree " + std::to_string(p) + " is inconsistent");
+      } else if (t.status & p2p::DELTA_NEED_BULK) {
+        // What a bulk round asks for in all: grown to hold it.  It is a bound; should the arenas not reach it, or ask
+        // again and again, the delta kernel goes on alone and asks for what its ops need.
+        const auto most = [](int32_t need, int32_t used) { return std::min(need, INT32_MAX / 2 - used / 2); };
+        t.need_node = most(t.need_node, t.n_node);
+        t.need_child = most(t.need_child, t.n_child);
+        t.need_label = most(t.need_label, t.n_label);
+        if (++bulk_grown > 8 * nt || grow_tree(r, p, true) != P2P_OK) {
+          use_bulk = false;
+          t.status = p2p::DELTA_OK;
+          t.need_node = t.need_child = t.need_label = t.need_root = 0;
+        }
+        again = true;
       } else if (t.status & p2p::DELTA_NEED_SPACE) {
         bool whole = false;
         if (!room.empty()) {
