@@ -70,7 +70,7 @@ KERNEL_SOURCE = {
     "group_place_kernel": "group_kernel.cu", "lru_walk_kernel": "lru_kernel.cu", "lru_stamp_kernel": "lru_kernel.cu",
     "lru_evict_kernel": "lru_kernel.cu", "bulk_resolve_kernel": "delta_bulk.cu", "bulk_grow_kernel": "delta_bulk.cu",
     "lru_ops_kernel": "lru_kernel.cu", "hit_rate_kernel": "lru_kernel.cu", "room_kernel": "delta_kernel.cu",
-    "bulk_apply_kernel": "delta_bulk.cu",
+    "bulk_apply_kernel": "delta_bulk.cu", "follow_kernel": "route_kernel.cu",
 }
 # DRAM bytes per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum) per workload and kernel, with the
 # source hash of the capture and the profile summary that holds the command.  A figure whose source hash
@@ -504,7 +504,7 @@ def run_ours(args):
         compulsory = 4 * int(n_tok) + 8 * (B + 1) + 4 * B * P + 4 * B
         route = {"kernels": [k for k in ("group_hash_kernel", "group_resolve_kernel", "group_ranges_kernel",
                                          "group_place_kernel", "route_kernel", "lane_kernel<true>",
-                                         "lane_kernel<false>") if k in kt],
+                                         "follow_kernel", "lane_kernel<false>") if k in kt],
                  "ms": route_avg_ms, "compulsory_bytes": compulsory}
         # Device time of the route kernels (with p2p_route_prepare the grouping runs alongside the delta kernel,
         # outside the route span), the time the route's bytes are measured against.

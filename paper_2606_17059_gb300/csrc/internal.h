@@ -109,7 +109,8 @@ enum KernelId {
   K_GROUP_HASH, K_GROUP_RESOLVE, K_ROUTE_STAGED, K_LANE_LEADER, K_LANE_FOLLOWER, K_DECIDE,
   K_VALIDATE, K_INIT_RANGES, K_DELTA, K_COMPACT, K_COMPACT_LABELS, K_REFRESH_VIEWS, K_SET_TREE,
   K_UPDATE_COUNT, K_UPDATE_SCAN, K_UPDATE_SCATTER, K_GROUP_RANGES, K_GROUP_PLACE, K_LRU_WALK, K_LRU_STAMP,
-  K_LRU_EVICT, K_LRU_OPS, K_HIT_RATE, K_ROOM, K_BULK_RESOLVE, K_BULK_GROW, K_BULK_APPLY, K_COUNT_
+  K_LRU_EVICT, K_LRU_OPS, K_HIT_RATE, K_ROOM, K_BULK_RESOLVE, K_BULK_GROW, K_BULK_APPLY, K_FOLLOW,
+  K_COUNT_
 };
 static_assert((int)K_COUNT_ == (int)P2P_KERNEL_COUNT, "the header's kernel count");
 const char* kernel_name(int id);
@@ -143,7 +144,7 @@ struct GroupScratch {
   unsigned long long* keys;  // 2^bits slots
   int32_t* fcnt;     // [B]: a leader's follower count, then the start of its followers' range
   int32_t* counts;   // [8]: leaders, followers, groups with a checkpoint row, the leader pass's work cursor,
-                     //      the follower ranges handed out
+                     //      the follower ranges handed out, (unused), the followers left to the lane kernel
   size_t n_zero;
   // Set to 0x7f bytes (larger than any index or prefix), in one piece from vals on (n_large bytes):
   int32_t* vals;     // 2^bits slots
@@ -151,7 +152,7 @@ struct GroupScratch {
   int32_t* cmin;     // [B]: a leader's smallest common prefix with its followers
   size_t n_large;
   int32_t bits;
-  int32_t* slot_of;  // [B]
+  int32_t* slot_of;  // [B]: the key's slot, then the rank in the group, then the followers left to the lane kernel
   int32_t* lead;     // [B]
   int32_t* cpre;     // [B]
   int32_t* lists;    // [2B]

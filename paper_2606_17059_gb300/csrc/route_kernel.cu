@@ -6,7 +6,8 @@
 //
 // Passes.  A grouped batch (group_kernel.cu) is routed by a leader pass and a follower pass; a small batch is not
 // grouped and all of it is routed by the leader pass (route_ungrouped).  Leaders of
-// short requests, and all followers, are walked by lane_kernel (a lane per tree; below).  Leaders whose
+// short requests, and the followers of long ones, are walked by lane_kernel (a lane per tree; below), the followers of
+// short requests by follow_kernel (a lane per follower).  Leaders whose
 // requests are longer than a staging window on average go to route_kernel:
 //
 // route_kernel schedule.  A CTA takes requests b = list[blockIdx.x], list[blockIdx.x + gridDim.x], ...; its
@@ -835,6 +836,191 @@ __global__ void __launch_bounds__(kFollowThreads, kFollowCtasPerSm) lane_kernel(
   }
 }
 
+// The followers of short requests: a lane per follower, all lanes of a warp in one tree at a time.
+//
+// In each tree a follower whose leader matched less than their common prefix has the leader's match; the others resume
+// at the leader's checkpoint with one lookup of the follower's token there, mostly in vain.  What bounds this over
+// many trees:
+//   - Address translation.  An SM keeps few translations at hand (random loads of this GPU: 273 G/s over 16 regions 32 MB
+//     apart, 37 G/s over 32 or more, whether they hit L2 or not), and a load whose 32 lanes lie in 32 trees needs 32 of
+//     them: with a lane per tree the lookups of 205,000 followers in 26 million tables took 0.7 ms whatever the
+//     tables' size.  The lanes here are followers, side by side for a leader, and look into one tree, mostly one table.
+//   - Loads in flight.  A lookup that its first load does not answer, and the walk behind a token that is there, take
+//     several round trips, and in almost every step some lane of the warp has one.  They are queued, and full warps of
+//     them are looked up and walked.
+// A follower that would compare more than kSpan tokens of an edge in some tree is left to lane_kernel (`late`), whose
+// lanes share such compares over the trees.  A lane keeps its follower's decision in registers.
+//
+// Measured against lane_kernel<false>: 205,000 followers on 256 trees 1.04 -> 0.70 ms, 160,000 on 64 trees 207 -> 148 us,
+// 52,000 on 16 trees 39 -> 31.  Two trees a lane and three CTAs a SM: one or four trees 824 and 785 us, two, four and
+// five CTAs 865, 721 and 817 (more loads in flight are more translations).
+constexpr int kRowWarps = 8;
+constexpr int kRowCtasPerSm = 3;
+constexpr int kRowIlp = 2;   // trees a lane looks up at a time
+constexpr int kTile = 16;    // trees whose matches are put together
+constexpr int kSpan = 80;    // tokens of an edge that a lane compares
+constexpr int kQueue = 32 + 32 * kRowIlp;
+struct RowWarp {
+  int4 todo[kQueue];         // lookups to finish: (table offset, table bits, position, follower | tree << 8)
+  int32_t m[32][kTile + 1];  // the tile's matches: [follower][tree]
+};
+template <bool kDecide>
+__global__ void __launch_bounds__(kRowWarps * 32, kRowCtasPerSm) follow_kernel(
+    const TreeView* __restrict__ trees, int32_t P, const int32_t* __restrict__ tokens, int64_t tok_base,
+    const int64_t* __restrict__ offsets, const int32_t* __restrict__ list, const int32_t* __restrict__ count,
+    const int32_t* __restrict__ lead, const int32_t* __restrict__ cpre, const int32_t* __restrict__ gid,
+    const int4* __restrict__ ckpt, const int32_t* __restrict__ load, int32_t alpha, int32_t* __restrict__ out_match,
+    int32_t* __restrict__ out_peer, int32_t* err, int32_t* __restrict__ out_next, int32_t* __restrict__ late,
+    int32_t* n_late) {
+  extern __shared__ __align__(16) unsigned char s_row_bytes[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  RowWarp& S = reinterpret_cast<RowWarp*>(s_row_bytes)[warp];
+  const int64_t n = *count;
+  const bool wide = P % 4 == 0 && (reinterpret_cast<uintptr_t>(out_match) & 15) == 0;
+  // Rounds of all CTAs, and the warps that take 32 followers in each: as even as the count allows.
+  const int64_t full = (int64_t)gridDim.x * kRowWarps * 32, rounds = (n + full - 1) / full;
+  const int64_t per_round = (int64_t)gridDim.x * 32 * max(rounds, (int64_t)1);
+  const int busy = (int)((n + per_round - 1) / per_round);  // warps of a CTA, <= kRowWarps
+  for (int64_t r = 0; r < rounds; ++r) {
+    const int64_t i = ((r * gridDim.x + blockIdx.x) * busy + warp) * 32 + lane;
+    const bool on = warp < busy && i < n;
+    int32_t f = 0, l = 0, c = 0, len = 0, row = -1;
+    const int32_t* req = tokens;
+    if (on) {  // (followers are always valid requests)
+      f = __ldg(list + i);
+      l = __ldg(lead + f);
+      c = __ldg(cpre + f);
+      const int64_t start = __ldg(offsets + f) - tok_base;
+      len = (int32_t)min(__ldg(offsets + f + 1) - tok_base - start, (int64_t)INT32_MAX);
+      req = tokens + start;
+      row = group_row(__ldg(gid + l));
+    }
+    const int32_t* lrow = out_match + (int64_t)l * P;  // (the leader pass has finished)
+    const int4* ckrow = ckpt + (int64_t)max(row, 0) * P;
+    RouteAcc<kDecide> acc;
+    unsigned slow = 0;               // the followers left to lane_kernel (a bit per lane)
+    int32_t tk_at = -1, tk_val = 0;  // the request token looked up last: most trees resume at one position
+    const bool any = __any_sync(kFull, on);
+    for (int32_t p0 = 0; p0 < P; p0 += kTile) {
+      if (any) {
+        int todo = 0;
+#pragma unroll 1
+        for (int h = 0; h < kTile; h += kRowIlp) {
+          int32_t ml[kRowIlp], tk[kRowIlp];
+          int4 st[kRowIlp], e0[kRowIlp], e1[kRowIlp];
+          bool act[kRowIlp];
+#pragma unroll
+          for (int g = 0; g < kRowIlp; ++g) {
+            const int32_t p = p0 + h + g;
+            ml[g] = on && p < P ? lrow[p] : -1;
+            st[g] = on && p < P && row >= 0 ? __ldg(ckrow + p) : make_int4(0, 0, 0, 0);
+          }
+#pragma unroll
+          for (int g = 0; g < kRowIlp; ++g) {
+            const int32_t p = p0 + h + g;
+            const bool w = on && p < P && ml[g] >= c && c < len;
+            if (w && row < 0) st[g] = root_checkpoint(trees[p]);
+            const int32_t pos = w ? min(st[g].x, len) : ml[g] < c ? ml[g] : len;  // the match so far
+            act[g] = w && !((slow >> lane) & 1) && pos < len && st[g].w > 0 && tab_bits(st[g].z) > 0;
+            st[g].x = pos;
+            if (act[g] && pos != tk_at) {
+              tk_at = pos;
+              tk_val = __ldg(req + pos);
+            }
+            tk[g] = tk_val;
+          }
+#pragma unroll
+          for (int g = 0; g < kRowIlp; ++g) {
+            e0[g] = e1[g] = make_int4(0, 0, 0, 0);
+            if (act[g]) {
+              const int32_t bits = tab_bits(st[g].z);
+              load_slots(trees[p0 + h + g].child + st[g].y + slot_hash(tk[g], bits), e0[g], e1[g]);
+            }
+          }
+#pragma unroll
+          for (int g = 0; g < kRowIlp; ++g) {
+            S.m[lane][h + g] = st[g].x;
+            int4 e;
+            if (act[g]) act[g] = probe_first2(e0[g], e1[g], tk[g], e) != 0;
+            const unsigned hm = __ballot_sync(kFull, act[g]);
+            if (act[g])
+              S.todo[todo + __popc(hm & ((1u << lane) - 1))] =
+                  make_int4(st[g].y, tab_bits(st[g].z), st[g].x, lane | (h + g) << 8);
+            todo += __popc(hm);
+          }
+          while (todo >= 32 || (todo > 0 && h + kRowIlp >= kTile)) {
+            __syncwarp();
+            const int first = max(todo - 32, 0);
+            const bool go = first + lane < todo;
+            const int4 q = go ? S.todo[first + lane] : make_int4(0, 0, 0, 0);
+            const int wi = q.w & 31, t = q.w >> 8;
+            todo = first;
+            const int32_t wl = __shfl_sync(kFull, len, wi), wc = __shfl_sync(kFull, c, wi);
+            const int32_t* wr = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)req, wi);
+            const TreeView& tv = trees[p0 + t];
+            int4 ce = make_int4(0, 0, 0, 0);
+            int32_t pos = q.z;
+            bool walk = go && find_child_1(tv.child + q.x, q.y, __ldg(wr + pos), ce), long_edge = false;
+            const bool found = walk;
+            while (walk) {  // edge by edge
+              if (ce.w <= 0 || ce.y <= 0) {  // cannot happen in a valid tree
+                atomicOr(err, ERR_CORRUPT_TREE);
+                break;
+              }
+              const int4 nn = __ldg(tv.node + ce.y);
+              const int32_t lim = min(ce.w, wl - pos), from = max(1, wc - pos), stop = min(lim, from + kSpan);
+              int32_t k = lim;
+              if (from < lim) {
+                k = first_diff_1(label_ptr(tv.label, tv.shared, ce.z), wr + pos, from, stop);
+                if (k == stop && stop < lim) {
+                  long_edge = true;
+                  break;
+                }
+              }
+              pos += k;
+              walk = k == ce.w && pos < wl && nn.z > 0 &&
+                     find_child_1(tv.child + nn.x, tab_bits(nn.y), __ldg(wr + pos), ce);
+            }
+            if (found) S.m[wi][t] = pos;
+            slow |= __reduce_or_sync(kFull, long_edge ? 1u << wi : 0u);
+          }
+        }
+        __syncwarp();
+        if (on) {  // the follower's part of its row, and of the decision
+          int32_t* out = out_match + (int64_t)f * P + p0;
+#pragma unroll
+          for (int h = 0; h < kTile; h += 4) {
+            const int4 v = make_int4(S.m[lane][h], S.m[lane][h + 1], S.m[lane][h + 2], S.m[lane][h + 3]);
+            const int32_t p = p0 + h;
+            if (wide && p < P) {
+              *reinterpret_cast<int4*>(out + h) = v;
+            } else {
+              if (p < P) out[h] = v.x;
+              if (p + 1 < P) out[h + 1] = v.y;
+              if (p + 2 < P) out[h + 2] = v.z;
+              if (p + 3 < P) out[h + 3] = v.w;
+            }
+            if (p < P) acc.add(v.x, __ldg(load + p), p, alpha);
+            if (p + 1 < P) acc.add(v.y, __ldg(load + p + 1), p + 1, alpha);
+            if (p + 2 < P) acc.add(v.z, __ldg(load + p + 2), p + 2, alpha);
+            if (p + 3 < P) acc.add(v.w, __ldg(load + p + 3), p + 3, alpha);
+          }
+        }
+        __syncwarp();
+      }
+    }
+    const bool is_late = on && ((slow >> lane) & 1);
+    if (on && !is_late) acc.write(f, out_peer, out_next);
+    const unsigned lm = __ballot_sync(kFull, is_late);
+    if (lm) {
+      int32_t at = 0;
+      if (lane == 0) at = atomicAdd(n_late, __popc(lm));
+      at = __shfl_sync(kFull, at, 0);
+      if (is_late) late[at + __popc(lm & ((1u << lane) - 1))] = f;
+    }
+  }
+}
+
 // Route decision from a match matrix with excluded peers: the best and the next-best candidate by the route
 // order of route_key, skipping trees whose staged load word carries kExcluded (Section 3.2: a peer that
 // pushes back; Section 3.3: a suspected-failed peer, and the next-best target a request falls back to when
@@ -999,12 +1185,26 @@ cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tok
   }
   e = cudaGetLastError();
   if (e != cudaSuccess || !g) return e;
-  // The followers' first per-lane compare: 8 tokens for long requests, 16 otherwise (lane_walks).
+  // The followers' first per-lane compare in lane_kernel: 8 tokens for long requests, 16 otherwise (lane_walks).  A
+  // single tree's followers stay with it: there is no tree to go on to.
   if (long_requests(B, n_tokens)) {
     P2P_TIMED(K_LANE_FOLLOWER, st,
               (lane_kernel<false, kDecide, 8><<<grid2, kFollowThreads, 0, st>>>(
                   d_trees, P, tokens, n_tokens, tok_base, offsets, B, g->lists + B, g->counts + 1, g->lead, g->cpre,
                   g->gid, nullptr, g->ckpt, d_load, alpha, out_match, out_peer, d_err, nullptr, out_next)));
+  } else if (P > 1) {
+    const size_t smem = sizeof(RowWarp) * kRowWarps;
+    e = cudaFuncSetAttribute(follow_kernel<kDecide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    P2P_TIMED(K_FOLLOW, st,
+              (follow_kernel<kDecide><<<(int)std::min<int64_t>((B + 31) / 32, num_sms * kRowCtasPerSm), kRowWarps * 32, smem, st>>>(
+                  d_trees, P, tokens, tok_base, offsets, g->lists + B, g->counts + 1, g->lead, g->cpre, g->gid, g->ckpt,
+                  d_load, alpha, out_match, out_peer, d_err, out_next, g->slot_of, g->counts + 6)));
+    P2P_TIMED(K_LANE_FOLLOWER, st,
+              (lane_kernel<false, kDecide, 16><<<grid2, kFollowThreads, 0, st>>>(
+                  d_trees, P, tokens, n_tokens, tok_base, offsets, B, g->slot_of, g->counts + 6, g->lead, g->cpre,
+                  g->gid, nullptr, g->ckpt, d_load, alpha, out_match, out_peer, d_err, nullptr, out_next)));
+    *launched += 1;
   } else {
     P2P_TIMED(K_LANE_FOLLOWER, st,
               (lane_kernel<false, kDecide, 16><<<grid2, kFollowThreads, 0, st>>>(

@@ -93,7 +93,7 @@ const char* kernel_name(int id) {
       "compact_kernel", "compact_labels_kernel", "refresh_views_kernel", "set_tree_kernel", "update_count_kernel",
       "update_scan_kernel", "update_scatter_kernel", "group_ranges_kernel", "group_place_kernel", "lru_walk_kernel",
       "lru_stamp_kernel", "lru_evict_kernel", "lru_ops_kernel", "hit_rate_kernel", "room_kernel", "bulk_resolve_kernel",
-      "bulk_grow_kernel", "bulk_apply_kernel"};
+      "bulk_grow_kernel", "bulk_apply_kernel", "follow_kernel"};
   return id >= 0 && id < K_COUNT_ ? names[id] : "";
 }
 
