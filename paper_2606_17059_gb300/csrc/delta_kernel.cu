@@ -1250,8 +1250,9 @@ struct CompactShared {
 // Copies the table of node cid (old record rec) into a fresh table of the same size, one thread.  The
 // slots are loaded kSlotBatch at a time; each batch takes its new ids and label space with one reservation,
 // and the thread places its entries by linear probing on a bit mask of the slots it has filled, so the new
-// table is written once, with no read-back.  Labels are not copied here: each child's scratch entry
-// records where its label moves, and compact_labels_kernel moves them all afterwards.
+// table is written once, with no read-back.  A big table (a level with more units than the warps' list holds)
+// does not fit the mask: it is zeroed first and probed in memory.  Labels are not copied here: each child's
+// scratch entry records where its label moves, and compact_labels_kernel moves them all afterwards.
 __device__ void compact_node_thread(CompactJob& J, CompactShared& S, int32_t cid, const int4& rec) {
   const int32_t bits = tab_bits(rec.y);
   int32_t noff = 0, live = 0;
@@ -1263,6 +1264,9 @@ __device__ void compact_node_thread(CompactJob& J, CompactShared& S, int32_t cid
       atomicOr(&S.fail, 1);
       return;
     }
+    const bool big = bits > kSmallBits;
+    if (big)
+      for (int32_t j = 0; j < size; ++j) J.nchild[noff + j] = make_int4(0, 0, 0, 0);
     uint32_t used = 0;
     for (int32_t j0 = 0; j0 < size; j0 += kSlotBatch) {
       int4 e[kSlotBatch];
@@ -1290,15 +1294,19 @@ __device__ void compact_node_thread(CompactJob& J, CompactShared& S, int32_t cid
         const int32_t z = own ? nz : e[u].z;
         J.queue[c] = make_int4(e[u].y, e[u].z, z, own ? e[u].w : 0);
         uint32_t sl = slot_hash(e[u].x, bits);
-        while ((used >> sl) & 1u) sl = (sl + 1) & mask;
-        used |= 1u << sl;
+        if (big) {
+          while (J.nchild[noff + sl].y) sl = (sl + 1) & mask;
+        } else {
+          while ((used >> sl) & 1u) sl = (sl + 1) & mask;
+          used |= 1u << sl;
+        }
         J.nchild[noff + sl] = make_int4(e[u].x, c, z, e[u].w);
         ++c;
         nz += own ? e[u].w : 0;
         ++live;
       }
     }
-    for (int32_t j = 0; j < size; ++j)
+    for (int32_t j = 0; !big && j < size; ++j)
       if (!((used >> j) & 1u)) J.nchild[noff + j] = make_int4(0, 0, 0, 0);
   }
   J.nnode[cid] = make_int4(noff, make_meta(bits, live), rec.z, rec.w);
