@@ -64,7 +64,7 @@ KERNEL_SOURCE = {
     "lane_kernel<true>": "route_kernel.cu", "lane_kernel<false>": "route_kernel.cu", "decide_kernel": "route_kernel.cu",
     "validate_kernel": "delta_kernel.cu", "init_ranges_kernel": "delta_kernel.cu", "delta_kernel": "delta_kernel.cu",
     "compact_kernel": "delta_kernel.cu", "compact_labels_kernel": "delta_kernel.cu",
-    "refresh_views_kernel": "delta_kernel.cu", "set_tree_kernel": "delta_kernel.cu",
+    "refresh_views_kernel": "delta_kernel.cu", "set_tree_kernel": "delta_kernel.cu", "upload_kernel": "delta_kernel.cu",
     "update_count_kernel": "update_kernel.cu", "update_scan_kernel": "update_kernel.cu",
     "update_scatter_kernel": "update_kernel.cu", "group_ranges_kernel": "group_kernel.cu",
     "group_place_kernel": "group_kernel.cu", "lru_walk_kernel": "lru_kernel.cu", "lru_stamp_kernel": "lru_kernel.cu",

@@ -1513,6 +1513,45 @@ __global__ void __launch_bounds__(kLabelThreads) compact_labels_kernel(const Com
   }
 }
 
+// The tables and own labels of an uploaded tree.  Eight lanes take an edge: the first puts it into its table (claimed by
+// its node id, with compare-and-swap: others fill the table too), all move its label, kUploadSteps tokens a lane at a
+// time.  Latency of a few round
+// trips; the snapshot's labels stay in L2: 13 us for 20,900 edges and 6.3 MB of own labels.  The host filled the tables
+// and packed the labels before: the upload of that tree 1.96 -> 0.76 ms (with it, a hash of labels in four chains
+// instead of one and a validity check without a search).
+constexpr int kUploadThreads = 256, kUploadLanes = 8, kUploadSteps = 8;
+__global__ void __launch_bounds__(kUploadThreads) upload_kernel(const UploadEdge* __restrict__ edge, int64_t n, int4* child,
+                                                                const int32_t* __restrict__ src, int32_t* dst) {
+  const int sub = threadIdx.x % kUploadLanes;
+  const int64_t step = (int64_t)gridDim.x * (kUploadThreads / kUploadLanes);
+  for (int64_t i = ((int64_t)blockIdx.x * kUploadThreads + threadIdx.x) / kUploadLanes; i < n; i += step) {
+    const int4 e = __ldg(&edge[i].slot), tab = __ldg(&edge[i].tab);
+    if (sub == 0) {
+      const uint32_t mask = (1u << tab.y) - 1;
+      uint32_t s = slot_hash(e.x, tab.y);
+      int4* slot = child + tab.x;
+      for (uint32_t k = 0; k <= mask; ++k, s = (s + 1) & mask)  // (a table has room for its edges)
+        if (atomicCAS(&slot[s].y, 0, e.y) == 0) {
+          slot[s].x = e.x;
+          slot[s].z = e.z;
+          slot[s].w = e.w;
+          break;
+        }
+    }
+    if (!src || e.z < 0) continue;
+    const int32_t *from = src + tab.z;
+    int32_t* to = dst + e.z;
+    for (int32_t b = sub; b < e.w; b += kUploadLanes * kUploadSteps) {
+      int32_t x[kUploadSteps];
+#pragma unroll
+      for (int u = 0; u < kUploadSteps; ++u) x[u] = b + u * kUploadLanes < e.w ? __ldg(from + b + u * kUploadLanes) : 0;
+#pragma unroll
+      for (int u = 0; u < kUploadSteps; ++u)
+        if (b + u * kUploadLanes < e.w) to[b + u * kUploadLanes] = x[u];
+    }
+  }
+}
+
 __global__ void set_tree_kernel(TreeState* st, TreeView* view, TreeState v, const int32_t* shared) {
   *st = v;
   const int4 root = v.node[0];
@@ -1615,6 +1654,13 @@ cudaError_t launch_room(const TreeState* d_states, int32_t nt, const uint8_t* do
 
 cudaError_t launch_init_ranges(TreeState* d_states, int32_t nt, const int64_t* peer_begin, int64_t n, cudaStream_t st) {
   P2P_TIMED(K_INIT_RANGES, st, (init_ranges_kernel<<<(nt + 127) / 128, 128, 0, st>>>(d_states, nt, peer_begin, n)));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_upload(const UploadEdge* edge, int64_t n, int4* child, const int32_t* src, int32_t* dst, int num_sms,
+                          cudaStream_t st) {
+  const int64_t per = kUploadThreads / kUploadLanes, ctas = std::min<int64_t>((n + per - 1) / per, (int64_t)num_sms * 8);
+  P2P_TIMED(K_UPLOAD, st, (upload_kernel<<<(int)ctas, kUploadThreads, 0, st>>>(edge, n, child, src, dst)));
   return cudaGetLastError();
 }
 

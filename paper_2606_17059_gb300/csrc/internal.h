@@ -110,7 +110,7 @@ enum KernelId {
   K_VALIDATE, K_INIT_RANGES, K_DELTA, K_COMPACT, K_COMPACT_LABELS, K_REFRESH_VIEWS, K_SET_TREE,
   K_UPDATE_COUNT, K_UPDATE_SCAN, K_UPDATE_SCATTER, K_GROUP_RANGES, K_GROUP_PLACE, K_LRU_WALK, K_LRU_STAMP,
   K_LRU_EVICT, K_LRU_OPS, K_HIT_RATE, K_ROOM, K_BULK_RESOLVE, K_BULK_GROW, K_BULK_APPLY, K_FOLLOW,
-  K_COUNT_
+  K_UPLOAD, K_COUNT_
 };
 static_assert((int)K_COUNT_ == (int)P2P_KERNEL_COUNT, "the header's kernel count");
 const char* kernel_name(int id);
@@ -291,6 +291,14 @@ __device__ __forceinline__ void load_slots(const int4* p, int4& a, int4& b) {
 
 // Writes a tree's state and view on the device (values passed as kernel parameters, so no host buffer
 // has to outlive the call).
+// An edge of a tree being uploaded.
+struct UploadEdge {
+  int4 slot;  // its slot: first token, node, label offset (< 0: in the shared pool), label length
+  int4 tab;   // the table it goes to: offset, bits; where an own label starts in the snapshot's labels; (unused)
+};
+// Puts n edges into their tables (zeroed) and moves the own labels from src (null: they are there already) to dst.
+cudaError_t launch_upload(const UploadEdge* edge, int64_t n, int4* child, const int32_t* src, int32_t* dst, int num_sms,
+                          cudaStream_t st);
 cudaError_t launch_set_tree(TreeState* d_state, TreeView* d_view, TreeState value, const int32_t* shared,
                             cudaStream_t st);
 

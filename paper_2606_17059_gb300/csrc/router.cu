@@ -55,14 +55,37 @@ constexpr int32_t kInternMin = 128;
 constexpr int32_t kHeadTokens = 64;
 constexpr size_t kHeadCandidates = 8;
 
-// 64-bit content hash of a token run (FNV-1a over the 32-bit tokens, then a final avalanche); interning
-// always verifies the content, so a collision only means a run is not shared.
+// 64-bit content hash of a token run: two tokens a step in four independent chains of multiplications (one chain waits
+// for the multiplier at every token), then a final avalanche.  Interning always verifies the content, so a collision
+// only means a run is not shared.
 uint64_t run_hash(const int32_t* p, int64_t n) {
-  uint64_t h = 0xcbf29ce484222325ull ^ (uint64_t)n;
-  for (int64_t i = 0; i < n; ++i) h = (h ^ (uint32_t)p[i]) * 0x100000001b3ull;
-  h ^= h >> 33;
-  h *= 0xff51afd7ed558ccdull;
-  return h ^ (h >> 33);
+  constexpr uint64_t kMul = 0x9e3779b97f4a7c15ull;
+  uint64_t h[4] = {0xcbf29ce484222325ull ^ (uint64_t)n, 1, 2, 3};
+  int64_t i = 0;
+  for (; i + 8 <= n; i += 8)
+    for (int j = 0; j < 4; ++j) {
+      uint64_t w;
+      std::memcpy(&w, p + i + 2 * j, sizeof(w));
+      h[j] = (h[j] ^ w) * kMul;
+      h[j] ^= h[j] >> 32;
+    }
+  for (; i < n; ++i) h[0] = (h[0] ^ (uint32_t)p[i]) * kMul;
+  uint64_t x = 0;
+  for (int j = 0; j < 4; ++j) {
+    x = (x ^ h[j]) * kMul;
+    x ^= x >> 32;
+  }
+  x *= 0xff51afd7ed558ccdull;
+  return x ^ (x >> 33);
+}
+
+// Length of the common prefix of two runs of n tokens.
+int32_t same_prefix(const int32_t* a, const int32_t* b, int32_t n) {
+  constexpr int32_t kBlock = 64;
+  int32_t i = 0;
+  while (i + kBlock <= n && std::memcmp(a + i, b + i, kBlock * sizeof(int32_t)) == 0) i += kBlock;
+  while (i < n && a[i] == b[i]) ++i;
+  return i;
 }
 
 // Children-table sizes (log2 slots): load factor <= 1/4 at upload (tables grow past 1/2); the root's table
@@ -93,7 +116,7 @@ const char* kernel_name(int id) {
       "compact_kernel", "compact_labels_kernel", "refresh_views_kernel", "set_tree_kernel", "update_count_kernel",
       "update_scan_kernel", "update_scatter_kernel", "group_ranges_kernel", "group_place_kernel", "lru_walk_kernel",
       "lru_stamp_kernel", "lru_evict_kernel", "lru_ops_kernel", "hit_rate_kernel", "room_kernel", "bulk_resolve_kernel",
-      "bulk_grow_kernel", "bulk_apply_kernel", "follow_kernel"};
+      "bulk_grow_kernel", "bulk_apply_kernel", "follow_kernel", "upload_kernel"};
   return id >= 0 && id < K_COUNT_ ? names[id] : "";
 }
 
@@ -534,12 +557,11 @@ int32_t longest_head(const p2p_router* r, const int32_t* src, int32_t len, int32
   auto it = r->heads.find(run_hash(src, kHeadTokens));
   if (it == r->heads.end()) return 0;
   for (const auto& [at, rl] : it->second) {
-    const int32_t m = std::min(len, rl);
-    const int32_t* a = r->h_shared.data() + at;
-    const int32_t lcp = (int32_t)(std::mismatch(a, a + m, src).first - a);
+    const int32_t lcp = same_prefix(r->h_shared.data() + at, src, std::min(len, rl));
     if (lcp > k) {
       k = lcp;
       best = at;
+      if (k == len) break;
     }
   }
   return best;
@@ -556,84 +578,82 @@ int upload_flat(p2p_router* r, int32_t peer, const p2p_flat_tree* t) {
   // no sequence continues with the rest.  Every tree holding the prefix then points at one copy, so a walk
   // compares it once for all of them (and the export merges the node back).  A label that is a prefix of an
   // interned run points at that run.
+  //
+  // The host decides what is interned and lays the arrays out; upload_kernel fills the tables and moves the own labels.
+  // It is given an edge per node (edge[c - 1] leads to node c).
   const int64_t shared_before = (int64_t)r->h_shared.size();
-  std::vector<int32_t> enc((size_t)N, 0), head_len((size_t)N, 0), tail_enc((size_t)N, 0), own;
-  own.reserve((size_t)NL);
-  int64_t n_split = 0;
+  std::vector<p2p::UploadEdge> edge((size_t)(N - 1));
+  struct Split {
+    int32_t v, at, len, tab;  // node v's label starts with len tokens of the run at `at`; its table's offset
+  };
+  std::vector<Split> split;
+  int64_t n_own = 0;
   for (int64_t v = 1; v < N; ++v) {
     const int32_t* src = t->labels + t->label_off[v];
     const int32_t len = t->label_len[v];
+    int32_t head = 0, enc = 0;  // tokens that a node of their own continues
     bool interned = false;
     if (len >= kInternMin) {
       int32_t k = 0;
       const int32_t at = longest_head(r, src, len, k);
       if (k == len) {
-        enc[(size_t)v] = ~at;
+        enc = ~at;
         interned = true;
       } else if (k >= kInternMin) {
-        enc[(size_t)v] = ~at;
-        head_len[(size_t)v] = k;
-        ++n_split;
-        const int32_t rest = len - k;
-        bool ok = false;
-        if (rest >= kInternMin) tail_enc[(size_t)v] = intern_label(r, src + k, rest, ok);
-        if (!ok) {
-          tail_enc[(size_t)v] = (int32_t)own.size();
-          own.insert(own.end(), src + k, src + len);
-        }
-        interned = true;
+        head = k;
+        split.push_back({(int32_t)v, ~at, k, 0});
+        if (len - k >= kInternMin) enc = intern_label(r, src + k, len - k, interned);
       } else {
-        enc[(size_t)v] = intern_label(r, src, len, interned);
+        enc = intern_label(r, src, len, interned);
       }
     }
     if (!interned) {
-      enc[(size_t)v] = (int32_t)own.size();
-      own.insert(own.end(), src, src + len);
+      enc = (int32_t)n_own;
+      n_own += len - head;
+      if (n_own > INT32_MAX) return fail(r, P2P_E_NOMEM, "labels exceed the int32 arena");
     }
+    // (The first token and the parent's table follow below.)
+    edge[(size_t)(v - 1)] = {make_int4(head ? src[head] : 0, (int32_t)v, enc, len - head),
+                             make_int4(0, 0, t->label_off[v] + head, head ? (int32_t)split.size() : 0)};
   }
   if (int rc = sync_shared_pool(r, shared_before)) return rc;
   // Children tables, laid out in node order in the child arena; the split nodes (ids N ..) after them.
-  const int64_t NN = N + n_split;
+  const int64_t NN = N + (int64_t)split.size();
   if (NN > INT32_MAX / 2) return fail(r, P2P_E_NOMEM, "too many nodes");
-  std::vector<int32_t> bits((size_t)NN), off((size_t)NN, 0), split_id((size_t)N, 0);
+  std::vector<int4> node((size_t)NN);
+  edge.resize((size_t)(NN - 1));
   int64_t slots = 0;
+  const auto take = [&slots](int32_t bits) {
+    const int64_t at = slots;
+    slots += bits ? (int64_t)1 << bits : 0;
+    return (int32_t)at;
+  };
   for (int64_t v = 0; v < N; ++v) {
-    bits[(size_t)v] = table_bits_for(t->child_count[v], v == 0);
-    if (bits[(size_t)v] > p2p::kMaxTabBits) return fail(r, P2P_E_NOMEM, "a node has too many children");
-    off[(size_t)v] = (int32_t)slots;
-    slots += bits[(size_t)v] ? (int64_t)1 << bits[(size_t)v] : 0;
+    const int32_t cnt = t->child_count[v], b = table_bits_for(cnt, v == 0);
+    if (b > p2p::kMaxTabBits) return fail(r, P2P_E_NOMEM, "a node has too many children");
+    const int32_t off = take(b);
     if (slots > INT32_MAX / 2) return fail(r, P2P_E_NOMEM, "children tables exceed the int32 arena");
-  }
-  for (int64_t v = 1, x = N; v < N; ++v)
-    if (head_len[(size_t)v]) {
-      split_id[(size_t)v] = (int32_t)x;
-      bits[(size_t)x] = p2p::kMinTabBits;
-      off[(size_t)x] = (int32_t)slots;
-      slots += (int64_t)1 << p2p::kMinTabBits;
-      if (slots > INT32_MAX / 2) return fail(r, P2P_E_NOMEM, "children tables exceed the int32 arena");
-      ++x;
-    }
-  std::vector<int4> node((size_t)NN), child((size_t)slots, make_int4(0, 0, 0, 0));
-  for (int64_t v = 0; v < N; ++v) {
-    const int32_t cnt = t->child_count[v], b = bits[(size_t)v];
-    node[(size_t)v] = make_int4(b ? off[(size_t)v] : 0, p2p::make_meta(b, cnt), cnt, t->term_count[v]);
+    node[(size_t)v] = make_int4(b ? off : 0, p2p::make_meta(b, cnt), cnt, t->term_count[v]);
     for (int64_t e = t->child_begin[v]; e < (int64_t)t->child_begin[v] + cnt; ++e) {
-      const int32_t c = t->child_idx[e];
-      const int32_t k = head_len[(size_t)c];
-      if (!k) {
-        table_put(child.data() + off[(size_t)v], b, make_int4(t->child_first_tok[e], c, enc[(size_t)c], t->label_len[c]));
-        continue;
-      }
-      // v -> x (the shared head) -> c (the rest of the label).
-      const int32_t x = split_id[(size_t)c];
-      table_put(child.data() + off[(size_t)v], b, make_int4(t->child_first_tok[e], x, enc[(size_t)c], k));
-      node[(size_t)x] = make_int4(off[(size_t)x], p2p::make_meta(p2p::kMinTabBits, 1), 1, 0);
-      const int32_t* src = t->labels + t->label_off[c];
-      table_put(child.data() + off[(size_t)x], p2p::kMinTabBits,
-                make_int4(src[k], c, tail_enc[(size_t)c], t->label_len[c] - k));
+      p2p::UploadEdge& E = edge[(size_t)t->child_idx[e] - 1];
+      E.tab.x = off;
+      E.tab.y = b;
+      if (!E.tab.w)
+        E.slot.x = t->child_first_tok[e];
+      else  // v -> x (the shared head) -> c (the rest of the label): the head's edge
+        edge[(size_t)(N + E.tab.w - 2)] = {make_int4(t->child_first_tok[e], (int32_t)(N + E.tab.w - 1),
+                                                     split[(size_t)E.tab.w - 1].at, split[(size_t)E.tab.w - 1].len),
+                                           make_int4(off, b, 0, 0)};
     }
   }
-  const int64_t n_own = (int64_t)own.size();
+  for (size_t i = 0; i < split.size(); ++i) {
+    const int32_t off = take(p2p::kMinTabBits);
+    if (slots > INT32_MAX / 2) return fail(r, P2P_E_NOMEM, "children tables exceed the int32 arena");
+    node[(size_t)N + i] = make_int4(off, p2p::make_meta(p2p::kMinTabBits, 1), 1, 0);
+    int4& tab = edge[(size_t)split[i].v - 1].tab;
+    tab.x = off;
+    tab.y = p2p::kMinTabBits;
+  }
   // Headroom for device deltas (no regrowth for a few anti-entropy rounds of a few percent each).
   const int32_t cap_node = clamp_i32(2 * NN + 1024);
   const int32_t cap_child = clamp_i32(2 * slots + 1024);
@@ -656,8 +676,26 @@ int upload_flat(p2p_router* r, int32_t peer, const p2p_flat_tree* t) {
     }
   }
   CK(cudaMemcpyAsync(nt.node, node.data(), (size_t)NN * sizeof(int4), cudaMemcpyHostToDevice, r->stream));
-  if (slots) CK(cudaMemcpyAsync(nt.child, child.data(), (size_t)slots * sizeof(int4), cudaMemcpyHostToDevice, r->stream));
-  if (n_own) CK(cudaMemcpyAsync(nt.label, own.data(), (size_t)n_own * sizeof(int32_t), cudaMemcpyHostToDevice, r->stream));
+  if (slots) CK(cudaMemsetAsync(nt.child, 0, (size_t)slots * sizeof(int4), r->stream));
+  // The snapshot's labels go as they are to the spare's label arena, which is free until a compaction, and upload_kernel
+  // moves the own ones from there; without that room they are put together here.
+  const bool staged = n_own > 0 && sp.label && NL <= sp.cap_label;
+  std::vector<int32_t> own;
+  if (staged) {
+    CK(cudaMemcpyAsync(sp.label, t->labels, (size_t)NL * sizeof(int32_t), cudaMemcpyHostToDevice, r->stream));
+  } else if (n_own) {
+    own.resize((size_t)n_own);
+    for (const p2p::UploadEdge& E : edge)
+      if (E.slot.z >= 0) std::memcpy(own.data() + E.slot.z, t->labels + E.tab.z, (size_t)E.slot.w * sizeof(int32_t));
+    CK(cudaMemcpyAsync(nt.label, own.data(), (size_t)n_own * sizeof(int32_t), cudaMemcpyHostToDevice, r->stream));
+  }
+  if (NN > 1) {
+    // The edges wait behind the tables: at most a quarter of a table's slots are taken, and the arena has twice them.
+    p2p::UploadEdge* d_edge = reinterpret_cast<p2p::UploadEdge*>(nt.child + slots);
+    CK(cudaMemcpyAsync(d_edge, edge.data(), edge.size() * sizeof(p2p::UploadEdge), cudaMemcpyHostToDevice, r->stream));
+    CK(p2p::launch_upload(d_edge, NN - 1, nt.child, staged ? sp.label : nullptr, nt.label, r->num_sms, r->stream));
+    r->launches += 1;
+  }
   nt.n_node = (int32_t)NN;
   nt.n_child = (int32_t)slots;
   nt.n_label = (int32_t)n_own;
@@ -674,7 +712,11 @@ int upload_flat(p2p_router* r, int32_t peer, const p2p_flat_tree* t) {
   old = nt;
   CK(p2p::launch_set_tree(r->d_states + peer, r->d_views + peer, nt, r->d_shared, r->stream));
   r->launches += 1;
-  // The host vectors above are released on return; pageable copies have consumed them by now.
+  // The host vectors above are released on return; pageable copies have consumed them by now.  Labels in page-locked
+  // memory are still being read.
+  cudaPointerAttributes pa = {};
+  if (staged && cudaPointerGetAttributes(&pa, t->labels) == cudaSuccess && pa.type != cudaMemoryTypeUnregistered)
+    CK(cudaStreamSynchronize(r->stream));
   return P2P_OK;
 }
 

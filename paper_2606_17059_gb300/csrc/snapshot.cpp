@@ -216,44 +216,67 @@ bool validate_flat(const p2p_flat_tree* t, std::string& err) {
     return err = "NULL node array", false;
   if ((N > 1 && (!t->child_first_tok || !t->child_idx)) || (NL > 0 && !t->labels)) return err = "NULL array", false;
   if (t->label_len[0] != 0) return err = "root label must be empty", false;
-  std::vector<int64_t> parent((size_t)N, -1);
   for (int64_t v = 0; v < N; ++v) {
     const int64_t off = t->label_off[v], len = t->label_len[v];
     if (off < 0 || len < 0 || off > NL - len) return err = "label of node " + std::to_string(v) + " out of range", false;
     if (v > 0 && len < 1) return err = "non-root node " + std::to_string(v) + " has an empty label", false;
     if (t->term_count[v] < 0) return err = "negative term_count", false;
+  }
+  // Child lists.  Where every child comes after its parent (preorder, as the library builds trees), path lengths add up
+  // on the way and a node is reachable from the root if it has a parent: no search is needed.
+  constexpr int64_t kAhead = 8;  // labels are far apart: their first tokens are fetched this many nodes ahead
+  std::vector<int64_t> depth((size_t)N, -1);  // -1: no path from the root so far
+  std::vector<uint8_t> has_parent((size_t)N, 0);
+  depth[0] = 0;
+  bool ordered = true, too_long = false;
+  int64_t seen = 1;
+  for (int64_t v = 0; v < N; ++v) {
     const int64_t cb = t->child_begin[v], cc = t->child_count[v];
     if (cb < 0 || cc < 0 || cb > (N - 1) - cc) return err = "child range of node " + std::to_string(v) + " out of range", false;
     for (int64_t e = cb; e < cb + cc; ++e) {
       const int64_t c = t->child_idx[e];
       if (c < 1 || c >= N) return err = "child index out of range", false;
-      if (parent[(size_t)c] != -1) return err = "node " + std::to_string(c) + " has two parents", false;
-      parent[(size_t)c] = v;
+      if (has_parent[(size_t)c]) return err = "node " + std::to_string(c) + " has two parents", false;
+      has_parent[(size_t)c] = 1;
+      if (e + kAhead < N - 1) {
+        const int64_t a = t->child_idx[e + kAhead];
+        if (a >= 1 && a < N) __builtin_prefetch(t->labels + t->label_off[a]);
+      }
       if (t->child_first_tok[e] != t->labels[t->label_off[c]])
         return err = "child_first_tok differs from the child's first label token", false;
       if (e > cb && !(t->child_first_tok[e - 1] < t->child_first_tok[e]))
         return err = "children of node " + std::to_string(v) + " not strictly ascending", false;
+      ordered = ordered && c > v;
+      if (ordered && depth[(size_t)v] >= 0) {
+        depth[(size_t)c] = depth[(size_t)v] + t->label_len[c];
+        too_long = too_long || depth[(size_t)c] > INT32_MAX;
+        ++seen;
+      }
     }
     if (v > 0 && cc <= 1 && t->term_count[v] == 0)
       return err = "non-root node " + std::to_string(v) + " with <= 1 child stores no sequence (not compressed)", false;
   }
-  // Reachability from the root and path lengths (a path of more than 2^31-1 tokens is rejected).
-  std::vector<int64_t> depth((size_t)N, -1);
-  std::vector<int64_t> st{0};
-  depth[0] = 0;
-  int64_t seen = 0;
-  while (!st.empty()) {
-    const int64_t v = st.back();
-    st.pop_back();
-    ++seen;
-    for (int64_t e = t->child_begin[v]; e < t->child_begin[v] + t->child_count[v]; ++e) {
-      const int64_t c = t->child_idx[e];
-      if (depth[(size_t)c] != -1) return err = "cycle in child lists", false;
-      depth[(size_t)c] = depth[(size_t)v] + t->label_len[c];
-      if (depth[(size_t)c] > INT32_MAX) return err = "a path is longer than 2^31-1 tokens", false;
-      st.push_back(c);
+  // Reachability from the root and path lengths (a path of more than 2^31-1 tokens is rejected) by a search otherwise.
+  if (!ordered) {
+    std::fill(depth.begin(), depth.end(), -1);
+    std::vector<int64_t> st{0};
+    depth[0] = 0;
+    seen = 0;
+    too_long = false;
+    while (!st.empty() && !too_long) {
+      const int64_t v = st.back();
+      st.pop_back();
+      ++seen;
+      for (int64_t e = t->child_begin[v]; e < t->child_begin[v] + t->child_count[v]; ++e) {
+        const int64_t c = t->child_idx[e];
+        if (depth[(size_t)c] != -1) return err = "cycle in child lists", false;
+        depth[(size_t)c] = depth[(size_t)v] + t->label_len[c];
+        too_long = too_long || depth[(size_t)c] > INT32_MAX;
+        st.push_back(c);
+      }
     }
   }
+  if (too_long) return err = "a path is longer than 2^31-1 tokens", false;
   if (seen != N) return err = "nodes unreachable from the root", false;
   return true;
 }
