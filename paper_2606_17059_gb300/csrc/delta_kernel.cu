@@ -1237,55 +1237,80 @@ __global__ void init_ranges_kernel(TreeState* states, int32_t nt, const int64_t*
 constexpr int kCompactThreads = 512;   // two CTAs per SM: every tree of a 256-tree router at once
 constexpr int kSmallBits = 4;   // tables of at most 16 slots are copied by one thread
 constexpr int kSlotBatch = 4;   // slots of a small table a thread loads before it handles them
-constexpr int kUnitSlots = 1024;  // slots of a big table per unit of warp work
+constexpr int kUnitSlots = 256;   // slots of a big table per unit of warp work, at least (unit_slots)
+constexpr int kMaxUnits = 512;    // units of a table
 constexpr int kUnitCap = 2048;    // units queued per level (a table whose units do not fit is copied by a thread)
 constexpr int kLabelThreads = 256;  // compact_labels_kernel: CTAs of 8 warps, a warp per 32 new nodes
 constexpr int kLabelCtasPerSm = 8;
 
 struct CompactShared {
   int node, child, label, fail, nunits;
-  int2 units[kUnitCap];  // (new node id, first slot) of kUnitSlots slots of a big table; id -1: none
+  int2 units[kUnitCap];  // (new node id, first slot) of a big table; id -1: none
 };
 
-// Copies the table of node cid (old record rec) into a fresh table of the same size, one thread.  The
-// slots are loaded kSlotBatch at a time; each batch takes its new ids and label space with one reservation,
-// and the thread places its entries by linear probing on a bit mask of the slots it has filled, so the new
-// table is written once, with no read-back.  A big table (a level with more units than the warps' list holds)
-// does not fit the mask: it is zeroed first and probed in memory.  Labels are not copied here: each child's
-// scratch entry records where its label moves, and compact_labels_kernel moves them all afterwards.
-__device__ void compact_node_thread(CompactJob& J, CompactShared& S, int32_t cid, const int4& rec) {
-  const int32_t bits = tab_bits(rec.y);
-  int32_t noff = 0, live = 0;
-  if (bits) {
-    const int32_t size = 1 << bits;
-    const uint32_t mask = (uint32_t)size - 1;
-    noff = atomicAdd(&S.child, size);
-    if ((int64_t)noff + size > J.cap_child) {
-      atomicOr(&S.fail, 1);
-      return;
+// Slots of a big table per unit: at most kMaxUnits units a table.
+__device__ __forceinline__ int32_t unit_slots(int32_t bits) { return max(kUnitSlots, (1 << bits) / kMaxUnits); }
+
+// Copies the tables of 32 nodes (old records rec; `on`: the lane has one, with at most 2^kSmallBits slots) into fresh
+// tables of the same sizes, a lane per node.  The warp counts its tables' entries first and takes slots, new ids and
+// label space for all of them with one reservation of each; a lane then places its entries by linear probing on a bit
+// mask of the slots it has filled, so the new table is written once, with no read-back.  Labels are not copied here:
+// each child's scratch entry records where its label moves, and compact_labels_kernel moves them all afterwards.
+__device__ void compact_nodes_warp(CompactJob& J, CompactShared& S, int32_t cid, const int4& rec, bool on, int lane) {
+  const int32_t bits = on ? tab_bits(rec.y) : 0, size = bits ? 1 << bits : 0;
+  const int4* old = J.child + rec.x;
+  int4 e[kSlotBatch];
+  int32_t cnt = 0, tot = 0;  // entries, and own label tokens
+#pragma unroll
+  for (int u = 0; u < kSlotBatch; ++u) {
+    e[u] = u < size ? __ldg(old + u) : make_int4(0, 0, 0, 0);
+    cnt += e[u].y >= 1;
+    tot += e[u].y >= 1 && e[u].z >= 0 ? e[u].w : 0;
+  }
+  for (int32_t j0 = kSlotBatch; j0 < size; j0 += kSlotBatch) {
+    int4 x[kSlotBatch];
+#pragma unroll
+    for (int u = 0; u < kSlotBatch; ++u) x[u] = __ldg(old + j0 + u);
+#pragma unroll
+    for (int u = 0; u < kSlotBatch; ++u) {
+      cnt += x[u].y >= 1;
+      tot += x[u].y >= 1 && x[u].z >= 0 ? x[u].w : 0;
     }
-    const bool big = bits > kSmallBits;
-    if (big)
-      for (int32_t j = 0; j < size; ++j) J.nchild[noff + j] = make_int4(0, 0, 0, 0);
+  }
+  int32_t noff = 0;
+  if (__any_sync(kFull, size > 0)) {
+    // Prefix sums over the warp: slots and entries (at most 2^kSmallBits a lane) in one word, label tokens.
+    const int32_t mine = size << 16 | cnt;
+    int32_t sum = mine, lsum = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(kFull, sum, o), ly = __shfl_up_sync(kFull, lsum, o);
+      if (lane >= o) {
+        sum += y;
+        lsum += ly;
+      }
+    }
+    const int32_t all = __shfl_sync(kFull, sum, 31), all_l = __shfl_sync(kFull, lsum, 31);
+    int32_t base = 0;
+    bool full = false;
+    if (lane < 3) {
+      int* counter = lane == 0 ? &S.node : lane == 1 ? &S.child : &S.label;
+      const int32_t want = lane == 0 ? all & 0xffff : lane == 1 ? all >> 16 : all_l;
+      const int32_t cap = lane == 0 ? J.cap_node : lane == 1 ? J.cap_child : J.cap_label;
+      base = want ? atomicAdd(counter, want) : 0;
+      full = (int64_t)base + want > cap;
+      if (full) atomicOr(&S.fail, 1);
+    }
+    if (__any_sync(kFull, full)) return;
+    int32_t c = __shfl_sync(kFull, base, 0) + ((sum - mine) & 0xffff);
+    noff = __shfl_sync(kFull, base, 1) + ((sum - mine) >> 16);
+    int32_t nz = __shfl_sync(kFull, base, 2) + lsum - tot;
+    const uint32_t mask = (uint32_t)size - 1;
     uint32_t used = 0;
     for (int32_t j0 = 0; j0 < size; j0 += kSlotBatch) {
-      int4 e[kSlotBatch];
+      if (j0) {
 #pragma unroll
-      for (int u = 0; u < kSlotBatch; ++u)
-        e[u] = j0 + u < size ? __ldg(J.child + rec.x + j0 + u) : make_int4(0, 0, 0, 0);
-      int32_t cnt = 0, tot = 0;
-#pragma unroll
-      for (int u = 0; u < kSlotBatch; ++u)
-        if (e[u].y >= 1) {
-          ++cnt;
-          tot += e[u].z >= 0 ? e[u].w : 0;
-        }
-      if (!cnt) continue;
-      int32_t c = atomicAdd(&S.node, cnt);
-      int32_t nz = tot ? atomicAdd(&S.label, tot) : 0;
-      if ((int64_t)c + cnt > J.cap_node || (int64_t)nz + tot > J.cap_label) {
-        atomicOr(&S.fail, 1);
-        return;
+        for (int u = 0; u < kSlotBatch; ++u) e[u] = __ldg(old + j0 + u);
       }
 #pragma unroll
       for (int u = 0; u < kSlotBatch; ++u) {
@@ -1294,40 +1319,101 @@ __device__ void compact_node_thread(CompactJob& J, CompactShared& S, int32_t cid
         const int32_t z = own ? nz : e[u].z;
         J.queue[c] = make_int4(e[u].y, e[u].z, z, own ? e[u].w : 0);
         uint32_t sl = slot_hash(e[u].x, bits);
-        if (big) {
-          while (J.nchild[noff + sl].y) sl = (sl + 1) & mask;
-        } else {
-          while ((used >> sl) & 1u) sl = (sl + 1) & mask;
-          used |= 1u << sl;
-        }
+        while ((used >> sl) & 1u) sl = (sl + 1) & mask;
+        used |= 1u << sl;
         J.nchild[noff + sl] = make_int4(e[u].x, c, z, e[u].w);
         ++c;
         nz += own ? e[u].w : 0;
-        ++live;
       }
     }
-    for (int32_t j = 0; !big && j < size; ++j)
+    for (int32_t j = 0; j < size; ++j)
       if (!((used >> j) & 1u)) J.nchild[noff + j] = make_int4(0, 0, 0, 0);
+  }
+  if (on) J.nnode[cid] = make_int4(size ? noff : 0, make_meta(bits, cnt), rec.z, rec.w);
+}
+
+// Copies a big table whose units do not fit the level's list, one thread: the new table is zeroed first and probed in
+// memory.
+__device__ void compact_node_thread(CompactJob& J, CompactShared& S, int32_t cid, const int4& rec) {
+  const int32_t bits = tab_bits(rec.y), size = 1 << bits;
+  const uint32_t mask = (uint32_t)size - 1;
+  const int32_t noff = atomicAdd(&S.child, size);
+  if ((int64_t)noff + size > J.cap_child) {
+    atomicOr(&S.fail, 1);
+    return;
+  }
+  for (int32_t j = 0; j < size; ++j) J.nchild[noff + j] = make_int4(0, 0, 0, 0);
+  int32_t live = 0;
+  for (int32_t j0 = 0; j0 < size; j0 += kSlotBatch) {
+    int4 e[kSlotBatch];
+    int32_t cnt = 0, tot = 0;
+#pragma unroll
+    for (int u = 0; u < kSlotBatch; ++u) {
+      e[u] = __ldg(J.child + rec.x + j0 + u);
+      cnt += e[u].y >= 1;
+      tot += e[u].y >= 1 && e[u].z >= 0 ? e[u].w : 0;
+    }
+    if (!cnt) continue;
+    int32_t c = atomicAdd(&S.node, cnt);
+    int32_t nz = tot ? atomicAdd(&S.label, tot) : 0;
+    if ((int64_t)c + cnt > J.cap_node || (int64_t)nz + tot > J.cap_label) {
+      atomicOr(&S.fail, 1);
+      return;
+    }
+#pragma unroll
+    for (int u = 0; u < kSlotBatch; ++u) {
+      if (e[u].y < 1) continue;
+      const bool own = e[u].z >= 0;
+      const int32_t z = own ? nz : e[u].z;
+      J.queue[c] = make_int4(e[u].y, e[u].z, z, own ? e[u].w : 0);
+      uint32_t sl = slot_hash(e[u].x, bits);
+      while (J.nchild[noff + sl].y) sl = (sl + 1) & mask;
+      J.nchild[noff + sl] = make_int4(e[u].x, c, z, e[u].w);
+      ++c;
+      nz += own ? e[u].w : 0;
+      ++live;
+    }
   }
   J.nnode[cid] = make_int4(noff, make_meta(bits, live), rec.z, rec.w);
 }
 
-// Copies slots [start, end) of a big table (old record rec) into its new table at noff, one warp: lane j
-// takes slot base + j, and new ids and label space for the live slots come from one reservation per 32
-// slots (ranks and a prefix sum of label lengths); entries go into the new table with a 64-bit
-// compare-and-swap, since other warps fill other ranges of the same table.  As for small tables, the
-// labels themselves move later.
+// Copies slots [start, end) of a big table (old record rec) into its new table at noff, one warp.  It counts the
+// entries first, takes new ids and label space for all of them with one reservation of each, then places them, lane j
+// slot base + j; entries go into the new table with a 64-bit compare-and-swap, since other warps fill other ranges of
+// the same table.  As for small tables, the labels themselves move later.
 __device__ void compact_range_warp(CompactJob& J, CompactShared& S, const int4& rec, int32_t noff, int32_t start,
                                    int32_t end, int lane) {
   const int32_t bits = tab_bits(rec.y);
   const uint32_t mask = (1u << bits) - 1;
-  for (int32_t base = start; base < end; base += 32) {
-    const int32_t j = base + lane;
-    const int4 e = j < end ? __ldg(J.child + rec.x + j) : make_int4(0, 0, 0, 0);
-    const bool is_live = j < end && e.y >= 1;
+  const int4* old = J.child + rec.x;
+  int32_t cnt = 0, tot = 0;
+  for (int32_t j0 = start + lane; j0 < end; j0 += 32 * kSlotBatch) {
+    int4 x[kSlotBatch];
+#pragma unroll
+    for (int u = 0; u < kSlotBatch; ++u) x[u] = j0 + 32 * u < end ? __ldg(old + j0 + 32 * u) : make_int4(0, 0, 0, 0);
+#pragma unroll
+    for (int u = 0; u < kSlotBatch; ++u) {
+      cnt += x[u].y >= 1;
+      tot += x[u].y >= 1 && x[u].z >= 0 ? x[u].w : 0;
+    }
+  }
+  cnt = __reduce_add_sync(kFull, cnt);
+  tot = __reduce_add_sync(kFull, tot);
+  if (!cnt) return;
+  int32_t base = 0;
+  bool full = false;
+  if (lane < 2) {
+    base = atomicAdd(lane == 0 ? &S.node : &S.label, lane == 0 ? cnt : tot);
+    full = (int64_t)base + (lane == 0 ? cnt : tot) > (lane == 0 ? J.cap_node : J.cap_label);
+    if (full) atomicOr(&S.fail, 1);
+  }
+  if (__any_sync(kFull, full)) return;
+  int32_t nbase = __shfl_sync(kFull, base, 0), lbase = __shfl_sync(kFull, base, 1);
+  for (int32_t b = start; b < end; b += 32) {
+    const int4 e = b + lane < end ? __ldg(old + b + lane) : make_int4(0, 0, 0, 0);
+    const bool is_live = e.y >= 1;
     const unsigned m = __ballot_sync(kFull, is_live);
     if (!m) continue;
-    const int32_t cnt = __popc(m), rank = __popc(m & ((1u << lane) - 1));
     const int32_t w = is_live && e.z >= 0 ? e.w : 0;
     int32_t incl = w;
 #pragma unroll
@@ -1335,22 +1421,11 @@ __device__ void compact_range_warp(CompactJob& J, CompactShared& S, const int4& 
       const int32_t y = __shfl_up_sync(kFull, incl, o);
       if (lane >= o) incl += y;
     }
-    const int32_t total = __shfl_sync(kFull, incl, 31);
-    int32_t lbase = 0, nbase = 0, bad = 0;
-    if (lane == 0) {
-      lbase = atomicAdd(&S.label, total);
-      nbase = atomicAdd(&S.node, cnt);
-      bad = (int64_t)lbase + total > J.cap_label || (int64_t)nbase + cnt > J.cap_node;
-      if (bad) atomicOr(&S.fail, 1);
-    }
-    if (__shfl_sync(kFull, bad, 0)) return;
-    lbase = __shfl_sync(kFull, lbase, 0);
-    nbase = __shfl_sync(kFull, nbase, 0);
     if (is_live) {
-      const int32_t cid = nbase + rank;
+      const int32_t c = nbase + __popc(m & ((1u << lane) - 1));
       const int32_t nz = e.z >= 0 ? lbase + incl - w : e.z;
-      J.queue[cid] = make_int4(e.y, e.z, nz, w);
-      const unsigned long long kv = (unsigned long long)(uint32_t)e.x | ((unsigned long long)(uint32_t)cid << 32);
+      J.queue[c] = make_int4(e.y, e.z, nz, w);
+      const unsigned long long kv = (unsigned long long)(uint32_t)e.x | ((unsigned long long)(uint32_t)c << 32);
       uint32_t sl = slot_hash(e.x, bits);
       for (uint32_t it = 0; it <= mask; ++it, sl = (sl + 1) & mask) {
         if (atomicCAS((unsigned long long*)&J.nchild[noff + sl], 0ull, kv) == 0ull) {
@@ -1360,16 +1435,22 @@ __device__ void compact_range_warp(CompactJob& J, CompactShared& S, const int4& 
         }
       }
     }
+    nbase += __popc(m);
+    lbase += __shfl_sync(kFull, incl, 31);
   }
 }
 
 // One cluster of kC CTAs per tree (kC = 1: a CTA): level-synchronous breadth-first copy of the structure from the root.  New ids are
 // handed out level by level, so the nodes of the next level are the ids [end, S.node) and the scratch
 // entry of id c (old id, old and new label offsets, own-arena label length) is written by the parent's
-// copy.  A thread takes each node of the level.  A node whose table has more than 2^kSmallBits slots gets
-// its new table range and record from that thread, and its slots are cut into units of kUnitSlots that all
-// warps then zero and fill; smaller tables are copied by the thread.  A big table's record counts its
+// copy.  A lane takes each node of the level.  A node whose table has more than 2^kSmallBits slots gets
+// its new table range and record from that lane, and its slots are cut into units (unit_slots) that all
+// warps then zero and fill; smaller tables are copied by the warp's lanes.  A big table's record counts its
 // children from the old record (the live-child count), so no pass has to count them.
+// What bounds it is the chain of round trips of each level and the reservations on the tree's three counters, so a warp
+// makes one of each for its 32 nodes, or for its unit.  Measured (a
+// reservation per table, units of 1,024 slots -> this): one tree of ~50,000 nodes by eight CTAs 194 -> 102 us, a wave of
+// 256 trees 1.70 -> 1.31 ms.
 //
 // Few trees are compacted by clusters: one tree's levels keep 512 threads busy for long (a tree of ~50,000 nodes
 // 0.61 ms by a CTA), while a wave of 256 trees fills the GPU with a CTA each.  The cluster's counters and units are
@@ -1392,7 +1473,7 @@ __device__ __forceinline__ void compact_sync() {
 }
 
 template <int kC>
-__global__ void __launch_bounds__(kCompactThreads) compact_kernel(CompactJob* jobs) {
+__global__ void __launch_bounds__(kCompactThreads, kC == 1 ? 2 : 1) compact_kernel(CompactJob* jobs) {
   CompactJob& J = jobs[blockIdx.x / kC];
   __shared__ CompactShared S_own;
   CompactShared& S = *compact_shared<kC>(&S_own);
@@ -1411,26 +1492,30 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(CompactJob* jo
   compact_sync<kC>();
   int begin = 0, end = 1;
   while (begin < end) {
-    for (int cid = begin + thread; cid < end; cid += kThreads) {
-      const int4 rec = __ldg(J.node + __ldcg(&J.queue[cid].x));
+    for (int first = begin + thread - lane; first < end; first += kThreads) {
+      const int cid = first + lane;
+      bool on = cid < end;
+      const int4 rec = on ? __ldg(J.node + __ldcg(&J.queue[cid].x)) : make_int4(0, 0, 0, 0);
       const int32_t bits = tab_bits(rec.y);
-      if (bits > kSmallBits) {
-        const int32_t size = 1 << bits, nu = (size + kUnitSlots - 1) / kUnitSlots;
+      if (on && bits > kSmallBits) {
+        on = false;
+        const int32_t size = 1 << bits, per = unit_slots(bits), nu = (size + per - 1) / per;
         const int u0 = atomicAdd(&S.nunits, nu);
         if (u0 + nu <= kUnitCap) {
           const int32_t noff = atomicAdd(&S.child, size);
-          if ((int64_t)noff + size > J.cap_child) {
+          const bool full = (int64_t)noff + size > J.cap_child;
+          if (full)
             atomicOr(&S.fail, 1);
-            for (int k = 0; k < nu; ++k) S.units[u0 + k] = make_int2(-1, 0);
-            continue;
-          }
-          J.nnode[cid] = make_int4(noff, make_meta(bits, rec.z), rec.z, rec.w);
-          for (int k = 0; k < nu; ++k) S.units[u0 + k] = make_int2(cid, k * kUnitSlots);
-          continue;
+          else
+            J.nnode[cid] = make_int4(noff, make_meta(bits, rec.z), rec.z, rec.w);
+          for (int k = 0; k < nu; ++k) S.units[u0 + k] = full ? make_int2(-1, 0) : make_int2(cid, k * per);
+        } else {
+          for (int k = u0; k < kUnitCap; ++k) S.units[k] = make_int2(-1, 0);  // no room: this thread copies it
+          compact_node_thread(J, S, cid, rec);
         }
-        for (int k = u0; k < kUnitCap; ++k) S.units[k] = make_int2(-1, 0);  // no room: this thread copies it
       }
-      compact_node_thread(J, S, cid, rec);
+      __syncwarp();
+      compact_nodes_warp(J, S, cid, rec, on, lane);
     }
     compact_sync<kC>();
     const int nunits = min(S.nunits, kUnitCap);
@@ -1438,7 +1523,7 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(CompactJob* jo
       const int2 u = S.units[k];
       if (u.x < 0) continue;
       const int4 nrec = __ldcg(J.nnode + u.x);
-      const int32_t n = min(kUnitSlots, (1 << tab_bits(nrec.y)) - u.y);
+      const int32_t bits = tab_bits(nrec.y), n = min(unit_slots(bits), (1 << bits) - u.y);
       for (int32_t j = lane; j < n; j += 32) J.nchild[nrec.x + u.y + j] = make_int4(0, 0, 0, 0);
     }
     compact_sync<kC>();
@@ -1447,7 +1532,8 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(CompactJob* jo
       if (u.x < 0 || __shfl_sync(kFull, *(volatile int*)&S.fail, 0)) continue;
       const int4 rec = __ldg(J.node + __ldcg(&J.queue[u.x].x));
       const int32_t noff = __ldcg(&J.nnode[u.x].x);
-      compact_range_warp(J, S, rec, noff, u.y, min(u.y + kUnitSlots, 1 << tab_bits(rec.y)), lane);
+      const int32_t bits = tab_bits(rec.y);
+      compact_range_warp(J, S, rec, noff, u.y, min(u.y + unit_slots(bits), 1 << bits), lane);
     }
     compact_sync<kC>();
     if (thread == 0) S.nunits = 0;

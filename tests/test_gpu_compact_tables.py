@@ -37,3 +37,17 @@ def test_more_big_tables_on_a_level_than_units(n_nodes, n_children):
     gm, gp = route_device(r, tok, off, [0], 1)
     om, op_, _ = oracle.route(o, tok, off, [0], 1)
     assert_same_route(gm, gp, om, op_, "after compaction")
+
+
+# A root of 32,768 slots (units of 256), and of 262,144 (units of 512).
+@pytest.mark.parametrize("n", [8000, 40000])
+def test_units_of_a_root(n):
+    rng = np.random.default_rng(n)
+    seqs = np.concatenate([np.arange(n)[:, None] * 7 + 1, rng.integers(1, 1 << 20, size=(n, 20))], axis=1).tolist()
+    r, o = router_from_seqlists([seqlist_from_lists(seqs)]), oracle.build_trees([seqlist_from_lists(seqs)])
+    gone = [s for k, s in enumerate(seqs) if k % 5 < 3]
+    sl, op = seqlist_from_lists(gone), np.ones(len(gone), np.int32)
+    assert r.apply_delta(0, op, sl) == 0
+    o[0].apply_ops(op, sl, 0, len(gone))
+    assert r.stats(0)["stale_label"] == 0
+    assert same_snapshot(r.download(0), o[0].export())
