@@ -343,7 +343,7 @@ cudaError_t launch_lru_stamp(const TreeState& s, TreeState* d_state, const int32
 struct LruScratch {
   int32_t *cnt, *big_cnt;     // [N + 2]: nodes found for a level, and its nodes with large tables
   unsigned long long* hist;   // [4 * 256]
-  unsigned long long* out;    // [8]: tokens of the tree, 1 if it is inconsistent, depth, cut level and cut
+  unsigned long long* out;    // [8]: tokens of the tree, 1 if it is inconsistent, depth, cut level, cut, largest stamp, largest ~stamp
   size_t zeroed;
   unsigned long long* sum;    // [N], by node: tokens of the threshold's stamp in its subtree
   int32_t *order, *parent, *cslot, *len;  // [N], by position in breadth-first order

@@ -178,11 +178,13 @@ __global__ void __launch_bounds__(kLruThreads) lru_stamp_kernel(LruTree t, TreeS
 // One cluster of kEvictCtas CTAs, so that its steps are ordered by the cluster's hardware barrier: an eviction has
 // about three steps per tree level and eight for the threshold.  With a launch per step (and per step of a global
 // bitonic sort of all siblings, and a host read per step of a binary search for the threshold) an eviction from
-// a trie of ~20,000 nodes took 240 launches and 100 host reads, 2.6 ms; now 0.2 ms.  What bounds it: the barriers and the
+// a trie of ~20,000 nodes took 240 launches and 100 host reads, 2.6 ms; now 0.11 ms (0.19 with large tables one after
+// another, 32 nodes a warp at every level, and four passes of every selection).  What bounds it: the barriers and the
 // dependent loads between them (a level's records, tables, stamps); 16 of the SMs stream the tables at ~1 TB/s,
 // which large tries need less than the steps do.
 constexpr int kEvictThreads = 1024;
 constexpr int kEvictCtas = 16;
+constexpr int kHeld = 8;        // slots a thread keeps of the table that the walk is at
 constexpr int kLaneBits = 4;    // tables of up to 16 slots are read by one lane,
 constexpr int kWarpBits = 8;    // up to 256 slots by one warp, larger ones by the whole cluster
 constexpr int kStBefore = 0, kStAfter = 1, kStOnPath = 2, kStGone = 4;
@@ -204,6 +206,7 @@ __device__ __forceinline__ uint32_t cluster_size() {
 struct EvictShared {
   unsigned long long hist[256];
   unsigned long long below, sum, best;
+  uint32_t least, most;  // of the keys of a selection
   int bin, child, len, tok;
 };
 
@@ -237,6 +240,11 @@ __device__ void pick_bin(EvictShared& S, unsigned long long r) {
   __syncthreads();
 }
 
+// The first pass of a radix selection by bytes over keys from lo to hi: those above it are the same in all keys.
+__device__ __forceinline__ int first_pass(uint32_t lo, uint32_t hi) { return min(3, __clz((int)(lo ^ hi)) / 8); }
+// The bytes of x above pass `pass`.
+__device__ __forceinline__ uint32_t bytes_above(uint32_t x, int pass) { return pass == 0 ? 0u : x >> (32 - 8 * pass); }
+
 // Adds w to bin k of S.hist: one addition for the warp when all of its lanes have the same bin (the high bytes
 // of the keys usually agree).  Every lane of the warp calls it; w = 0 adds nothing.
 __device__ __forceinline__ void add_bin(EvictShared& S, int k, unsigned long long w) {
@@ -268,20 +276,34 @@ __global__ void __launch_bounds__(kEvictThreads, 1) lru_evict_kernel(LruTree t, 
   }
   cluster_sync();
   // Breadth-first order, a level at a time.  By position in the order: node, parent, slot, edge length, stamp.
+  uint32_t newest = 0, oldest = ~0u;  // stamps this thread has put
   auto put = [&](int32_t at, int32_t v, int32_t slot, const int4& e) {
     if (at >= N) return;  // (more nodes than the tree has: reported below)
+    const uint32_t x = t.stamp[e.y];
     s.order[at] = e.y;
     s.parent[at] = v;
     s.cslot[at] = slot;
     s.len[at] = e.w;
-    s.stamp[at] = t.stamp[e.y];
+    s.stamp[at] = x;
     s.sum[e.y] = 0;
+    newest = max(newest, x);
+    oldest = min(oldest, x);
+  };
+  // (Ahead of a barrier that follows the last put.)
+  auto put_range = [&]() {
+    const uint32_t hi = __reduce_max_sync(kFull, newest), lo = __reduce_min_sync(kFull, oldest);
+    if (lane == 0 && lo <= hi) {
+      atomicMax(&s.out[5], (unsigned long long)hi);
+      atomicMax(&s.out[6], (unsigned long long)~lo);
+    }
   };
   int32_t begin = 0, end = 1, L = 0;
   for (;;) {
-    for (int32_t b0 = begin + gw * 32; b0 < end; b0 += n_warps * 32) {
+    // Nodes per warp: few enough that every warp has some, since a warp reads its nodes' larger tables one by one.
+    const int32_t per = max(1, min(32, (end - begin) / n_warps));
+    for (int32_t b0 = begin + gw * per; b0 < end; b0 += n_warps * per) {
       const int32_t i = b0 + lane;
-      const int32_t v = i < end ? __ldcg(s.order + i) : -1;
+      const int32_t v = lane < per && i < end ? __ldcg(s.order + i) : -1;
       const int4 nd = v >= 0 ? t.node[v] : make_int4(0, 0, 0, 0);
       const int32_t bits = tab_bits(nd.y);
       const int32_t z = bits > 0 && bits <= kWarpBits ? max(nd.z, 0) : 0;  // its children, placed side by side
@@ -324,21 +346,35 @@ __global__ void __launch_bounds__(kEvictThreads, 1) lru_evict_kernel(LruTree t, 
         }
       }
     }
+    put_range();
     cluster_sync();
     const int32_t nb = min(__ldcg(s.big_cnt + L), N);
     if (nb) {
-      for (int32_t k = 0; k < nb; ++k) {
-        const int32_t v = __ldcg(s.big + k);
-        const int4 nd = t.node[v];
-        for (int32_t j0 = gw * 32; j0 < (1 << tab_bits(nd.y)); j0 += n_warps * 32) {
-          const int4 e = t.child[nd.x + j0 + lane];
+      // 32 large tables at a time: a warp takes 32 slots of any of them.
+      for (int32_t k0 = 0; k0 < nb; k0 += 32) {
+        const int32_t v = k0 + lane < nb ? __ldcg(s.big + k0 + lane) : -1;
+        const int4 nd = v >= 0 ? t.node[v] : make_int4(0, 0, 0, 0);
+        const int32_t parts = v >= 0 ? 1 << (tab_bits(nd.y) - 5) : 0;
+        int32_t incl = parts;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int32_t y = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += y;
+        }
+        const int32_t parts_all = __shfl_sync(kFull, incl, 31);
+        for (int32_t c = gw; c < parts_all; c += n_warps) {
+          const int j = __popc(__ballot_sync(kFull, incl <= c));  // part c is the j-th table's
+          const int32_t vj = __shfl_sync(kFull, v, j);
+          const int32_t slot = __shfl_sync(kFull, nd.x, j) + 32 * (c - __shfl_sync(kFull, incl - parts, j)) + lane;
+          const int4 e = t.child[slot];
           const unsigned lm = __ballot_sync(kFull, e.y >= 1);
           int32_t base = 0;
           if (lane == 0 && lm) base = atomicAdd(&s.cnt[L + 1], __popc(lm));
           base = __shfl_sync(kFull, base, 0);
-          if (e.y >= 1) put(end + base + __popc(lm & ((1u << lane) - 1)), v, nd.x + j0 + lane, e);
+          if (e.y >= 1) put(end + base + __popc(lm & ((1u << lane) - 1)), vj, slot, e);
         }
       }
+      put_range();
       cluster_sync();
     }
     const int32_t c = __ldcg(s.cnt + L + 1);
@@ -354,17 +390,19 @@ __global__ void __launch_bounds__(kEvictThreads, 1) lru_evict_kernel(LruTree t, 
   }
   const int32_t total = end;
   // The stamp S of the threshold: a radix selection of unit `want` of the edge lengths by stamp.
-  uint32_t cut_stamp = 0;
+  const uint32_t stamp_hi = (uint32_t)__ldcg(s.out + 5), stamp_lo = ~(uint32_t)__ldcg(s.out + 6);
+  const int stamp_pass = first_pass(stamp_lo, stamp_hi);
+  uint32_t cut_stamp = bytes_above(stamp_hi, stamp_pass);
   unsigned long long rest = want;
   bool all = false;
-  for (int pass = 0; pass < 4; ++pass) {
+  for (int pass = stamp_pass; pass < 4; ++pass) {
     const int shift = 24 - 8 * pass;
     for (int k = threadIdx.x; k < 256; k += kEvictThreads) S.hist[k] = 0;
     __syncthreads();
     for (int32_t i0 = 1 + gw * 32; i0 < total; i0 += n_threads) {
       const int32_t i = i0 + lane;
       const uint32_t x = i < total ? __ldcg(s.stamp + i) : 0u;
-      const bool in = i < total && (pass == 0 || (x >> (shift + 8)) == cut_stamp);
+      const bool in = i < total && bytes_above(x, pass) == cut_stamp;
       add_bin(S, (int)((x >> shift) & 255u), in ? (unsigned long long)__ldcg(s.len + i) : 0ull);
     }
     __syncthreads();
@@ -373,7 +411,7 @@ __global__ void __launch_bounds__(kEvictThreads, 1) lru_evict_kernel(LruTree t, 
     cluster_sync();
     for (int k = threadIdx.x; k < 256; k += kEvictThreads) S.hist[k] = __ldcg(&s.hist[pass * 256 + k]);
     pick_bin(S, rest);
-    if (pass == 0) {
+    if (pass == stamp_pass) {
       if (lead) s.out[0] = S.sum;
       if (rest >= S.sum) {
         all = true;
@@ -407,47 +445,87 @@ __global__ void __launch_bounds__(kEvictThreads, 1) lru_evict_kernel(LruTree t, 
         const int32_t size = tab_bits(nd.y) ? 1 << tab_bits(nd.y) : 0;
         const bool same = u != 0 && t.stamp[u] == cut_stamp;
         if (same) carry += (unsigned long long)len_u;
-        // A table of up to one slot per thread is read once; larger ones once per step.
-        const bool held = size <= kEvictThreads;
-        int4 e0 = make_int4(0, 0, 0, 0);
-        if (held && (int)threadIdx.x < size) e0 = t.child[nd.x + threadIdx.x];
-        unsigned long long T0 = e0.y >= 1 ? __ldcg(s.sum + e0.y) : 0ull;
+        // The children's keys and weights, kept by the threads for a table of up to kHeld slots a thread, and read again
+        // by each step for a larger one.
+        const bool held = size <= kHeld * kEvictThreads;
+        uint32_t kx[kHeld] = {};
+        unsigned long long kw[kHeld] = {};
+        if (held) {
+#pragma unroll
+          for (int c = 0; c < kHeld; ++c) {
+            const int32_t j = c * kEvictThreads + (int32_t)threadIdx.x;
+            const int4 e = j < size ? t.child[nd.x + j] : make_int4(0, 0, 0, 0);
+            kx[c] = (uint32_t)e.x ^ 0x80000000u;
+            kw[c] = e.y >= 1 ? __ldcg(s.sum + e.y) : 0ull;
+          }
+        }
         if (threadIdx.x == 0) {
           S.best = 0;
           S.child = S.len = S.tok = 0;
+          S.least = ~0u;
+          S.most = 0;
         }
         __syncthreads();
         if (same)
           for (int32_t j = threadIdx.x; j < size; j += kEvictThreads) {
-            const int4 e = held ? e0 : t.child[nd.x + j];
+            const int4 e = t.child[nd.x + j];
             if (e.y >= 1 && t.stamp[e.y] == cut_stamp)
               atomicMax(&S.best, ((unsigned long long)((uint32_t)e.x ^ 0x80000000u) << 32) | (uint32_t)e.y);
           }
         __syncthreads();
         const int32_t best = (int32_t)(S.best & 0xffffffffull);
         if (same && best == 0) break;  // the carried edges end here
-        if (held && same && e0.y == best && e0.y >= 1) T0 += carry;
-        uint32_t key = 0;
-        for (int pass = 0; pass < 4; ++pass) {
+        const uint32_t best_key = (uint32_t)(S.best >> 32);
+        // f(key, weight) for every slot; all of a warp's lanes come to it together.
+        auto each = [&](auto f) {
+          if (held) {
+#pragma unroll
+            for (int c = 0; c < kHeld; ++c)
+              if (c * kEvictThreads < size) f(kx[c], kw[c]);
+          } else {
+            for (int32_t j0 = 0; j0 < size; j0 += kEvictThreads) {
+              const int4 e = t.child[nd.x + j0 + (int32_t)threadIdx.x];  // (a table this large is a multiple of the CTA)
+              const uint32_t x = (uint32_t)e.x ^ 0x80000000u;
+              const unsigned long long w = e.y >= 1 ? __ldcg(s.sum + e.y) : 0ull;
+              f(x, w && same && x == best_key ? w + carry : w);
+            }
+          }
+        };
+        if (held && same) {  // (best stands for tokens of its own, so its weight is not 0; a tombstone's is)
+#pragma unroll
+          for (int c = 0; c < kHeld; ++c)
+            if (kw[c] && kx[c] == best_key) kw[c] += carry;
+        }
+        uint32_t least = ~0u, most = 0;
+        each([&](uint32_t x, unsigned long long w) {
+          if (w) {
+            least = min(least, x);
+            most = max(most, x);
+          }
+        });
+        least = __reduce_min_sync(kFull, least);
+        most = __reduce_max_sync(kFull, most);
+        if (lane == 0 && least <= most) {
+          atomicMin(&S.least, least);
+          atomicMax(&S.most, most);
+        }
+        __syncthreads();
+        const int key_pass = first_pass(S.least, S.most);
+        uint32_t key = bytes_above(S.most, key_pass);
+        for (int pass = key_pass; pass < 4; ++pass) {
           const int shift = 24 - 8 * pass;
           for (int k = threadIdx.x; k < 256; k += kEvictThreads) S.hist[k] = 0;
           __syncthreads();
-          for (int32_t j0 = 0; j0 < size; j0 += kEvictThreads) {
-            const int32_t j = j0 + (int32_t)threadIdx.x;
-            const int4 e = held ? e0 : j < size ? t.child[nd.x + j] : make_int4(0, 0, 0, 0);
-            const uint32_t x = (uint32_t)e.x ^ 0x80000000u;
-            const bool in = j < size && e.y >= 1 && (pass == 0 || (x >> (shift + 8)) == key);
-            unsigned long long w = 0;
-            if (in) w = held ? T0 : __ldcg(s.sum + e.y) + (same && e.y == best ? carry : 0ull);
-            add_bin(S, (int)((x >> shift) & 255u), w);
-          }
+          each([&](uint32_t x, unsigned long long w) {
+            add_bin(S, (int)((x >> shift) & 255u), bytes_above(x, pass) == key ? w : 0ull);
+          });
           pick_bin(S, r);
           r -= S.below;
           key = (key << 8) | (uint32_t)S.bin;
           __syncthreads();
         }
         for (int32_t j = threadIdx.x; j < size; j += kEvictThreads) {
-          const int4 e = held ? e0 : t.child[nd.x + j];
+          const int4 e = t.child[nd.x + j];
           if (e.y >= 1 && ((uint32_t)e.x ^ 0x80000000u) == key) {
             S.child = e.y;
             S.len = e.w;

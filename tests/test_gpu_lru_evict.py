@@ -69,3 +69,22 @@ def test_eviction_along_chains():
             assert _access(r, 0, reqs, t).tolist() == [o.access(s, t) for s in reqs]
         _evict_both(r, o, n)
         _evict_both(r, o, n)
+
+
+@pytest.mark.parametrize("fan,inner,kids", [(4500, 0, 0), (60, 40, 140)])
+def test_eviction_of_large_tables(fan, inner, kids):
+    """A root larger than the threads keep (8,192 slots), and more than 32 nodes of one level with tables that the
+    whole cluster reads; stamps that differ in every byte, in one, and not at all."""
+    rng = random.Random(fan)
+    seqs = [[rng.randrange(-(1 << 31), 1 << 31), 3][: rng.randint(1, 2)] for _ in range(fan)]
+    seqs += [[i, 7, 7, rng.randrange(1 << 20)] for i in range(inner) for _ in range(kids)]
+    r, o = g.Router(1), LRUTrie()
+    g.p2p_lru_enable(r.handle, 0)
+    _insert(r, 0, seqs, 5)
+    for s in seqs:
+        o.insert(s, 5)
+    _evict_both(r, o, 30)
+    for t in (6, 300, 70000, (1 << 24) + 9, (1 << 32) - 2):
+        reqs = [list(rng.choice(seqs)) for _ in range(40)]
+        assert _access(r, 0, reqs, t).tolist() == [o.access(s, t) for s in reqs]
+        _evict_both(r, o, 25)
