@@ -45,8 +45,8 @@
 // other edges and look again.
 //
 // Measured, the delta of a call (delta_kernel alone -> these rounds and delta_kernel behind them): 16,384 routed
-// requests into 16 trees, most into one, 8.2 -> 0.21 ms; 4,096 requests into one cache trie 2.46 -> 0.12 ms; 300 ops
-// into one tree 189 -> 77 us; 1,024,000 ops on 256 trees of 40,000 sequences 3.58 -> 1.46 ms.
+// requests into 16 trees, most into one, 8.2 -> 0.18 ms; 4,096 requests into one cache trie 2.46 -> 0.12 ms; 300 ops
+// into one tree 189 -> 77 us; 1,024,000 ops on 256 trees of 40,000 sequences 3.58 -> 1.44 ms.
 #include "internal.h"
 
 namespace p2p {
@@ -70,7 +70,10 @@ constexpr int kBulkThreads = 256;
 constexpr int kBulkWarps = kBulkThreads / 32;
 constexpr int kBulkCtasPerSm = 4;   // at most 64 registers a thread (80 and 3 CTAs: the resolve launches of a step of
                                     // 1,024,000 ops 0.90 ms instead of 0.81)
-constexpr int kLaneSpan = 128;      // label tokens after the first eight that a lane compares alone
+// Label tokens after the first eight that a lane compares alone: a warp of few ops has its lanes compare them together
+// instead (one round trip an op, where the lane takes one per eight tokens).  16,384 routed requests, four ops a warp:
+// the first resolve launch 8% shorter; a warp of 16 ops or more keeps its 128.
+constexpr int kLaneSpan = 128, kLaneSpanPerOp = 8;
 constexpr int kLaneBits = 5;        // tables up to 32 slots are moved by one lane
 constexpr int kMaxProbes = 64;      // of the key and node tables
 constexpr int kMemoProbes = 4;
@@ -268,8 +271,10 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
   const int lane = threadIdx.x & 31;
   const int64_t total = list_size(A, round);
   const int64_t warps = (int64_t)gridDim.x * kBulkWarps;
-  // Ops per warp: few enough that every warp has some, since a warp's long compares follow one another.
-  const int32_t per = (int32_t)max((int64_t)1, min((int64_t)32, total / warps));
+  // Ops per warp: few enough that every warp has some, since a warp's long compares follow one another, and rounded up,
+  // since a few warps with a second turn double the launch (16,384 ops: 3.4 a warp, the resolve launches 34 -> 30 us).
+  const int32_t per = (int32_t)max((int64_t)1, min((int64_t)32, (total + warps - 1) / warps));
+  const int32_t lane_span = min(kLaneSpan, kLaneSpanPerOp * per);
   const int32_t* list = A.lists + (round & 1) * A.n;
   for (int64_t t = (int64_t)blockIdx.x * kBulkThreads + threadIdx.x; t < A.n_trees; t += (int64_t)gridDim.x * kBulkThreads) {
     const TreeState& s = A.states[t];  // the arenas' use ahead of this round's reservations
@@ -327,7 +332,7 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
           first = min(lim, 9);
           k = diff_lane(lab, q, pos, 1, first);
           if (k == first && first < lim) {
-            if (lim - first <= kLaneSpan) {
+            if (lim - first <= lane_span) {
               k = diff_lane(lab, q, pos, first, lim);
             } else {
               need = true;
@@ -739,7 +744,7 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
   const int lane = threadIdx.x & 31;
   const int64_t total = list_size(A, round);
   const int64_t warps = (int64_t)gridDim.x * kBulkWarps;
-  const int32_t per = (int32_t)max((int64_t)1, min((int64_t)32, total / warps));
+  const int32_t per = (int32_t)max((int64_t)1, min((int64_t)32, (total + warps - 1) / warps));
   const int32_t* list = A.lists + (round & 1) * A.n;
   int32_t* next = A.lists + ((round + 1) & 1) * A.n;
   for (int64_t b0 = (((int64_t)blockIdx.x * kBulkThreads + threadIdx.x) >> 5) * per; b0 < total; b0 += warps * per) {

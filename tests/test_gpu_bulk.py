@@ -142,3 +142,25 @@ def test_room_running_out(seed):
     for p in range(4):
         seqs = [[rng.randrange(60) for _ in range(rng.randint(1, 90))] for _ in range(2500)]
         _check(r, trees, [(p, [0] * 2500, seqlist_from_lists(seqs))], seqs[:50])
+
+
+@pytest.mark.parametrize("n_fill", [0, 6000])
+def test_edges_left_around_the_lane_spans(n_fill):
+    """INSERTs that leave an edge, and DELETEs and repeats that follow it, after every count of tokens around those that
+    a lane compares alone (9, then 8 per op of its warp, 128 at most), in one pool run and in two; with and without
+    enough other ops that a warp has two."""
+    rng = random.Random(n_fill)
+    lens = [1, 8, 9, 10, 16, 17, 18, 24, 25, 26, 33, 127, 128, 136, 137, 138, 300]
+    base = [[i] + [rng.randrange(1000) for _ in range(320)] for i in range(len(lens))]
+    r, o = router_from_seqlists([seqlist_from_lists(base)]), oracle.build_trees([seqlist_from_lists(base)])
+    for cuts in (0, 1):
+        ops, seqs = [], []
+        for i, k in enumerate(lens):
+            seqs += [base[i][:k] + [1000 + cuts, 5], base[i][:k] + [1000 + cuts], base[i], base[i][:k]]
+            ops += [0, 1, 0, 1]
+        fill = [[5000 + cuts * n_fill + j, 1] for j in range(n_fill)]
+        ops, seqs = np.array(ops + [0] * n_fill, np.int32), seqs + fill
+        sl = _runs(seqs, [min(len(s), 1 + 7 * (i % 30)) if cuts else len(s) for i, s in enumerate(seqs)])
+        r.apply_delta(0, ops, sl)
+        o[0].apply_ops(ops, sl, 0, len(ops))
+        assert same_snapshot(r.download(0), o[0].export()), cuts
