@@ -33,7 +33,8 @@ constexpr int kWarps = 16;              // warps per CTA
 constexpr int kThreads = kWarps * 32;
 constexpr int kSlots = 4;               // requests staged at a time per CTA
 constexpr int kCtasPerSm = 2;           // 32 warps per SM: 64 KB of slots and <= 64 registers per thread
-constexpr int kUnroll = 16;             // label loads in flight per lane on long labels (512 tokens per step)
+constexpr int kUnroll = 24;             // label loads in flight per lane on long labels (768 tokens per step; 16: the
+                                        // leader pass of 8,191 requests of 11,400 tokens 120 us instead of 98)
 constexpr int kMaxGroup = 8;            // trees per work item, at most
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kSpinLimit = 1 << 24;     // bounded waits (~1 s): the kernel flags ERR_STALL and stops
@@ -156,7 +157,8 @@ __device__ __forceinline__ int32_t compare_tail(const int32_t* __restrict__ lab,
 // First j in [j0, end) with lab[j] != req[j], or -1.  After one block at j0 the label side continues at a
 // 128-byte-aligned position at or below j0 + 32 (re-comparing <= 31 tokens): a warp's 32 consecutive label
 // tokens are then one cache line, and its 32 request tokens in shared memory fall in 32 distinct banks at
-// any alignment, so each load is a single wavefront on both sides.
+// any alignment, so each load is a single wavefront on both sides.  What is left of a large step goes by steps of 16
+// and 8 loads before the last ones of four.
 template <int U, bool kGlobal>
 __device__ __forceinline__ int32_t compare_range(const int32_t* __restrict__ lab, const int32_t* req, int32_t j0,
                                                  int32_t end, int lane) {
@@ -169,6 +171,18 @@ __device__ __forceinline__ int32_t compare_range(const int32_t* __restrict__ lab
       const int32_t k2 = compare_full<U, kGlobal>(lab, req, j0, lane);
       if (k2 >= 0) return k2;
     }
+    if constexpr (U > 16)
+      if (j0 + 16 * 32 <= end) {
+        const int32_t k2 = compare_full<16, kGlobal>(lab, req, j0, lane);
+        if (k2 >= 0) return k2;
+        j0 += 16 * 32;
+      }
+    if constexpr (U > 8)
+      if (j0 + 8 * 32 <= end) {
+        const int32_t k2 = compare_full<8, kGlobal>(lab, req, j0, lane);
+        if (k2 >= 0) return k2;
+        j0 += 8 * 32;
+      }
   }
   for (; j0 < end; j0 += 128) {
     const int32_t k = compare_tail<kGlobal>(lab, req, j0, end, lane);
@@ -574,6 +588,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) route_kernel(
 constexpr int kFollowThreads = 256;
 constexpr int kFollowCtasPerSm = 4;
 constexpr int kThreadSpan = 64;
+// Long requests' followers spend their time in compares of thousands of tokens by the warp, a round trip per step: 1,024
+// tokens a step and 16 warps on a SM (eight loads and 32 warps: the follower pass of 8,191 requests of 11,400 tokens
+// on 32 trees 150 us, 16 and 32: 96, 32 and 24: 68, 32 and 16: 59).  The others compare little: leaders of
+// short requests with 16 loads instead of eight took 579 us instead of 467 (a step's 262,144 on 256 trees).
+template <bool kLeader, int kFirst>
+constexpr int kLaneUnroll = !kLeader && kFirst == 8 ? 32 : 8;
+template <bool kLeader, int kFirst>
+constexpr int kLaneCtas = !kLeader && kFirst == 8 ? 2 : kFollowCtasPerSm;
 constexpr int kFollowIlp = 2;  // trees a follower's lane takes per iteration (their first loads overlap; 3 or 4 spill)
 
 // One thread: the child with first token tok in a table of 2^bits (>= 4) slots, two slots (a sector) per step of
@@ -669,7 +691,8 @@ __device__ __forceinline__ void lane_walks(const TreeView* __restrict__ trees, i
       int32_t cmax = mine ? lim - from2 : 0;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) cmax = max(cmax, __shfl_xor_sync(kFull, cmax, o));
-      const int32_t kk = compare_range<8, true>(reinterpret_cast<const int32_t*>(la), req + rp, 0, cmax, lane);
+      const int32_t kk = compare_range<kLaneUnroll<kLeader, kFirst>, true>(reinterpret_cast<const int32_t*>(la),
+                                                                           req + rp, 0, cmax, lane);
       if (mine) {
         k = from2 + min(kk < 0 ? cmax : kk, lim - from2);
         need = false;
@@ -710,7 +733,7 @@ __device__ __forceinline__ int probe_first2(const int4& a, const int4& b, int32_
 //   tokens.  A lane takes kFollowIlp trees at a time (p, p + 32, ...): the leader's matches, the
 //   checkpoints and the first probe step of each are loaded before any of them is looked at.
 template <bool kLeader, bool kDecide, int kFirst = 8, bool kGrouped = true>
-__global__ void __launch_bounds__(kFollowThreads, kFollowCtasPerSm) lane_kernel(
+__global__ void __launch_bounds__(kFollowThreads, kLaneCtas<kLeader, kFirst>) lane_kernel(
     const TreeView* __restrict__ trees, int32_t P, const int32_t* __restrict__ tokens, int64_t n_tokens,
     int64_t tok_base, const int64_t* __restrict__ offsets, int64_t B, const int32_t* __restrict__ list,
     const int32_t* __restrict__ count, const int32_t* __restrict__ lead, const int32_t* __restrict__ cpre,
@@ -1188,8 +1211,9 @@ cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tok
   // The followers' first per-lane compare in lane_kernel: 8 tokens for long requests, 16 otherwise (lane_walks).  A
   // single tree's followers stay with it: there is no tree to go on to.
   if (long_requests(B, n_tokens)) {
+    const int grid_long = (int)std::min<int64_t>(want, (int64_t)num_sms * kLaneCtas<false, 8>);
     P2P_TIMED(K_LANE_FOLLOWER, st,
-              (lane_kernel<false, kDecide, 8><<<grid2, kFollowThreads, 0, st>>>(
+              (lane_kernel<false, kDecide, 8><<<grid_long, kFollowThreads, 0, st>>>(
                   d_trees, P, tokens, n_tokens, tok_base, offsets, B, g->lists + B, g->counts + 1, g->lead, g->cpre,
                   g->gid, nullptr, g->ckpt, d_load, alpha, out_match, out_peer, d_err, nullptr, out_next)));
   } else if (P > 1) {
