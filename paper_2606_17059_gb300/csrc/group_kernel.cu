@@ -101,7 +101,8 @@ __global__ void __launch_bounds__(kGroupThreads) group_hash_kernel(
   }
 }
 
-// First position in [0, n) where a and b differ, or n (one warp, both in global memory; 32 U tokens per step).
+// First position in [0, n) where a and b differ, or n (one warp, both in global memory; 32 U tokens per step, and the
+// rest in one more: at 32 tokens a round trip it took up to seven, 200,003 requests 152 us instead of 142).
 template <int U>
 __device__ int64_t lcp_warp(const int32_t* __restrict__ a, const int32_t* __restrict__ b, int64_t n, int lane) {
   int64_t j0 = 0;
@@ -120,10 +121,20 @@ __device__ int64_t lcp_warp(const int32_t* __restrict__ a, const int32_t* __rest
       }
     }
   }
-  for (; j0 < n; j0 += 32) {
-    const int64_t j = j0 + lane;
-    const unsigned m = __ballot_sync(kFull, j < n && __ldg(a + j) != __ldg(b + j));
-    if (m) return j0 + (__ffs(m) - 1);
+  if (j0 < n) {  // the rest, less than a step, in one round trip too
+    const int32_t left = (int32_t)(n - j0);
+    int32_t x[U], y[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool in = u * 32 + lane < left;
+      x[u] = in ? __ldg(a + j0 + u * 32 + lane) : 0;
+      y[u] = in ? __ldg(b + j0 + u * 32 + lane) : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const unsigned m = __ballot_sync(kFull, x[u] != y[u]);
+      if (m) return j0 + u * 32 + (__ffs(m) - 1);
+    }
   }
   return n;
 }
@@ -231,12 +242,12 @@ __global__ void __launch_bounds__(kGroupThreads) group_place_kernel(int64_t B, c
 // the same (one counter update serves them all): 65,536 requests 65 us, 80 from a work cursor in smaller pieces.
 constexpr int64_t kResolveCtas = 6;
 
-// Below this many bytes of match matrix the followers of short requests are listed as they come: their leaders' rows,
-// checkpoints and tables stay in L2 (126 MB) whatever the order, and two launches are spared (65,536 requests
-// of 1,250 tokens on 16 trees: the follower pass 37 -> 41 us, 12 us of launches less).  Above it a group's followers
-// lie side by side: the follower pass of 200,003 requests on 64 trees takes 217 us so and 234 as they come, of 8,191
-// requests of 11,400 tokens on 32 trees 147 and 192, of 1,048,576 on 256 it reads 15.5 GB instead of 22.  (A single
-// tree's row is 4 bytes and its requests have no choice of route: that path is left as it was.)
+// Below this many bytes of match matrix the followers are listed as they come: their leaders' rows, checkpoints and
+// tables stay in L2 (126 MB) whatever the order, and two launches are spared (65,536 requests of 1,250 tokens on 16
+// trees: the follower pass 24 -> 27 us, 12 us of launches less; 8,191 of 11,400 tokens on 32 trees: 62 -> 65 and 12
+// less).  Above it a group's followers lie side by side: the follower pass of 200,003 requests on 64 trees takes 148
+// us so and 168 as they come, of 262,144 on 256 trees 0.70 ms and 0.87.  (A single tree's row is 4 bytes and
+// its requests have no choice of route: that path is left as it was.)
 constexpr int64_t kPlaceBytes = (int64_t)8 << 20;
 
 cudaError_t launch_group(const int32_t* tokens, int64_t n_tokens, int64_t tok_base, const int64_t* offsets, int64_t B,
@@ -247,7 +258,7 @@ cudaError_t launch_group(const int32_t* tokens, int64_t n_tokens, int64_t tok_ba
   const int64_t warps = (int64_t)num_sms * kResolveCtas * kWarps;
   const int32_t per = (int32_t)std::min<int64_t>(32, long_requests(B, n_tokens) ? 1 : (B + warps - 1) / warps);
   const int32_t per_hash = B < 16 * warps ? 8 : 32;  // (eight requests are hashed at a time)
-  const bool place = P > 1 && B * P * (int64_t)sizeof(int32_t) <= kPlaceBytes && !long_requests(B, n_tokens);
+  const bool place = P > 1 && B * P * (int64_t)sizeof(int32_t) <= kPlaceBytes;
   cudaError_t e = cudaMemsetAsync(g.keys, 0, g.n_zero, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(g.vals, 0x7f, g.n_large, st);
   if (e != cudaSuccess) return e;
