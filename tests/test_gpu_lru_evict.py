@@ -88,3 +88,21 @@ def test_eviction_of_large_tables(fan, inner, kids):
         reqs = [list(rng.choice(seqs)) for _ in range(40)]
         assert _access(r, 0, reqs, t).tolist() == [o.access(s, t) for s in reqs]
         _evict_both(r, o, 25)
+
+
+def test_accesses_that_end_around_the_steps_of_a_compare():
+    """Edges left, or followed to the end, after every count of tokens around 32, 256, 512 and 1,024."""
+    rng = random.Random(11)
+    edges = [n + d for n in (32, 256, 512, 544, 768, 1024, 1056) for d in (-1, 0, 1)]
+    base = [rng.randrange(1000) for _ in range(1100)]
+    r, o = g.Router(1), LRUTrie()
+    g.p2p_lru_enable(r.handle, 0)
+    seqs = [base, base[:512] + [2000, 1]]
+    _insert(r, 0, seqs, 1)
+    for s in seqs:
+        o.insert(s, 1)
+    for t, k in enumerate(edges, 2):
+        for reqs in ([base[:k] + [3000]], [base[:k]]):
+            assert _access(r, 0, reqs, t).tolist() == [o.access(s, t) for s in reqs]
+    assert same_snapshot(r.download(0), _oracle_export(o))
+    _evict_both(r, o, 40)
