@@ -145,7 +145,9 @@ __device__ int64_t lcp_warp(const int32_t* __restrict__ a, const int32_t* __rest
 // each follower takes its rank in its group (fcnt[leader] counts them; the rank goes to slot_of[b]) and
 // group_ranges_kernel and group_place_kernel make the list.  A leader with followers gets the smallest of their common
 // prefixes in cmin and, while rows last, a checkpoint row in gid (one update per distinct leader of the warp's
-// followers).  U: 16 for long requests, whose longest compares bound the kernel, else 8 (more resident warps).
+// followers).  U: 24 for long requests, whose longest compares bound the kernel (8,191 of 11,400 tokens 65 us; 16: 70, 32:
+// 75), else 8 and more resident warps (200,003 of 1,250 tokens 142 us; 16: 148) -- but 16 beside a delta, whose
+// kernels leave room for few warps (262,144 requests 0.43 ms; 8: 0.53).
 template <int U>
 __global__ void __launch_bounds__(kGroupThreads) group_resolve_kernel(
     const int32_t* __restrict__ tokens, int64_t n_tokens, int64_t tok_base, const int64_t* __restrict__ offsets,
@@ -251,7 +253,7 @@ constexpr int64_t kResolveCtas = 6;
 constexpr int64_t kPlaceBytes = (int64_t)8 << 20;
 
 cudaError_t launch_group(const int32_t* tokens, int64_t n_tokens, int64_t tok_base, const int64_t* offsets, int64_t B,
-                         int32_t P, const GroupScratch& g, int num_sms, cudaStream_t st, int* launched) {
+                         int32_t P, const GroupScratch& g, bool beside, int num_sms, cudaStream_t st, int* launched) {
   *launched = 0;
   if (B <= 0) return cudaSuccess;
   constexpr int kWarps = kGroupThreads / 32;
@@ -268,7 +270,9 @@ cudaError_t launch_group(const int32_t* tokens, int64_t n_tokens, int64_t tok_ba
   P2P_TIMED(K_GROUP_HASH, st,
             (group_hash_kernel<<<grid_for(B, (int64_t)kWarps * per_hash), kGroupThreads, 0, st>>>(
                 tokens, n_tokens, tok_base, offsets, B, per_hash, g.keys, g.vals, g.bits, g.slot_of)));
-  const auto resolve = long_requests(B, n_tokens) ? group_resolve_kernel<16> : group_resolve_kernel<8>;
+  const auto resolve = long_requests(B, n_tokens) ? group_resolve_kernel<24>
+                       : beside                   ? group_resolve_kernel<16>
+                                                  : group_resolve_kernel<8>;
   P2P_TIMED(K_GROUP_RESOLVE, st,
             (resolve<<<grid_for(B, (int64_t)kWarps * per), kGroupThreads, 0, st>>>(
                 tokens, n_tokens, tok_base, offsets, B, per, place, g.vals, g.slot_of, g.lead, g.cpre, g.lists,

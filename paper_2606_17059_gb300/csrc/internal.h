@@ -164,8 +164,9 @@ inline __host__ __device__ int32_t group_row(int32_t gid) { return gid == kNoRow
 // Requests of a staging window (of route_kernel.cu's staged pass) or longer on average.
 constexpr int kSlotTokens = 4096;  // tokens of a request kept in shared memory (16 KB per slot)
 inline bool long_requests(int64_t B, int64_t n_tokens) { return n_tokens >= B * (int64_t)kSlotTokens; }
+// beside: the launch runs alongside a delta's kernels, which leave it few warps.
 cudaError_t launch_group(const int32_t* tokens, int64_t n_tokens, int64_t tok_base, const int64_t* offsets, int64_t B,
-                         int32_t P, const GroupScratch& g, int num_sms, cudaStream_t st, int* launched);
+                         int32_t P, const GroupScratch& g, bool beside, int num_sms, cudaStream_t st, int* launched);
 
 // Staged load words (d_load) carry the load in the low 16 bits and kLoadExcluded for a tree that the
 // decision with excluded trees takes out.

@@ -364,7 +364,7 @@ int route(p2p_router* r, const int32_t* tokens, int64_t n_tokens, int64_t tok_ba
   if (group) {
     CK(group_scratch(r, B, g));
     if (!grouped) {
-      CK(p2p::launch_group(tokens, n_tokens, tok_base, offsets, B, r->P, g, r->num_sms, r->stream, &launched));
+      CK(p2p::launch_group(tokens, n_tokens, tok_base, offsets, B, r->P, g, false, r->num_sms, r->stream, &launched));
       r->launches += launched;
     }
   }
@@ -393,7 +393,7 @@ int launch_prepared(p2p_router* r) {
   CK(group_scratch(r, r->prep.B, g));  // the buffers of prepare_scratch (no allocation)
   CK(cudaStreamWaitEvent(r->grp_stream, r->grp_start, 0));
   int launched = 0;
-  CK(p2p::launch_group(r->prep.tokens, r->prep.n_tokens, 0, r->prep.offsets, r->prep.B, r->P, g, r->num_sms,
+  CK(p2p::launch_group(r->prep.tokens, r->prep.n_tokens, 0, r->prep.offsets, r->prep.B, r->P, g, true, r->num_sms,
                        r->grp_stream, &launched));
   CK(cudaEventRecord(r->grp_done, r->grp_stream));
   r->launches += launched;

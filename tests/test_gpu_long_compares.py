@@ -68,6 +68,14 @@ def test_common_prefixes_around_the_steps():
     r, o = router_from_seqlists(sls), oracle.build_trees(sls)
     tok, off = csr_from_lists(reqs)
     om, op, _ = oracle.route(o, tok, off, [0, 0], 1)
-    m, p = r.route(torch.from_numpy(tok).cuda(), torch.from_numpy(off).cuda(), [0, 0], 1)
+    t, f = torch.from_numpy(tok).cuda(), torch.from_numpy(off).cuda()
+    m, p = r.route(t, f, [0, 0], 1)
     r.sync()
     assert_same_route(m.cpu().numpy(), p.cpu().numpy(), om, op, "common prefixes")
+    # Grouped beside a delta (that leaves the trees as they were).
+    g.p2p_route_prepare(r.handle, t, t.numel(), f, len(reqs))
+    sl = seqlist_from_lists([[7, 7, 7], [7, 7, 7]])
+    r.apply_delta(0, np.array([0, 1], np.int32), sl)
+    m, p = r.route(t, f, [0, 0], 1)
+    r.sync()
+    assert_same_route(m.cpu().numpy(), p.cpu().numpy(), om, op, "grouped beside a delta")
