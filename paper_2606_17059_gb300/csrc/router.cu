@@ -1269,6 +1269,7 @@ constexpr int64_t kPartOps = 16384;
 // kernel's slabs are behind them.
 constexpr int64_t kBulkMaxOps = (int64_t)1 << 24;
 constexpr int32_t kBulkSlabShift = 3;
+constexpr int kBulkGrowths = 16;  // launches of a call after which trees are no longer grown for its bulk rounds
 static int split_trees(p2p_router* r, int32_t peer, const p2p_delta* d, const int64_t* d_pb, int32_t p0, int32_t nt,
                 int64_t n, int32_t& n_blocks, const int32_t*& d_parts) {
   n_blocks = nt;
@@ -1407,7 +1408,6 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
   // ops, as a rule) goes to the delta kernel, whose warps then take smaller slabs.
   p2p::BulkArgs bulk = {};
   bool use_bulk = max_runs <= 2 && n <= kBulkMaxOps;
-  int32_t bulk_grown = 0;
   if (use_bulk) {
     if (ensure(r, r->bulk, p2p::bulk_scratch(n, nt, nullptr, bulk)) != cudaSuccess) {
       (void)cudaGetLastError();
@@ -1472,13 +1472,12 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
       if (t.status & p2p::DELTA_CORRUPT) {
         rc = fail(r, P2P_E_DEVICE, "tree " + std::to_string(p) + " is inconsistent");
       } else if (t.status & p2p::DELTA_NEED_BULK) {
-        // What a bulk round asks for in all: grown to hold it.  It is a bound; should the arenas not reach it, or ask
-        // again and again, the delta kernel goes on alone and asks for what its ops need.
-        const auto most = [](int32_t need, int32_t used) { return std::min(need, INT32_MAX / 2 - used / 2); };
-        t.need_node = most(t.need_node, t.n_node);
-        t.need_child = most(t.need_child, t.n_child);
-        t.need_label = most(t.need_label, t.n_label);
-        if (++bulk_grown > 8 * nt || grow_tree(r, p, true) != P2P_OK) {
+        // What a bulk round asks for in all: grown to hold it.  It is a bound (many requests that bring one new prompt
+        // count it each); should the arenas not reach it, or ask again and again, the delta kernel goes on alone and
+        // asks for what its ops need.
+        const auto reach = [](int32_t need, int32_t used) { return need <= INT32_MAX / 2 - used / 2; };
+        if (!reach(t.need_node, t.n_node) || !reach(t.need_child, t.n_child) || !reach(t.need_label, t.n_label) ||
+            round >= kBulkGrowths || grow_tree(r, p, true) != P2P_OK) {
           use_bulk = false;
           t.status = p2p::DELTA_OK;
           t.need_node = t.need_child = t.need_label = t.need_root = 0;

@@ -164,3 +164,23 @@ def test_edges_left_around_the_lane_spans(n_fill):
         r.apply_delta(0, ops, sl)
         o[0].apply_ops(ops, sl, 0, len(ops))
         assert same_snapshot(r.download(0), o[0].export()), cuts
+
+
+def test_a_round_that_asks_for_more_than_an_arena_can_hold():
+    """Many INSERTs of one long new prompt: a round's bound counts it for each of them (1.15 G tokens, past the arenas'
+    reach), though together they take it once.  The delta kernel applies them without bulk rounds."""
+    n, L = 1100, 1 << 20
+    rng = np.random.default_rng(3)
+    pool = np.concatenate([rng.integers(0, 1000, size=L), np.arange(n)]).astype(np.int32)
+    sb = np.arange(0, 2 * n + 1, 2, dtype=np.int64)
+    so = np.stack([np.zeros(n), L + np.arange(n)], axis=1).astype(np.int64).reshape(-1)
+    sl = np.tile([L, 1], n).astype(np.int32)
+    seqs = wl.SeqList(sb, so, sl, pool)
+    r = router_from_seqlists([seqlist_from_lists([[5]])])
+    r.apply_delta(0, np.zeros(n, np.int32), seqs)
+    st = r.download(0)
+    lens = np.sort(np.asarray(st["label_len"]))
+    assert len(lens) == n + 3 and lens[-1] == L and (lens[1:-1] == 1).all() and int(np.sum(st["term_count"])) == n + 1
+    tok, off = csr_from_lists([pool[:L].tolist() + [3], pool[: L // 2].tolist() + [-1], [5]])
+    gm, _ = route_device(r, tok, off, [0], 1)
+    assert gm.ravel().tolist() == [L + 1, L // 2, 1]
