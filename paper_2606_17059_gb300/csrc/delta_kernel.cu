@@ -1235,7 +1235,8 @@ __global__ void init_ranges_kernel(TreeState* states, int32_t nt, const int64_t*
 
 
 constexpr int kCompactThreads = 512;   // two CTAs per SM: every tree of a 256-tree router at once
-constexpr int kSmallBits = 4;   // tables of at most 16 slots are copied by one thread
+constexpr int kSmallBits = 4;   // tables of at most 16 slots are copied by one lane,
+constexpr int kWarpTabBits = 7; // of at most 128 by one warp, larger ones in units by all warps
 constexpr int kSlotBatch = 4;   // slots of a small table a thread loads before it handles them
 constexpr int kUnitSlots = 256;   // slots of a big table per unit of warp work, at least (unit_slots)
 constexpr int kMaxUnits = 512;    // units of a table
@@ -1330,6 +1331,63 @@ __device__ void compact_nodes_warp(CompactJob& J, CompactShared& S, int32_t cid,
       if (!((used >> j) & 1u)) J.nchild[noff + j] = make_int4(0, 0, 0, 0);
   }
   if (on) J.nnode[cid] = make_int4(size ? noff : 0, make_meta(bits, cnt), rec.z, rec.w);
+}
+
+// Copies the table of node cid (old record rec; more than 2^kSmallBits and at most 2^kWarpTabBits slots), one warp: all
+// loads in flight at once, one reservation of each counter, entries placed by a bit mask in shared memory, so that the
+// new table is written once here too.
+__device__ void compact_table_warp(CompactJob& J, CompactShared& S, int32_t cid, const int4& rec, uint32_t* used, int lane) {
+  constexpr int kSteps = (1 << kWarpTabBits) / 32;
+  const int32_t bits = tab_bits(rec.y), size = 1 << bits;
+  const uint32_t mask = (uint32_t)size - 1;
+  int4 e[kSteps];
+  int32_t cnt = 0, tot = 0;
+#pragma unroll
+  for (int c = 0; c < kSteps; ++c) {
+    e[c] = c * 32 < size ? __ldg(J.child + rec.x + c * 32 + lane) : make_int4(0, 0, 0, 0);
+    cnt += e[c].y >= 1;
+    tot += e[c].y >= 1 && e[c].z >= 0 ? e[c].w : 0;
+  }
+  int32_t incl = cnt, lincl = tot;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t y = __shfl_up_sync(kFull, incl, o), ly = __shfl_up_sync(kFull, lincl, o);
+    if (lane >= o) {
+      incl += y;
+      lincl += ly;
+    }
+  }
+  const int32_t all = __shfl_sync(kFull, incl, 31), all_l = __shfl_sync(kFull, lincl, 31);
+  if (lane < kSteps) used[lane] = 0;
+  int32_t base = 0;
+  bool full = false;
+  if (lane < 3) {
+    const int32_t want = lane == 0 ? all : lane == 1 ? size : all_l;
+    base = want ? atomicAdd(lane == 0 ? &S.node : lane == 1 ? &S.child : &S.label, want) : 0;
+    full = (int64_t)base + want > (lane == 0 ? J.cap_node : lane == 1 ? J.cap_child : J.cap_label);
+    if (full) atomicOr(&S.fail, 1);
+  }
+  if (__any_sync(kFull, full)) return;
+  __syncwarp();
+  int32_t id = __shfl_sync(kFull, base, 0) + incl - cnt, nz = __shfl_sync(kFull, base, 2) + lincl - tot;
+  const int32_t noff = __shfl_sync(kFull, base, 1);
+#pragma unroll
+  for (int c = 0; c < kSteps; ++c) {
+    if (e[c].y < 1) continue;
+    const bool own = e[c].z >= 0;
+    const int32_t z = own ? nz : e[c].z;
+    J.queue[id] = make_int4(e[c].y, e[c].z, z, own ? e[c].w : 0);
+    uint32_t sl = slot_hash(e[c].x, bits);
+    while (atomicOr(&used[sl >> 5], 1u << (sl & 31)) >> (sl & 31) & 1u) sl = (sl + 1) & mask;  // (never full)
+    J.nchild[noff + sl] = make_int4(e[c].x, id, z, e[c].w);
+    ++id;
+    nz += own ? e[c].w : 0;
+  }
+  __syncwarp();
+  for (int32_t j = lane; j < size; j += 32)
+    if (!((used[j >> 5] >> (j & 31)) & 1u)) J.nchild[noff + j] = make_int4(0, 0, 0, 0);
+  if (lane == 0) J.nnode[cid] = make_int4(noff, make_meta(bits, all), rec.z, rec.w);
+  __syncwarp();
 }
 
 // Copies a big table whose units do not fit the level's list, one thread: the new table is zeroed first and probed in
@@ -1443,14 +1501,15 @@ __device__ void compact_range_warp(CompactJob& J, CompactShared& S, const int4& 
 // One cluster of kC CTAs per tree (kC = 1: a CTA): level-synchronous breadth-first copy of the structure from the root.  New ids are
 // handed out level by level, so the nodes of the next level are the ids [end, S.node) and the scratch
 // entry of id c (old id, old and new label offsets, own-arena label length) is written by the parent's
-// copy.  A lane takes each node of the level.  A node whose table has more than 2^kSmallBits slots gets
+// copy.  A lane takes each node of the level.  A node whose table has more than 2^kWarpTabBits slots gets
 // its new table range and record from that lane, and its slots are cut into units (unit_slots) that all
-// warps then zero and fill; smaller tables are copied by the warp's lanes.  A big table's record counts its
+// warps then zero and fill; the others are copied by the warp, those of up to 2^kSmallBits slots a lane each.  A big table's record counts its
 // children from the old record (the live-child count), so no pass has to count them.
 // What bounds it is the chain of round trips of each level and the reservations on the tree's three counters, so a warp
-// makes one of each for its 32 nodes, or for its unit.  Measured (a
-// reservation per table, units of 1,024 slots -> this): one tree of ~50,000 nodes by eight CTAs 194 -> 102 us, a wave of
-// 256 trees 1.70 -> 1.31 ms.
+// makes one of each for its small tables, for a table of up to 128 slots, or for a unit.  Measured (a reservation per
+// table, units of 1,024 slots -> this): one tree of ~50,000 nodes by eight CTAs 194 -> 96 us, a wave of 256 trees of 40,000
+// sequences 1.70 -> 1.19 ms, of 100,000 3.8 -> 3.0 (20.6 with their 10,000 tables of 64 slots a tree as units: past 2,048
+// of them, a thread each).
 //
 // Few trees are compacted by clusters: one tree's levels keep 512 threads busy for long (a tree of ~50,000 nodes
 // 0.61 ms by a CTA), while a wave of 256 trees fills the GPU with a CTA each.  The cluster's counters and units are
@@ -1476,10 +1535,11 @@ template <int kC>
 __global__ void __launch_bounds__(kCompactThreads, kC == 1 ? 2 : 1) compact_kernel(CompactJob* jobs) {
   CompactJob& J = jobs[blockIdx.x / kC];
   __shared__ CompactShared S_own;
+  __shared__ uint32_t s_used[kCompactThreads / 32][(1 << kWarpTabBits) / 32];
   CompactShared& S = *compact_shared<kC>(&S_own);
   const int rank = kC > 1 ? (int)(blockIdx.x % kC) : 0;
   const int lane = threadIdx.x & 31, warp = rank * (kCompactThreads / 32) + (threadIdx.x >> 5);
-  constexpr int kThreads = kCompactThreads * kC, kWarps = kThreads / 32;
+  constexpr int kWarps = kCompactThreads * kC / 32;
   const int thread = rank * kCompactThreads + (int)threadIdx.x;
   if (thread == 0) {
     S.node = 1;
@@ -1492,12 +1552,15 @@ __global__ void __launch_bounds__(kCompactThreads, kC == 1 ? 2 : 1) compact_kern
   compact_sync<kC>();
   int begin = 0, end = 1;
   while (begin < end) {
-    for (int first = begin + thread - lane; first < end; first += kThreads) {
+    // Nodes per warp: few enough that every warp has some.
+    const int per = max(1, min(32, (end - begin + kWarps - 1) / kWarps));
+    for (int first = begin + warp * per; first < end; first += kWarps * per) {
       const int cid = first + lane;
-      bool on = cid < end;
+      bool on = lane < per && cid < end;
       const int4 rec = on ? __ldg(J.node + __ldcg(&J.queue[cid].x)) : make_int4(0, 0, 0, 0);
       const int32_t bits = tab_bits(rec.y);
-      if (on && bits > kSmallBits) {
+      const unsigned mid = __ballot_sync(kFull, on && bits > kSmallBits && bits <= kWarpTabBits);
+      if (on && bits > kWarpTabBits) {
         on = false;
         const int32_t size = 1 << bits, per = unit_slots(bits), nu = (size + per - 1) / per;
         const int u0 = atomicAdd(&S.nunits, nu);
@@ -1515,7 +1578,13 @@ __global__ void __launch_bounds__(kCompactThreads, kC == 1 ? 2 : 1) compact_kern
         }
       }
       __syncwarp();
-      compact_nodes_warp(J, S, cid, rec, on, lane);
+      compact_nodes_warp(J, S, cid, rec, on && bits <= kSmallBits, lane);
+      for (unsigned m = mid; m; m &= m - 1) {
+        const int j = __ffs(m) - 1;
+        const int4 r = make_int4(__shfl_sync(kFull, rec.x, j), __shfl_sync(kFull, rec.y, j), __shfl_sync(kFull, rec.z, j),
+                                 __shfl_sync(kFull, rec.w, j));
+        compact_table_warp(J, S, first + j, r, s_used[threadIdx.x >> 5], lane);
+      }
     }
     compact_sync<kC>();
     const int nunits = min(S.nunits, kUnitCap);
