@@ -46,7 +46,7 @@
 //
 // Measured, the delta of a call (delta_kernel alone -> these rounds and delta_kernel behind them): 16,384 routed
 // requests into 16 trees, most into one, 8.2 -> 0.18 ms; 4,096 requests into one cache trie 2.46 -> 0.12 ms; 300 ops
-// into one tree 189 -> 77 us; 1,024,000 ops on 256 trees of 40,000 sequences 3.58 -> 1.44 ms.
+// into one tree 189 -> 77 us; 1,024,000 ops on 256 trees of 40,000 sequences 3.58 -> 1.37 ms.
 #include "internal.h"
 
 namespace p2p {
@@ -74,7 +74,9 @@ constexpr int kBulkCtasPerSm = 4;   // at most 64 registers a thread (80 and 3 C
 // instead (one round trip an op, where the lane takes one per eight tokens).  16,384 routed requests, four ops a warp:
 // the first resolve launch 8% shorter; a warp of 16 ops or more keeps its 128.
 constexpr int kLaneSpan = 128, kLaneSpanPerOp = 8;
-constexpr int kLaneBits = 5;        // tables up to 32 slots are moved by one lane
+constexpr int kLaneBits = 5;        // tables up to 32 slots are moved by one lane,
+constexpr int kMaskBits = 9;        // up to 512 by one warp with a bit mask of the slots it has filled
+constexpr int kMaskWords = 1 << (kMaskBits - 5);
 constexpr int kMaxProbes = 64;      // of the key and node tables
 constexpr int kMemoProbes = 4;
 constexpr int kMemoWaits = 256;     // looks at a pair another warp compares before the lane's warp compares it too
@@ -447,10 +449,14 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
           atomicAdd(&e->shared, 1u);
           if (what == B_LEAF && !(flags & BF_REVIVE)) {
             const uint32_t rank = atomicAdd(&e->leaves, 1u);
-            // The first leaf under a node puts its table on the list of those that may have to grow.  The root's table
-            // grows between launches only; a leaf past its half waits for that.
-            if (pu != 0) grow = rank == 0;
-            else if (tab_full(tab_bits(nd.y), (int64_t)tab_used(nd.y) + rank + 1)) flags |= BF_LATER;
+            // The leaf that takes a node's table past its half puts it on the list of those to grow.  (The root's table
+            // grows between launches only; a leaf past its half waits for that.)
+            const int32_t bits = tab_bits(nd.y);
+            const int64_t used = (int64_t)tab_used(nd.y) + rank;
+            if (tab_full(bits, used + 1)) {
+              if (pu == 0) flags |= BF_LATER;
+              else grow = rank == 0 || !tab_full(bits, used);
+            }
           }
           if (what == B_REMOVE && g != 0 && gw == 0 && (int64_t)atomicAdd(&e->removals, 1u) > (int64_t)gz - 3)
             flags |= BF_LATER;
@@ -556,6 +562,32 @@ __device__ void move_table_lane(int4* child, int32_t off, int32_t bits, int32_t 
     if (!((used >> t) & 1u)) child[dst + t] = make_int4(0, 0, 0, 0);
 }
 
+// The same for up to 2^kMaskBits slots, one warp, with a bit mask in shared memory.
+__device__ void move_table_mask(int4* child, int32_t off, int32_t bits, int32_t dst, int32_t nb, uint32_t* used, int lane) {
+  const uint32_t mask = (1u << nb) - 1;
+  if (lane < kMaskWords) used[lane] = 0;
+  __syncwarp();
+  for (int32_t t0 = 0; bits && t0 < (1 << bits); t0 += 128) {
+    int4 e[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int32_t t = t0 + c * 32 + lane;
+      e[c] = t < (1 << bits) ? __ldcg(child + off + t) : make_int4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (e[c].y < 1) continue;
+      uint32_t sl = slot_hash(e[c].x, nb);
+      while (atomicOr(&used[sl >> 5], 1u << (sl & 31)) >> (sl & 31) & 1u) sl = (sl + 1) & mask;  // (at most 1/2 taken)
+      child[dst + sl] = e[c];
+    }
+  }
+  __syncwarp();
+  for (int32_t t = lane; t < (1 << nb); t += 32)
+    if (!((used[t >> 5] >> (t & 31)) & 1u)) child[dst + t] = make_int4(0, 0, 0, 0);
+  __syncwarp();
+}
+
 // The same for any size, one warp.
 __device__ void move_table_warp(int4* child, int32_t off, int32_t bits, int32_t dst, int32_t nb, int lane) {
   const uint32_t mask = (1u << nb) - 1;
@@ -584,15 +616,22 @@ __device__ void move_table_warp(int4* child, int32_t off, int32_t bits, int32_t 
   __syncwarp();
 }
 
-// A lane per listed node: if the round's leaves would take its table past 1/2 claimed, it moves to one of at most 1/4
+// A lane per listed node: the round's leaves take its table past 1/2 claimed, so it moves to one of at most 1/4
 // live load (as delta_kernel grows tables), small ones by the lane and larger ones by the warp.  A table that cannot
-// grow (no room in the arena) marks the node's entry, and its leaves wait.
+// grow (no room in the arena) marks the node's entry, and its leaves wait.  (With every node that gets a leaf listed, and
+// tables of 64 slots and more zeroed and filled by compare-and-swap, a step of 1,024,000 ops took 130 us of these
+// launches; now 47.)
 __global__ void __launch_bounds__(kBulkThreads) bulk_grow_kernel(BulkArgs A, int round) {
+  __shared__ uint32_t s_used[kBulkWarps][kMaskWords];
   const int lane = threadIdx.x & 31;
   const int32_t total = A.counts[kBulkRounds + 1 + round];
-  const int32_t stride = (int32_t)gridDim.x * kBulkThreads;
-  for (int32_t b0 = ((int32_t)blockIdx.x * kBulkWarps + (int32_t)(threadIdx.x >> 5)) * 32; b0 < total; b0 += stride) {
-    const bool valid = b0 + lane < total;
+  const int32_t warps = (int32_t)gridDim.x * kBulkWarps;
+  // Nodes per warp: few, since a warp moves its larger tables one after another, but not one, since each warp reserves
+  // its room in a tree's arena.
+  const int32_t per = max(4, min(32, (total + warps - 1) / warps));
+  for (int64_t b0 = (int64_t)((int32_t)blockIdx.x * kBulkWarps + (int32_t)(threadIdx.x >> 5)) * per; b0 < total;
+       b0 += (int64_t)warps * per) {
+    const bool valid = lane < per && b0 + lane < total;
     const int4 gr = valid ? A.grow[b0 + lane] : make_int4(-1, 0, 0, 0);
     const int32_t tree = gr.x, u = gr.y;
     int32_t nb = 0, c0 = 0;
@@ -655,8 +694,11 @@ __global__ void __launch_bounds__(kBulkThreads) bulk_grow_kernel(BulkArgs A, int
     if (nb > 0 && nb <= kLaneBits) move_table_lane(child, rec.x, bits, c0, nb);
     for (unsigned m = __ballot_sync(kFull, nb > kLaneBits); m; m &= m - 1) {
       const int j = __ffs(m) - 1;
-      move_table_warp((int4*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)child, j), __shfl_sync(kFull, rec.x, j),
-                      __shfl_sync(kFull, bits, j), __shfl_sync(kFull, c0, j), __shfl_sync(kFull, nb, j), lane);
+      int4* cj = (int4*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)child, j);
+      const int32_t off = __shfl_sync(kFull, rec.x, j), bj = __shfl_sync(kFull, bits, j), dst = __shfl_sync(kFull, c0, j),
+                    nj = __shfl_sync(kFull, nb, j);
+      if (nj <= kMaskBits) move_table_mask(cj, off, bj, dst, nj, s_used[threadIdx.x >> 5], lane);
+      else move_table_warp(cj, off, bj, dst, nj, lane);
     }
     if (nb > 0) s->node[u] = make_int4(c0, make_meta(nb, rec.z), rec.z, rec.w);
   }

@@ -184,3 +184,26 @@ def test_a_round_that_asks_for_more_than_an_arena_can_hold():
     tok, off = csr_from_lists([pool[:L].tolist() + [3], pool[: L // 2].tolist() + [-1], [5]])
     gm, _ = route_device(r, tok, off, [0], 1)
     assert gm.ravel().tolist() == [L + 1, L // 2, 1]
+
+
+@pytest.mark.parametrize("held,new", [(0, 1), (0, 3), (2, 1), (2, 30), (8, 1), (8, 9), (30, 3), (60, 70), (130, 1), (200, 900), (1000, 1100)])
+def test_tables_that_grow_within_a_round(held, new):
+    """Nodes with `held` children that get `new` leaves in one call (and one with a single one, and a few that are left
+    alone): tables of every size class move, by a lane, by a warp with a bit mask, and by compare-and-swap."""
+    rng = random.Random(held * 31 + new)
+    kids = [rng.sample(range(-(1 << 31), 1 << 31), held + new) for _ in range(6)]
+    base = [[i, 7, c, 1] for i in range(6) for c in kids[i][:held]] + [[i, 7] for i in range(6)]
+    add = [[i, 7, c, 1] for i in range(4) for c in kids[i][held:]] + [[4, 7, kids[4][held], 1]]
+    rng.shuffle(add)
+    r, o = router_from_seqlists([seqlist_from_lists(base)] * 2), oracle.build_trees([seqlist_from_lists(base)] * 2)
+    sl, op = seqlist_from_lists(add + add), np.zeros(2 * len(add), np.int32)
+    pb = np.array([0, len(add), 2 * len(add)], np.int64)
+    assert r.apply_delta(-1, op, sl, pb) == 0
+    reqs = [s[: rng.randint(2, 4)] for s in rng.sample(base + add, min(300, len(base + add)))]
+    tok, off = csr_from_lists(reqs)
+    for p in range(2):
+        o[p].apply_ops(op, sl, int(pb[p]), int(pb[p + 1]))
+        assert same_snapshot(r.download(p), o[p].export()), p
+    gm, gp = route_device(r, tok, off, [0, 0], 1)
+    om, op_, _ = oracle.route(o, tok, off, [0, 0], 1)
+    assert_same_route(gm, gp, om, op_, "grown tables")
