@@ -77,16 +77,20 @@ KERNEL_SOURCE = {
 # differs from the current source is not reported (the kernel changed since it was taken).
 TRAFFIC: dict = {
     "cfg4": {k: dict(v, profile="profiles/traffic_workload4.md") for k, v in {
-        "delta_kernel": {"bytes": 6722955162, "source": "e2ef36bc7089a1f9"},
-        "validate_kernel": {"bytes": 99170202, "source": "e2ef36bc7089a1f9"},
-        "compact_kernel": {"bytes": 10286514944, "source": "e2ef36bc7089a1f9"},
-        "compact_labels_kernel": {"bytes": 24298933760, "source": "e2ef36bc7089a1f9"},
-        "group_hash_kernel": {"bytes": 491484160, "source": "5dbd6a2a3cb8351d"},
-        "group_resolve32_kernel": {"bytes": 9457201050, "source": "5dbd6a2a3cb8351d"},
-        "group_ranges_kernel": {"bytes": 4005018, "source": "5dbd6a2a3cb8351d"},
-        "group_place_kernel": {"bytes": 8143744, "source": "5dbd6a2a3cb8351d"},
-        "lane_kernel<true>": {"bytes": 6151677824, "source": "73d5d75a48fec1cc"},
-        "lane_kernel<false>": {"bytes": 16206268134, "source": "73d5d75a48fec1cc"},
+        "bulk_resolve_kernel": {"bytes": 1329090569, "source": "a715ce49b4ce5629"},
+        "bulk_grow_kernel": {"bytes": 6032316, "source": "a715ce49b4ce5629"},
+        "bulk_apply_kernel": {"bytes": 1294768290, "source": "a715ce49b4ce5629"},
+        "delta_kernel": {"bytes": 140046182, "source": "8685ed8ca885cceb"},
+        "validate_kernel": {"bytes": 108518477, "source": "8685ed8ca885cceb"},
+        "compact_kernel": {"bytes": 10303667456, "source": "8685ed8ca885cceb"},
+        "compact_labels_kernel": {"bytes": 24837504000, "source": "8685ed8ca885cceb"},
+        "group_hash_kernel": {"bytes": 485369267, "source": "3bbb2ca20c911727"},
+        "group_resolve_kernel": {"bytes": 9566132454, "source": "3bbb2ca20c911727"},
+        "group_ranges_kernel": {"bytes": 4062259, "source": "3bbb2ca20c911727"},
+        "group_place_kernel": {"bytes": 8227840, "source": "3bbb2ca20c911727"},
+        "lane_kernel<true>": {"bytes": 6063724314, "source": "0eed343382562327"},
+        "follow_kernel": {"bytes": 14547960499, "source": "0eed343382562327"},
+        "lane_kernel<false>": {"bytes": 52710, "source": "0eed343382562327"},
     }.items()},
 }
 
