@@ -347,7 +347,8 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
         need = true;
         held = false;
       }
-      // A pair of an interned label and a pool run: how much of it is known to be equal.  One lane of the warp at a time
+      // A pair of an interned label and a pool run: how much of it is known to be equal, as far as this op's first run
+      // goes (another op's may start at the same place and be longer).  One lane of the warp at a time
       // takes on a pair that nobody has compared yet, so that a launch's first compares spread over all warps (a
       // warp that took on each of its lanes' pairs had 20 of them to do, one after another, with the others waiting).
       int32_t free_at = -1;
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
               break;
             }
             if (have == key) {
-              const int32_t known = __ldcg(A.memo_vals + s);
+              const int32_t known = min(__ldcg(A.memo_vals + s), q.na - pos);
               if (known == 0 && ++waits < kMemoWaits) {
                 held = true;
               } else if (known >= lim) {

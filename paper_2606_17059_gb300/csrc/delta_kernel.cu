@@ -357,7 +357,8 @@ __device__ int64_t first_diff_arrays(const int32_t* a, const int32_t* b, int64_t
 }
 
 // First j in [from, lim) with lab[j] != q[pos + j], or lim.  Lane k looks at memo entry k, so a lookup is
-// one step.  The sequence side is compared run by run (its first pool run, then the second), so both
+// one step; what it finds holds as far as q's first pool run goes (another op's may start at the same place and be
+// longer).  The sequence side is compared run by run (its first pool run, then the second), so both
 // sides of every compare are contiguous.
 __device__ int64_t first_diff(const int32_t* lab, int32_t loff, const Seq& q, int64_t pos, int64_t from, int64_t lim,
                               int lane, Memo& memo) {
@@ -365,14 +366,15 @@ __device__ int64_t first_diff(const int32_t* lab, int32_t loff, const Seq& q, in
   const unsigned long long gkey = in_a ? global_memo_key(memo, q, loff, pos) : 0ull;
   if (in_a) {
     int32_t skip = 0;
+    const int64_t own = min(lim, q.na - pos);
     if (lane < kMemoSlots) {
       const MemoEntry m = memo.e[lane];
       const int64_t dl = lab - m.lab, ds = (q.a + pos) - m.seq;
-      if (m.lab && dl == ds && dl >= 0 && dl < m.n) skip = (int32_t)min(lim, m.n - dl);
+      if (m.lab && dl == ds && dl >= 0 && dl < m.n) skip = (int32_t)min(own, m.n - dl);
     }
     if (gkey && lane >= kMemoSlots && lane < kMemoSlots + kGlobalMemoProbes) {
       const uint32_t s = (global_memo_slot(gkey, memo.gmask) + (uint32_t)(lane - kMemoSlots)) & memo.gmask;
-      if (__ldcg(memo.gkeys + s) == gkey) skip = (int32_t)min(lim, (int64_t)__ldcg(memo.gvals + s));
+      if (__ldcg(memo.gkeys + s) == gkey) skip = (int32_t)min(own, (int64_t)__ldcg(memo.gvals + s));
     }
     from = max(from, (int64_t)__reduce_max_sync(kFull, (unsigned)skip));
   }
