@@ -362,7 +362,8 @@ __device__ int64_t first_diff_arrays(const int32_t* a, const int32_t* b, int64_t
 // sides of every compare are contiguous.
 __device__ int64_t first_diff(const int32_t* lab, int32_t loff, const Seq& q, int64_t pos, int64_t from, int64_t lim,
                               int lane, Memo& memo) {
-  const bool in_a = pos < q.na;  // q[pos ..] starts in the first pool run, which the memo can describe
+  // q[pos ..] starts in the first pool run, which the memo can describe (scratch holds another sequence soon).
+  const bool in_a = q.pooled && pos < q.na;
   const unsigned long long gkey = in_a ? global_memo_key(memo, q, loff, pos) : 0ull;
   if (in_a) {
     int32_t skip = 0;
@@ -465,7 +466,7 @@ __device__ bool ensure_room(Tree& t, int32_t cur, int4& nd, int32_t extra, int l
 // A shortcut to an anchor, shared by the CTA's warps for one chunk's parallel phase.  Nothing above an
 // anchor changes in that phase, so an op whose first pool run is the run (same address, same tokens) of
 // the op that first reached the anchor, and covers the anchor's position, reaches it by the same path: it
-// may start there.  The first op to reach the anchor claims the entry, writes pos and rec, and publishes
+// may start there.  (Not one gathered into scratch, whose address says nothing of its tokens.)  The first op to reach the anchor claims the entry, writes pos and rec, and publishes
 // seq last; the entry is not written again in the phase.
 struct AnchorEntry {
   const int32_t* seq;  // the first pool run of the op that reached the anchor (NULL: not published)
@@ -478,7 +479,7 @@ struct AnchorEntry {
 // anchor of entry ae.
 __device__ __forceinline__ bool anchor_start(const AnchorEntry* ae, const Seq& q, int lane, int64_t& pos, int4& rec) {
   int ok = 0;
-  if (lane == 0 && ae) {
+  if (lane == 0 && ae && q.pooled) {
     const int32_t* sp = *(const int32_t* const volatile*)&ae->seq;
     ok = sp == q.a && sp != nullptr;
   }
@@ -493,7 +494,7 @@ __device__ __forceinline__ bool anchor_start(const AnchorEntry* ae, const Seq& q
 // Publishes the shortcut for the op that first reached its anchor (at pos, record rec), if the entry is free
 // and the op's first pool run covers the anchor's position.
 __device__ __forceinline__ void anchor_publish(AnchorEntry* ae, const Seq& q, int64_t pos, const int4& rec, int lane) {
-  if (lane == 0 && ae && pos <= q.na && atomicCAS(&ae->claim, 0, 1) == 0) {
+  if (lane == 0 && ae && q.pooled && pos <= q.na && atomicCAS(&ae->claim, 0, 1) == 0) {
     ae->pos = (int32_t)pos;
     ae->rec = rec;
     __threadfence_block();

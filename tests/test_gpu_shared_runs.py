@@ -64,3 +64,37 @@ def test_runs_of_one_start_and_several_lengths(cut, order, alone):
     op = np.array(ops, np.int32)
     assert r.apply_delta(0, op, q) == o[0].apply_ops(op, q)
     assert same_snapshot(r.download(0), o[0].export())
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_sequences_of_many_runs_share_nothing_by_their_place(seed):
+    """Ops of three runs are put together in scratch, where one sequence after another has the same place: what the
+    last one matched says nothing of the next.  They differ early or late within a label, below a node of few
+    children and of many (which the kernel starts from directly)."""
+    rng = np.random.default_rng(seed)
+    L, n = 200, 40
+    labels = [np.concatenate([[5000 + k], rng.integers(0, 50, L - 1)]) for k in range(n)]
+    held, seqs, ops = [], [], []
+    for k in range(n):
+        held += [np.concatenate([labels[k], [7000 + j, 1, 2]]) for j in range(2 if k % 2 else 70)]
+        for j in range(4):
+            off = labels[k].copy()
+            off[[1, 70, 130, L - 1][j]] += 1000
+            seqs += [np.concatenate([labels[k], [9000 + j]]), np.concatenate([off, [7000 + j, 1, 2]])]
+            ops += [0, int(rng.integers(2))]
+        seqs += [held[-1], np.concatenate([labels[k][: L - 1], [6000, 7000]])]
+        ops += [1, 0]
+    sb, so, sl, pool = [0], [], [], []
+    for s in seqs:
+        a, b = sorted(rng.integers(0, len(s) + 1, 2))
+        for lo, hi in ((0, a), (a, b), (b, len(s))):
+            so.append(len(pool))
+            sl.append(hi - lo)
+            pool.extend(s[lo:hi])
+        sb.append(len(so))
+    q = wl.SeqList(np.array(sb, np.int64), np.array(so, np.int64), np.array(sl, np.int32), np.array(pool, np.int32))
+    sls = [seqlist_from_lists([x.tolist() for x in held])]
+    r, o = router_from_seqlists(sls), oracle.build_trees(sls)
+    op = np.array(ops, np.int32)
+    assert r.apply_delta(0, op, q) == o[0].apply_ops(op, q)
+    assert same_snapshot(r.download(0), o[0].export())
