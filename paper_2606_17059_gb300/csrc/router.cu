@@ -287,6 +287,7 @@ int fail(p2p_router* r, int code, const std::string& msg) {
 }
 
 int cuda_fail(p2p_router* r, cudaError_t e, const char* what) {
+  (void)cudaGetLastError();  // reported here: the launch of a later call must not find it again
   return fail(r, P2P_E_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
@@ -296,8 +297,11 @@ int cuda_fail(p2p_router* r, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(r, e_, #call); \
   } while (0)
 
+// (Without memory, the call may go on some other way: the runtime's last error is not left for its next launch to find.)
 cudaError_t dalloc(p2p_router* r, void** p, size_t bytes) {
-  return cudaMallocFromPoolAsync(p, bytes ? bytes : 16, r->pool, r->stream);
+  const cudaError_t e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, r->pool, r->stream);
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e;
 }
 void dfree(p2p_router* r, void* p) {
   if (p) cudaFreeAsync(p, r->stream);
@@ -670,10 +674,7 @@ int upload_flat(p2p_router* r, int32_t peer, const p2p_flat_tree* t) {
                 sp_label = clamp_i32(cap_label + (int64_t)cap_label / 4);
   if (sp.cap_node < sp_node || sp.cap_child < sp_child || sp.cap_label < sp_label) {
     free_tree_arrays(r, sp);
-    if (alloc_tree_arrays(r, sp, sp_node, sp_child, sp_label) != cudaSuccess) {
-      sp = TreeState{};
-      (void)cudaGetLastError();
-    }
+    if (alloc_tree_arrays(r, sp, sp_node, sp_child, sp_label) != cudaSuccess) sp = TreeState{};
   }
   CK(cudaMemcpyAsync(nt.node, node.data(), (size_t)NN * sizeof(int4), cudaMemcpyHostToDevice, r->stream));
   if (slots) CK(cudaMemsetAsync(nt.child, 0, (size_t)slots * sizeof(int4), r->stream));
@@ -1035,6 +1036,7 @@ int p2p_router_create(int32_t P, p2p_router** out) {
   p2p_router* r = new p2p_router();
   r->P = P;
   auto bail = [&](int code) {
+    (void)cudaGetLastError();
     p2p::set_global_error(r->err);
     p2p_router_destroy(r);
     return code;
@@ -1410,7 +1412,6 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
   bool use_bulk = max_runs <= 2 && n <= kBulkMaxOps;
   if (use_bulk) {
     if (ensure(r, r->bulk, p2p::bulk_scratch(n, nt, nullptr, bulk)) != cudaSuccess) {
-      (void)cudaGetLastError();
       use_bulk = false;
     } else {
       p2p::bulk_scratch(n, nt, r->bulk.p, bulk);

@@ -1,0 +1,79 @@
+"""Allocations that fail while a delta call grows a tree: the router's host code over a fake CUDA runtime (host/), whose
+launchers check the arrays they are given."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_2606_17059_gb300 as g
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2606_17059_gb300", "csrc")
+CUDA = os.path.dirname(os.path.dirname(g._build.NVCC)) if os.sep in g._build.NVCC else "/usr/local/cuda"
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("host") / "libhost.so")
+    cmd = ["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-I", os.path.join(CUDA, "include"), "-I", CSRC, "-I",
+           os.path.join(ROOT, "include"), "-o", so, "-x", "c++", os.path.join(CSRC, "router.cu"),
+           os.path.join(CSRC, "snapshot.cpp"), os.path.join(ROOT, "tests", "host", "fake_cuda.cpp")]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-3000:]
+    L = ctypes.CDLL(so)
+    L.fake_fail_sizes.argtypes = [ctypes.c_int64, ctypes.c_int64]
+    L.p2p_last_error.restype = ctypes.c_char_p
+    return L
+
+
+class Host:
+    """A router of the fake library with two trees; one INSERT of a token as the delta."""
+
+    def __init__(self, lib):
+        self.lib, self.h = lib, ctypes.c_void_p()
+        assert lib.p2p_router_create(2, ctypes.byref(self.h)) == 0
+        self.bad = lib.fake_bad_arrays()
+
+    def delta(self, n=64):
+        op, sb, so = np.zeros(n, np.int32), np.arange(n + 1, dtype=np.int64), np.zeros(n, np.int64)
+        sl, pool = np.ones(n, np.int32), np.array([7], np.int32)
+        a = lambda x: x.ctypes.data
+        d = g.Delta(a(op), g.Seqs(n, a(sb), a(so), a(sl), a(pool), n, 1), None, g.P2P_MEM_HOST)
+        self.keep = (op, sb, so, sl, pool)
+        return self.lib.p2p_tree_apply_delta(self.h, 0, ctypes.byref(d), None)
+
+    def lru_insert(self, n=64):
+        tok, off = np.full(n, 7, np.int32), np.arange(n + 1, dtype=np.int64)
+        return self.lib.p2p_lru_insert(self.h, 0, ctypes.c_void_p(tok.ctypes.data), ctypes.c_int64(n),
+                                       ctypes.c_void_p(off.ctypes.data), ctypes.c_int64(n), ctypes.c_int64(1))
+
+    def close(self):
+        assert self.lib.fake_bad_arrays() == self.bad
+        self.lib.p2p_router_destroy(self.h)
+
+
+# What the bulk rounds find no room for: nodes, slots, label tokens.
+@pytest.mark.parametrize("ask", [(1 << 20, 0, 0), (0, 1 << 20, 0), (0, 0, 1 << 24), (1 << 20, 1 << 20, 1 << 24)])
+def test_a_tree_that_cannot_grow_for_the_bulk_rounds(lib, ask):
+    """The call goes on with the delta kernel alone, on the arrays as they were."""
+    r = Host(lib)
+    assert r.delta() == 0
+    bulk, delta = lib.fake_bulk_calls(), lib.fake_delta_calls()
+    lib.fake_ask(*ask)
+    lib.fake_fail_sizes(1 << 20, 1 << 62)
+    rc = r.delta()
+    lib.fake_fail_sizes(0, 0)
+    assert rc == 0, lib.p2p_last_error(r.h)
+    assert lib.fake_bulk_calls() - bulk == 1 and lib.fake_delta_calls() - delta == 2
+    r.close()
+
+
+def test_a_failed_allocation_is_not_reported_by_a_later_call(lib):
+    r = Host(lib)
+    lib.fake_fail_sizes(1 << 22, 1 << 62)
+    assert r.delta(1 << 20) != 0  # no room for its op arrays
+    lib.fake_fail_sizes(0, 0)
+    assert r.delta() == 0, lib.p2p_last_error(r.h)
+    r.close()
