@@ -769,7 +769,8 @@ int regrow_root(p2p_router* r, int32_t p, int64_t extra = 0) {
 }
 
 // Grows the arenas of tree p so that the largest op that did not fit does (at least doubling them), or, with
-// whole, so that need_* -- the room the rest of the call may take -- fits with an eighth to spare.
+// whole, so that need_* -- the room the rest of the call may take -- fits with an eighth to spare.  Every array is
+// allocated before one is replaced: without memory the tree stays as it was.
 int grow_tree(p2p_router* r, int32_t p, bool whole = false) {
   TreeState& t = r->hs[(size_t)p];
   auto newcap = [whole](int64_t cap, int64_t used, int64_t need) -> int64_t {
@@ -790,7 +791,9 @@ int grow_tree(p2p_router* r, int32_t p, bool whole = false) {
   int4* nn = t.node;
   int4* nc = t.child;
   int32_t* nl = t.label;
+  uint32_t* ns = t.stamp;  // an LRU tree's stamps follow its node slots; new slots start at time 0
   cudaError_t e = cudaSuccess;
+  if (grow_n && t.stamp) e = dalloc(r, (void**)&ns, (size_t)cn * sizeof(uint32_t));
   if (grow_n && e == cudaSuccess) e = dalloc(r, (void**)&nn, (size_t)cn * sizeof(int4));
   if (grow_c && e == cudaSuccess) e = dalloc(r, (void**)&nc, (size_t)cc * sizeof(int4));
   if (grow_l && e == cudaSuccess) e = dalloc(r, (void**)&nl, (size_t)cl * sizeof(int32_t));
@@ -798,18 +801,16 @@ int grow_tree(p2p_router* r, int32_t p, bool whole = false) {
     if (nn != t.node) dfree(r, nn);
     if (nc != t.child) dfree(r, nc);
     if (nl != t.label) dfree(r, nl);
+    if (ns != t.stamp) dfree(r, ns);
     return fail(r, P2P_E_NOMEM, std::string("growing a tree: ") + cudaGetErrorString(e));
   }
   if (grow_n) {
     CK(cudaMemcpyAsync(nn, t.node, (size_t)t.n_node * sizeof(int4), cudaMemcpyDeviceToDevice, r->stream));
     dfree(r, t.node);
-    if (t.stamp) {  // an LRU tree's stamps follow its node slots; new slots start at time 0
-      uint32_t* ns = nullptr;
-      CK(dalloc(r, (void**)&ns, (size_t)cn * sizeof(uint32_t)));
+    if (t.stamp) {
       CK(cudaMemcpyAsync(ns, t.stamp, (size_t)t.n_node * sizeof(uint32_t), cudaMemcpyDeviceToDevice, r->stream));
       CK(cudaMemsetAsync(ns + t.n_node, 0, (size_t)(cn - t.n_node) * sizeof(uint32_t), r->stream));
       dfree(r, t.stamp);
-      t.stamp = ns;
     }
   }
   if (grow_c) {
@@ -823,6 +824,7 @@ int grow_tree(p2p_router* r, int32_t p, bool whole = false) {
   t.node = nn;
   t.child = nc;
   t.label = nl;
+  t.stamp = ns;
   t.cap_node = (int32_t)cn;
   t.cap_child = (int32_t)cc;
   t.cap_label = (int32_t)cl;

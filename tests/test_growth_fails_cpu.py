@@ -70,6 +70,21 @@ def test_a_tree_that_cannot_grow_for_the_bulk_rounds(lib, ask):
     r.close()
 
 
+@pytest.mark.parametrize("nth", [1, 2, 3, 4, 5])
+def test_a_growth_that_fails_half_way_changes_nothing(lib, nth):
+    """An LRU tree's growth allocates nodes, slots, labels and stamps; whichever fails, the arrays stay as they were."""
+    r = Host(lib)
+    assert lib.p2p_lru_enable(r.h, 0) == 0 and r.lru_insert() == 0
+    lib.fake_ask(1 << 16, 1 << 16, 1 << 20)
+    lib.fake_fail_sizes(0, 0)
+    lib.fake_fail_after(nth)
+    rc = r.lru_insert()
+    lib.fake_fail_after(0)
+    assert rc == 0, lib.p2p_last_error(r.h)
+    assert r.lru_insert() == 0
+    r.close()
+
+
 def test_a_failed_allocation_is_not_reported_by_a_later_call(lib):
     r = Host(lib)
     lib.fake_fail_sizes(1 << 22, 1 << 62)
