@@ -31,8 +31,8 @@
 //   bulk_apply_kernel    an op that won its places, and whose node nobody shares if it needs it alone (and no op of
 //                        smaller index needs it alone too), is applied: room for the warp's ops with one reservation
 //                        per tree and arena, labels copied by the whole warp, slots, records and counts by the op's
-//                        lane.  The others go to the next round's list.  A tree whose arenas may not hold what the
-//                        round asks for is grown by the host first: its ops that need room all wait.
+//                        lane.  The others go to the next round's list, and with them those that found no room: the
+//                        host then grows their tree, by what the round's ops that could go came to.
 // Of the removals under a node with z children that stores nothing only the first z - 2 to arrive go in one round, so
 // no node is left with fewer than 2 children unless it is folded.  A leaf's record and what hangs from it are
 // changed only by ops that hold its place.  Ops on one sequence always name the same place first, the one with the
@@ -427,7 +427,6 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
         }
       }
     }
-    int3 want = make_int3(0, 0, 0);
     bool grow = false;
     int4 mine_grow = make_int4(0, 0, 0, 0);
     if (valid) {
@@ -500,11 +499,7 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
         flags |= BF_MORE;
         out[2] = make_int4(key2, key3, ent_u, ent_y);
         out[3] = make_int4(gg, ggpos, 0, 0);
-        if (what == B_FOLD) want = make_int3(0, 0, ppos - ggpos + y.w);
       }
-      // At most this much room.
-      if (what == B_LEAF) want = make_int3(1, 0, q.n - ppos);
-      if (what == B_SPLIT) want = make_int3(2, 1 << kMinTabBits, q.n - ppos - k);
       out[0] = make_int4(what | flags | tree << kTreeShift, pu, tok, slot);
       out[1] = make_int4(key, arg, ent, ppos);
       if (grow) mine_grow = make_int4(tree, pu, ent, 0);
@@ -517,22 +512,6 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
       if (lane == 0) at = atomicAdd(&A.counts[kBulkRounds + 1 + round], __popc(gm));
       at = __shfl_sync(kFull, at, 0);
       if (grow) A.grow[at + __popc(gm & ((1u << lane) - 1))] = mine_grow;
-    }
-    // The room the round may take, once per tree and warp.
-    for (unsigned m = __ballot_sync(kFull, want.x | want.y | want.z); m;) {
-      const int32_t t = __shfl_sync(kFull, tree, __ffs(m) - 1);
-      const bool mine = (want.x | want.y | want.z) && tree == t;
-      m &= ~__ballot_sync(kFull, mine);
-      unsigned n = mine ? want.x : 0, c = mine ? want.y : 0;
-      unsigned long long l = mine ? want.z : 0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        n += __shfl_xor_sync(kFull, n, o);
-        c += __shfl_xor_sync(kFull, c, o);
-        l += __shfl_xor_sync(kFull, l, o);
-      }
-      const unsigned long long v = lane == 0 ? n : lane == 1 ? c : l;
-      if (lane < 3 && v) atomicAdd(&A.want[((int64_t)round * A.n_trees + t) * 3 + lane], v);
     }
   }
 }
@@ -874,8 +853,8 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
       want_n = want_l > 0 ? 2 : 1;
       want_c = 1 << kMinTabBits;
     }
-    // Room, once per tree and warp.  Everything the round may take fits (an addition then cannot go too far, so none
-    // has to be taken back), or the tree's ops that need room all wait until the host has grown it.
+    // Room, once per tree and warp.  Tickets count on past an arena's end, so none has to be taken back and no two get
+    // the same room; an op past the end waits until the host has grown the tree, by what the tickets came to.
     int32_t n0 = 0, c0 = 0, l0 = 0;
     for (unsigned m = __ballot_sync(kFull, want_n | want_c | want_l); m;) {
       const int32_t t = __shfl_sync(kFull, tree, __ffs(m) - 1);
@@ -892,24 +871,23 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
       const int32_t tn = __shfl_sync(kFull, sn, 31), tc = __shfl_sync(kFull, sc, 31);
       const int64_t tl = __shfl_sync(kFull, sl, 31);
       TreeState* ts = A.states + t;
-      int32_t r = 0;
-      bool fits = true;
-      if (lane < 3) {
-        const unsigned long long most = A.want[((int64_t)round * A.n_trees + t) * 3 + lane];
-        const int32_t cap = lane == 0 ? ts->cap_node : lane == 1 ? ts->cap_child : ts->cap_label;
-        fits = most == 0 || (unsigned long long)A.base[3 * t + lane] + most <= (unsigned long long)cap;
-        if (!fits) {
-          atomicOr(&ts->status, DELTA_NEED_SPACE | DELTA_NEED_BULK);
-          atomicMax(lane == 0 ? &ts->need_node : lane == 1 ? &ts->need_child : &ts->need_label,
-                    (int32_t)min(most, (unsigned long long)INT32_MAX));
-        }
+      const int64_t k = lane == 0 ? tn : lane == 1 ? tc : lane == 2 ? tl : 0;
+      int64_t at = 0, cap = 0;
+      if (k) {
+        at = A.base[3 * t + lane] + (int64_t)atomicAdd(&A.taken[((int64_t)round * A.n_trees + t) * 3 + lane], (unsigned long long)k);
+        cap = lane == 0 ? ts->cap_node : lane == 1 ? ts->cap_child : ts->cap_label;
       }
-      const bool ok = __all_sync(kFull, fits);
-      if (ok && lane < 3) {
-        const int32_t k = lane == 0 ? tn : lane == 1 ? tc : (int32_t)tl;
-        if (k) r = atomicAdd(lane == 0 ? &ts->n_node : lane == 1 ? &ts->n_child : &ts->n_label, k);
+      const bool ok = __all_sync(kFull, at + k <= cap);
+      if (k && at + k <= cap) {
+        atomicMax(lane == 0 ? &ts->n_node : lane == 1 ? &ts->n_child : &ts->n_label, (int32_t)(at + k));
+        if (!ok) add64(lane == 0 ? &ts->dead_nodes : lane == 1 ? &ts->stale_child : &ts->stale_label, k);
+      } else if (k) {
+        atomicOr(&ts->status, DELTA_NEED_SPACE | DELTA_NEED_BULK);
+        atomicMax(lane == 0 ? &ts->need_node : lane == 1 ? &ts->need_child : &ts->need_label,
+                  (int32_t)min(at + k - cap, (int64_t)INT32_MAX));
       }
-      const int32_t bn = __shfl_sync(kFull, r, 0), bc = __shfl_sync(kFull, r, 1), bl = __shfl_sync(kFull, r, 2);
+      const int32_t bn = __shfl_sync(kFull, (int32_t)at, 0), bc = __shfl_sync(kFull, (int32_t)at, 1),
+                    bl = __shfl_sync(kFull, (int32_t)at, 2);
       if (mine) {
         go = ok;
         n0 = bn + sn - want_n;
@@ -1077,7 +1055,7 @@ size_t bulk_scratch(int64_t n, int32_t n_trees, void* base, BulkArgs& A) {
   A.tab.key_mask = (uint32_t)(keys - 1);
   A.tab.nodes = static_cast<BulkNode*>(take((size_t)nodes * sizeof(BulkNode)));
   A.tab.node_mask = (uint32_t)(nodes - 1);
-  A.want = static_cast<unsigned long long*>(take((size_t)kBulkRounds * n_trees * 3 * sizeof(unsigned long long)));
+  A.taken = static_cast<unsigned long long*>(take((size_t)kBulkRounds * n_trees * 3 * sizeof(unsigned long long)));
   A.counts = static_cast<int32_t*>(take((2 * kBulkRounds + 1) * sizeof(int32_t)));
   A.n_zero = at;  // cleared by the launch up to here
   A.base = static_cast<int32_t*>(take((size_t)n_trees * 3 * sizeof(int32_t)));

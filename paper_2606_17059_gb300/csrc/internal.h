@@ -81,7 +81,7 @@ struct TreeState {
   int64_t stale_child, stale_label, dead_nodes;  // unreachable arena space
 };
 
-// DELTA_NEED_BULK: the room asked for (need_*) is what a bulk round takes in all, not the largest op.
+// DELTA_NEED_BULK: need_* is how far past the arenas' ends a bulk round's ops came, not the largest op.
 enum { DELTA_OK = 0, DELTA_NEED_SPACE = 1, DELTA_CORRUPT = 2, DELTA_NEED_BULK = 4 };
 
 // Delta kernel: ops are bucketed by a hash of their first token (kDeltaBuckets per tree); one CTA of
@@ -244,7 +244,7 @@ struct BulkArgs {
   int32_t* lists;  // [2n]: the op indices of odd and even rounds
   int4* grow;      // [n]: (tree, node, node entry) of the tables that may have to grow in a round
   int32_t* base;   // [3 * n_trees]: the arenas' use ahead of the round's ops
-  unsigned long long* want;  // [kBulkRounds * n_trees * 3]: nodes, slots and tokens a round may take, at most
+  unsigned long long* taken;  // [kBulkRounds * n_trees * 3]: nodes, slots and tokens a round's ops have asked for
   int32_t* counts;           // [2 * kBulkRounds + 1]: list sizes by round, then the sizes of its grow lists
   size_t n_zero;             // bytes from tab.keys on that the launch clears
 };

@@ -1475,12 +1475,18 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
       if (t.status & p2p::DELTA_CORRUPT) {
         rc = fail(r, P2P_E_DEVICE, "tree " + std::to_string(p) + " is inconsistent");
       } else if (t.status & p2p::DELTA_NEED_BULK) {
-        // What a bulk round asks for in all: grown to hold it.  It is a bound (many requests that bring one new prompt
-        // count it each); should the arenas not reach it, or ask again and again, the delta kernel goes on alone and
-        // asks for what its ops need.
-        const auto reach = [](int32_t need, int32_t used) { return need <= INT32_MAX / 2 - used / 2; };
-        if (!reach(t.need_node, t.n_node) || !reach(t.need_child, t.n_child) || !reach(t.need_label, t.n_label) ||
-            round >= kBulkGrowths || grow_tree(r, p, true) != P2P_OK) {
+        // Grown by what the round lacked (each op that could go counted once) and a quarter, so that what the later ops
+        // bring does not ask again and again.  Should that not be had, or not be enough, the delta kernel goes on alone
+        // and asks for what its ops need.
+        const auto lacks = [](int32_t past, int32_t cap, int32_t used) {
+          if (!past) return 0;
+          const int64_t least = (int64_t)past + cap - used, room = INT32_MAX - (int64_t)used;
+          return (int32_t)std::min<int64_t>(std::max(least, std::min(least + cap / 4, room)), INT32_MAX);
+        };
+        t.need_node = lacks(t.need_node, t.cap_node, t.n_node);
+        t.need_child = lacks(t.need_child, t.cap_child, t.n_child);
+        t.need_label = lacks(t.need_label, t.cap_label, t.n_label);
+        if (round >= kBulkGrowths || grow_tree(r, p, true) != P2P_OK) {
           use_bulk = false;
           t.status = p2p::DELTA_OK;
           t.need_node = t.need_child = t.need_label = t.need_root = 0;

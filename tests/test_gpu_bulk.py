@@ -167,8 +167,8 @@ def test_edges_left_around_the_lane_spans(n_fill):
 
 
 def test_a_round_that_asks_for_more_than_an_arena_can_hold():
-    """Many INSERTs of one long new prompt: a round's bound counts it for each of them (1.15 G tokens, past the arenas'
-    reach), though together they take it once.  The delta kernel applies them without bulk rounds."""
+    """Many INSERTs of one long new prompt: counted for each of them they ask for 1.15 G tokens, past the arenas' reach,
+    though together they take it once."""
     n, L = 1100, 1 << 20
     rng = np.random.default_rng(3)
     pool = np.concatenate([rng.integers(0, 1000, size=L), np.arange(n)]).astype(np.int32)
@@ -184,6 +184,20 @@ def test_a_round_that_asks_for_more_than_an_arena_can_hold():
     tok, off = csr_from_lists([pool[:L].tolist() + [3], pool[: L // 2].tolist() + [-1], [5]])
     gm, _ = route_device(r, tok, off, [0], 1)
     assert gm.ravel().tolist() == [L + 1, L // 2, 1]
+
+
+@pytest.mark.parametrize("n", [5, 32, 60])
+def test_a_tree_with_room_is_not_grown(n):
+    """INSERTs of one new prompt, which together take it once: the arenas that hold them (and a next call like it) stay
+    as they are, though n prompts would not fit."""
+    r, trees = router_from_seqlists([seqlist_from_lists([[1, 2, 3]])]), oracle.build_trees([seqlist_from_lists([[1, 2, 3]])])
+    before = r.stats(0)
+    prompt = list(range(1000, 1000 + before["cap_label"] // 4))
+    sl, op = _runs([prompt + [k] for k in range(n)], [len(prompt)] * n), np.zeros(n, np.int32)
+    assert r.apply_delta(0, op, sl) == trees[0].apply_ops(op, sl)
+    assert same_snapshot(r.download(0), trees[0].export())
+    after = r.stats(0)
+    assert all(after[k] == before[k] for k in ("cap_node", "cap_child", "cap_label")), (before, after)
 
 
 @pytest.mark.parametrize("held,new", [(0, 1), (0, 3), (2, 1), (2, 30), (8, 1), (8, 9), (30, 3), (60, 70), (130, 1), (200, 900), (1000, 1100)])
