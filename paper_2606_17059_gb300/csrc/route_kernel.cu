@@ -6,8 +6,8 @@
 //
 // Passes.  A grouped batch (group_kernel.cu) is routed by a leader pass and a follower pass; a small batch is not
 // grouped and all of it is routed by the leader pass (route_ungrouped).  Leaders of
-// short requests, and the followers of long ones, are walked by lane_kernel (a lane per tree; below), the followers of
-// short requests by follow_kernel (a lane per follower).  Leaders whose
+// short requests, and followers, are walked by lane_kernel (a lane per tree; below), the followers of short requests in
+// a large batch by follow_kernel (a lane per follower).  Leaders whose
 // requests are longer than a staging window on average go to route_kernel:
 //
 // route_kernel schedule.  A CTA takes requests b = list[blockIdx.x], list[blockIdx.x + gridDim.x], ...; its
@@ -859,7 +859,7 @@ __global__ void __launch_bounds__(kFollowThreads, kLaneCtas<kLeader, kFirst>) la
   }
 }
 
-// The followers of short requests: a lane per follower, all lanes of a warp in one tree at a time.
+// The followers of short requests in a large batch: a lane per follower, all lanes of a warp in one tree at a time.
 //
 // In each tree a follower whose leader matched less than their common prefix has the leader's match; the others resume
 // at the leader's checkpoint with one lookup of the follower's token there, mostly in vain.  What bounds this over
@@ -870,18 +870,34 @@ __global__ void __launch_bounds__(kFollowThreads, kLaneCtas<kLeader, kFirst>) la
 //     tables' size.  The lanes here are followers, side by side for a leader, and look into one tree, mostly one table.
 //   - Loads in flight.  A lookup that its first load does not answer, and the walk behind a token that is there, take
 //     several round trips, and in almost every step some lane of the warp has one.  They are queued, and full warps of
-//     them are looked up and walked.
-// A follower that would compare more than kSpan tokens of an edge in some tree is left to lane_kernel (`late`), whose
-// lanes share such compares over the trees.  A lane keeps its follower's decision in registers.
+//     them are looked up and walked; what is left of an edge after kOwn tokens is compared by the warp.
+// A follower whose token is there in many trees (kMinHits, and more than a third) has little of this to gain: there
+// lane_kernel's lanes share the request's tokens, and the follower is left to it (`late`), from its first trees on as a
+// rule; so is one that comes to more than kFar tokens of an edge in a second tree, or together with many others whose
+// tokens are there in most trees.  A lane keeps its follower's decision in registers.
 //
-// Measured against lane_kernel<false>: 205,000 followers on 256 trees 1.04 -> 0.70 ms, 160,000 on 64 trees 207 -> 148 us,
-// 52,000 on 16 trees 39 -> 31.  Two trees a lane and three CTAs a SM: one or four trees 824 and 785 us, two, four and
-// five CTAs 865, 721 and 817 (more loads in flight are more translations).
+// Measured against lane_kernel<false> (us): 205,000 followers on 256 trees 725 -> 435, 160,000 on 64 trees 155 -> 117,
+// 52,000 on 16 trees 34 -> 28; conversations cached in one tree each behind one of 64 prompts: 200,000 of 300 tokens on 16
+// trees 272 -> 192, of 100 on 64 trees 361 -> 193, 100,000 of 600 on 64 trees 221 -> 179.  Where every tree holds every
+// follower's next 70 tokens: 200,000 on 64 trees 1,439 -> 1,573 (2,500 with none left to lane_kernel before its trees are
+// through), on 16 trees 456 -> 557.  Two trees a lane and three CTAs a SM: one or four trees 824 and 785 us, two, four and
+// five CTAs 865, 721 and 817 where these took 697 (more loads in flight are more translations).
 constexpr int kRowWarps = 8;
 constexpr int kRowCtasPerSm = 3;
 constexpr int kRowIlp = 2;   // trees a lane looks up at a time
 constexpr int kTile = 16;    // trees whose matches are put together
-constexpr int kSpan = 80;    // tokens of an edge that a lane compares
+constexpr int kOwn = 8;      // tokens of an edge that a lane compares (16: the conversations on 64 trees 315 -> 324)
+constexpr int kFar = 128;    // ... and that the warp compares in one round trip
+constexpr int kFarLanes = 8;  // far compares of a warp at a time
+constexpr int kMinHits = 4;
+// Followers of a full wave of lanes.  With fewer the warps that there are walk tree after tree while the GPU idles, where
+// lane_kernel has a warp for each follower (a route of 8,192 requests on 256 trees 437 us, 227 by lane_kernel; of 65,536
+// 579 and 539, of 90,000 650 and 665; on 64 trees 65,536 214 and 214, 90,000 243 and 257; on 32 trees 48,000 159 and 149,
+// 100,000 224 and 238).  A single tile of trees is walked soon (48,000 on 16 trees 137 and 138, on 4 130 and 135).
+inline int64_t follow_line(int32_t P, int num_sms) {
+  const int64_t lanes = (int64_t)num_sms * kRowCtasPerSm * kRowWarps * 32;
+  return P <= kTile ? lanes / 2 : lanes * 3 / 4;
+}
 constexpr int kQueue = 32 + 32 * kRowIlp;
 struct RowWarp {
   int4 todo[kQueue];         // lookups to finish: (table offset, table bits, position, follower | tree << 8)
@@ -922,6 +938,8 @@ __global__ void __launch_bounds__(kRowWarps * 32, kRowCtasPerSm) follow_kernel(
     const int4* ckrow = ckpt + (int64_t)max(row, 0) * P;
     RouteAcc<kDecide> acc;
     unsigned slow = 0;               // the followers left to lane_kernel (a bit per lane)
+    unsigned far_once = 0;           // ... and those with a tree of more than kFar tokens to compare
+    int hits = 0;                    // lookups that were not answered at once
     int32_t tk_at = -1, tk_val = 0;  // the request token looked up last: most trees resume at one position
     const bool any = __any_sync(kFull, on);
     for (int32_t p0 = 0; p0 < P; p0 += kTile) {
@@ -965,47 +983,81 @@ __global__ void __launch_bounds__(kRowWarps * 32, kRowCtasPerSm) follow_kernel(
             S.m[lane][h + g] = st[g].x;
             int4 e;
             if (act[g]) act[g] = probe_first2(e0[g], e1[g], tk[g], e) != 0;
+            hits += act[g];
             const unsigned hm = __ballot_sync(kFull, act[g]);
             if (act[g])
               S.todo[todo + __popc(hm & ((1u << lane) - 1))] =
                   make_int4(st[g].y, tab_bits(st[g].z), st[g].x, lane | (h + g) << 8);
             todo += __popc(hm);
           }
+          slow |= __ballot_sync(kFull, hits >= kMinHits && 3 * hits > p0 + h + kRowIlp + 6 && 2 * (p0 + h + kRowIlp) <= P);
           while (todo >= 32 || (todo > 0 && h + kRowIlp >= kTile)) {
             __syncwarp();
             const int first = max(todo - 32, 0);
-            const bool go = first + lane < todo;
+            bool go = first + lane < todo;
             const int4 q = go ? S.todo[first + lane] : make_int4(0, 0, 0, 0);
             const int wi = q.w & 31, t = q.w >> 8;
+            go = go && !((slow >> wi) & 1);
             todo = first;
             const int32_t wl = __shfl_sync(kFull, len, wi), wc = __shfl_sync(kFull, c, wi);
             const int32_t* wr = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)req, wi);
             const TreeView& tv = trees[p0 + t];
             int4 ce = make_int4(0, 0, 0, 0);
+            const int wh = __shfl_sync(kFull, hits, wi);
             int32_t pos = q.z;
-            bool walk = go && find_child_1(tv.child + q.x, q.y, __ldg(wr + pos), ce), long_edge = false;
+            bool far = false, left = false;  // a far compare in this walk; the follower is left to lane_kernel
+            bool walk = go && find_child_1(tv.child + q.x, q.y, __ldg(wr + pos), ce);
             const bool found = walk;
-            while (walk) {  // edge by edge
-              if (ce.w <= 0 || ce.y <= 0) {  // cannot happen in a valid tree
-                atomicOr(err, ERR_CORRUPT_TREE);
-                break;
-              }
-              const int4 nn = __ldg(tv.node + ce.y);
-              const int32_t lim = min(ce.w, wl - pos), from = max(1, wc - pos), stop = min(lim, from + kSpan);
-              int32_t k = lim;
-              if (from < lim) {
-                k = first_diff_1(label_ptr(tv.label, tv.shared, ce.z), wr + pos, from, stop);
-                if (k == stop && stop < lim) {
-                  long_edge = true;
-                  break;
+            while (__any_sync(kFull, walk)) {  // edge by edge
+              int4 nn = make_int4(0, 0, 0, 0);
+              int32_t k = 0, lim = 0, from = 0;
+              const int32_t* lab = nullptr;
+              bool need = false;
+              if (walk) {
+                if (ce.w <= 0 || ce.y <= 0) {  // cannot happen in a valid tree
+                  atomicOr(err, ERR_CORRUPT_TREE);
+                  walk = false;
+                } else {
+                  nn = __ldg(tv.node + ce.y);
+                  lim = k = min(ce.w, wl - pos);
+                  from = max(1, wc - pos);
+                  if (from < lim) {
+                    lab = label_ptr(tv.label, tv.shared, ce.z);
+                    const int32_t stop = min(lim, from + kOwn);
+                    k = first_diff_1(lab, wr + pos, from, stop);
+                    need = k == stop && stop < lim;
+                    from = stop;
+                  }
                 }
               }
-              pos += k;
-              walk = k == ce.w && pos < wl && nn.z > 0 &&
-                     find_child_1(tv.child + nn.x, tab_bits(nn.y), __ldg(wr + pos), ce);
+              const bool far_now = need && !far && lim - from > kFar;
+              const unsigned fm = __ballot_sync(kFull, far_now);
+              if (fm) {
+                const unsigned same = __match_any_sync(kFull, far_now ? wi : 32 + lane);
+                if (far_now) {
+                  far = true;
+                  left = ((far_once >> wi) & 1) || __popc(same) > 1 || (__popc(fm) > kFarLanes && 2 * wh > p0 + h);
+                  if (left) need = walk = false;
+                }
+                far_once |= __reduce_or_sync(kFull, far_now ? 1u << wi : 0u);
+              }
+              for (unsigned m = __ballot_sync(kFull, need); m; m &= m - 1) {
+                const int j = __ffs(m) - 1;
+                const int32_t* lj = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)lab, j);
+                const int32_t* rj = (const int32_t*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)(wr + pos), j);
+                const int32_t f = __shfl_sync(kFull, from, j), to = __shfl_sync(kFull, lim, j);
+                const int32_t kk = to - f <= kFar ? compare_tail<true>(lj, rj, f, to, lane)
+                                                 : compare_range<8, true>(lj, rj, f, to, lane);
+                if (lane == j) k = kk < 0 ? to : kk;
+              }
+              if (walk) {
+                pos += k;
+                walk = k == ce.w && pos < wl && nn.z > 0 &&
+                       find_child_1(tv.child + nn.x, tab_bits(nn.y), __ldg(wr + pos), ce);
+              }
             }
             if (found) S.m[wi][t] = pos;
-            slow |= __reduce_or_sync(kFull, long_edge ? 1u << wi : 0u);
+            slow |= __reduce_or_sync(kFull, left ? 1u << wi : 0u);
           }
         }
         __syncwarp();
@@ -1209,14 +1261,14 @@ cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tok
   e = cudaGetLastError();
   if (e != cudaSuccess || !g) return e;
   // The followers' first per-lane compare in lane_kernel: 8 tokens for long requests, 16 otherwise (lane_walks).  A
-  // single tree's followers stay with it: there is no tree to go on to.
+  // single tree's followers stay with it (there is no tree to go on to), and those of smaller batches (follow_line).
   if (long_requests(B, n_tokens)) {
     const int grid_long = (int)std::min<int64_t>(want, (int64_t)num_sms * kLaneCtas<false, 8>);
     P2P_TIMED(K_LANE_FOLLOWER, st,
               (lane_kernel<false, kDecide, 8><<<grid_long, kFollowThreads, 0, st>>>(
                   d_trees, P, tokens, n_tokens, tok_base, offsets, B, g->lists + B, g->counts + 1, g->lead, g->cpre,
                   g->gid, nullptr, g->ckpt, d_load, alpha, out_match, out_peer, d_err, nullptr, out_next)));
-  } else if (P > 1) {
+  } else if (P > 1 && B >= follow_line(P, num_sms)) {
     const size_t smem = sizeof(RowWarp) * kRowWarps;
     e = cudaFuncSetAttribute(follow_kernel<kDecide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
