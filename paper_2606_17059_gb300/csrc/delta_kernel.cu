@@ -1134,7 +1134,7 @@ __global__ void __launch_bounds__(kDeltaWarps * 32, 2)
 }
 
 // Validates a device-resident delta into header (int32 words: [0..1] longest sequence as u64, [2] error
-// bits STATIC_*, [3] most pool runs of one op); the header must be zero on entry.
+// bits STATIC_*, [3] most pool runs of one op, [4] most ops of one tree); the header must be zero on entry.
 __global__ void validate_kernel(int32_t* header, const int32_t* __restrict__ op, const int64_t* __restrict__ seg_begin,
                                 const int64_t* __restrict__ seg_off, const int32_t* __restrict__ seg_len, int64_t n,
                                 int64_t n_segs, int64_t n_pool, const int64_t* __restrict__ peer_begin, int32_t P) {
@@ -1178,12 +1178,17 @@ __global__ void validate_kernel(int32_t* header, const int32_t* __restrict__ op,
     if (my_runs) atomicMax(max_runs, my_runs);
     if (my_bits) atomicOr(err, my_bits);
   }
-  if (peer_begin && blockIdx.x == 0) {
+  if (!peer_begin) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) header[4] = (int32_t)min(n, (int64_t)INT32_MAX);
+  } else if (blockIdx.x == 0) {
+    int32_t most = 0;
     for (int32_t p = threadIdx.x; p <= P; p += blockDim.x) {
-      const int64_t v = peer_begin[p];
-      if ((p == 0 && v != 0) || (p == P && v != n) || (p > 0 && v < peer_begin[p - 1]))
-        atomicOr(err, STATIC_BAD_PEER_BEGIN);
+      const int64_t v = peer_begin[p], before = p > 0 ? peer_begin[p - 1] : 0;
+      if ((p == 0 && v != 0) || (p == P && v != n) || v < before) atomicOr(err, STATIC_BAD_PEER_BEGIN);
+      most = max(most, (int32_t)min(max(v - before, (int64_t)0), (int64_t)INT32_MAX));
     }
+    most = __reduce_max_sync(kFull, most);
+    if ((threadIdx.x & 31) == 0) atomicMax(header + 4, most);
   }
 }
 

@@ -312,7 +312,7 @@ enum { STATIC_BAD_OP = 1, STATIC_BAD_SEGMENT = 2, STATIC_BAD_PEER_BEGIN = 4, STA
 int64_t static_scratch_tokens();
 cudaError_t static_scratch(int device, int32_t** header, int32_t** tokens);
 // Validates a device-resident delta on the device into a kStaticHeaderInts-word header (zeroed first):
-// [0..1] longest sequence (u64), [2] STATIC_* error bits, [3] most pool runs of one op.
+// [0..1] longest sequence (u64), [2] STATIC_* error bits, [3] most pool runs of one op, [4] most ops of one tree.
 cudaError_t launch_validate(int32_t* header, const p2p_delta* d, int32_t peer, int32_t P, cudaStream_t st);
 cudaError_t launch_init_ranges(TreeState* d_states, int32_t nt, const int64_t* peer_begin, int64_t n, cudaStream_t st);
 // Per tree that stopped for room (DELTA_NEED_SPACE): room[2i] = label tokens and room[2i + 1] = INSERTs of its ops

@@ -1269,6 +1269,15 @@ int p2p_tree_apply_delta(p2p_router* r, int32_t peer, const p2p_delta* d, int64_
 // routed mostly to one tree and inserted with p2p_update_estimates, for one).  n_blocks = nt and
 // d_parts = NULL when no tree is split.
 constexpr int64_t kPartOps = 16384;
+// Deltas that the delta kernel takes alone: its CTA of a tree has 16 ops in work at a time, and the rounds' nine launches
+// take 28 us whatever the ops.  A call of 1, 4, 8, 16, 64 ops on one tree, alone and with the rounds: 96, 95, 122, 141,
+// 223 us and 123, 125, 126, 133, 131; of 1, 8, 12, 16 ops on each of 256 trees 98, 134, 154, 166 and 141, 165, 167, 170.
+// With more trees than the SMs hold CTAs of that kernel they wait for one another: 1, 2, 4 ops on each of 1,024 trees 173,
+// 190, 246 and 176, 177, 207.
+constexpr int64_t kAloneOps = 12;
+static bool few_ops(int64_t n, int64_t max_ops, int32_t n_trees, int num_sms) {
+  return max_ops <= kAloneOps && (n_trees <= 2 * num_sms || n <= 8 * (int64_t)num_sms);
+}
 // Largest delta of the bulk rounds (their scratch takes up to 200 bytes per op), and how much smaller the delta
 // kernel's slabs are behind them.
 constexpr int64_t kBulkMaxOps = (int64_t)1 << 24;
@@ -1325,7 +1334,7 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
   const int32_t nt = p1 - p0;
   if (!lru_ok)
     if (int rc = reject_lru_ops(r, peer, d)) return rc;
-  int64_t max_len = 0, max_runs = 0;
+  int64_t max_len = 0, max_runs = 0, max_ops = 0;  // of one op, of one op, of one tree
   const int32_t* d_op = d->op;
   const int64_t *d_sb = S.seg_begin, *d_so = S.seg_off, *d_pb = d->peer_begin;
   const int32_t *d_sl = S.seg_len, *d_pool = S.pool;
@@ -1368,12 +1377,13 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
     // Validate on the device; only the 16-byte result comes back.
     CK(p2p::launch_validate(r->d_hdr, &dv, peer, r->P, r->stream));
     r->launches += 1;
-    int32_t h[4] = {0, 0, 0, 0};
+    int32_t h[5] = {0, 0, 0, 0, 0};
     CK(d2h(r, h, r->d_hdr, sizeof(h)));
     unsigned long long ml = 0;
     std::memcpy(&ml, h, sizeof(ml));
     max_len = (int64_t)ml;
     max_runs = h[3];
+    max_ops = h[4];
     if (h[2] & p2p::STATIC_BAD_OP) return fail(r, P2P_E_INVAL, "bad op code in the delta");
     if (h[2] & p2p::STATIC_BAD_SEGMENT) return fail(r, P2P_E_INVAL, "seg_begin or a segment is malformed or outside the pool");
     if (h[2] & p2p::STATIC_TOO_LONG) return fail(r, P2P_E_INVAL, "a sequence is longer than 2^31-1 tokens");
@@ -1408,10 +1418,10 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
                      reinterpret_cast<int32_t*>(static_cast<unsigned long long*>(r->gmemo.p) + gslots),
                      (uint32_t)(gslots - 1)};
   CK(cudaMemsetAsync(r->gmemo.p, 0, gslots * (sizeof(unsigned long long) + sizeof(int32_t)), r->stream));
-  // Bulk rounds first, where the ops are of at most two pool runs and the scratch can be had; what they leave (few
-  // ops, as a rule) goes to the delta kernel, whose warps then take smaller slabs.
+  // Bulk rounds first, where there are ops for them, of at most two pool runs, and the scratch can be had; what they leave
+  // (few ops, as a rule) goes to the delta kernel, whose warps then take smaller slabs.
   p2p::BulkArgs bulk = {};
-  bool use_bulk = max_runs <= 2 && n <= kBulkMaxOps;
+  bool use_bulk = max_runs <= 2 && n <= kBulkMaxOps && !few_ops(n, max_ops, nt, r->num_sms);
   if (use_bulk) {
     if (ensure(r, r->bulk, p2p::bulk_scratch(n, nt, nullptr, bulk)) != cudaSuccess) {
       use_bulk = false;

@@ -134,7 +134,7 @@ cudaError_t static_scratch(int, int32_t**, int32_t**) { return cudaErrorNotSuppo
 cudaError_t launch_validate(int32_t* h, const p2p_delta* d, int32_t, int32_t, cudaStream_t) {
   std::memset(h, 0, kStaticHeaderInts * 4);
   h[0] = h[3] = 1;
-  (void)d;
+  h[4] = (int32_t)d->seqs.n;
   return cudaGetLastError();
 }
 cudaError_t launch_init_ranges(TreeState* s, int32_t nt, const int64_t*, int64_t n, cudaStream_t) {

@@ -186,6 +186,36 @@ def test_a_round_that_asks_for_more_than_an_arena_can_hold():
     assert gm.ravel().tolist() == [L + 1, L // 2, 1]
 
 
+@pytest.mark.parametrize("P,per,one", [(1, 1, 0), (1, 12, 0), (1, 13, 0), (5, 12, 3), (5, 2, 13), (5, 0, 1), (5, 0, 40),
+                                       (310, 3, 2), (310, 6, 0)])
+def test_deltas_of_a_few_ops(P, per, one):
+    """Up to 12 ops a tree the delta kernel takes a delta alone (fewer in all on many trees), from host and from device
+    memory; `one` more go to the last tree."""
+    import torch
+    rng = random.Random(P * 100 + per)
+    stored = [[[rng.randrange(4) for _ in range(rng.randint(1, 20))] for _ in range(12)] for _ in range(P)]
+    sls = [seqlist_from_lists(s) for s in stored]
+    r, trees = router_from_seqlists(sls), oracle.build_trees(sls)
+    ops, seqs, pb = [], [], [0]
+    for p in range(P):
+        for _ in range(per + (one if p == P - 1 else 0)):
+            ops.append(rng.randrange(2))
+            seqs.append(rng.choice(stored[p])[: rng.randint(0, 20)] + [rng.randrange(4)])
+        pb.append(len(ops))
+    sl, op, pb = seqlist_from_lists(seqs), np.array(ops, np.int32), np.array(pb, np.int64)
+    dev = wl.SeqList(*(torch.from_numpy(x).cuda() for x in (sl.seg_begin, sl.seg_off, sl.seg_len, sl.pool)))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    few = max(np.diff(pb)) <= 12 and (P <= 2 * sms or len(ops) <= 8 * sms)
+    for turn in range(2):
+        r.kernel_clock(True)
+        got = r.apply_delta(-1, op, sl, pb) if turn else r.apply_delta(-1, torch.from_numpy(op).cuda(), dev, torch.from_numpy(pb).cuda(), on_device=True)
+        assert got == sum(t.apply_ops(op, sl, int(pb[p]), int(pb[p + 1])) for p, t in enumerate(trees))
+        assert ("bulk_resolve_kernel" in r.kernel_times()) != few
+    for p in range(0, P, max(1, P // 7)):
+        assert same_snapshot(r.download(p), trees[p].export()), p
+    assert same_snapshot(r.download(P - 1), trees[P - 1].export())
+
+
 @pytest.mark.parametrize("n", [5, 32, 60])
 def test_a_tree_with_room_is_not_grown(n):
     """INSERTs of one new prompt, which together take it once: the arenas that hold them (and a next call like it) stay
