@@ -871,7 +871,7 @@ __global__ void __launch_bounds__(kFollowThreads, kLaneCtas<kLeader, kFirst>) la
 //   - Loads in flight.  A lookup that its first load does not answer, and the walk behind a token that is there, take
 //     several round trips, and in almost every step some lane of the warp has one.  They are queued, and full warps of
 //     them are looked up and walked; what is left of an edge after kOwn tokens is compared by the warp.
-// A follower whose token is there in many trees (kMinHits, and more than a third) has little of this to gain: there
+// A follower whose token is there in many trees (kMinHits, and more than half) has little of this to gain: there
 // lane_kernel's lanes share the request's tokens, and the follower is left to it (`late`), from its first trees on as a
 // rule; so is one that comes to more than kFar tokens of an edge in a second tree, or together with many others whose
 // tokens are there in most trees.  A lane keeps its follower's decision in registers.
@@ -939,7 +939,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, kRowCtasPerSm) follow_kernel(
     RouteAcc<kDecide> acc;
     unsigned slow = 0;               // the followers left to lane_kernel (a bit per lane)
     unsigned far_once = 0;           // ... and those with a tree of more than kFar tokens to compare
-    int hits = 0;                    // lookups that were not answered at once
+    int hits = 0;                    // lookups past the common prefix that were not answered at once
     int32_t tk_at = -1, tk_val = 0;  // the request token looked up last: most trees resume at one position
     const bool any = __any_sync(kFull, on);
     for (int32_t p0 = 0; p0 < P; p0 += kTile) {
@@ -983,15 +983,15 @@ __global__ void __launch_bounds__(kRowWarps * 32, kRowCtasPerSm) follow_kernel(
             S.m[lane][h + g] = st[g].x;
             int4 e;
             if (act[g]) act[g] = probe_first2(e0[g], e1[g], tk[g], e) != 0;
-            hits += act[g];
+            hits += act[g] && st[g].x >= c;
             const unsigned hm = __ballot_sync(kFull, act[g]);
             if (act[g])
               S.todo[todo + __popc(hm & ((1u << lane) - 1))] =
                   make_int4(st[g].y, tab_bits(st[g].z), st[g].x, lane | (h + g) << 8);
             todo += __popc(hm);
           }
-          slow |= __ballot_sync(kFull, hits >= kMinHits && 3 * hits > p0 + h + kRowIlp + 6 && 2 * (p0 + h + kRowIlp) <= P);
           while (todo >= 32 || (todo > 0 && h + kRowIlp >= kTile)) {
+            slow |= __ballot_sync(kFull, hits >= kMinHits && 2 * hits > p0 + h + kRowIlp + 2 && 2 * (p0 + h + kRowIlp) <= P);
             __syncwarp();
             const int first = max(todo - 32, 0);
             bool go = first + lane < todo;
