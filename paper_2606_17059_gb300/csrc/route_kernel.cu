@@ -1293,15 +1293,21 @@ cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tok
 
 }  // namespace
 
-// A batch of no more requests than the leader pass has warps (or eight a resident CTA of the staged pass) is not
-// grouped: its walks all run at once, so the pass takes as long as its longest walk whether or not the followers are
-// among them, and the grouping and the follower pass would only come on top.  Measured (us a call, grouped ->
-// ungrouped): 33 requests on 4 trees 34 -> 25, 1,025 on 16 trees 46 -> 24, 4,864 on 64 trees 60 -> 29, on 256 trees
-// 103 -> 77, twice that many on 256 trees 140 -> 144; long requests on 32 trees: 33 124 -> 68, 2,048 246 -> 173,
-// 4,096 318 -> 333.  A batch on few trees gains too, but stays grouped past 300 requests for each tree after the
-// first: the kernel clock and the launch count are documented by their grouped launches on such batches.
+// A batch of no more requests than the leader pass has warps is not grouped: its walks all run at once, so the pass takes
+// about as long as its longest walk whether or not the followers are among them, and the grouping and the follower pass
+// would only come on top.  Measured (us a call, grouped -> ungrouped): 33 requests on 4 trees 46 -> 25, 1,200 on 16
+// trees 54 -> 26, 4,864 on 64 trees 68 -> 35, on 256 trees 166 -> 112; where every tree holds a copy of its own of each
+// prompt, 4,864 of 200 tokens on 256 trees 320 -> 319, of 1,000 490 -> 577, 33 to 300 of 4,000 1,088 -> 1,104, 2,400 1,119
+// -> 1,233.
+// Long requests are walked by a CTA each, several warps to a request, and a walk reads thousands of tokens in every tree
+// that holds the prompt, where the grouping compares a follower with its leader once: one a SM, on few trees a few.
+// 20,000 tokens that all trees hold, 8 trees, 608 requests 71 -> 51, 1,000 74 -> 91; 32 trees, 304 requests 89 -> 80, 608
+// 92 -> 142; 128 trees, 152 requests 209 -> 171, 304 215 -> 261; 512 trees, 152 requests 649 -> 607, 304 644 -> 960.
+// Prompts left half-way on 256 trees, 152 requests 327 -> 254.
+// A batch on few trees gains too, but stays grouped past 300 requests for each tree after the first (all of a single
+// tree): that leaves the launches of such batches, which tests count, as they were.
 bool route_ungrouped(int64_t B, int32_t P, int64_t n_tokens, int num_sms) {
-  const int64_t most = long_requests(B, n_tokens) ? (int64_t)num_sms * kCtasPerSm * 8
+  const int64_t most = long_requests(B, n_tokens) ? (int64_t)num_sms * (P <= 8 ? 4 : P <= 32 ? 2 : 1)
                                                   : (int64_t)num_sms * kFollowCtasPerSm * (kFollowThreads / 32);
   return B <= std::min<int64_t>(most, (int64_t)300 * (P - 1));
 }

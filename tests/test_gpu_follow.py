@@ -89,8 +89,9 @@ def test_followers_of_large_batches(P, far, held):
 
 @pytest.mark.parametrize("P,far", [(2, 200), (3, 90), (4, 500), (15, 83), (16, 200), (17, 161), (33, 82), (64, 300), (97, 100)])
 def test_followers(P, far):
+    import torch
     rng = random.Random(P * 31 + far)
-    line = min(4864, 300 * (P - 1))  # batches above it are grouped on 152 SMs
+    line = min(torch.cuda.get_device_properties(0).multi_processor_count * 32, 300 * (P - 1))  # batches above it are grouped
     sizes = [1, 2, 31, 32, 33, 34, 64, 65, 300]
     while sum(sizes) <= line:
         sizes.append(rng.choice([2, 33, 200, 700]))

@@ -48,11 +48,24 @@ def _case(rng, P, B, stem_len, tail):
     return trees, reqs
 
 
-# P trees: the line lies at min(4864, 300 (P - 1)) requests of ordinary length on 152 SMs.
-@pytest.mark.parametrize("P,B", [(1, 1), (1, 40), (2, 299), (2, 300), (2, 301), (2, 309), (4, 900), (4, 901), (20, 4864), (20, 4865),
-                                 (3, 33), (33, 7), (45, 5300)])
+def _line(P, long):
+    """The most requests that are routed without grouping on P trees."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return min(sms * (4 if P <= 8 else 2 if P <= 32 else 1) if long else sms * 32, 300 * (P - 1))
+
+
+def _requests(P, B, long):
+    """B requests, or (a text) that many more than the line."""
+    return B if isinstance(B, int) else _line(P, long) + int(B)
+
+
+# Batches around the line, around the CTA sizes of the ungrouped pass (a warp, two and eight a SM) and well off both.
+@pytest.mark.parametrize("P,B", [(1, 1), (1, 40), (2, 299), (2, "+0"), (2, "+1"), (2, 309), (4, "+0"), (4, "+1"), (20, "+0"), (20, "+1"),
+                                 (3, 33), (33, 7), (45, 5300), (20, 152), (20, 153), (20, 1217)])
 def test_both_sides_of_the_grouping_line(P, B):
     import torch
+    B = _requests(P, B, False)
     rng = random.Random(P * 10007 + B)
     trees, reqs = _case(rng, P, B, 200, 12)
     sls = [seqlist_from_lists(t) for t in trees]
@@ -61,7 +74,9 @@ def test_both_sides_of_the_grouping_line(P, B):
     load = [rng.randrange(5) for _ in range(P)]
     om, op, _ = oracle.route(o, tok, off, load, 2)
     t, f = torch.from_numpy(tok).cuda(), torch.from_numpy(off).cuda()
+    n0 = r.launch_count()
     m, p = r.route(t, f, load, 2)
+    assert (r.launch_count() - n0 == 1) == (B <= _line(P, False))
     assert_same_route(m.cpu().numpy(), p.cpu().numpy(), om, op, "route")
     ex = np.array([rng.random() < 0.4 for _ in range(P)], np.uint8)
     m, p, n = r.route_decide(t, f, load, 2, ex)
@@ -84,10 +99,10 @@ def test_both_sides_of_the_grouping_line(P, B):
     assert not m.cpu().numpy()[-1].any() and int(p[-1]) == -1
 
 
-# Long requests: 304 resident CTAs take eight requests each before the batch is grouped.
-@pytest.mark.parametrize("P,B", [(2, 3), (3, 599), (3, 601), (9, 2390)])
+@pytest.mark.parametrize("P,B", [(2, 3), (3, "+0"), (3, "+1"), (9, "+0"), (9, "+1"), (9, 2390), (33, "+0"), (33, "+1")])
 def test_long_requests_on_both_sides(P, B):
     import torch
+    B = _requests(P, B, True)
     rng = random.Random(P + B)
     trees, reqs = _case(rng, P, 40, 9000, 30)
     full = [q + [rng.randrange(9) for _ in range(max(0, 4200 - len(q)))] for q in reqs]
@@ -97,8 +112,10 @@ def test_long_requests_on_both_sides(P, B):
     tok, off = csr_from_lists(reqs)
     om, op, _ = oracle.route(o, tok, off, [0] * P, 1)
     t, f = torch.from_numpy(tok).cuda(), torch.from_numpy(off).cuda()
+    n0 = r.launch_count()
     m, p = r.route(t, f, [0] * P, 1)
     r.sync()
+    assert (r.launch_count() - n0 == 1) == (B <= _line(P, True))
     assert_same_route(m.cpu().numpy(), p.cpu().numpy(), om, op, "long")
     ex = np.zeros(P, np.uint8)
     ex[0] = 1
