@@ -742,13 +742,13 @@ __global__ void __launch_bounds__(kFollowThreads, kLaneCtas<kLeader, kFirst>) la
     int32_t* err, int32_t* cursor, int32_t* __restrict__ out_next) {
   __shared__ unsigned long long s_top[kDecide ? kFollowThreads / 32 : 1][kDecide ? 64 : 1];
   const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (kFollowThreads / 32);
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
   const int64_t n = kGrouped ? *count : B;
   // Requests go to warps in a fixed stride, or, with a cursor (zero at launch), one at a time as warps
   // become free: leaders' walks differ widely in length.  The next index is fetched while the warp
   // routes the current request.
   int32_t nxt = 0;
-  int64_t i0 = ((int64_t)blockIdx.x * kFollowThreads + threadIdx.x) >> 5;
+  int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (cursor) {
     if (lane == 0) nxt = atomicAdd(cursor, 1);
     i0 = __shfl_sync(kFull, nxt, 0);
@@ -1252,8 +1252,12 @@ cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tok
   } else {
     // Shorter requests: most leader walks end within a few tokens, so each lane walks its own tree.
     const auto kernel = g ? lane_kernel<true, kDecide, 8, true> : lane_kernel<true, kDecide, 8, false>;
+    // A small ungrouped batch is spread over all SMs, where a warp shares loads and translations with few others (33
+    // requests of 4,000 tokens that 256 trees hold a copy each of: 1,177 us by CTAs of eight warps, 1,088 so).
+    const int warps = g ? kFollowThreads / 32 : (int)std::min<int64_t>(kFollowThreads / 32, (B + num_sms - 1) / num_sms);
+    const int grid1 = g ? grid2 : (int)std::min<int64_t>((B + warps - 1) / warps, (int64_t)num_sms * kFollowCtasPerSm);
     P2P_TIMED(K_LANE_LEADER, st,
-              (kernel<<<grid2, kFollowThreads, 0, st>>>(
+              (kernel<<<grid1, warps * 32, 0, st>>>(
                   d_trees, P, tokens, n_tokens, tok_base, offsets, B, lists, counts, nullptr, nullptr, gid, cmin, ckpt,
                   d_load, alpha, out_match, out_peer, d_err, g ? g->counts + 3 : nullptr, out_next)));
     *launched = 1;
