@@ -250,6 +250,7 @@ struct p2p_router {
   int32_t* d_shared = nullptr;
   int64_t shared_cap = 0;
   std::vector<int32_t> h_shared;
+  int64_t shared_synced = 0;  // tokens of the mirror that the device array holds
   std::unordered_map<uint64_t, int32_t> intern;
   // Interned runs by a hash of their first kHeadTokens tokens: (pool offset, length), a few per head.
   std::unordered_map<uint64_t, std::vector<std::pair<int32_t, int32_t>>> heads;
@@ -508,10 +509,10 @@ int do_sync(p2p_router* r) {
 
 int push_states(p2p_router* r, int32_t p0, int32_t p1);
 
-// Makes the device shared pool hold the host mirror's tokens [from, end): grows it (stream-ordered copy)
-// if needed, in which case every tree's view is refreshed with the new pool address.
-int sync_shared_pool(p2p_router* r, int64_t from) {
-  const int64_t n = (int64_t)r->h_shared.size();
+// Makes the device shared pool hold all of the host mirror's tokens (also those of an upload that failed before it got
+// here): grows it (stream-ordered copy) if needed, in which case every tree's view is refreshed with the new pool address.
+int sync_shared_pool(p2p_router* r) {
+  const int64_t n = (int64_t)r->h_shared.size(), from = r->shared_synced;
   if (n == from) return P2P_OK;
   if (n > r->shared_cap) {
     const int64_t cap = std::min<int64_t>(std::max<int64_t>(2 * r->shared_cap, n + (1 << 20)), INT32_MAX);
@@ -529,6 +530,7 @@ int sync_shared_pool(p2p_router* r, int64_t from) {
   CK(cudaMemcpyAsync(r->d_shared + from, r->h_shared.data() + from, (size_t)(n - from) * sizeof(int32_t),
                      cudaMemcpyHostToDevice, r->stream));
   CK(cudaStreamSynchronize(r->stream));  // the mirror may reallocate on the next append
+  r->shared_synced = n;
   return P2P_OK;
 }
 
@@ -585,7 +587,6 @@ int upload_flat(p2p_router* r, int32_t peer, const p2p_flat_tree* t) {
   //
   // The host decides what is interned and lays the arrays out; upload_kernel fills the tables and moves the own labels.
   // It is given an edge per node (edge[c - 1] leads to node c).
-  const int64_t shared_before = (int64_t)r->h_shared.size();
   std::vector<p2p::UploadEdge> edge((size_t)(N - 1));
   struct Split {
     int32_t v, at, len, tab;  // node v's label starts with len tokens of the run at `at`; its table's offset
@@ -620,7 +621,7 @@ int upload_flat(p2p_router* r, int32_t peer, const p2p_flat_tree* t) {
     edge[(size_t)(v - 1)] = {make_int4(head ? src[head] : 0, (int32_t)v, enc, len - head),
                              make_int4(0, 0, t->label_off[v] + head, head ? (int32_t)split.size() : 0)};
   }
-  if (int rc = sync_shared_pool(r, shared_before)) return rc;
+  if (int rc = sync_shared_pool(r)) return rc;
   // Children tables, laid out in node order in the child arena; the split nodes (ids N ..) after them.
   const int64_t NN = N + (int64_t)split.size();
   if (NN > INT32_MAX / 2) return fail(r, P2P_E_NOMEM, "too many nodes");

@@ -13,6 +13,8 @@ cudaError_t last = cudaSuccess;
 size_t fail_from = 0, fail_to = 0;  // allocations of fail_from .. fail_to bytes fail (0: none)
 int fail_after = 0;                 // > 0: the allocation after that many more fails
 int ask_node = 0, ask_child = 0, ask_label = 0;  // what the next bulk rounds find no room for
+int64_t pool_end = 0;                // of the interned labels that the last upload's edges point at
+int32_t pool_at = 0, pool_tok = 0;  // one of them, and its first token
 int bad_arrays = 0, bulk_calls = 0, delta_calls = 0;
 
 cudaError_t err(cudaError_t e) {
@@ -123,8 +125,22 @@ cudaError_t launch_bulk(const BulkArgs& A, int, cudaStream_t, int* l) {
   return cudaGetLastError();
 }
 cudaError_t launch_compact(CompactJob*, int32_t, int32_t, int, cudaStream_t) { return cudaGetLastError(); }
-cudaError_t launch_upload(const UploadEdge*, int64_t, int4*, const int32_t*, int32_t*, int, cudaStream_t) { return cudaGetLastError(); }
-cudaError_t launch_set_tree(TreeState* s, TreeView*, TreeState v, const int32_t*, cudaStream_t) { return *s = v, cudaGetLastError(); }
+cudaError_t launch_upload(const UploadEdge* e, int64_t n, int4*, const int32_t*, int32_t*, int, cudaStream_t) {
+  pool_end = 0;
+  for (int64_t i = 0; i < n; ++i)
+    if (e[i].slot.z < 0 && (int64_t)~e[i].slot.z + e[i].slot.w > pool_end) {
+      pool_end = (int64_t)~e[i].slot.z + e[i].slot.w;
+      pool_at = ~e[i].slot.z;
+      pool_tok = e[i].slot.x;
+    }
+  return cudaGetLastError();
+}
+cudaError_t launch_set_tree(TreeState* s, TreeView*, TreeState v, const int32_t* shared, cudaStream_t) {
+  *s = v;
+  if (pool_end && (!holds(shared, (size_t)pool_end * 4) || shared[pool_at] != pool_tok)) ++bad_arrays;
+  pool_end = 0;
+  return cudaGetLastError();
+}
 cudaError_t launch_refresh_views(const TreeState* s, TreeView*, int32_t n, const int32_t*, cudaStream_t) {
   look(s, n);
   return cudaGetLastError();

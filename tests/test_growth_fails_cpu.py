@@ -49,6 +49,13 @@ class Host:
         return self.lib.p2p_lru_insert(self.h, 0, ctypes.c_void_p(tok.ctypes.data), ctypes.c_int64(n),
                                        ctypes.c_void_p(off.ctypes.data), ctypes.c_int64(n), ctypes.c_int64(1))
 
+    def build(self, tokens):
+        """One sequence as tree 1."""
+        sb, so = np.array([0, 1], np.int64), np.zeros(1, np.int64)
+        sl, pool = np.array([len(tokens)], np.int32), np.array(tokens, np.int32)
+        a = lambda x: x.ctypes.data
+        return self.lib.p2p_tree_build(self.h, 1, ctypes.byref(g.Seqs(1, a(sb), a(so), a(sl), a(pool), 1, len(tokens))))
+
     def close(self):
         assert self.lib.fake_bad_arrays() == self.bad
         self.lib.p2p_router_destroy(self.h)
@@ -82,6 +89,18 @@ def test_a_growth_that_fails_half_way_changes_nothing(lib, nth):
     lib.fake_fail_after(0)
     assert rc == 0, lib.p2p_last_error(r.h)
     assert r.lru_insert() == 0
+    r.close()
+
+
+def test_labels_of_an_upload_that_failed_are_there_for_the_next(lib):
+    """The pool of shared long labels cannot grow: the upload fails, and the next one with the same label brings it."""
+    r = Host(lib)
+    label = list(range(5, 1005))
+    lib.fake_fail_sizes(1 << 21, 1 << 62)  # (the pool starts with 4 MB, the tree's own arrays take less)
+    assert r.build(label) != 0
+    lib.fake_fail_sizes(0, 0)
+    assert r.build(label) == 0, lib.p2p_last_error(r.h)
+    assert r.build(label[:500]) == 0 and r.build([7] * 300) == 0
     r.close()
 
 
