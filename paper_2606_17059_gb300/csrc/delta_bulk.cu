@@ -53,8 +53,8 @@ namespace p2p {
 
 // What an op would do, as found by the walk.  u, tok: its place, which was slot `slot` of u's table at table offset
 // `tab` then; key: its entry.  Then by kind: k where a split cuts the edge, the leaf a removal takes, the node of a
-// count (arg) and its entry (ent); a leaf's entry of u (ent).  The second half only for a fold (v = arg; g, gpos: u's own
-// place) and a leaf under a leaf (key2).
+// count (arg) and its entry (ent); a leaf's entry of u (ent).  The second half only for a fold (v = arg; g, gpos: u's
+// own place) and a leaf under a leaf (key2).
 struct __align__(32) BulkOp {
   int32_t what;  // B_* | BF_* flags | tree << kTreeShift
   int32_t u, tok, slot;
@@ -85,12 +85,6 @@ constexpr int kFoldBits = 6;        // tables a lane searches for the one other 
 enum { B_NONE = 0, B_LEAF, B_SPLIT, B_COUNT, B_REMOVE, B_FOLD, B_ABSENT, B_LEFT };
 enum { BF_ALONE = 16, BF_REVIVE = 32, BF_MORE = 64, BF_LATER = 128 };  // BF_MORE: the record's second half holds
 constexpr int kTreeShift = 8;  // (a tree index has 16 bits)
-
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {  // SplitMix64's output function
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  return z ^ (z >> 31);
-}
 
 // Enters (tree, u, tok) of this round for op idx; the table's index, or -1 if it has no room near the key's home.  An
 // entry is 32 bits of the place's hash over the complement of the smallest op index.  Two places that share those
@@ -210,7 +204,8 @@ __device__ __forceinline__ int32_t ld_ahead(const int32_t* p) {
 // short, so that lanes with ends of their own stay together (with a tested tail per lane the resolve launch had
 // three times the instructions in this loop).  Only labels under eight tokens and steps across the two pool runs take
 // a token at a time.
-__device__ __forceinline__ int32_t diff_lane(const int32_t* lab, const LaneSeq& q, int32_t pos, int32_t from, int32_t to) {
+__device__ __forceinline__ int32_t diff_lane(const int32_t* lab, const LaneSeq& q, int32_t pos, int32_t from,
+                                             int32_t to) {
   for (int32_t j0 = from; j0 < to; j0 += 8) {
     const int32_t s0 = min(j0, to - 8), p0 = pos + s0;
     if (s0 < 0 || (p0 < q.na && q.na - p0 < 8)) {
@@ -267,7 +262,9 @@ __device__ int32_t diff_warp(const int32_t* a, const int32_t* b, int32_t from, i
   return to;
 }
 
-__device__ __forceinline__ int64_t list_size(const BulkArgs& A, int round) { return round == 0 ? A.n : A.counts[round]; }
+__device__ __forceinline__ int64_t list_size(const BulkArgs& A, int round) {
+  return round == 0 ? A.n : A.counts[round];
+}
 
 __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_kernel(BulkArgs A, int round) {
   const int lane = threadIdx.x & 31;
@@ -278,7 +275,8 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_resolve_ker
   const int32_t per = (int32_t)max((int64_t)1, min((int64_t)32, (total + warps - 1) / warps));
   const int32_t lane_span = min(kLaneSpan, kLaneSpanPerOp * per);
   const int32_t* list = A.lists + (round & 1) * A.n;
-  for (int64_t t = (int64_t)blockIdx.x * kBulkThreads + threadIdx.x; t < A.n_trees; t += (int64_t)gridDim.x * kBulkThreads) {
+  for (int64_t t = (int64_t)blockIdx.x * kBulkThreads + threadIdx.x; t < A.n_trees;
+       t += (int64_t)gridDim.x * kBulkThreads) {
     const TreeState& s = A.states[t];  // the arenas' use ahead of this round's reservations
     A.base[3 * t] = s.n_node;
     A.base[3 * t + 1] = s.n_child;
@@ -543,7 +541,8 @@ __device__ void move_table_lane(int4* child, int32_t off, int32_t bits, int32_t 
 }
 
 // The same for up to 2^kMaskBits slots, one warp, with a bit mask in shared memory.
-__device__ void move_table_mask(int4* child, int32_t off, int32_t bits, int32_t dst, int32_t nb, uint32_t* used, int lane) {
+__device__ void move_table_mask(int4* child, int32_t off, int32_t bits, int32_t dst, int32_t nb, uint32_t* used,
+                                int lane) {
   const uint32_t mask = (1u << nb) - 1;
   if (lane < kMaskWords) used[lane] = 0;
   __syncwarp();
@@ -596,9 +595,9 @@ __device__ void move_table_warp(int4* child, int32_t off, int32_t bits, int32_t 
   __syncwarp();
 }
 
-// A lane per listed node: the round's leaves take its table past 1/2 claimed, so it moves to one of at most 1/4
-// live load (as delta_kernel grows tables), small ones by the lane and larger ones by the warp.  A table that cannot
-// grow (no room in the arena) marks the node's entry, and its leaves wait.  (With every node that gets a leaf listed, and
+// A lane per listed node: the round's leaves take its table past 1/2 claimed, so it moves to one of at most 1/4 live
+// load (as delta_kernel grows tables), small ones by the lane and larger ones by the warp.  A table that cannot grow
+// (no room in the arena) marks the node's entry, and its leaves wait.  (With every node that gets a leaf listed, and
 // tables of 64 slots and more zeroed and filled by compare-and-swap, a step of 1,024,000 ops took 130 us of these
 // launches; now 47.)
 __global__ void __launch_bounds__(kBulkThreads) bulk_grow_kernel(BulkArgs A, int round) {
@@ -675,8 +674,8 @@ __global__ void __launch_bounds__(kBulkThreads) bulk_grow_kernel(BulkArgs A, int
     for (unsigned m = __ballot_sync(kFull, nb > kLaneBits); m; m &= m - 1) {
       const int j = __ffs(m) - 1;
       int4* cj = (int4*)__shfl_sync(kFull, (unsigned long long)(uintptr_t)child, j);
-      const int32_t off = __shfl_sync(kFull, rec.x, j), bj = __shfl_sync(kFull, bits, j), dst = __shfl_sync(kFull, c0, j),
-                    nj = __shfl_sync(kFull, nb, j);
+      const int32_t off = __shfl_sync(kFull, rec.x, j), bj = __shfl_sync(kFull, bits, j);
+      const int32_t dst = __shfl_sync(kFull, c0, j), nj = __shfl_sync(kFull, nb, j);
       if (nj <= kMaskBits) move_table_mask(cj, off, bj, dst, nj, s_used[threadIdx.x >> 5], lane);
       else move_table_warp(cj, off, bj, dst, nj, lane);
     }
@@ -808,7 +807,8 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
         if (go && what == B_FOLD)
           go = alone(A, z.z, idx) && (z.y >= 0 ? won(A, z.y, idx) : alone(A, z.w, idx));
       }
-      if (what == B_LEFT) valid = A.seg_begin[i + 1] > A.seg_begin[i] && lane_seq(A, i).n > 0;  // (not an empty sequence)
+      if (what == B_LEFT)  // (not an empty sequence)
+        valid = A.seg_begin[i + 1] > A.seg_begin[i] && lane_seq(A, i).n > 0;
       if (go && (what == B_LEAF || what == B_SPLIT || what == B_FOLD)) q = lane_seq(A, i);
       // The place, as the walk found it or, where the table has moved since, looked up again.
       if (go && what <= B_FOLD && what != B_COUNT) {
@@ -874,7 +874,8 @@ __global__ void __launch_bounds__(kBulkThreads, kBulkCtasPerSm) bulk_apply_kerne
       const int64_t k = lane == 0 ? tn : lane == 1 ? tc : lane == 2 ? tl : 0;
       int64_t at = 0, cap = 0;
       if (k) {
-        at = A.base[3 * t + lane] + (int64_t)atomicAdd(&A.taken[((int64_t)round * A.n_trees + t) * 3 + lane], (unsigned long long)k);
+        at = A.base[3 * t + lane] + (int64_t)atomicAdd(&A.taken[((int64_t)round * A.n_trees + t) * 3 + lane],
+                                                       (unsigned long long)k);
         cap = lane == 0 ? ts->cap_node : lane == 1 ? ts->cap_child : ts->cap_label;
       }
       const bool ok = __all_sync(kFull, at + k <= cap);

@@ -464,10 +464,10 @@ __device__ bool ensure_room(Tree& t, int32_t cur, int4& nd, int32_t extra, int l
 }
 
 // A shortcut to an anchor, shared by the CTA's warps for one chunk's parallel phase.  Nothing above an
-// anchor changes in that phase, so an op whose first pool run is the run (same address, same tokens) of
-// the op that first reached the anchor, and covers the anchor's position, reaches it by the same path: it
-// may start there.  (Not one gathered into scratch, whose address says nothing of its tokens.)  The first op to reach the anchor claims the entry, writes pos and rec, and publishes
-// seq last; the entry is not written again in the phase.
+// anchor changes in that phase, so an op whose first pool run is the run (same address, same tokens) of the op that
+// first reached the anchor, and covers the anchor's position, reaches it by the same path: it may start there.  (Not
+// one gathered into scratch, whose address says nothing of its tokens.)  The first op to reach the anchor claims the
+// entry, writes pos and rec, and publishes seq last; the entry is not written again in the phase.
 struct AnchorEntry {
   const int32_t* seq;  // the first pool run of the op that reached the anchor (NULL: not published)
   int32_t pos;         // tokens consumed on reaching it
@@ -1344,7 +1344,8 @@ __device__ void compact_nodes_warp(CompactJob& J, CompactShared& S, int32_t cid,
 // Copies the table of node cid (old record rec; more than 2^kSmallBits and at most 2^kWarpTabBits slots), one warp: all
 // loads in flight at once, one reservation of each counter, entries placed by a bit mask in shared memory, so that the
 // new table is written once here too.
-__device__ void compact_table_warp(CompactJob& J, CompactShared& S, int32_t cid, const int4& rec, uint32_t* used, int lane) {
+__device__ void compact_table_warp(CompactJob& J, CompactShared& S, int32_t cid, const int4& rec, uint32_t* used,
+                                   int lane) {
   constexpr int kSteps = (1 << kWarpTabBits) / 32;
   const int32_t bits = tab_bits(rec.y), size = 1 << bits;
   const uint32_t mask = (uint32_t)size - 1;
@@ -1506,22 +1507,6 @@ __device__ void compact_range_warp(CompactJob& J, CompactShared& S, const int4& 
   }
 }
 
-// One cluster of kC CTAs per tree (kC = 1: a CTA): level-synchronous breadth-first copy of the structure from the root.  New ids are
-// handed out level by level, so the nodes of the next level are the ids [end, S.node) and the scratch
-// entry of id c (old id, old and new label offsets, own-arena label length) is written by the parent's
-// copy.  A lane takes each node of the level.  A node whose table has more than 2^kWarpTabBits slots gets
-// its new table range and record from that lane, and its slots are cut into units (unit_slots) that all
-// warps then zero and fill; the others are copied by the warp, those of up to 2^kSmallBits slots a lane each.  A big table's record counts its
-// children from the old record (the live-child count), so no pass has to count them.
-// What bounds it is the chain of round trips of each level and the reservations on the tree's three counters, so a warp
-// makes one of each for its small tables, for a table of up to 128 slots, or for a unit.  Measured (a reservation per
-// table, units of 1,024 slots -> this): one tree of ~50,000 nodes by eight CTAs 194 -> 96 us, a wave of 256 trees of 40,000
-// sequences 1.70 -> 1.19 ms, of 100,000 3.8 -> 3.0 (20.6 with their 10,000 tables of 64 slots a tree as units: past 2,048
-// of them, a thread each).
-//
-// Few trees are compacted by clusters: one tree's levels keep 512 threads busy for long (a tree of ~50,000 nodes
-// 0.61 ms by a CTA), while a wave of 256 trees fills the GPU with a CTA each.  The cluster's counters and units are
-// in its first CTA's shared memory.
 // The cluster's shared counters, and a barrier of the cluster (or of the CTA).
 template <int kC>
 __device__ __forceinline__ CompactShared* compact_shared(CompactShared* own) {
@@ -1535,10 +1520,25 @@ __device__ __forceinline__ void compact_sync() {
   if constexpr (kC == 1) {
     __syncthreads();
   } else {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_sync();
   }
 }
 
+// One cluster of kC CTAs per tree (kC = 1: a CTA): level-synchronous breadth-first copy of the structure from the root.
+// New ids are handed out level by level, so the nodes of the next level are the ids [end, S.node) and the scratch entry
+// of id c (old id, old and new label offsets, own-arena label length) is written by the parent's copy.  A lane takes
+// each node of the level.  A node whose table has more than 2^kWarpTabBits slots gets its new table range and record
+// from that lane, and its slots are cut into units (unit_slots) that all warps then zero and fill; the others are
+// copied by the warp, those of up to 2^kSmallBits slots a lane each.  A big table's record counts its children from the
+// old record (the live-child count), so no pass has to count them. What bounds it is the chain of round trips of each
+// level and the reservations on the tree's three counters, so a warp makes one of each for its small tables, for a
+// table of up to 128 slots, or for a unit.  Measured (a reservation per table, units of 1,024 slots -> this): one tree
+// of ~50,000 nodes by eight CTAs 194 -> 96 us, a wave of 256 trees of 40,000 sequences 1.70 -> 1.19 ms, of 100,000 3.8
+// -> 3.0 (20.6 with their 10,000 tables of 64 slots a tree as units: past 2,048 of them, a thread each).
+//
+// Few trees are compacted by clusters: one tree's levels keep 512 threads busy for long (a tree of ~50,000 nodes
+// 0.61 ms by a CTA), while a wave of 256 trees fills the GPU with a CTA each.  The cluster's counters and units are
+// in its first CTA's shared memory.
 template <int kC>
 __global__ void __launch_bounds__(kCompactThreads, kC == 1 ? 2 : 1) compact_kernel(CompactJob* jobs) {
   CompactJob& J = jobs[blockIdx.x / kC];
@@ -1589,8 +1589,8 @@ __global__ void __launch_bounds__(kCompactThreads, kC == 1 ? 2 : 1) compact_kern
       compact_nodes_warp(J, S, cid, rec, on && bits <= kSmallBits, lane);
       for (unsigned m = mid; m; m &= m - 1) {
         const int j = __ffs(m) - 1;
-        const int4 r = make_int4(__shfl_sync(kFull, rec.x, j), __shfl_sync(kFull, rec.y, j), __shfl_sync(kFull, rec.z, j),
-                                 __shfl_sync(kFull, rec.w, j));
+        const int4 r = make_int4(__shfl_sync(kFull, rec.x, j), __shfl_sync(kFull, rec.y, j),
+                                 __shfl_sync(kFull, rec.z, j), __shfl_sync(kFull, rec.w, j));
         compact_table_warp(J, S, first + j, r, s_used[threadIdx.x >> 5], lane);
       }
     }
@@ -1676,15 +1676,15 @@ __global__ void __launch_bounds__(kLabelThreads) compact_labels_kernel(const Com
   }
 }
 
-// The tables and own labels of an uploaded tree.  Eight lanes take an edge: the first puts it into its table (claimed by
-// its node id, with compare-and-swap: others fill the table too), all move its label, kUploadSteps tokens a lane at a
-// time.  Latency of a few round
-// trips; the snapshot's labels stay in L2: 13 us for 20,900 edges and 6.3 MB of own labels.  The host filled the tables
-// and packed the labels before: the upload of that tree 1.96 -> 0.76 ms (with it, a hash of labels in four chains
-// instead of one and a validity check without a search).
+// The tables and own labels of an uploaded tree.  Eight lanes take an edge: the first puts it into its table (claimed
+// by its node id, with compare-and-swap: others fill the table too), all move its label, kUploadSteps tokens a lane at
+// a time.  Latency of a few round trips; the snapshot's labels stay in L2: 13 us for 20,900 edges and 6.3 MB of own
+// labels.  The host filled the tables and packed the labels before: the upload of that tree 1.96 -> 0.76 ms (with it, a
+// hash of labels in four chains instead of one and a validity check without a search).
 constexpr int kUploadThreads = 256, kUploadLanes = 8, kUploadSteps = 8;
-__global__ void __launch_bounds__(kUploadThreads) upload_kernel(const UploadEdge* __restrict__ edge, int64_t n, int4* child,
-                                                                const int32_t* __restrict__ src, int32_t* dst) {
+__global__ void __launch_bounds__(kUploadThreads) upload_kernel(const UploadEdge* __restrict__ edge, int64_t n,
+                                                                int4* child, const int32_t* __restrict__ src,
+                                                                int32_t* dst) {
   const int sub = threadIdx.x % kUploadLanes;
   const int64_t step = (int64_t)gridDim.x * (kUploadThreads / kUploadLanes);
   for (int64_t i = ((int64_t)blockIdx.x * kUploadThreads + threadIdx.x) / kUploadLanes; i < n; i += step) {
@@ -1822,7 +1822,8 @@ cudaError_t launch_init_ranges(TreeState* d_states, int32_t nt, const int64_t* p
 
 cudaError_t launch_upload(const UploadEdge* edge, int64_t n, int4* child, const int32_t* src, int32_t* dst, int num_sms,
                           cudaStream_t st) {
-  const int64_t per = kUploadThreads / kUploadLanes, ctas = std::min<int64_t>((n + per - 1) / per, (int64_t)num_sms * 8);
+  const int64_t per = kUploadThreads / kUploadLanes;
+  const int64_t ctas = std::min<int64_t>((n + per - 1) / per, (int64_t)num_sms * 8);
   P2P_TIMED(K_UPLOAD, st, (upload_kernel<<<(int)ctas, kUploadThreads, 0, st>>>(edge, n, child, src, dst)));
   return cudaGetLastError();
 }

@@ -24,13 +24,6 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kGroupThreads = 256;
 
-// SplitMix64 output function (Steele, Lea & Flood 2014; constants published by Vigna).
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  return z ^ (z >> 31);
-}
-
 __device__ __forceinline__ bool request_range(const int64_t* offsets, int64_t b, int64_t tok_base, int64_t n_tokens,
                                               int64_t& start, int64_t& len) {
   start = offsets[b] - tok_base;
@@ -40,10 +33,10 @@ __device__ __forceinline__ bool request_range(const int64_t* offsets, int64_t b,
 }
 
 // One warp per `per` consecutive requests (lane i < per owns request base + i).  Eight lanes hash a request: four
-// requests a step and two steps in flight, each lane eight tokens of each (token 8 j + s by lane s), mixed with
-// their positions and summed.  (A request at a time by the whole warp, 32 in series, took 31 us for 65,536
-// requests and 30 for 8,191; now 17 and 9.)  Then every distinct key of the warp is looked up or claimed once, by its lowest lane, which also
-// lowers the key's leader index to that lane's request (the smallest of the warp's requests with the key).
+// requests a step and two steps in flight, each lane eight tokens of each (token 8 j + s by lane s), mixed with their
+// positions and summed.  (A request at a time by the whole warp, 32 in series, took 31 us for 65,536 requests and 30
+// for 8,191; now 17 and 9.)  Then every distinct key of the warp is looked up or claimed once, by its lowest lane,
+// which also lowers the key's leader index to that lane's request (the smallest of the warp's requests with the key).
 __global__ void __launch_bounds__(kGroupThreads) group_hash_kernel(
     const int32_t* __restrict__ tokens, int64_t n_tokens, int64_t tok_base, const int64_t* __restrict__ offsets,
     int64_t B, int32_t per, unsigned long long* keys, int32_t* vals, int32_t bits, int32_t* slot_of) {
@@ -139,14 +132,14 @@ __device__ int64_t lcp_warp(const int32_t* __restrict__ a, const int32_t* __rest
   return n;
 }
 
-// One warp per `per` consecutive requests (lane i < per owns request base + i): each request's leader; for each follower
-// in turn, the exact common prefix with its leader (the whole warp compares); then the warp's leaders are
+// One warp per `per` consecutive requests (lane i < per owns request base + i): each request's leader; for each
+// follower in turn, the exact common prefix with its leader (the whole warp compares); then the warp's leaders are
 // appended to lists[0 ..) with one counter update, and so are its followers to lists[B ..) if `place` is set; if not,
 // each follower takes its rank in its group (fcnt[leader] counts them; the rank goes to slot_of[b]) and
 // group_ranges_kernel and group_place_kernel make the list.  A leader with followers gets the smallest of their common
 // prefixes in cmin and, while rows last, a checkpoint row in gid (one update per distinct leader of the warp's
-// followers).  U: 24 for long requests, whose longest compares bound the kernel (8,191 of 11,400 tokens 65 us; 16: 70, 32:
-// 75), else 8 and more resident warps (200,003 of 1,250 tokens 142 us; 16: 148) -- but 16 beside a delta, whose
+// followers).  U: 24 for long requests, whose longest compares bound the kernel (8,191 of 11,400 tokens 65 us; 16: 70,
+// 32: 75), else 8 and more resident warps (200,003 of 1,250 tokens 142 us; 16: 148) -- but 16 beside a delta, whose
 // kernels leave room for few warps (262,144 requests 0.43 ms; 8: 0.53).
 template <int U>
 __global__ void __launch_bounds__(kGroupThreads) group_resolve_kernel(

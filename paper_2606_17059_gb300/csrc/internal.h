@@ -144,7 +144,7 @@ struct GroupScratch {
   unsigned long long* keys;  // 2^bits slots
   int32_t* fcnt;     // [B]: a leader's follower count, then the start of its followers' range
   int32_t* counts;   // [8]: leaders, followers, groups with a checkpoint row, the leader pass's work cursor,
-                     //      the follower ranges handed out, (unused), the followers left to the lane kernel
+                     //      the follower ranges handed out, the followers left to the lane kernel
   size_t n_zero;
   // Set to 0x7f bytes (larger than any index or prefix), in one piece from vals on (n_large bytes):
   int32_t* vals;     // 2^bits slots
@@ -176,10 +176,10 @@ cudaError_t launch_decide(const int32_t* match, int64_t B, int32_t P, const int3
                           int32_t* out_peer, int32_t* out_next, int num_sms, cudaStream_t st);
 // Whether a batch is routed without grouping: every request is walked as a leader (route_kernel.cu has the rule).
 bool route_ungrouped(int64_t B, int32_t P, int64_t n_tokens, int num_sms);
-// Route kernels (lookup + route decision) of a grouped batch, see route_kernel.cu: a leader pass and a
-// follower pass; with g = NULL the batch is not grouped and the leader pass takes every request.  *launched is set to the number of kernels launched.  With decide (load
-// words carrying kLoadExcluded) or out_next (device [B]) the passes make the decision with excluded trees
-// and the next-best target instead of the plain argmax.
+// Route kernels (lookup + route decision) of a grouped batch, see route_kernel.cu: a leader pass and a follower pass;
+// with g = NULL the batch is not grouped and the leader pass takes every request.  *launched is set to the number of
+// kernels launched.  With decide (load words carrying kLoadExcluded) or out_next (device [B]) the passes make the
+// decision with excluded trees and the next-best target instead of the plain argmax.
 cudaError_t launch_route(const TreeView* d_trees, int32_t P, const int32_t* tokens, int64_t n_tokens,
                          int64_t tok_base, const int64_t* offsets, int64_t B, const int32_t* d_load, int32_t alpha,
                          int32_t* out_match, int32_t* out_peer, int32_t* d_err, const GroupScratch* g, int num_sms,
@@ -288,10 +288,20 @@ __device__ __forceinline__ void load_slots(const int4* p, int4& a, int4& b) {
       : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
       : "l"(p));
 }
+
+// SplitMix64 output function (Steele, Lea & Flood 2014; constants published by Vigna).
+__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  return z ^ (z >> 31);
+}
+
+// A barrier of all threads of the cluster, which also orders their memory accesses.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 #endif
 
-// Writes a tree's state and view on the device (values passed as kernel parameters, so no host buffer
-// has to outlive the call).
 // An edge of a tree being uploaded.
 struct UploadEdge {
   int4 slot;  // its slot: first token, node, label offset (< 0: in the shared pool), label length
@@ -300,6 +310,8 @@ struct UploadEdge {
 // Puts n edges into their tables (zeroed) and moves the own labels from src (null: they are there already) to dst.
 cudaError_t launch_upload(const UploadEdge* edge, int64_t n, int4* child, const int32_t* src, int32_t* dst, int num_sms,
                           cudaStream_t st);
+// Writes a tree's state and view on the device (values passed as kernel parameters, so no host buffer
+// has to outlive the call).
 cudaError_t launch_set_tree(TreeState* d_state, TreeView* d_view, TreeState value, const int32_t* shared,
                             cudaStream_t st);
 
@@ -344,7 +356,8 @@ cudaError_t launch_lru_stamp(const TreeState& s, TreeState* d_state, const int32
 struct LruScratch {
   int32_t *cnt, *big_cnt;     // [N + 2]: nodes found for a level, and its nodes with large tables
   unsigned long long* hist;   // [4 * 256]
-  unsigned long long* out;    // [8]: tokens of the tree, 1 if it is inconsistent, depth, cut level, cut, largest stamp, largest ~stamp
+  unsigned long long* out;    // [8]: tokens of the tree, 1 if it is inconsistent, depth, cut level, cut, largest stamp,
+                              //      largest ~stamp
   size_t zeroed;
   unsigned long long* sum;    // [N], by node: tokens of the threshold's stamp in its subtree
   int32_t *order, *parent, *cslot, *len;  // [N], by position in breadth-first order

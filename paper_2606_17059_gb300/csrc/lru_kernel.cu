@@ -20,10 +20,10 @@
 // So n tokens are removed at once: the nodes whose key is below a threshold, and the tail of the one node at it.
 //
 // The threshold needs no sort and no rank of the nodes.  Its stamp S comes from a radix selection over the stamps,
-// weighted by edge lengths; the r tokens left over are the first r of stamp S in the order of (end, deeper first), found
-// by walking down from the root.  At a node u, `carry` is the length of the edges above (u's included) whose end
-// lies in u's subtree: they are a run of stamp S down to u, each the largest same-stamp child of the one before.
-// A child c then stands for T(c) tokens, the edge lengths of stamp S in its subtree, and for carry too if it is u's
+// weighted by edge lengths; the r tokens left over are the first r of stamp S in the order of (end, deeper first),
+// found by walking down from the root.  At a node u, `carry` is the length of the edges above (u's included) whose end
+// lies in u's subtree: they are a run of stamp S down to u, each the largest same-stamp child of the one before. A
+// child c then stands for T(c) tokens, the edge lengths of stamp S in its subtree, and for carry too if it is u's
 // largest same-stamp child; the children are taken in token order, and the walk goes on in the one that holds token r.
 // At a u of stamp S without a same-stamp child the carried edges end: the r tokens are taken from the deepest up.  A
 // node of stamp S is removed if it precedes the walked path x in preorder or is one of those whole edges: one that
@@ -199,9 +199,6 @@ constexpr int kLaneBits = 4;    // tables of up to 16 slots are read by one lane
 constexpr int kWarpBits = 8;    // up to 256 slots by one warp, larger ones by the whole cluster
 constexpr int kStBefore = 0, kStAfter = 1, kStOnPath = 2, kStGone = 4;
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -455,8 +452,8 @@ __global__ void __launch_bounds__(kEvictThreads, 1) lru_evict_kernel(LruTree t, 
         const int32_t size = tab_bits(nd.y) ? 1 << tab_bits(nd.y) : 0;
         const bool same = u != 0 && t.stamp[u] == cut_stamp;
         if (same) carry += (unsigned long long)len_u;
-        // The children's keys and weights, kept by the threads for a table of up to kHeld slots a thread, and read again
-        // by each step for a larger one.
+        // The children's keys and weights, kept by the threads for a table of up to kHeld slots a thread, and read
+        // again by each step for a larger one.
         const bool held = size <= kHeld * kEvictThreads;
         uint32_t kx[kHeld] = {};
         unsigned long long kw[kHeld] = {};
@@ -494,7 +491,8 @@ __global__ void __launch_bounds__(kEvictThreads, 1) lru_evict_kernel(LruTree t, 
               if (c * kEvictThreads < size) f(kx[c], kw[c]);
           } else {
             for (int32_t j0 = 0; j0 < size; j0 += kEvictThreads) {
-              const int4 e = t.child[nd.x + j0 + (int32_t)threadIdx.x];  // (a table this large is a multiple of the CTA)
+              // (A table this large is a multiple of the CTA.)
+              const int4 e = t.child[nd.x + j0 + (int32_t)threadIdx.x];
               const uint32_t x = (uint32_t)e.x ^ 0x80000000u;
               const unsigned long long w = e.y >= 1 ? __ldcg(s.sum + e.y) : 0ull;
               f(x, w && same && x == best_key ? w + carry : w);
@@ -729,7 +727,8 @@ cudaError_t launch_lru_evict(const TreeState& tree, TreeState* d_state, const Lr
     attr[0].val.clusterDim.x = 8;  // the portable size
     cfg.gridDim = dim3(8);
   }
-  P2P_TIMED(K_LRU_EVICT, st, (e = cudaLaunchKernelEx(&cfg, lru_evict_kernel, lru_tree(tree, nullptr), d_state, s, N, want)));
+  P2P_TIMED(K_LRU_EVICT, st,
+            (e = cudaLaunchKernelEx(&cfg, lru_evict_kernel, lru_tree(tree, nullptr), d_state, s, N, want)));
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 

@@ -364,9 +364,9 @@ struct LaneAcc<true> {
   }
 };
 
-// Routes the leaders list[0 .. *count) of a grouped batch, or (kGrouped = false) all B requests, with full walks.  kDecide: the decision with
-// excluded trees and the next-best target (RouteAcc<true>), made by the request's last warp from its match
-// row once every item of the request has written its part.
+// Routes the leaders list[0 .. *count) of a grouped batch, or (kGrouped = false) all B requests, with full walks.
+// kDecide: the decision with excluded trees and the next-best target (RouteAcc<true>), made by the request's last warp
+// from its match row once every item of the request has written its part.
 template <bool kDecide, bool kGrouped>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) route_kernel(
     const TreeView* __restrict__ trees, int32_t P, const int32_t* __restrict__ tokens, int64_t n_tokens,
@@ -588,10 +588,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) route_kernel(
 constexpr int kFollowThreads = 256;
 constexpr int kFollowCtasPerSm = 4;
 constexpr int kThreadSpan = 64;
-// Long requests' followers spend their time in compares of thousands of tokens by the warp, a round trip per step: 1,024
-// tokens a step and 16 warps on a SM (eight loads and 32 warps: the follower pass of 8,191 requests of 11,400 tokens
-// on 32 trees 150 us, 16 and 32: 96, 32 and 24: 68, 32 and 16: 59).  The others compare little: leaders of
-// short requests with 16 loads instead of eight took 579 us instead of 467 (a step's 262,144 on 256 trees).
+// Long requests' followers spend their time in compares of thousands of tokens by the warp, a round trip per step:
+// 1,024 tokens a step and 16 warps on a SM (eight loads and 32 warps: the follower pass of 8,191 requests of 11,400
+// tokens on 32 trees 150 us, 16 and 32: 96, 32 and 24: 68, 32 and 16: 59).  The others compare little: leaders of short
+// requests with 16 loads instead of eight took 579 us instead of 467 (a step's 262,144 on 256 trees).
 template <bool kLeader, int kFirst>
 constexpr int kLaneUnroll = !kLeader && kFirst == 8 ? 32 : 8;
 template <bool kLeader, int kFirst>
@@ -864,9 +864,9 @@ __global__ void __launch_bounds__(kFollowThreads, kLaneCtas<kLeader, kFirst>) la
 // In each tree a follower whose leader matched less than their common prefix has the leader's match; the others resume
 // at the leader's checkpoint with one lookup of the follower's token there, mostly in vain.  What bounds this over
 // many trees:
-//   - Address translation.  An SM keeps few translations at hand (random loads of this GPU: 273 G/s over 16 regions 32 MB
-//     apart, 37 G/s over 32 or more, whether they hit L2 or not), and a load whose 32 lanes lie in 32 trees needs 32 of
-//     them: with a lane per tree the lookups of 205,000 followers in 26 million tables took 0.7 ms whatever the
+//   - Address translation.  An SM keeps few translations at hand (random loads of this GPU: 273 G/s over 16 regions
+//     32 MB apart, 37 G/s over 32 or more, whether they hit L2 or not), and a load whose 32 lanes lie in 32 trees needs
+//     32 of them: with a lane per tree the lookups of 205,000 followers in 26 million tables took 0.7 ms whatever the
 //     tables' size.  The lanes here are followers, side by side for a leader, and look into one tree, mostly one table.
 //   - Loads in flight.  A lookup that its first load does not answer, and the walk behind a token that is there, take
 //     several round trips, and in almost every step some lane of the warp has one.  They are queued, and full warps of
@@ -877,11 +877,11 @@ __global__ void __launch_bounds__(kFollowThreads, kLaneCtas<kLeader, kFirst>) la
 // tokens are there in most trees.  A lane keeps its follower's decision in registers.
 //
 // Measured against lane_kernel<false> (us): 205,000 followers on 256 trees 725 -> 435, 160,000 on 64 trees 155 -> 117,
-// 52,000 on 16 trees 34 -> 28; conversations cached in one tree each behind one of 64 prompts: 200,000 of 300 tokens on 16
-// trees 272 -> 192, of 100 on 64 trees 361 -> 193, 100,000 of 600 on 64 trees 221 -> 179.  Where every tree holds every
-// follower's next 70 tokens: 200,000 on 64 trees 1,439 -> 1,573 (2,500 with none left to lane_kernel before its trees are
-// through), on 16 trees 456 -> 557.  Two trees a lane and three CTAs a SM: one or four trees 824 and 785 us, two, four and
-// five CTAs 865, 721 and 817 where these took 697 (more loads in flight are more translations).
+// 52,000 on 16 trees 34 -> 28; conversations cached in one tree each behind one of 64 prompts: 200,000 of 300 tokens on
+// 16 trees 272 -> 192, of 100 on 64 trees 361 -> 193, 100,000 of 600 on 64 trees 221 -> 179.  Where every tree holds
+// every follower's next 70 tokens: 200,000 on 64 trees 1,439 -> 1,573 (2,500 with none left to lane_kernel before its
+// trees are through), on 16 trees 456 -> 557.  Two trees a lane and three CTAs a SM: one or four trees 824 and 785 us,
+// two, four and five CTAs 865, 721 and 817 where these took 697 (more loads in flight are more translations).
 constexpr int kRowWarps = 8;
 constexpr int kRowCtasPerSm = 3;
 constexpr int kRowIlp = 2;   // trees a lane looks up at a time
@@ -890,10 +890,11 @@ constexpr int kOwn = 8;      // tokens of an edge that a lane compares (16: the 
 constexpr int kFar = 128;    // ... and that the warp compares in one round trip
 constexpr int kFarLanes = 8;  // far compares of a warp at a time
 constexpr int kMinHits = 4;
-// Followers of a full wave of lanes.  With fewer the warps that there are walk tree after tree while the GPU idles, where
-// lane_kernel has a warp for each follower (a route of 8,192 requests on 256 trees 437 us, 227 by lane_kernel; of 65,536
-// 579 and 539, of 90,000 650 and 665; on 64 trees 65,536 214 and 214, 90,000 243 and 257; on 32 trees 48,000 159 and 149,
-// 100,000 224 and 238).  A single tile of trees is walked soon (48,000 on 16 trees 137 and 138, on 4 130 and 135).
+// Followers of a full wave of lanes.  With fewer the warps that there are walk tree after tree while the GPU idles,
+// where lane_kernel has a warp for each follower (a route of 8,192 requests on 256 trees 437 us, 227 by lane_kernel; of
+// 65,536 579 and 539, of 90,000 650 and 665; on 64 trees 65,536 214 and 214, 90,000 243 and 257; on 32 trees 48,000 159
+// and 149, 100,000 224 and 238).  A single tile of trees is walked soon (48,000 on 16 trees 137 and 138, on 4 130 and
+// 135).
 inline int64_t follow_line(int32_t P, int num_sms) {
   const int64_t lanes = (int64_t)num_sms * kRowCtasPerSm * kRowWarps * 32;
   return P <= kTile ? lanes / 2 : lanes * 3 / 4;
@@ -991,7 +992,8 @@ __global__ void __launch_bounds__(kRowWarps * 32, kRowCtasPerSm) follow_kernel(
             todo += __popc(hm);
           }
           while (todo >= 32 || (todo > 0 && h + kRowIlp >= kTile)) {
-            slow |= __ballot_sync(kFull, hits >= kMinHits && 2 * hits > p0 + h + kRowIlp + 2 && 2 * (p0 + h + kRowIlp) <= P);
+            const int32_t seen = p0 + h + kRowIlp;
+            slow |= __ballot_sync(kFull, hits >= kMinHits && 2 * hits > seen + 2 && 2 * seen <= P);
             __syncwarp();
             const int first = max(todo - 32, 0);
             bool go = first + lane < todo;
@@ -1254,7 +1256,7 @@ cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tok
     const auto kernel = g ? lane_kernel<true, kDecide, 8, true> : lane_kernel<true, kDecide, 8, false>;
     // A small ungrouped batch is spread over all SMs, where a warp shares loads and translations with few others (33
     // requests of 4,000 tokens that 256 trees hold a copy each of: 1,177 us by CTAs of eight warps, 1,088 so).
-    const int warps = g ? kFollowThreads / 32 : (int)std::min<int64_t>(kFollowThreads / 32, (B + num_sms - 1) / num_sms);
+    const int most = kFollowThreads / 32, warps = g ? most : (int)std::min<int64_t>(most, (B + num_sms - 1) / num_sms);
     const int grid1 = g ? grid2 : (int)std::min<int64_t>((B + warps - 1) / warps, (int64_t)num_sms * kFollowCtasPerSm);
     P2P_TIMED(K_LANE_LEADER, st,
               (kernel<<<grid1, warps * 32, 0, st>>>(
@@ -1276,13 +1278,14 @@ cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tok
     const size_t smem = sizeof(RowWarp) * kRowWarps;
     e = cudaFuncSetAttribute(follow_kernel<kDecide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    const int grid_row = (int)std::min<int64_t>((B + 31) / 32, (int64_t)num_sms * kRowCtasPerSm);
     P2P_TIMED(K_FOLLOW, st,
-              (follow_kernel<kDecide><<<(int)std::min<int64_t>((B + 31) / 32, num_sms * kRowCtasPerSm), kRowWarps * 32, smem, st>>>(
+              (follow_kernel<kDecide><<<grid_row, kRowWarps * 32, smem, st>>>(
                   d_trees, P, tokens, tok_base, offsets, g->lists + B, g->counts + 1, g->lead, g->cpre, g->gid, g->ckpt,
-                  d_load, alpha, out_match, out_peer, d_err, out_next, g->slot_of, g->counts + 6)));
+                  d_load, alpha, out_match, out_peer, d_err, out_next, g->slot_of, g->counts + 5)));
     P2P_TIMED(K_LANE_FOLLOWER, st,
               (lane_kernel<false, kDecide, 16><<<grid2, kFollowThreads, 0, st>>>(
-                  d_trees, P, tokens, n_tokens, tok_base, offsets, B, g->slot_of, g->counts + 6, g->lead, g->cpre,
+                  d_trees, P, tokens, n_tokens, tok_base, offsets, B, g->slot_of, g->counts + 5, g->lead, g->cpre,
                   g->gid, nullptr, g->ckpt, d_load, alpha, out_match, out_peer, d_err, nullptr, out_next)));
     *launched += 1;
   } else {
@@ -1297,19 +1300,18 @@ cudaError_t launch_passes(const TreeView* d_trees, int32_t P, const int32_t* tok
 
 }  // namespace
 
-// A batch of no more requests than the leader pass has warps is not grouped: its walks all run at once, so the pass takes
-// about as long as its longest walk whether or not the followers are among them, and the grouping and the follower pass
-// would only come on top.  Measured (us a call, grouped -> ungrouped): 33 requests on 4 trees 46 -> 25, 1,200 on 16
-// trees 54 -> 26, 4,864 on 64 trees 68 -> 35, on 256 trees 166 -> 112; where every tree holds a copy of its own of each
-// prompt, 4,864 of 200 tokens on 256 trees 320 -> 319, of 1,000 490 -> 577, 33 to 300 of 4,000 1,088 -> 1,104, 2,400 1,119
-// -> 1,233.
-// Long requests are walked by a CTA each, several warps to a request, and a walk reads thousands of tokens in every tree
-// that holds the prompt, where the grouping compares a follower with its leader once: one a SM, on few trees a few.
-// 20,000 tokens that all trees hold, 8 trees, 608 requests 71 -> 51, 1,000 74 -> 91; 32 trees, 304 requests 89 -> 80, 608
-// 92 -> 142; 128 trees, 152 requests 209 -> 171, 304 215 -> 261; 512 trees, 152 requests 649 -> 607, 304 644 -> 960.
-// Prompts left half-way on 256 trees, 152 requests 327 -> 254.
-// A batch on few trees gains too, but stays grouped past 300 requests for each tree after the first (all of a single
-// tree): that leaves the launches of such batches, which tests count, as they were.
+// A batch of no more requests than the leader pass has warps is not grouped: its walks all run at once, so the pass
+// takes about as long as its longest walk whether or not the followers are among them, and the grouping and the
+// follower pass would only come on top.  Measured (us a call, grouped -> ungrouped): 33 requests on 4 trees 46 -> 25,
+// 1,200 on 16 trees 54 -> 26, 4,864 on 64 trees 68 -> 35, on 256 trees 166 -> 112; where every tree holds a copy of its
+// own of each prompt, 4,864 of 200 tokens on 256 trees 320 -> 319, of 1,000 490 -> 577, 33 to 300 of 4,000 1,088 ->
+// 1,104, 2,400 1,119 -> 1,233. Long requests are walked by a CTA each, several warps to a request, and a walk reads
+// thousands of tokens in every tree that holds the prompt, where the grouping compares a follower with its leader once:
+// one a SM, on few trees a few. 20,000 tokens that all trees hold, 8 trees, 608 requests 71 -> 51, 1,000 74 -> 91; 32
+// trees, 304 requests 89 -> 80, 608 92 -> 142; 128 trees, 152 requests 209 -> 171, 304 215 -> 261; 512 trees, 152
+// requests 649 -> 607, 304 644 -> 960. Prompts left half-way on 256 trees, 152 requests 327 -> 254. A batch on few
+// trees gains too, but stays grouped past 300 requests for each tree after the first (all of a single tree): that
+// leaves the launches of such batches, which tests count, as they were.
 bool route_ungrouped(int64_t B, int32_t P, int64_t n_tokens, int num_sms) {
   const int64_t most = long_requests(B, n_tokens) ? (int64_t)num_sms * (P <= 8 ? 4 : P <= 32 ? 2 : 1)
                                                   : (int64_t)num_sms * kFollowCtasPerSm * (kFollowThreads / 32);

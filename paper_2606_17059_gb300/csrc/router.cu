@@ -56,7 +56,8 @@ constexpr int32_t kHeadTokens = 64;
 constexpr size_t kHeadCandidates = 8;
 
 // 64-bit content hash of a token run: two tokens a step in four independent chains of multiplications (one chain waits
-// for the multiplier at every token), then a final avalanche.  Interning always verifies the content, so a collision
+// for the multiplier at every token) by 2^64 over the golden ratio (Knuth's multiplicative hashing), then a final
+// avalanche with a multiplier of MurmurHash3's 64-bit finalizer (Appleby, public domain).  Interning always verifies the content, so a collision
 // only means a run is not shared.
 uint64_t run_hash(const int32_t* p, int64_t n) {
   constexpr uint64_t kMul = 0x9e3779b97f4a7c15ull;
@@ -298,7 +299,8 @@ int cuda_fail(p2p_router* r, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(r, e_, #call); \
   } while (0)
 
-// (Without memory, the call may go on some other way: the runtime's last error is not left for its next launch to find.)
+// (Without memory, the call may go on some other way: the runtime's last error is not left for its next launch to
+// find.)
 cudaError_t dalloc(p2p_router* r, void** p, size_t bytes) {
   const cudaError_t e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, r->pool, r->stream);
   if (e != cudaSuccess) (void)cudaGetLastError();
@@ -320,9 +322,10 @@ cudaError_t ensure(p2p_router* r, DevBuf& b, size_t bytes) {
   return e;
 }
 
-// Scratch of the shared-prefix grouping for a batch of B requests (B <= 2^30): a key table of at least 2B
-// slots with fcnt (B) and eight counts behind the keys, gid and cmin (B each) behind the values; slot_of, lead and
-// cpre (B each) and the two request lists (2B); and checkpoint rows, as many as fit in 256 MB (and at most B/2 + 1, one per leader with followers).
+// Scratch of the shared-prefix grouping for a batch of B requests (B <= 2^30): a key table of at least 2B slots with
+// fcnt (B) and eight counts behind the keys, gid and cmin (B each) behind the values; slot_of, lead and cpre (B each)
+// and the two request lists (2B); and checkpoint rows, as many as fit in 256 MB (and at most B/2 + 1, one per leader
+// with followers).
 cudaError_t group_scratch(p2p_router* r, int64_t B, p2p::GroupScratch& g) {
   const int64_t slots = std::max<int64_t>(next_pow2(2 * B), 1024);
   const int64_t gcap = std::max<int64_t>(1, std::min<int64_t>(B / 2 + 1, ((int64_t)256 << 20) / ((int64_t)r->P * 16)));
@@ -350,10 +353,9 @@ cudaError_t group_scratch(p2p_router* r, int64_t B, p2p::GroupScratch& g) {
   return cudaSuccess;
 }
 
-// Groups the batch by shared prefix (unless it is small) and routes it (leaders, then followers).  The callers check B <= kMaxBatch
-// (request indices and list positions are 32-bit).
-// With decide (an excluded-peer mask staged with the load) or out_next, the passes make the decision with
-// excluded trees and the next-best target.
+// Groups the batch by shared prefix (unless it is small) and routes it (leaders, then followers).  The callers check B
+// <= kMaxBatch (request indices and list positions are 32-bit). With decide (an excluded-peer mask staged with the
+// load) or out_next, the passes make the decision with excluded trees and the next-best target.
 int route(p2p_router* r, const int32_t* tokens, int64_t n_tokens, int64_t tok_base, const int64_t* offsets, int64_t B,
           int32_t alpha, int32_t* out_match, int32_t* out_peer, bool decide = false, int32_t* out_next = nullptr) {
   const auto& pr = r->prep;
@@ -510,7 +512,8 @@ int do_sync(p2p_router* r) {
 int push_states(p2p_router* r, int32_t p0, int32_t p1);
 
 // Makes the device shared pool hold all of the host mirror's tokens (also those of an upload that failed before it got
-// here): grows it (stream-ordered copy) if needed, in which case every tree's view is refreshed with the new pool address.
+// here): grows it (stream-ordered copy) if needed, in which case every tree's view is refreshed with the new pool
+// address.
 int sync_shared_pool(p2p_router* r) {
   const int64_t n = (int64_t)r->h_shared.size(), from = r->shared_synced;
   if (n == from) return P2P_OK;
@@ -679,8 +682,8 @@ int upload_flat(p2p_router* r, int32_t peer, const p2p_flat_tree* t) {
   }
   CK(cudaMemcpyAsync(nt.node, node.data(), (size_t)NN * sizeof(int4), cudaMemcpyHostToDevice, r->stream));
   if (slots) CK(cudaMemsetAsync(nt.child, 0, (size_t)slots * sizeof(int4), r->stream));
-  // The snapshot's labels go as they are to the spare's label arena, which is free until a compaction, and upload_kernel
-  // moves the own ones from there; without that room they are put together here.
+  // The snapshot's labels go as they are to the spare's label arena, which is free until a compaction, and
+  // upload_kernel moves the own ones from there; without that room they are put together here.
   const bool staged = n_own > 0 && sp.label && NL <= sp.cap_label;
   std::vector<int32_t> own;
   if (staged) {
@@ -1270,11 +1273,11 @@ int p2p_tree_apply_delta(p2p_router* r, int32_t peer, const p2p_delta* d, int64_
 // routed mostly to one tree and inserted with p2p_update_estimates, for one).  n_blocks = nt and
 // d_parts = NULL when no tree is split.
 constexpr int64_t kPartOps = 16384;
-// Deltas that the delta kernel takes alone: its CTA of a tree has 16 ops in work at a time, and the rounds' nine launches
-// take 28 us whatever the ops.  A call of 1, 4, 8, 16, 64 ops on one tree, alone and with the rounds: 96, 95, 122, 141,
-// 223 us and 123, 125, 126, 133, 131; of 1, 8, 12, 16 ops on each of 256 trees 98, 134, 154, 166 and 141, 165, 167, 170.
-// With more trees than the SMs hold CTAs of that kernel they wait for one another: 1, 2, 4 ops on each of 1,024 trees 173,
-// 190, 246 and 176, 177, 207.
+// Deltas that the delta kernel takes alone: its CTA of a tree has 16 ops in work at a time, and the rounds' nine
+// launches take 28 us whatever the ops.  A call of 1, 4, 8, 16, 64 ops on one tree, alone and with the rounds: 96, 95,
+// 122, 141, 223 us and 123, 125, 126, 133, 131; of 1, 8, 12, 16 ops on each of 256 trees 98, 134, 154, 166 and 141,
+// 165, 167, 170. With more trees than the SMs hold CTAs of that kernel they wait for one another: 1, 2, 4 ops on each
+// of 1,024 trees 173, 190, 246 and 176, 177, 207.
 constexpr int64_t kAloneOps = 12;
 static bool few_ops(int64_t n, int64_t max_ops, int32_t n_trees, int num_sms) {
   return max_ops <= kAloneOps && (n_trees <= 2 * num_sms || n <= 8 * (int64_t)num_sms);
@@ -1419,8 +1422,8 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
                      reinterpret_cast<int32_t*>(static_cast<unsigned long long*>(r->gmemo.p) + gslots),
                      (uint32_t)(gslots - 1)};
   CK(cudaMemsetAsync(r->gmemo.p, 0, gslots * (sizeof(unsigned long long) + sizeof(int32_t)), r->stream));
-  // Bulk rounds first, where there are ops for them, of at most two pool runs, and the scratch can be had; what they leave
-  // (few ops, as a rule) goes to the delta kernel, whose warps then take smaller slabs.
+  // Bulk rounds first, where there are ops for them, of at most two pool runs, and the scratch can be had; what they
+  // leave (few ops, as a rule) goes to the delta kernel, whose warps then take smaller slabs.
   p2p::BulkArgs bulk = {};
   bool use_bulk = max_runs <= 2 && n <= kBulkMaxOps && !few_ops(n, max_ops, nt, r->num_sms);
   if (use_bulk) {
@@ -1466,7 +1469,8 @@ static int apply_delta_impl(p2p_router* r, int32_t peer, const p2p_delta* d, int
     if (int e = pull_states(r, p0, p1)) return e;
     bool again = false, stopped = false;
     for (int32_t p = p0; p < p1; ++p)
-      stopped = stopped || (r->hs[(size_t)p].status & (p2p::DELTA_NEED_SPACE | p2p::DELTA_NEED_BULK)) == p2p::DELTA_NEED_SPACE;
+      stopped = stopped || (r->hs[(size_t)p].status & (p2p::DELTA_NEED_SPACE | p2p::DELTA_NEED_BULK)) ==
+                               p2p::DELTA_NEED_SPACE;
     // The first stop for room: the room every op not yet applied may take, per tree (room_kernel), so that a
     // tree is grown once for the rest of the call (a delta that brings many new sequences to one tree would
     // otherwise stop at every doubling).  The bound counts INSERTs only; a later stop (a DELETE's fold needs
