@@ -17,7 +17,7 @@ CUDA = os.path.dirname(os.path.dirname(g._build.NVCC)) if os.sep in g._build.NVC
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
     so = str(tmp_path_factory.mktemp("host") / "libhost.so")
-    cmd = ["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-I", os.path.join(CUDA, "include"), "-I", CSRC, "-I",
+    cmd = ["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I", os.path.join(CUDA, "include"), "-I", CSRC, "-I",
            os.path.join(ROOT, "include"), "-o", so, "-x", "c++", os.path.join(CSRC, "router.cu"),
            os.path.join(CSRC, "snapshot.cpp"), os.path.join(ROOT, "tests", "host", "fake_cuda.cpp")]
     r = subprocess.run(cmd, capture_output=True, text=True)
