@@ -576,6 +576,11 @@ int32_t longest_head(const p2p_router* r, const int32_t* src, int32_t len, int32
   return best;
 }
 
+// Largest tree whose tables and own labels the host puts together: upload_kernel takes two launches more and copies an
+// edge's 32 bytes for its slot's 16 (an upload of 100, 200, 300, 400, 1,000 sequences 57, 73, 91, 102, 160 us so and 71,
+// 82, 89, 98, 126 by the kernel; 300 are about 450 nodes).
+constexpr int64_t kHostNodes = 512;
+
 int upload_flat(p2p_router* r, int32_t peer, const p2p_flat_tree* t) {
   std::string err;
   if (!p2p::validate_flat(t, err)) return fail(r, P2P_E_FORMAT, err);
@@ -681,10 +686,20 @@ int upload_flat(p2p_router* r, int32_t peer, const p2p_flat_tree* t) {
     if (alloc_tree_arrays(r, sp, sp_node, sp_child, sp_label) != cudaSuccess) sp = TreeState{};
   }
   CK(cudaMemcpyAsync(nt.node, node.data(), (size_t)NN * sizeof(int4), cudaMemcpyHostToDevice, r->stream));
-  if (slots) CK(cudaMemsetAsync(nt.child, 0, (size_t)slots * sizeof(int4), r->stream));
-  // The snapshot's labels go as they are to the spare's label arena, which is free until a compaction, and
-  // upload_kernel moves the own ones from there; without that room they are put together here.
-  const bool staged = n_own > 0 && sp.label && NL <= sp.cap_label;
+  // A small tree's tables and own labels are put together here, a larger one's by upload_kernel.
+  const bool small = NN <= kHostNodes;
+  std::vector<int4> child;
+  if (small) {
+    child.assign((size_t)slots, make_int4(0, 0, 0, 0));
+    for (const p2p::UploadEdge& E : edge) table_put(child.data() + E.tab.x, E.tab.y, E.slot);
+    if (slots)
+      CK(cudaMemcpyAsync(nt.child, child.data(), child.size() * sizeof(int4), cudaMemcpyHostToDevice, r->stream));
+  } else {
+    CK(cudaMemsetAsync(nt.child, 0, (size_t)slots * sizeof(int4), r->stream));
+  }
+  // Its labels go as they are to the spare's label arena, which is free until a compaction, and the kernel moves the
+  // own ones from there; without that room they are put together here too.
+  const bool staged = !small && n_own > 0 && sp.label && NL <= sp.cap_label;
   std::vector<int32_t> own;
   if (staged) {
     CK(cudaMemcpyAsync(sp.label, t->labels, (size_t)NL * sizeof(int32_t), cudaMemcpyHostToDevice, r->stream));
@@ -694,7 +709,7 @@ int upload_flat(p2p_router* r, int32_t peer, const p2p_flat_tree* t) {
       if (E.slot.z >= 0) std::memcpy(own.data() + E.slot.z, t->labels + E.tab.z, (size_t)E.slot.w * sizeof(int32_t));
     CK(cudaMemcpyAsync(nt.label, own.data(), (size_t)n_own * sizeof(int32_t), cudaMemcpyHostToDevice, r->stream));
   }
-  if (NN > 1) {
+  if (!small) {
     // The edges wait behind the tables: at most a quarter of a table's slots are taken, and the arena has twice them.
     p2p::UploadEdge* d_edge = reinterpret_cast<p2p::UploadEdge*>(nt.child + slots);
     CK(cudaMemcpyAsync(d_edge, edge.data(), edge.size() * sizeof(p2p::UploadEdge), cudaMemcpyHostToDevice, r->stream));

@@ -77,3 +77,23 @@ def test_upload(trees, form):
     gm, gp = route_device(r, tok, off, [0] * len(o), 1)
     om, op, _ = oracle.route(o, tok, off, [0] * len(o), 1)
     assert_same_route(gm, gp, om, op, form)
+
+
+@pytest.mark.parametrize("kids", [1, 510, 511, 512])
+def test_both_sides_of_the_line_between_host_and_device(kids):
+    """Trees of up to 512 nodes are put together on the host, with own, shared and split labels on both sides."""
+    rng = np.random.default_rng(kids)
+    long = rng.integers(0, 30000, size=300).tolist()
+    r = g.Router(2)
+    r.upload(1, _flat([long + [1], long + [2]]))
+    seqs = [[40000 + i] + rng.integers(0, 9, size=rng.integers(0, 140)).tolist() for i in range(kids - 1)] + [long + [3, 3]]
+    flat = _flat(seqs)  # (the last one's label is split where the shared run ends: a node more)
+    r.kernel_clock(True)
+    r.upload(0, flat)
+    assert ("upload_kernel" in r.kernel_times()) == (kids + 2 > 512)
+    assert same_snapshot(r.download(0), flat)
+    o = oracle.build_trees([seqlist_from_lists(seqs), seqlist_from_lists([long + [1], long + [2]])])
+    tok, off = csr_from_lists([s[: len(s) // 2 + 1] + [9] for s in seqs])
+    gm, gp = route_device(r, tok, off, [0, 0], 1)
+    om, op, _ = oracle.route(o, tok, off, [0, 0], 1)
+    assert_same_route(gm, gp, om, op, "line")
